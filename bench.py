@@ -318,6 +318,15 @@ def kernel_models(block):
     }
 
 
+def integer_hop_models(block):
+    """The FP64-accurate hops as they run (kinds 2 and 4 on two-limb integers, hop_x_kernel): bound by HBM, 196 bytes a
+    spinor in limbs, 148 a link, 192 an FP64 spinor."""
+    k = hops_kept(block)
+    return {2: ("hop_x_kernel (FP64 accuracy on integers), whole lattice", "hbm", 196 + 8 * 148 + 194, 1368, "site"),
+            4: ("hop_x_kernel (FP64 accuracy on integers), Dirichlet blocks", "hbm", 196 + 148 * k + 194,
+                48 + FLOPS_PER_HOP * k, "site")}
+
+
 def peaks_alu(stream):
     """FP64/FP32 FMA peaks measured live by the library (derived from unit
     counts and the maximum clock if the probe fails), and where they came from."""
@@ -455,7 +464,7 @@ def run_gpu(args, cfg):
     est = cfg["n_global"] * args.steps * world
     value = job_rate(cfg["n_global"] * args.steps, world, t_max)
     peak, peak_src = peaks()
-    models = kernel_models(cfg["block"])
+    models = {**kernel_models(cfg["block"]), **integer_hop_models(cfg["block"])}
     # persistent block solver: its unit is a block site x inner iteration
     units = {k: timing[k][2] for k in timing}
     units[7] = stats["block_solver"]["site_iterations"]

@@ -52,7 +52,7 @@ struct Reduce {
 
 // One formatted copy of a gauge field.
 struct FieldSlot {
-    double2* eo64;   // eo layout, FP64, 9 chunks, [parity][dir][chunk][Vh]
+    int4* eox;       // eo layout, two-limb integers (LinkX, FP64 accuracy): [parity][dir][9][Vh], then exponents
     float4* eo32;    // eo layout, FP32 rows 0-1, 3 chunks
     uint2* eo16;     // eo layout, FP16 rows 0-1, 3 chunks
     double2* dd64;   // block order, FP64 [blockpos][dir][chunk][bsites]
@@ -68,8 +68,11 @@ struct SolverVecs {
     double2* xe;   // FP64 even solution
     double2* xo;   // FP64 odd solution
     double2* re;   // FP64 residual
-    double2* t64;  // FP64 temporary (odd)
-    double2* t64b; // FP64 temporary (even)
+    int4* tx;      // odd temporary of the FP64 operator (SpinorX: limbs, exponents)
+    int* txe;
+    int4* px;      // SpinorX copy of the operator's input (x, or p of the plain FP64 solver)
+    int* pxe;
+    int* rxe;      // exponents of the SpinorX copies kept in xo (b_o at the start, then r of the plain FP64 solver)
     double2* x64;  // FP64 inner vectors of the plain FP64 solver
     double2* p64;
     double2* q64;
@@ -307,7 +310,7 @@ int block_filter_exact(dd_handle* h, const double* U_old, const double* U_new, i
 inline int grid_for(long long n, int threads) { return (int)((n + threads - 1) / threads); }
 
 // field formatting (lattice.cu)
-int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eo64, bool eo32, bool eo16, bool dd64, bool dd32);
+int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eox, bool eo32, bool eo16, bool dd64, bool dd32);
 // spinor packing between canonical FP64 and eo FP64 (lattice.cu)
 void launch_pack_spinor_eo(dd_handle* h, const double* in, double2* out, int parity, int nrhs, long long in_rhs_stride);
 void launch_unpack_spinor_eo(dd_handle* h, const double2* in, double* out, int parity, int nrhs, long long out_rhs_stride);

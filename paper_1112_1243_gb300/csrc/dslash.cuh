@@ -15,6 +15,7 @@
 
 #include "dd_internal.h"
 #include "reduce.cuh"
+#include "xfix.cuh"
 
 // per-rhs shifted copies of storage descriptors (contiguous per-rhs blocks)
 DD_DEV SpinorF64 at_rhs(SpinorF64 s, int r) {
@@ -49,8 +50,9 @@ struct HopArgs {
     unsigned long long* sites;  // timed launches: output sites processed (may be null)
     // three-value reductions (BiCGStab): 0 off; 1: <rhat, out>; 2: <out, xin> and |out|^2
     int red3 = 0;
-    SX rhat;
+    SX rhat;                    // red3 == 1: the shadow residual; resid: the right-hand side
     SiteSet S = {nullptr, -1};  // output sites (n < 0: all Vh sites of parity p)
+    int resid = 0;              // FP64 hops: out = rhat - (xin + b * hops)
 };
 
 template <class LK>
@@ -189,12 +191,121 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
     }
 }
 
+// FP64 hop on the two-limb integers of xfix.cuh (in: SpinorX, links: LinkX).
+// SOut = SpinorX: out = hops; SOut = SpinorF64: out = (has_x ? xin : 0) + b *
+// hops, or rhat - (xin + b * hops) with resid, and |out|^2 to A.red.
+template <class SX, class SOut, int MASK>
+__global__ void __launch_bounds__(128, 4) hop_x_kernel(HopArgs<SpinorX, SX, SOut, LinkX> A) {
+    __shared__ double sh[34];
+    const int rhs = blockIdx.y;
+    if (A.st && !A.st[rhs].active) return;
+    const Geo& g = A.g;
+    const long long Vh = g.Vh;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (A.sites && threadIdx.x == 0)
+        atomicAdd(A.sites, (unsigned long long)min((long long)blockDim.x, A.S.n - (long long)blockIdx.x * blockDim.x));
+    double nrm = 0.0;
+    if (t < A.S.n) {
+        int x[4];
+        int h;
+        if (A.S.colour >= 0) {
+            h = colour_site(g, A.S.colour, (int)t, A.p, x);
+        } else {
+            h = (int)A.S.at(t);
+            eo_coords(g, A.p, h, x);
+        }
+        const int s = canon_index(g, x);
+        const SpinorX in = at_rhs(A.in, rhs);
+        const int4* lk = A.lk.p + (long long)rhs * A.lk_rhs_stride;
+        const int* le = LinkX{lk, A.lk.stride}.exps();
+        // neighbour d = 2 a (forward) or 2 a + 1 (backward): its index, the
+        // index and parity of the link; false when the hop is dropped
+        auto hop_at = [&](int d, int& yh, long long& lrow) {
+            const int a = d >> 1;
+            const bool fwd = !(d & 1);
+            const int xa = a == 0 ? x[0] : a == 1 ? x[1] : a == 2 ? x[2] : x[3];
+            const int La = g.L[a];
+            const bool edge = xa == (fwd ? La - 1 : 0);
+            const int step = edge ? -(La - 1) * g.st[a] : g.st[a];
+            yh = (fwd ? s + step : s - step) >> 1;
+            lrow = (long long)((fwd ? A.p : 1 - A.p) * 4 + a);
+            if (MASK) {
+                const int loc = xa - fast_div(xa, g.b[a], g.mb[a]) * g.b[a];
+                const bool face = loc == (fwd ? g.b[a] - 1 : 0);
+                if (MASK == 1 ? face : !face) return false;
+            }
+            return true;
+        };
+        int eout = 2 * X_ZERO;
+#pragma unroll 4
+        for (int d = 0; d < 8; ++d) {
+            int yh;
+            long long lrow;
+            if (hop_at(d, yh, lrow)) eout = max(eout, in.e[yh] + le[lrow * Vh + ((d & 1) ? yh : h)]);
+        }
+        xacc acc[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k].x = acc[k].y = 0;
+#pragma unroll 1
+        for (int d = 0; d < 8; ++d) {
+            int yh;
+            long long lrow;
+            if (!hop_at(d, yh, lrow)) continue;
+            const int a = d >> 1;
+            const bool fwd = !(d & 1);
+            const int lh = fwd ? h : yh;
+            const int shift = min(eout - (in.e[yh] + le[lrow * Vh + lh]), 62);
+            const bool flip = a == 3 && g.bc < 0 && x[3] == (fwd ? g.L[3] - 1 : 0);
+            x_hop(a, fwd, A.g5in ? -1 : 0, flip, shift, in, yh, lk + lrow * 9 * Vh + lh, Vh, acc);
+        }
+        if constexpr (std::is_same<SOut, SpinorX>::value) {
+            x_store_acc(at_rhs(A.out, rhs), h, acc, eout);
+        } else {
+            const bool bad = eout >= X_BAD_MIN;
+            double sc = 0.0;
+            const bool one = x_scale(eout, A.b, sc);
+            const bool none = eout <= X_ZERO / 2;
+            auto value = [&](long long v) -> double {
+                if (one) return (double)v;
+                if (bad) return __longlong_as_double(0x7ff8000000000000ll);
+                return none ? 0.0 : scalbn((double)v, eout - 56) * A.b;  // far from the exponents of one multiplier
+            };
+            if (!one) sc = 1.0;
+            const bool zeroed = A.colour_mask != 3 && !((A.colour_mask >> block_colour_of(g, x)) & 1);
+            const double sg = A.g5out ? -sc : sc;
+            Spinor<double> res;
+            if (A.has_x)
+                at_rhs(A.xin, rhs).load(h, res);
+            else
+                zero(res);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {
+                const double f = k < 6 ? sc : sg;
+                res.c[k].x = fma(f, value(acc[k].x), res.c[k].x);
+                res.c[k].y = fma(f, value(acc[k].y), res.c[k].y);
+            }
+            if (A.resid) {
+                Spinor<double> bv;
+                at_rhs(A.rhat, rhs).load(h, bv);
+#pragma unroll
+                for (int k = 0; k < 12; ++k) res.c[k] = bv.c[k] - res.c[k];
+            }
+            if (zeroed) zero(res);
+            at_rhs(A.out, rhs).store(h, res);
+            if (A.red.op != FIN_NONE) nrm = snorm2(res);
+        }
+    }
+    if constexpr (!std::is_same<SOut, SpinorX>::value) {
+        if (A.red.op != FIN_NONE) grid_reduce(A.red, rhs, nrm, sh);
+    }
+}
+
 // timing class of a hop kernel instance (see dd_handle::timer_*), -1: not timed
 template <class SIn, class SOut>
 constexpr int hop_kind() {
     return std::is_same<SIn, SpinorF16>::value && std::is_same<SOut, SpinorF16>::value   ? 0
            : std::is_same<SIn, SpinorF16>::value && std::is_same<SOut, SpinorF32>::value ? 1
-           : std::is_same<SIn, SpinorF64>::value                                          ? 2
+           : std::is_same<SIn, SpinorX>::value                                            ? 2
                                                                                           : -1;
 }
 
@@ -202,13 +313,14 @@ template <class R, class SIn, class SX, class SOut, class LK, int MASK>
 inline void launch_hop(const HopArgs<SIn, SX, SOut, LK>& A, int nrhs, dd_handle* h) {
     HopArgs<SIn, SX, SOut, LK> B = A;
     if (B.S.n < 0) B.S = SiteSet{nullptr, (long long)A.g.Vh};
-    // tile shape from the handle's tuning (threads x sites per thread >= 64,
+    // tile shape from the handle's tuning (threads x sites per thread >= 32,
     // which keeps the grid within the reduction partials)
-    const bool f64 = std::is_same<R, double>::value;
-    const int tpb = std::min(f64 ? h->tune.hop64_tpb : h->tune.hop_tpb, 128);  // the kernels' launch bound
-    // two sites per thread only for the FP32-arithmetic kernels (the FP64
-    // kernel needs 130-150 registers for one site)
-    constexpr int SPT2 = std::is_same<R, double>::value ? 1 : 2;
+    constexpr bool f64 = std::is_same<SIn, SpinorX>::value;
+    int tpb = std::min(f64 ? h->tune.hop64_tpb : h->tune.hop_tpb, 128);  // the kernels' launch bound
+    // one warp per thread block while that leaves SMs without work (the FP64
+    // hop of one site is about 4000 instructions long)
+    if (f64)
+        while (tpb > 32 && (long long)grid_for(B.S.n, tpb) * nrhs < h->num_sms) tpb >>= 1;
     const int spt = (!f64 && h->tune.hop_spt == 2) ? 2 : 1;
     dim3 grid(grid_for(B.S.n, (long long)tpb * spt), nrhs);
     constexpr int kind0 = hop_kind<SIn, SOut>();
@@ -224,12 +336,14 @@ inline void launch_hop(const HopArgs<SIn, SX, SOut, LK>& A, int nrhs, dd_handle*
         if (e) cudaEventRecord(e, h->stream);
         B.sites = h->d_sites + kind;
     }
-    if (A.red3 == 1)
-        DD_KLAUNCH(h, (spt == 2 ? hop_eo_kernel<R, SIn, SX, SOut, LK, MASK, 1, SPT2> : hop_eo_kernel<R, SIn, SX, SOut, LK, MASK, 1, 1>)<<<grid, tpb, 0, h->stream>>>(B));
+    if constexpr (f64) {
+        DD_KLAUNCH(h, hop_x_kernel<SX, SOut, MASK><<<grid, tpb, 0, h->stream>>>(B));
+    } else if (A.red3 == 1)
+        DD_KLAUNCH(h, (spt == 2 ? hop_eo_kernel<R, SIn, SX, SOut, LK, MASK, 1, 2> : hop_eo_kernel<R, SIn, SX, SOut, LK, MASK, 1, 1>)<<<grid, tpb, 0, h->stream>>>(B));
     else if (A.red3 == 2)
-        DD_KLAUNCH(h, (spt == 2 ? hop_eo_kernel<R, SIn, SX, SOut, LK, MASK, 2, SPT2> : hop_eo_kernel<R, SIn, SX, SOut, LK, MASK, 2, 1>)<<<grid, tpb, 0, h->stream>>>(B));
+        DD_KLAUNCH(h, (spt == 2 ? hop_eo_kernel<R, SIn, SX, SOut, LK, MASK, 2, 2> : hop_eo_kernel<R, SIn, SX, SOut, LK, MASK, 2, 1>)<<<grid, tpb, 0, h->stream>>>(B));
     else
-        DD_KLAUNCH(h, (spt == 2 ? hop_eo_kernel<R, SIn, SX, SOut, LK, MASK, 0, SPT2> : hop_eo_kernel<R, SIn, SX, SOut, LK, MASK, 0, 1>)<<<grid, tpb, 0, h->stream>>>(B));
+        DD_KLAUNCH(h, (spt == 2 ? hop_eo_kernel<R, SIn, SX, SOut, LK, MASK, 0, 2> : hop_eo_kernel<R, SIn, SX, SOut, LK, MASK, 0, 1>)<<<grid, tpb, 0, h->stream>>>(B));
     if (timed) {
         cudaEvent_t e = dd_timer_event(h, kind);
         if (e) cudaEventRecord(e, h->stream);

@@ -138,11 +138,8 @@ __global__ void format_gauge_kernel(Geo g, const double* __restrict__ U, FieldSl
     const long long nb = g.bsites;
     for (int a = 0; a < 4; ++a) {
         const double* u = U + ((long long)s * 4 + a) * 18;
-        if (f.eo64) {
-            double2* o = f.eo64 + ((long long)par * 4 + a) * 9 * Vh + h;
-            for (int k = 0; k < 9; ++k) o[k * Vh] = make_double2(u[2 * k], u[2 * k + 1]);
-        }
-        if (f.eo64 && f.eodf) {
+        if (f.eox) x_store_link(f.eox, Vh, par, a, h, u);
+        if (f.eox && f.eodf) {
             float4* o = f.eodf + ((long long)par * 4 + a) * 9 * Vh + h;
             for (int k = 0; k < 9; ++k) {
                 const float rh = (float)u[2 * k], ih = (float)u[2 * k + 1];
@@ -176,9 +173,9 @@ __global__ void format_gauge_kernel(Geo g, const double* __restrict__ U, FieldSl
     }
 }
 
-int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eo64, bool eo32, bool eo16, bool dd64, bool dd32) {
+int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eox, bool eo32, bool eo16, bool dd64, bool dd32) {
     FieldSlot t = f;
-    if (!eo64) t.eo64 = nullptr;
+    if (!eox) t.eox = nullptr;
     if (!eo32) t.eo32 = nullptr;
     if (!eo16) t.eo16 = nullptr;
     if (!dd64) t.dd64 = nullptr;
@@ -342,7 +339,7 @@ void plan(dd_handle* h, char* base) {
     h->fields.assign(R + 1, FieldSlot{});
     for (int k = 0; k <= (est ? R : 0); ++k) {
         FieldSlot& f = h->fields[k];
-        f.eo64 = c.take<double2>((size_t)2 * 4 * 9 * Vh);
+        f.eox = c.take<int4>((size_t)LinkX::field_chunks(Vh));
         f.eo32 = c.take<float4>((size_t)2 * 4 * 3 * Vh);
         f.eo16 = c.take<uint2>((size_t)2 * 4 * 3 * Vh);
         f.eodf = h->prm.outer_prec == DD_PREC_DF64 ? c.take<float4>((size_t)2 * 4 * 9 * Vh) : nullptr;
@@ -366,8 +363,11 @@ void plan(dd_handle* h, char* base) {
     v.xe = c.take<double2>((size_t)R * 12 * Vh);
     v.xo = c.take<double2>((size_t)R * 12 * Vh);
     v.re = c.take<double2>((size_t)R * 12 * Vh);
-    v.t64 = c.take<double2>((size_t)R * 12 * Vh);
-    v.t64b = c.take<double2>((size_t)R * 12 * Vh);
+    v.tx = c.take<int4>((size_t)R * 12 * Vh);
+    v.txe = c.take<int>((size_t)R * Vh);
+    v.px = c.take<int4>((size_t)R * 12 * Vh);
+    v.pxe = c.take<int>((size_t)R * Vh);
+    v.rxe = c.take<int>((size_t)R * Vh);
     v.x64 = c.take<double2>((size_t)R * 12 * Vh);
     v.p64 = c.take<double2>((size_t)R * 12 * Vh);
     v.q64 = c.take<double2>((size_t)R * 12 * Vh);
@@ -788,14 +788,15 @@ extern "C" int dd_finalize(dd_t h) {
 // ------------------------------------------------------ operator application
 namespace {
 
-template <class SS, class LK>
-int apply_eo_ops(dd_handle* h, int op, SS in_e, SS in_o, SS out_e, SS out_o, LK lk, int nrhs, int colour_mask,
-                 int mask_mode) {
+// SH: storage of the hop inputs (in_e, in_o, th), SS: of the results and of
+// the terms that enter without a hop (x_e, x_o); the same for FP32 and FP16
+template <class R, class SH, class SS, class LK>
+int apply_eo_ops(dd_handle* h, int op, SH in_e, SH in_o, SS x_e, SS x_o, SH th, SS out_e, SS out_o, LK lk, int nrhs,
+                 int colour_mask, int mask_mode) {
     const Geo& g = h->g;
     const double k = h->prm.kappa;
-    typedef typename SS::real R;
-    auto mk_args = [&](int p, SS in, SS x, SS out, double a, double b, int hasx, int g5) {
-        HopArgs<SS, SS, SS, LK> A;
+    auto mk_args = [&](int p, SH in, SS x, auto out, double a, double b, int hasx, int g5) {
+        HopArgs<SH, SS, decltype(out), LK> A;
         A.g = g;
         A.p = p;
         A.in = in;
@@ -816,34 +817,34 @@ int apply_eo_ops(dd_handle* h, int op, SS in_e, SS in_o, SS out_e, SS out_o, LK 
     cudaStream_t s = h->stream;
     if (op == DD_OP_D || op == DD_OP_DDAG) {
         int g5 = (op == DD_OP_DDAG);
-        auto A0 = mk_args(0, in_o, in_e, out_e, 1.0, -k, 1, g5);
-        auto A1 = mk_args(1, in_e, in_o, out_o, 1.0, -k, 1, g5);
+        auto A0 = mk_args(0, in_o, x_e, out_e, 1.0, -k, 1, g5);
+        auto A1 = mk_args(1, in_e, x_o, out_o, 1.0, -k, 1, g5);
         if (mask_mode == 1) {
-            launch_hop<R, SS, SS, SS, LK, 1>(A0, nrhs, h);
-            launch_hop<R, SS, SS, SS, LK, 1>(A1, nrhs, h);
+            launch_hop<R, SH, SS, SS, LK, 1>(A0, nrhs, h);
+            launch_hop<R, SH, SS, SS, LK, 1>(A1, nrhs, h);
         } else {
-            launch_hop<R, SS, SS, SS, LK, 0>(A0, nrhs, h);
-            launch_hop<R, SS, SS, SS, LK, 0>(A1, nrhs, h);
+            launch_hop<R, SH, SS, SS, LK, 0>(A0, nrhs, h);
+            launch_hop<R, SH, SS, SS, LK, 0>(A1, nrhs, h);
         }
     } else if (op == DD_OP_INTER) {
-        auto A0 = mk_args(0, in_o, in_e, out_e, 0.0, -k, 0, 0);
-        auto A1 = mk_args(1, in_e, in_o, out_o, 0.0, -k, 0, 0);
-        launch_hop<R, SS, SS, SS, LK, 2>(A0, nrhs, h);
-        launch_hop<R, SS, SS, SS, LK, 2>(A1, nrhs, h);
+        auto A0 = mk_args(0, in_o, x_e, out_e, 0.0, -k, 0, 0);
+        auto A1 = mk_args(1, in_e, x_o, out_o, 0.0, -k, 0, 0);
+        launch_hop<R, SH, SS, SS, LK, 2>(A0, nrhs, h);
+        launch_hop<R, SH, SS, SS, LK, 2>(A1, nrhs, h);
     } else if (op == DD_OP_DTILDE || op == DD_OP_DTILDE_DAG) {
-        // out_o used as the odd temporary: t = H_oe psi_e; out_e = psi_e - k^2 H_eo t
+        // t = H_oe psi_e (odd temporary); out_e = psi_e - k^2 H_eo t
         int g5 = (op == DD_OP_DTILDE_DAG);
-        auto A1 = mk_args(1, in_e, in_e, out_o, 0.0, 1.0, 0, 0);
+        auto A1 = mk_args(1, in_e, x_e, th, 0.0, 1.0, 0, 0);
         A1.g5in = g5;
         A1.g5out = 0;
-        auto A0 = mk_args(0, out_o, in_e, out_e, 1.0, -k * k, 1, 0);
+        auto A0 = mk_args(0, th, x_e, out_e, 1.0, -k * k, 1, 0);
         A0.g5in = 0;
         A0.g5out = g5;
-        launch_hop<R, SS, SS, SS, LK, 0>(A1, nrhs, h);
-        launch_hop<R, SS, SS, SS, LK, 0>(A0, nrhs, h);
+        launch_hop<R, SH, SS, SH, LK, 0>(A1, nrhs, h);
+        launch_hop<R, SH, SS, SS, LK, 0>(A0, nrhs, h);
     } else if (op == DD_OP_HEO) {
-        auto A0 = mk_args(0, in_o, in_e, out_e, 0.0, 1.0, 0, 0);
-        launch_hop<R, SS, SS, SS, LK, 0>(A0, nrhs, h);
+        auto A0 = mk_args(0, in_o, x_e, out_e, 0.0, 1.0, 0, 0);
+        launch_hop<R, SH, SS, SS, LK, 0>(A0, nrhs, h);
     } else {
         return DD_ERR_INVALID_ARG;
     }
@@ -883,14 +884,18 @@ static int apply_common(dd_handle* h, void* out, const void* in, const void* U, 
     dim3 cg(grid_for(Vh, 128), nrhs);
     SpinorF64 be{v.be, Vh}, bo{v.bo, Vh}, xe{v.xe, Vh}, xo{v.xo, Vh};
     if (prec == DD_PREC_F64) {
-        LinkF64 lk{f.eo64, Vh};
-        rc = apply_eo_ops(h, op, be, bo, xe, xo, lk, nrhs, colour_mask, mask_mode);
+        // hop inputs in limbs: even in px, odd in the buffer of re
+        const LinkX lk{f.eox, Vh};
+        const SpinorX ie{v.px, v.pxe, Vh}, io{reinterpret_cast<int4*>(v.re), v.rxe, Vh}, th{v.tx, v.txe, Vh};
+        if (!odd_in) DD_KLAUNCH(h, convert_from64_kernel<<<cg, 128, 0, h->stream>>>(Vh, be, ie));
+        if (!even_in) DD_KLAUNCH(h, convert_from64_kernel<<<cg, 128, 0, h->stream>>>(Vh, bo, io));
+        rc = apply_eo_ops<double>(h, op, ie, io, be, bo, th, xe, xo, lk, nrhs, colour_mask, mask_mode);
     } else if (prec == DD_PREC_F32) {
         SpinorF32 ie{v.r32, Vh}, io{v.t32, Vh}, oe{v.p32, Vh}, oo{v.q32, Vh};
         DD_KLAUNCH(h, convert_from64_kernel<<<cg, 128, 0, h->stream>>>(Vh, be, ie));
         DD_KLAUNCH(h, convert_from64_kernel<<<cg, 128, 0, h->stream>>>(Vh, bo, io));
         LinkF32 lk{f.eo32, Vh};
-        rc = apply_eo_ops(h, op, ie, io, oe, oo, lk, nrhs, colour_mask, mask_mode);
+        rc = apply_eo_ops<float>(h, op, ie, io, ie, io, oo, oe, oo, lk, nrhs, colour_mask, mask_mode);
         DD_KLAUNCH(h, convert_to64_kernel<<<cg, 128, 0, h->stream>>>(Vh, oe, xe));
         DD_KLAUNCH(h, convert_to64_kernel<<<cg, 128, 0, h->stream>>>(Vh, oo, xo));
     } else {
@@ -898,7 +903,7 @@ static int apply_common(dd_handle* h, void* out, const void* in, const void* U, 
         DD_KLAUNCH(h, convert_from64_kernel<<<cg, 128, 0, h->stream>>>(Vh, be, ie));
         DD_KLAUNCH(h, convert_from64_kernel<<<cg, 128, 0, h->stream>>>(Vh, bo, io));
         LinkF16 lk{f.eo16, Vh};
-        rc = apply_eo_ops(h, op, ie, io, oe, oo, lk, nrhs, colour_mask, mask_mode);
+        rc = apply_eo_ops<float>(h, op, ie, io, ie, io, oo, oe, oo, lk, nrhs, colour_mask, mask_mode);
         DD_KLAUNCH(h, convert_to64_kernel<<<cg, 128, 0, h->stream>>>(Vh, oe, xe));
         DD_KLAUNCH(h, convert_to64_kernel<<<cg, 128, 0, h->stream>>>(Vh, oo, xo));
     }

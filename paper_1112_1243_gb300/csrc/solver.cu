@@ -146,9 +146,9 @@ __global__ void outer_arm_kernel(int nrhs, CGState* outer, const double* bb, dou
 }
 
 // x64 += scale * e (any storage; scale = |r_outer| when the inner system was
-// normalised, rr = null: 1), r64 = b - t (with |r|^2), v = 0, copies
+// normalised, rr = null: 1), px = x in limbs for the residual's hop
 template <class SE>
-__global__ void add_correction_kernel(SiteSet S, SpinorF64 x, SE e, const double* rr, const CGState* outer) {
+__global__ void add_correction_kernel(SiteSet S, SpinorF64 x, SpinorX px, SE e, const double* rr, const CGState* outer) {
     const int rhs = blockIdx.y;
     if (outer && !outer[rhs].active) return;
     const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -161,6 +161,7 @@ __global__ void add_correction_kernel(SiteSet S, SpinorF64 x, SE e, const double
 #pragma unroll
     for (int k = 0; k < 12; ++k) a.c[k] = a.c[k] + sc * b.c[k];
     at_rhs(x, rhs).store(i, a);
+    at_rhs(px, rhs).store(i, a);
 }
 // out = in / |in| (|in|^2 given per rhs): the inner solver always sees a
 // unit-norm right-hand side, so FP32 squares neither underflow nor overflow
@@ -181,25 +182,6 @@ __global__ void normalised_copy_kernel(SiteSet S, SpinorF64 in, SOut out, const 
 __global__ void fill_kernel(int n, double* p, double v) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) p[i] = v;
-}
-__global__ void __launch_bounds__(128) residual_kernel(SiteSet S, SpinorF64 b, SpinorF64 t, SpinorF64 r,
-                                                       const CGState* outer, Reduce red) {
-    __shared__ double sh[34];
-    const int rhs = blockIdx.y;
-    if (outer && !outer[rhs].active) return;
-    const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    double nrm = 0.0;
-    if (ti < S.n) {
-        const long long i = S.at(ti);
-        Spinor<double> a, c;
-        at_rhs(b, rhs).load(i, a);
-        at_rhs(t, rhs).load(i, c);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) a.c[k] = a.c[k] - c.c[k];
-        at_rhs(r, rhs).store(i, a);
-        nrm = snorm2(a);
-    }
-    grid_reduce(red, rhs, nrm, sh);
 }
 template <class SV>
 __global__ void __launch_bounds__(128) norm2_kernel(SiteSet S, SV v, Reduce red) {
@@ -226,7 +208,8 @@ __global__ void copy_kernel(SiteSet S, SIn in, SOut out, const CGState* outer) {
     at_rhs(in, rhs).load(i, a);
     at_rhs(out, rhs).store(i, a);
 }
-__global__ void zero64_kernel(SiteSet S, SpinorF64 v) {
+// v = 0, and (pxe given) the exponents of its copy in limbs
+__global__ void zero64_kernel(SiteSet S, SpinorF64 v, int* pxe) {
     const int rhs = blockIdx.y;
     const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (ti >= S.n) return;
@@ -234,6 +217,7 @@ __global__ void zero64_kernel(SiteSet S, SpinorF64 v) {
     Spinor<double> z;
     zero(z);
     at_rhs(v, rhs).store(i, z);
+    if (pxe) pxe[(long long)rhs * v.stride + i] = X_ZERO;
 }
 
 // ------------------------------------------------------------ CGNR runner
@@ -592,8 +576,8 @@ struct BiCGStab {
 template <class LK>
 LK field_links(dd_handle* h, int slot);
 template <>
-LinkF64 field_links<LinkF64>(dd_handle* h, int slot) {
-    return LinkF64{h->fields[slot].eo64, h->g.Vh};
+LinkX field_links<LinkX>(dd_handle* h, int slot) {
+    return LinkX{h->fields[slot].eox, h->g.Vh};
 }
 template <>
 LinkF32 field_links<LinkF32>(dd_handle* h, int slot) {
@@ -621,11 +605,12 @@ Reduce store_reduce(dd_handle* h, double* out) {
     return R_;
 }
 
-// FP64 hop helper on eo FP64 vectors
-template <int MASK>
-void hop64(dd_handle* h, SiteSet S, int nrhs, int par, SpinorF64 in, SpinorF64 xin, SpinorF64 out, double a, double b,
-           int hasx, LinkF64 lk, long long lk_rs, const CGState* st, Reduce red) {
-    HopArgs<SpinorF64, SpinorF64, SpinorF64, LinkF64> A;
+// FP64 hop (in limbs, xfix.cuh): out = (hasx ? xin : 0) + b * hops of in, or
+// bvec - that with resid (SOut SpinorF64), or the hops alone (SOut SpinorX)
+template <int MASK, class SOut>
+void hop64(dd_handle* h, SiteSet S, int nrhs, int par, SpinorX in, SpinorF64 xin, SOut out, double b, int hasx,
+           LinkX lk, long long lk_rs, const CGState* st, Reduce red, const SpinorF64* bvec = nullptr) {
+    HopArgs<SpinorX, SpinorF64, SOut, LinkX> A;
     A.g = h->g;
     A.p = par;
     A.in = in;
@@ -633,7 +618,7 @@ void hop64(dd_handle* h, SiteSet S, int nrhs, int par, SpinorF64 in, SpinorF64 x
     A.out = out;
     A.lk = lk;
     A.lk_rhs_stride = lk_rs;
-    A.a = a;
+    A.a = 1.0;
     A.b = b;
     A.has_x = hasx;
     A.g5in = 0;
@@ -642,7 +627,9 @@ void hop64(dd_handle* h, SiteSet S, int nrhs, int par, SpinorF64 in, SpinorF64 x
     A.st = st;
     A.red = red;
     A.S = S;
-    launch_hop<double, SpinorF64, SpinorF64, SpinorF64, LinkF64, MASK>(A, nrhs, h);
+    A.rhat = bvec ? *bvec : xin;
+    A.resid = bvec != nullptr;
+    launch_hop<double, SpinorX, SpinorF64, SOut, LinkX, MASK>(A, nrhs, h);
 }
 
 __global__ void not_converged_kernel(int nrhs, const CGState* outer, int* status) {
@@ -677,10 +664,10 @@ int defect_correction(dd_handle* h, int nrhs, int field0, int step, Inner& cg, b
     const double kappa = h->prm.kappa;
     const SiteSet S = cg.S;
     dim3 grid(grid_for(S.n, 128), nrhs);
-    SpinorF64 be{v.be, Vh}, bo{v.bo, Vh}, xe{v.xe, Vh}, xo{v.xo, Vh}, re{v.re, Vh}, t64{v.t64, Vh},
-        t64b{v.t64b, Vh};
-    LinkF64 lk64 = field_links<LinkF64>(h, field0);
-    const long long rs64 = field_stride<LinkF64>(h, step);
+    SpinorF64 be{v.be, Vh}, bo{v.bo, Vh}, xe{v.xe, Vh}, xo{v.xo, Vh}, re{v.re, Vh};
+    const SpinorX tx{v.tx, v.txe, Vh}, px{v.px, v.pxe, Vh}, box{reinterpret_cast<int4*>(v.xo), v.rxe, Vh};
+    LinkX lk64 = field_links<LinkX>(h, field0);
+    const long long rs64 = field_stride<LinkX>(h, step);
     CGState* outer = h->d_cg + h->prm.max_rhs;
     double* bb = h->d_scalars;
     double* tmp = h->d_scalars + nrhs;
@@ -692,9 +679,10 @@ int defect_correction(dd_handle* h, int nrhs, int field0, int step, Inner& cg, b
     DD_KLAUNCH(h, norm2_kernel<SpinorF64><<<grid, 128, 0, h->stream>>>(S, be, store_reduce(h, bb)));
     DD_KLAUNCH(h, norm2_kernel<SpinorF64><<<grid, 128, 0, h->stream>>>(S, bo, store_reduce(h, tmp)));
     DD_KLAUNCH(h, add_scalars_kernel<<<1, 64, 0, h->stream>>>(nrhs, bb, tmp));
-    hop64<MASK>(h, S, nrhs, 0, bo, be, be, 1.0, kappa, 1, lk64, rs64, nullptr, none);
+    DD_KLAUNCH(h, copy_kernel<SpinorF64, SpinorX><<<grid, 128, 0, h->stream>>>(S, bo, box, nullptr));
+    hop64<MASK>(h, S, nrhs, 0, box, be, be, kappa, 1, lk64, rs64, nullptr, none);
     DD_KLAUNCH(h, outer_arm_kernel<<<1, 64, 0, h->stream>>>(nrhs, outer, bb, tol));
-    DD_KLAUNCH(h, zero64_kernel<<<grid, 128, 0, h->stream>>>(S, xe));
+    DD_KLAUNCH(h, zero64_kernel<<<grid, 128, 0, h->stream>>>(S, xe, v.pxe));
     DD_KLAUNCH(h, copy_kernel<SpinorF64, SpinorF64><<<grid, 128, 0, h->stream>>>(S, be, re, nullptr));
     DD_KLAUNCH(h, norm2_kernel<SpinorF64><<<grid, 128, 0, h->stream>>>(S, re, store_reduce(h, rr)));
     DD_KLAUNCH(h, outer_update_kernel<<<1, 64, 0, h->stream>>>(nrhs, outer, rr, h->d_status));
@@ -716,12 +704,11 @@ int defect_correction(dd_handle* h, int nrhs, int field0, int step, Inner& cg, b
         int rc = cg.run(fp64_inner ? rr : ones, tol_inner, fp64_inner ? 0.25 : -1.0, maxit - total, 16, &it);
         total += it;
         if (rc) return rc;
-        DD_KLAUNCH(h, add_correction_kernel<SM><<<grid, 128, 0, h->stream>>>(S, xe, cg.x, fp64_inner ? nullptr : rr,
-                                                                          outer));
+        DD_KLAUNCH(h, add_correction_kernel<SM><<<grid, 128, 0, h->stream>>>(S, xe, px, cg.x,
+                                                                          fp64_inner ? nullptr : rr, outer));
         // true residual r = b~ - Dtilde x (FP64)
-        hop64<MASK>(h, S, nrhs, 1, xe, xe, t64, 0.0, 1.0, 0, lk64, rs64, outer, none);
-        hop64<MASK>(h, S, nrhs, 0, t64, xe, t64b, 1.0, -kappa * kappa, 1, lk64, rs64, outer, none);
-        DD_KLAUNCH(h, residual_kernel<<<grid, 128, 0, h->stream>>>(S, be, t64b, re, outer, store_reduce(h, rr)));
+        hop64<MASK>(h, S, nrhs, 1, px, xe, tx, 1.0, 0, lk64, rs64, outer, none);
+        hop64<MASK>(h, S, nrhs, 0, tx, xe, re, -kappa * kappa, 1, lk64, rs64, outer, store_reduce(h, rr), &be);
         DD_KLAUNCH(h, outer_update_kernel<<<1, 64, 0, h->stream>>>(nrhs, outer, rr, h->d_status));
         return cudaGetLastError() == cudaSuccess ? DD_OK : DD_ERR_CUDA;
     };
@@ -743,7 +730,7 @@ int defect_correction(dd_handle* h, int nrhs, int field0, int step, Inner& cg, b
     int rc = dd_loop(h, body, more, lc);
     if (rc) return rc;
     // x_o = b_o + kappa H_oe x_e
-    hop64<MASK>(h, S, nrhs, 1, xe, bo, xo, 1.0, kappa, 1, lk64, rs64, nullptr, none);
+    hop64<MASK>(h, S, nrhs, 1, px, bo, xo, kappa, 1, lk64, rs64, nullptr, none);
     if (cudaGetLastError() != cudaSuccess) return DD_ERR_CUDA;
     if (!polled) {
         // captured: a solve that missed its target is reported in the status word
@@ -947,7 +934,7 @@ int defect_correction_df(dd_handle* h, int nrhs, int field0, int step, Inner& cg
     A.c = df_from_double(kappa);
     hopdf<MASK, 1>(h, nrhs, A);
     DD_KLAUNCH(h, outer_arm_kernel<<<1, 64, 0, h->stream>>>(nrhs, outer, bb, tol));
-    DD_KLAUNCH(h, zero64_kernel<<<grid, 128, 0, h->stream>>>(S, SpinorF64{v.x64, Vh}));
+    DD_KLAUNCH(h, zero64_kernel<<<grid, 128, 0, h->stream>>>(S, SpinorF64{v.x64, Vh}, nullptr));
     DD_KLAUNCH(h, df_round_kernel<<<grid, 128, 0, h->stream>>>(S, btd, r32, sig, store_reduce(h, rr)));
     DD_KLAUNCH(h, outer_update_kernel<<<1, 64, 0, h->stream>>>(nrhs, outer, rr, h->d_status));
     if (cudaGetLastError() != cudaSuccess) return DD_ERR_CUDA;
@@ -1061,7 +1048,7 @@ static int solve_packed_mask(dd_handle* h, SiteSet S, int nrhs, int field0, int 
     CGState* inner = h->d_cg;
     CGState* outer = h->d_cg + h->prm.max_rhs;
     if (prec == DD_PREC_F64) {
-        NormalCG<double, SpinorF64, SpinorF64, LinkF64, MASK> cg;
+        NormalCG<double, SpinorF64, SpinorX, LinkX, MASK> cg;
         cg.h = h;
         cg.nrhs = nrhs;
         // the inner x must not alias the residual temporaries: x64
@@ -1070,12 +1057,12 @@ static int solve_packed_mask(dd_handle* h, SiteSet S, int nrhs, int field0, int 
         cg.p = SpinorF64{v.p64, Vh};
         cg.q = SpinorF64{v.q64, Vh};
         cg.z = SpinorF64{v.z64, Vh};
-        cg.ph = cg.p;
-        cg.rh = cg.r;
-        cg.th = SpinorF64{v.t64, Vh};
-        cg.copies = 0;
-        cg.lk = field_links<LinkF64>(h, field0);
-        cg.lk_rs = field_stride<LinkF64>(h, step);
+        cg.ph = SpinorX{v.px, v.pxe, Vh};
+        cg.rh = SpinorX{reinterpret_cast<int4*>(v.xo), v.rxe, Vh};  // xo is written after the last iteration
+        cg.th = SpinorX{v.tx, v.txe, Vh};
+        cg.copies = 1;
+        cg.lk = field_links<LinkX>(h, field0);
+        cg.lk_rs = field_stride<LinkX>(h, step);
         cg.st = inner;
         cg.outer = outer;
         cg.S = S;

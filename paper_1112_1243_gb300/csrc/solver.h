@@ -8,7 +8,7 @@
 // Solve D x = b for nrhs systems whose right-hand sides are already packed
 // into h->vecs[0].be / .bo (FP64 eo chunks, system r at offset r*12*Vh).
 // System r uses the gauge field of slot field0 + r*field_step (field_step 0:
-// one shared field, 1: consecutive slots), formatted in eo64 and in the
+// one shared field, 1: consecutive slots), formatted in eox and in the
 // inner precision.  On return vecs[0].xe / .xo hold the solution.
 // relres (host, nrhs, may be null) receives ||b - D x|| / ||b||, iters (may
 // be null) the total inner iterations.  prec: DD_PREC_F64 (plain FP64 CG) or

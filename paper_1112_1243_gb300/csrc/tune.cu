@@ -144,7 +144,8 @@ extern "C" int dd_autotune(dd_t h, int what, const void* U_old, const void* U_ne
             DD_CUDA(h, cudaMemsetAsync(v.p16n, 0, sizeof(float) * Vh * R, h->stream));
             DD_CUDA(h, cudaMemsetAsync(v.x32, 0, sizeof(float4) * 6 * Vh * R, h->stream));
             DD_CUDA(h, cudaMemsetAsync(v.be, 0, sizeof(double2) * 12 * Vh * R, h->stream));
-            DD_CUDA(h, cudaMemsetAsync(v.bo, 0, sizeof(double2) * 12 * Vh * R, h->stream));
+            DD_CUDA(h, cudaMemsetAsync(v.px, 0, sizeof(int4) * 12 * Vh * R, h->stream));
+            DD_CUDA(h, cudaMemsetAsync(v.pxe, 0, sizeof(int) * Vh * R, h->stream));
             const double k2 = h->prm.kappa * h->prm.kappa;
             // the hop of the mixed inner solver: FP16 in, FP32 out with xpay
             HopArgs<SpinorF16, SpinorF32, SpinorF32, LinkF16> A;
@@ -179,13 +180,13 @@ extern "C" int dd_autotune(dd_t h, int what, const void* U_old, const void* U_ne
             }
             r.hop_ms = best;
             // FP64 hop of the defect-correction residual
-            HopArgs<SpinorF64, SpinorF64, SpinorF64, LinkF64> B;
+            HopArgs<SpinorX, SpinorF64, SpinorF64, LinkX> B;
             B.g = h->g;
             B.p = 0;
-            B.in = SpinorF64{v.bo, Vh};
+            B.in = SpinorX{v.px, v.pxe, Vh};
             B.xin = SpinorF64{v.be, Vh};
             B.out = SpinorF64{v.xe, Vh};
-            B.lk = LinkF64{h->fields[0].eo64, Vh};
+            B.lk = LinkX{h->fields[0].eox, Vh};
             B.lk_rhs_stride = 0;
             B.a = 1.0;
             B.b = -k2;
@@ -200,7 +201,7 @@ extern "C" int dd_autotune(dd_t h, int what, const void* U_old, const void* U_ne
                 h->tune.hop64_tpb = s.tpb;
                 h->tune.hop64_spt = s.spt;
                 float ms = time_launches(h, std::max(2, reps / 4), [&] {
-                    launch_hop<double, SpinorF64, SpinorF64, SpinorF64, LinkF64, 0>(B, R, h);
+                    launch_hop<double, SpinorX, SpinorF64, SpinorF64, LinkX, 0>(B, R, h);
                 });
                 if (ms < 0) return dd_fail(h, DD_ERR_CUDA, "dd_autotune: FP64 hop timing failed");
                 if (s.tpb == 128 && s.spt == 1) r.hop64_default_ms = ms;
