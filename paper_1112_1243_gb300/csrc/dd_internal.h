@@ -42,8 +42,10 @@ enum FinOp {
 };
 
 struct Reduce {
-    double* partials;     // [rhs][gridDim.x]
+    double* partials;     // [rhs][value][gridDim.x], then the sums of groups of thread blocks
     unsigned* counters;   // [rhs]
+    unsigned* groups;     // [rhs][gmax] tickets of the groups
+    int gmax;
     CGState* st;          // [rhs] (FIN_ALPHA / RR / BETA / ZZ_INIT)
     double* out;          // [rhs] (FIN_STORE)
     int op;
@@ -112,6 +114,9 @@ struct SapVecs {
     float4* at(int k) const { return halves + (size_t)k * half; }
 };
 
+// thread blocks of one group of a grid reduction (grid_reduce_n)
+constexpr int DD_REDUCE_GROUP = 64;
+
 constexpr int DD_BLOCK_CTAS_MAX = 4;
 // timed kernel kinds: whole-lattice hops 0 FP16 -> FP16, 1 FP16 -> FP32 (xpay),
 // 2 FP64, 3 double-float residual; Dirichlet (block-restricted) hops 4 FP64,
@@ -154,7 +159,8 @@ struct dd_handle {
     CGState* d_cg = nullptr;         // [3 * max_rhs + 2]: inner, outer, SAP block-solver states
     SapVecs sap;                     // SAP-preconditioned GCR (krylov DD_KRYLOV_SAP_GCR)
     double* d_partials = nullptr;    // reduction partials
-    unsigned* d_counters = nullptr;  // reduction tickets
+    unsigned* d_counters = nullptr;  // reduction tickets: [4 * (max_rhs + 1) + 64], then [max_rhs + 1][reduce_gmax]
+    int reduce_gmax = 0;
     size_t partials_cap = 0;
     double* d_scalars = nullptr;     // scratch doubles [64 * max_rhs]
     char* block_scratch = nullptr;   // persistent block-solver slots
@@ -271,6 +277,23 @@ int dd_loop(dd_handle* h, const std::function<int()>& body, const std::function<
 
 // Launch a kernel and count it: DD_KLAUNCH(h, kern<<<grid, block, 0, h->stream>>>(args));
 #define DD_KLAUNCH(h, ...) ((__VA_ARGS__), ++(h)->launches)
+
+inline size_t dd_counter_count(const dd_handle* h) {
+    return (size_t)4 * (h->prm.max_rhs + 1) + 64 + (size_t)(h->prm.max_rhs + 1) * h->reduce_gmax;
+}
+// a grid reduction on the handle's tickets and partials
+inline Reduce dd_reduce(dd_handle* h, int op, CGState* st, double* out) {
+    Reduce r;
+    r.partials = h->d_partials;
+    r.counters = h->d_counters;
+    r.groups = h->d_counters + (size_t)4 * (h->prm.max_rhs + 1) + 64;
+    r.gmax = h->reduce_gmax;
+    r.st = st;
+    r.out = out;
+    r.op = op;
+    r.status = h->d_status;
+    return r;
+}
 
 // next timing event of a kind (pool grows on demand)
 inline cudaEvent_t dd_timer_event(dd_handle* h, int kind) {

@@ -236,7 +236,6 @@ DD_DEV void df_hop(int a, float sg, float ph, int yh, const float4* lk_site, con
 // MODE 0: out = H in; MODE 1: out = xin + c H in; MODE 2: rout = bin - xin + c H in with |rout|^2 / sigma^2
 template <int MASK, int MODE>
 __global__ void __launch_bounds__(128) hop_df_kernel(DFHopArgs A) {
-    __shared__ double sh[34];
     const int rhs = blockIdx.y;
     if (A.st && !A.st[rhs].active) return;
     if (A.sites && threadIdx.x == 0)
@@ -306,5 +305,5 @@ __global__ void __launch_bounds__(128) hop_df_kernel(DFHopArgs A) {
             }
         }
     }
-    if (MODE == 2) grid_reduce(A.red, rhs, nrm, sh);
+    if (MODE == 2) grid_reduce(A.red, rhs, nrm);
 }

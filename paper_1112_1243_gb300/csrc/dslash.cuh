@@ -114,7 +114,6 @@ DD_DEV void hop_site(const Geo& g, int p, int h, const int x[4], const SIn& in, 
 template <class R, class SIn, class SX, class SOut, class LK, int MASK, int RED3, int SPT>
 __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
     hop_eo_kernel(HopArgs<SIn, SX, SOut, LK> A) {
-    __shared__ double sh[34];
     const int rhs = blockIdx.y;
     if (A.st && !A.st[rhs].active) return;
     const long long Vh = A.g.Vh;
@@ -185,9 +184,9 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
         }
     }
     if (RED3) {
-        grid_reduce3(A.red, rhs, v3, sh);
+        grid_reduce3(A.red, rhs, v3);
     } else if (A.red.op != FIN_NONE) {
-        grid_reduce(A.red, rhs, nrm, sh);
+        grid_reduce(A.red, rhs, nrm);
     }
 }
 
@@ -196,7 +195,6 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
 // hops, or rhat - (xin + b * hops) with resid, and |out|^2 to A.red.
 template <class SX, class SOut, int MASK>
 __global__ void __launch_bounds__(128, 4) hop_x_kernel(HopArgs<SpinorX, SX, SOut, LinkX> A) {
-    __shared__ double sh[34];
     const int rhs = blockIdx.y;
     if (A.st && !A.st[rhs].active) return;
     const Geo& g = A.g;
@@ -296,7 +294,7 @@ __global__ void __launch_bounds__(128, 4) hop_x_kernel(HopArgs<SpinorX, SX, SOut
         }
     }
     if constexpr (!std::is_same<SOut, SpinorX>::value) {
-        if (A.red.op != FIN_NONE) grid_reduce(A.red, rhs, nrm, sh);
+        if (A.red.op != FIN_NONE) grid_reduce(A.red, rhs, nrm);
     }
 }
 

@@ -171,7 +171,6 @@ __global__ void dd_to_eo_kernel(Geo g, BlockCtx c, const double2* bank, long lon
 // ln_i = -sum_black (2 Re<eta, d> + |d|^2), d from the eo solution
 __global__ void __launch_bounds__(128) estimate_kernel(Geo g, BlockCtx c, const double2* eta_bank, long long vs,
                                                        const double2* xe, const double2* xo, Reduce red) {
-    __shared__ double sh[34];
     long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     int i = blockIdx.y;
     double acc = 0.0;
@@ -189,7 +188,7 @@ __global__ void __launch_bounds__(128) estimate_kernel(Geo g, BlockCtx c, const 
         for (int k = 0; k < 12; ++k) acc += 2.0 * (e.c[k].x * d.c[k].x + e.c[k].y * d.c[k].y) + norm2(d.c[k]);
         acc = -acc;
     }
-    grid_reduce(red, i, acc, sh);
+    grid_reduce(red, i, acc);
 }
 
 // ln_b[b] = sum of the n item results of block b (0 for blocks without
@@ -991,13 +990,7 @@ extern "C" int dd_det_ratio_estimate(dd_t h, const void* U_old, const void* U_ne
                       nullptr);
     if (rc && rc != DD_ERR_NOT_CONVERGED) return dd_fail(h, rc, "dd_det_ratio_estimate: global solve failed");
     // 8. ln r_i
-    Reduce red;
-    red.partials = h->d_partials;
-    red.counters = h->d_counters;
-    red.st = nullptr;
-    red.out = ln_out;
-    red.op = FIN_STORE;
-    red.status = h->d_status;
+    const Reduce red = dd_reduce(h, FIN_STORE, nullptr, ln_out);
     dim3 gb(grid_for(g.V / 2, 128), n);
     DD_KLAUNCH(h, estimate_kernel<<<gb, 128, 0, h->stream>>>(g, c, bank[0], vs, v.xe, v.xo, red));
     DD_LAUNCH_CHECK(h, "estimate_kernel");

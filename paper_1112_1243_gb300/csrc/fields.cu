@@ -125,7 +125,6 @@ extern "C" int dd_interpolate(dd_t h, void* U_t, const void* U, const void* U_ne
 
 // ---------------------------------------------------------------- plaquette
 __global__ void __launch_bounds__(128) plaquette_kernel(Geo g, const double* __restrict__ U, Reduce red) {
-    __shared__ double sh[34];
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     double acc = 0.0;
     if (s < g.V) {
@@ -142,7 +141,7 @@ __global__ void __launch_bounds__(128) plaquette_kernel(Geo g, const double* __r
                 acc += p.m[0][0].x + p.m[1][1].x + p.m[2][2].x;
             }
     }
-    grid_reduce(red, 0, acc, sh);
+    grid_reduce(red, 0, acc);
 }
 __global__ void plaquette_scale_kernel(double* out, double inv) { out[0] *= inv; }
 
@@ -150,13 +149,7 @@ extern "C" int dd_plaquette(dd_t h, const void* U, double* out) {
     int rc = dd_require_ws(h);
     if (rc) return rc;
     if (!U || !out) return dd_fail(h, DD_ERR_INVALID_ARG, "dd_plaquette: bad arguments");
-    Reduce R_;
-    R_.partials = h->d_partials;
-    R_.counters = h->d_counters;
-    R_.st = nullptr;
-    R_.out = out;
-    R_.op = FIN_STORE;
-    R_.status = h->d_status;
+    const Reduce R_ = dd_reduce(h, FIN_STORE, nullptr, out);
     DD_KLAUNCH(h, plaquette_kernel<<<grid_for(h->g.V, 128), 128, 0, h->stream>>>(h->g, (const double*)U, R_));
     DD_KLAUNCH(h, plaquette_scale_kernel<<<1, 1, 0, h->stream>>>(out, 1.0 / (18.0 * h->g.V)));
     DD_LAUNCH_CHECK(h, "plaquette_kernel");

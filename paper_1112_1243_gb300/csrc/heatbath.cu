@@ -188,7 +188,6 @@ __global__ void __launch_bounds__(128) gauge_fix_kernel(Geo g, const double* __r
 // sum Re tr(U^dag U'^g) accumulated into *F (may be null)
 __global__ void __launch_bounds__(128) gauge_apply_kernel(Geo g, const double* __restrict__ U, const double* G,
                                                           double* Up, Reduce red) {
-    __shared__ double sh[34];
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     double f = 0.0;
     if (s < g.V) {
@@ -203,7 +202,7 @@ __global__ void __launch_bounds__(128) gauge_apply_kernel(Geo g, const double* _
             f += t.m[0][0].x + t.m[1][1].x + t.m[2][2].x;
         }
     }
-    if (red.op != FIN_NONE) grid_reduce(red, 0, f, sh);
+    if (red.op != FIN_NONE) grid_reduce(red, 0, f);
 }
 
 }  // namespace
@@ -221,13 +220,7 @@ extern "C" int dd_relative_gauge_fix(dd_t h, const void* U, void* U_new, int swe
         for (int par = 0; par < 2; ++par)
             DD_KLAUNCH(h, gauge_fix_kernel<<<grid_for(g.Vh, 128), 128, 0, h->stream>>>(g, (const double*)U,
                                                                                    (const double*)U_new, G, par));
-    Reduce red;
-    red.partials = h->d_partials;
-    red.counters = h->d_counters;
-    red.st = nullptr;
-    red.out = functional;
-    red.op = functional ? FIN_STORE : FIN_NONE;
-    red.status = h->d_status;
+    const Reduce red = dd_reduce(h, functional ? FIN_STORE : FIN_NONE, nullptr, functional);
     DD_KLAUNCH(h, gauge_apply_kernel<<<grid_for(g.V, 128), 128, 0, h->stream>>>(g, (const double*)U, G,
                                                                               (double*)U_new, red));
     DD_LAUNCH_CHECK(h, "dd_relative_gauge_fix");

@@ -410,7 +410,8 @@ void plan(dd_handle* h, char* base) {
     // partials of grid reductions with tiles of 64 sites or more (3 values per tile)
     h->partials_cap = (size_t)(grid_for(std::max(Vh, V), 64) + 64) * (R + 1) * 2;
     h->d_partials = c.take<double>(h->partials_cap);
-    h->d_counters = c.take<unsigned>((size_t)4 * (R + 1) + 64);
+    h->reduce_gmax = (int)((grid_for(std::max(Vh, V), 64) + 64 + DD_REDUCE_GROUP - 1) / DD_REDUCE_GROUP);
+    h->d_counters = c.take<unsigned>(dd_counter_count(h));
     h->d_scalars = c.take<double>((size_t)64 * (R + 2));
     // persistent block-solver slots
     const long long nb = h->g.bsites;
@@ -643,7 +644,7 @@ extern "C" int dd_set_workspace(dd_t h, void* dev_ptr, size_t bytes) {
     h->ws_size = bytes;
     plan(h, h->ws);
     // reduction tickets and solver states start from zero
-    DD_CUDA(h, cudaMemsetAsync(h->d_counters, 0, sizeof(unsigned) * (4 * (h->prm.max_rhs + 1) + 64), h->stream));
+    DD_CUDA(h, cudaMemsetAsync(h->d_counters, 0, sizeof(unsigned) * dd_counter_count(h), h->stream));
     DD_CUDA(h, cudaMemsetAsync(h->d_cg, 0, sizeof(CGState) * (3 * h->prm.max_rhs + 2), h->stream));
     return DD_OK;
 }

@@ -141,59 +141,83 @@ DD_DEV void finish3(const Reduce& R, int rhs, const double* s) {
     }
 }
 
-// Three-value variant: partials [rhs][gridDim.x][3].  `sh` needs 34 doubles.
-DD_DEV void grid_reduce3(const Reduce& R, int rhs, const double* v, double* sh) {
-    double b[3];
+// Sum of N values a thread over the grid row of rhs; the last thread block
+// runs the finisher.  Every thread of the block calls this (at most 128
+// threads).  Deterministic: all sums are taken in a fixed order.
+//
+// FP64 additions are the scarce resource (1.6 lanes a clock): the block sum
+// goes through shared memory, 32 lanes a value, about 8 warp additions a
+// value instead of 5 a warp.  Above 4096 partial sums the reduction has two
+// levels: the last block of a group of DD_REDUCE_GROUP adds its members, the
+// last group the groups.  With one level the last block of a grid of 6144
+// had 18432 additions to make: the three-value kernels of a solve at
+// 32^3 x 48 took 100 us instead of 66.  Below the line the second ticket
+// costs more than it saves (135 blocks of one value: 1.5 us a launch).
+template <int N>
+DD_DEV void grid_reduce_n(const Reduce& R, int rhs, const double* v, void (*fin)(const Reduce&, int, const double*)) {
+    __shared__ double buf[N][128];
+    __shared__ double tot[N];
+    __shared__ int last;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
+    const int nblk = gridDim.x;
+    auto block_total = [&](const double* w) {  // tot[k] = sum of w[k] over the block
 #pragma unroll
-    for (int k = 0; k < 3; ++k) b[k] = block_sum(v[k], sh);
-    int* last = reinterpret_cast<int*>(&sh[33]);
-    if (threadIdx.x == 0) {
-        double* p = R.partials + ((long long)rhs * gridDim.x + blockIdx.x) * 3;
-        p[0] = b[0];
-        p[1] = b[1];
-        p[2] = b[2];
-        __threadfence();
-        unsigned t = atomicAdd(&R.counters[rhs], 1u);
-        *last = (t == gridDim.x - 1);
-    }
+        for (int k = 0; k < N; ++k) buf[k][tid] = w[k];
+        __syncthreads();
+        for (int k = wid; k < N; k += nw) {
+            double s = 0.0;
+            for (int j = lane; j < (int)blockDim.x; j += 32) s += buf[k][j];
+            s = warp_sum(s);
+            if (lane == 0) tot[k] = s;
+        }
+        __syncthreads();
+    };
+    // true in every thread of the block that arrives last at a counter
+    auto ticket = [&](unsigned* c, unsigned members) {
+        if (tid == 0) {
+            __threadfence();
+            last = atomicAdd(c, 1u) == members - 1;
+            if (last) *c = 0;
+        }
+        __syncthreads();
+        const bool l = last;
+        if (l) __threadfence();
+        return l;
+    };
+    // partial sums p[k * n + i], i in [lo, hi), added up by the whole block
+    auto gather = [&](const double* p, int n, int lo, int hi) {
+        double s[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) s[k] = 0.0;
+#pragma unroll 4
+        for (int i = lo + tid; i < hi; i += blockDim.x)
+#pragma unroll
+            for (int k = 0; k < N; ++k) s[k] += __ldcg(p + (long long)k * n + i);
+        block_total(s);
+    };
+    block_total(v);
+    double* part = R.partials + (long long)rhs * N * nblk;
+    if (tid < N) part[(long long)tid * nblk + blockIdx.x] = tot[tid];
+    if (tid < N) __threadfence();
     __syncthreads();
-    if (*last) {
-        __threadfence();
-        double s[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            double a = 0.0;
-            for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x)
-                a += __ldcg(&R.partials[((long long)rhs * gridDim.x + i) * 3 + k]);
-            s[k] = block_sum(a, sh);
-        }
-        if (threadIdx.x == 0) {
-            finish3(R, rhs, s);
-            R.counters[rhs] = 0;
-        }
+    const int ngrp = (nblk + DD_REDUCE_GROUP - 1) / DD_REDUCE_GROUP;
+    if (N * nblk > 4096) {
+        const int grp = blockIdx.x / DD_REDUCE_GROUP, lo = grp * DD_REDUCE_GROUP, hi = min(lo + DD_REDUCE_GROUP, nblk);
+        if (!ticket(R.groups + (long long)rhs * R.gmax + grp, (unsigned)(hi - lo))) return;
+        gather(part, nblk, lo, hi);
+        double* gpart = R.partials + (long long)gridDim.y * N * nblk + (long long)rhs * N * ngrp;
+        if (tid < N) gpart[(long long)tid * ngrp + grp] = tot[tid];
+        if (tid < N) __threadfence();
+        __syncthreads();
+        if (!ticket(&R.counters[rhs], (unsigned)ngrp)) return;
+        gather(gpart, ngrp, 0, ngrp);
+    } else {
+        if (!ticket(&R.counters[rhs], (unsigned)nblk)) return;
+        gather(part, nblk, 0, nblk);
     }
+    if (tid == 0) fin(R, rhs, tot);
 }
 
-// Every thread of the block calls this with its contribution.  `sh` needs 34 doubles.
-DD_DEV void grid_reduce(const Reduce& R, int rhs, double v, double* sh) {
-    double bsum = block_sum(v, sh);
-    int* last = reinterpret_cast<int*>(&sh[33]);
-    if (threadIdx.x == 0) {
-        R.partials[(long long)rhs * gridDim.x + blockIdx.x] = bsum;
-        __threadfence();
-        unsigned t = atomicAdd(&R.counters[rhs], 1u);
-        *last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (*last) {
-        __threadfence();
-        double s = 0.0;
-        for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x)
-            s += __ldcg(&R.partials[(long long)rhs * gridDim.x + i]);
-        s = block_sum(s, sh);
-        if (threadIdx.x == 0) {
-            finish(R, rhs, s);
-            R.counters[rhs] = 0;
-        }
-    }
-}
+DD_DEV void finish1(const Reduce& R, int rhs, const double* s) { finish(R, rhs, s[0]); }
+DD_DEV void grid_reduce3(const Reduce& R, int rhs, const double* v) { grid_reduce_n<3>(R, rhs, v, finish3); }
+DD_DEV void grid_reduce(const Reduce& R, int rhs, double v) { grid_reduce_n<1>(R, rhs, &v, finish1); }

@@ -283,7 +283,6 @@ __global__ void __launch_bounds__(128) sap_update_kernel(SiteSet Sc, FullF32 Z, 
 
 // |v|^2 of an even-sized FP32 vector on the sites of S (per system), to `out`
 __global__ void __launch_bounds__(128) sap_norm_kernel(SiteSet S, SpinorF32 v, const CGState* st, Reduce red) {
-    __shared__ double sh[34];
     const int rhs = blockIdx.y;
     if (st && !st[rhs].active) return;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -293,7 +292,7 @@ __global__ void __launch_bounds__(128) sap_norm_kernel(SiteSet S, SpinorF32 v, c
         at_rhs(v, rhs).load(S.at(t), a);
         nrm = (double)snorm2(a);
     }
-    grid_reduce(red, rhs, nrm, sh);
+    grid_reduce(red, rhs, nrm);
 }
 
 // hop-storage view of a SAP half vector (FP16: chunks, then the per-site scales)

@@ -28,7 +28,6 @@ namespace {
 template <class R, class SM, class SH>
 __global__ void __launch_bounds__(128) cg_xr_kernel(SiteSet S, SM x, SM r, SM p, SM q, SH rh, int copy,
                                                     const CGState* st, Reduce red) {
-    __shared__ double sh[34];
     const int rhs = blockIdx.y;
     if (!st[rhs].active) return;
     const R alpha = (R)st[rhs].alpha;
@@ -51,7 +50,7 @@ __global__ void __launch_bounds__(128) cg_xr_kernel(SiteSet S, SM x, SM r, SM p,
         if (copy) at_rhs(rh, rhs).store(i, a);
         nrm = (double)snorm2(a);
     }
-    grid_reduce(red, rhs, nrm, sh);
+    grid_reduce(red, rhs, nrm);
 }
 
 template <class R, class SM, class SH>
@@ -185,7 +184,6 @@ __global__ void fill_kernel(int n, double* p, double v) {
 }
 template <class SV>
 __global__ void __launch_bounds__(128) norm2_kernel(SiteSet S, SV v, Reduce red) {
-    __shared__ double sh[34];
     const int rhs = blockIdx.y;
     const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     double nrm = 0.0;
@@ -195,7 +193,7 @@ __global__ void __launch_bounds__(128) norm2_kernel(SiteSet S, SV v, Reduce red)
         at_rhs(v, rhs).load(i, a);
         nrm = snorm2(a);
     }
-    grid_reduce(red, rhs, nrm, sh);
+    grid_reduce(red, rhs, nrm);
 }
 template <class SIn, class SOut>
 __global__ void copy_kernel(SiteSet S, SIn in, SOut out, const CGState* outer) {
@@ -234,16 +232,7 @@ struct NormalCG {
     const CGState* outer;
     SiteSet S;  // the sites of the solve (all even sites, or one block colour's)
 
-    Reduce red(int op) const {
-        Reduce R_;
-        R_.partials = h->d_partials;
-        R_.counters = h->d_counters;
-        R_.st = st;
-        R_.out = nullptr;
-        R_.op = op;
-        R_.status = h->d_status;
-        return R_;
-    }
+    Reduce red(int op) const { return dd_reduce(h, op, st, nullptr); }
     template <class SIn, class SX, class SOut>
     HopArgs<SIn, SX, SOut, LK> args(int par, SIn in, SX xin, SOut out, double a, double b, int hasx, int g5in,
                                     int g5out, int op) const {
@@ -366,7 +355,6 @@ __global__ void bicg_arm_kernel(int nrhs, CGState* st) {
 
 template <class R, class SM, class SH>
 __global__ void __launch_bounds__(128) bicg_rho_kernel(SiteSet S, SH rhat, SM r, const CGState* st, Reduce red) {
-    __shared__ double sh[34];
     const int rhs = blockIdx.y;
     if (!st[rhs].active) return;
     const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -386,7 +374,7 @@ __global__ void __launch_bounds__(128) bicg_rho_kernel(SiteSet S, SH rhat, SM r,
         v[1] = (double)d1;
         v[2] = (double)snorm2(b);
     }
-    grid_reduce3(red, rhs, v, sh);
+    grid_reduce3(red, rhs, v);
 }
 
 // p = r + beta (p - omega v)
@@ -432,7 +420,6 @@ __global__ void __launch_bounds__(128) bicg_s_kernel(SiteSet S, SM s, SM r, SM v
 template <class R, class SM, class SH>
 __global__ void __launch_bounds__(128) bicg_xr_kernel(SiteSet S, SM x, SM r, SH p, SM s, SM t, SH rhat,
                                                       const CGState* st, Reduce red) {
-    __shared__ double sh[34];
     const int rhs = blockIdx.y;
     if (!st[rhs].active) return;
     const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -463,7 +450,7 @@ __global__ void __launch_bounds__(128) bicg_xr_kernel(SiteSet S, SM x, SM r, SH 
         v[1] = (double)d1;
         v[2] = (double)snorm2(ss);
     }
-    grid_reduce3(red, rhs, v, sh);
+    grid_reduce3(red, rhs, v);
 }
 
 template <class R, class SM, class SH, class LK, int MASK = 0>
@@ -479,16 +466,7 @@ struct BiCGStab {
     const CGState* outer;
     SiteSet S;  // the sites of the solve (all even sites, or one block colour's)
 
-    Reduce red(int op) const {
-        Reduce R_;
-        R_.partials = h->d_partials;
-        R_.counters = h->d_counters;
-        R_.st = st;
-        R_.out = nullptr;
-        R_.op = op;
-        R_.status = h->d_status;
-        return R_;
-    }
+    Reduce red(int op) const { return dd_reduce(h, op, st, nullptr); }
     template <class SIn, class SX, class SOut>
     HopArgs<SIn, SX, SOut, LK> args(int par, SIn in, SX xin, SOut out, double a, double b, int hasx, int op,
                                     int red3) const {
@@ -594,16 +572,7 @@ long long field_stride(dd_handle* h, int step) {
     return (long long)(b.p - a.p);
 }
 
-Reduce store_reduce(dd_handle* h, double* out) {
-    Reduce R_;
-    R_.partials = h->d_partials;
-    R_.counters = h->d_counters;
-    R_.st = nullptr;
-    R_.out = out;
-    R_.op = FIN_STORE;
-    R_.status = h->d_status;
-    return R_;
-}
+Reduce store_reduce(dd_handle* h, double* out) { return dd_reduce(h, FIN_STORE, nullptr, out); }
 
 // FP64 hop (in limbs, xfix.cuh): out = (hasx ? xin : 0) + b * hops of in, or
 // bvec - that with resid (SOut SpinorF64), or the hops alone (SOut SpinorX)
@@ -810,7 +779,6 @@ __global__ void __launch_bounds__(128) from_df_kernel(SiteSet S, SpinorDF in, Sp
 // r = in rounded to FP32, |r|^2 / sigma^2 (the residual of x = 0)
 __global__ void __launch_bounds__(128) df_round_kernel(SiteSet S, SpinorDF in, SpinorF32 r, const double* sig_exp,
                                                        Reduce red) {
-    __shared__ double sh[34];
     const int rhs = blockIdx.y;
     const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     double nrm = 0.0;
@@ -828,7 +796,7 @@ __global__ void __launch_bounds__(128) df_round_kernel(SiteSet S, SpinorDF in, S
         at_rhs(r, rhs).store(i, v);
         nrm = ldexp((double)n2, -2 * (int)sig_exp[rhs]);
     }
-    grid_reduce(red, rhs, nrm, sh);
+    grid_reduce(red, rhs, nrm);
 }
 // r /= sigma |r| (the inner solver's unit-norm right-hand side)
 __global__ void __launch_bounds__(128) df_normalise_kernel(SiteSet S, SpinorF32 r, const double* rr,
