@@ -67,6 +67,14 @@ struct Link {
     cpx<R> m[3][3];
 };
 
+// complex number i of a caller's field (al16: the field starts on a 16-byte
+// boundary; the C ABI asks only for that of a double)
+DD_DEV double2 load_c(const double* p, long long i, bool al16) {
+    if (al16) return reinterpret_cast<const double2*>(p)[i];
+    return make_double2(p[2 * i], p[2 * i + 1]);
+}
+inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 // ----------------------------------------------------------- storage formats
 // All fields are stored as 16-byte (or 8-byte) chunks, chunk-major:
 // chunk k of site i lives at base[k * stride + i], so consecutive threads

@@ -60,47 +60,65 @@ __global__ void interpolate_kernel(long long nlinks, const double* __restrict__ 
     store_m3(o, mul(u, wt));
 }
 
-// Every slot k = 0 .. nslots - 1 of one chain U_{k/den} (slot k at out +
-// k * slot_stride doubles): the eigen-decomposition of U^dag U' is computed
-// once per link for all slots.
-__global__ void interpolate_slots_kernel(long long nlinks, const double* __restrict__ U, const double* __restrict__ Up,
-                                         const uint8_t* __restrict__ active, double* out, long long slot_stride,
-                                         int nslots, int den) {
-    long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= nlinks) return;
+// The chain U_{k/den}, k = 0 .. nslots - 1 (slot k at out + k * slot_stride
+// doubles), in two launches: every link of U into every slot, then the links
+// of the list (null: all links) along the path.  One launch over all links
+// made nearly every warp wait for the eigen-decompositions of the 8% of its
+// lanes with an active link: 3750 us for 13 slots at 16^3 x 32 against
+// 160 + 645 us.
+__global__ void __launch_bounds__(256) copy_slots_kernel(long long n, const double* __restrict__ U, bool al16,
+                                                         double* out, long long slot_stride, int nslots) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double2 v = load_c(U, i, al16);
+    for (int s = 0; s < nslots; ++s) reinterpret_cast<double2*>(out + s * slot_stride)[i] = v;
+}
+
+// U W^t = sum_k e^{i t theta_k} (U v_k) v_k^dag with the eigenvectors v_k of
+// W = U^dag U': FP64 arithmetic bound, so the decomposition and U v_k are
+// made once a link and every slot costs three sincos and 144 FMAs.
+__global__ void __launch_bounds__(64) interpolate_slots_kernel(long long n, const int* __restrict__ links,
+                                                               const double* __restrict__ U,
+                                                               const double* __restrict__ Up, double* out,
+                                                               long long slot_stride, int nslots, int den) {
+    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const long long l = links ? links[k] : k;
     const double* a = U + l * 18;
     const double* b = Up + l * 18;
     bool same = true;
-    for (int k = 0; k < 18; ++k) same = same && (a[k] == b[k]);
-    if ((active && !active[l]) || same) {
-        for (int s = 0; s < nslots; ++s) {
-            const double* src = (s == den && !(active && !active[l])) ? b : a;
-            double* o = out + s * slot_stride + l * 18;
-            for (int k = 0; k < 18; ++k) o[k] = src[k];
-        }
-        return;
-    }
-    M3 u = load_m3(a), up = load_m3(b);
-    M3 V;
+    for (int e = 0; e < 18; ++e) same = same && (a[e] == b[e]);
+    if (den < nslots)
+        for (int e = 0; e < 18; ++e) out[den * slot_stride + l * 18 + e] = b[e];
+    // an unchanged link (e.g. in a rejected block) stays on the path
+    if (same || den == 1) return;
+    M3 u = load_m3(a), V;
     double th[3];
-    su3_eig(mul_dag_left(u, up), V, th);
-    for (int s = 0; s < nslots; ++s) {
-        double* o = out + s * slot_stride + l * 18;
-        if (s == 0) {
-            for (int k = 0; k < 18; ++k) o[k] = a[k];
-        } else if (s == den) {
-            for (int k = 0; k < 18; ++k) o[k] = b[k];
-        } else {
-            store_m3(o, mul(u, su3_power_eig(V, th, (double)s / (double)den)));
+    su3_eig(mul_dag_left(u, load_m3(b)), V, th);
+    u = mul(u, V);
+    for (int s = 1; s < nslots && s < den; ++s) {
+        const double t = (double)s / (double)den;
+        M3 w;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            double sn, cs;
+            sincos(t * th[c], &sn, &cs);
+#pragma unroll
+            for (int r = 0; r < 3; ++r) w.m[r][c] = cmul(u.m[r][c], mk<double>(cs, sn));
         }
+        store_m3(out + s * slot_stride + l * 18, mul_dag_right(w, V));
     }
 }
 
 int launch_interpolate_slots(dd_handle* h, const double* U, const double* Up, double* out, long long slot_stride,
                              int nslots, int den, bool all_links) {
-    const long long n = (long long)h->g.V * 4;
-    DD_KLAUNCH(h, interpolate_slots_kernel<<<grid_for(n, 128), 128, 0, h->stream>>>(
-                      n, U, Up, all_links ? nullptr : h->d_active_mask, out, slot_stride, nslots, den));
+    const long long nl = (long long)h->g.V * 4, n2 = nl * 9;
+    DD_KLAUNCH(h, copy_slots_kernel<<<(int)((n2 + 255) / 256), 256, 0, h->stream>>>(n2, U, aligned16(U), out,
+                                                                                   slot_stride, nslots));
+    const long long n = all_links ? nl : h->n_active;
+    if (n > 0)
+        DD_KLAUNCH(h, interpolate_slots_kernel<<<grid_for(n, 64), 64, 0, h->stream>>>(
+                          n, all_links ? nullptr : h->d_active_links, U, Up, out, slot_stride, nslots, den));
     DD_LAUNCH_CHECK(h, "interpolate_slots_kernel");
     return DD_OK;
 }

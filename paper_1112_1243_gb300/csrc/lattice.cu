@@ -125,8 +125,10 @@ std::vector<uint8_t> active_links(const HostGeo& G, int mode) {
 }  // namespace
 
 // --------------------------------------------------------- field formatting
-__global__ void format_gauge_kernel(Geo g, const double* __restrict__ U, FieldSlot f) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
+// one thread a link (blockIdx.y: its direction)
+__global__ void __launch_bounds__(128) format_gauge_kernel(Geo g, const double* __restrict__ U, bool al16,
+                                                           FieldSlot f) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x, a = blockIdx.y;
     if (s >= g.V) return;
     int x[4];
     canon_coords(g, s, x);
@@ -136,40 +138,44 @@ __global__ void format_gauge_kernel(Geo g, const double* __restrict__ U, FieldSl
     const long long q = dd_position(g, x);
     const long long bpos = q / g.bsites, j = q % g.bsites;
     const long long nb = g.bsites;
-    for (int a = 0; a < 4; ++a) {
-        const double* u = U + ((long long)s * 4 + a) * 18;
-        if (f.eox) x_store_link(f.eox, Vh, par, a, h, u);
-        if (f.eox && f.eodf) {
-            float4* o = f.eodf + ((long long)par * 4 + a) * 9 * Vh + h;
-            for (int k = 0; k < 9; ++k) {
-                const float rh = (float)u[2 * k], ih = (float)u[2 * k + 1];
-                o[k * Vh] = make_float4(rh, ih, (float)(u[2 * k] - (double)rh), (float)(u[2 * k + 1] - (double)ih));
-            }
+    double u[18];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const double2 v = load_c(U, ((long long)s * 4 + a) * 9 + k, al16);
+        u[2 * k] = v.x;
+        u[2 * k + 1] = v.y;
+    }
+    if (f.eox) x_store_link(f.eox, Vh, par, a, h, u);
+    if (f.eox && f.eodf) {
+        float4* o = f.eodf + ((long long)par * 4 + a) * 9 * Vh + h;
+        for (int k = 0; k < 9; ++k) {
+            const float rh = (float)u[2 * k], ih = (float)u[2 * k + 1];
+            o[k * Vh] = make_float4(rh, ih, (float)(u[2 * k] - (double)rh), (float)(u[2 * k + 1] - (double)ih));
         }
-        if (f.eo32) {
-            float4* o = f.eo32 + ((long long)par * 4 + a) * 3 * Vh + h;
-            for (int k = 0; k < 3; ++k)
-                o[k * Vh] = make_float4((float)u[4 * k], (float)u[4 * k + 1], (float)u[4 * k + 2], (float)u[4 * k + 3]);
+    }
+    if (f.eo32) {
+        float4* o = f.eo32 + ((long long)par * 4 + a) * 3 * Vh + h;
+        for (int k = 0; k < 3; ++k)
+            o[k * Vh] = make_float4((float)u[4 * k], (float)u[4 * k + 1], (float)u[4 * k + 2], (float)u[4 * k + 3]);
+    }
+    if (f.eo16) {
+        uint2* o = f.eo16 + ((long long)par * 4 + a) * 3 * Vh + h;
+        for (int k = 0; k < 3; ++k) {
+            uint2 v;
+            __half2* hh = reinterpret_cast<__half2*>(&v);
+            hh[0] = __floats2half2_rn((float)u[4 * k], (float)u[4 * k + 1]);
+            hh[1] = __floats2half2_rn((float)u[4 * k + 2], (float)u[4 * k + 3]);
+            o[k * Vh] = v;
         }
-        if (f.eo16) {
-            uint2* o = f.eo16 + ((long long)par * 4 + a) * 3 * Vh + h;
-            for (int k = 0; k < 3; ++k) {
-                uint2 v;
-                __half2* hh = reinterpret_cast<__half2*>(&v);
-                hh[0] = __floats2half2_rn((float)u[4 * k], (float)u[4 * k + 1]);
-                hh[1] = __floats2half2_rn((float)u[4 * k + 2], (float)u[4 * k + 3]);
-                o[k * Vh] = v;
-            }
-        }
-        if (f.dd64) {
-            double2* o = f.dd64 + (bpos * 4 + a) * 9 * nb + j;
-            for (int k = 0; k < 9; ++k) o[k * nb] = make_double2(u[2 * k], u[2 * k + 1]);
-        }
-        if (f.dd32) {
-            float4* o = f.dd32 + (bpos * 4 + a) * 3 * nb + j;
-            for (int k = 0; k < 3; ++k)
-                o[k * nb] = make_float4((float)u[4 * k], (float)u[4 * k + 1], (float)u[4 * k + 2], (float)u[4 * k + 3]);
-        }
+    }
+    if (f.dd64) {
+        double2* o = f.dd64 + (bpos * 4 + a) * 9 * nb + j;
+        for (int k = 0; k < 9; ++k) o[k * nb] = make_double2(u[2 * k], u[2 * k + 1]);
+    }
+    if (f.dd32) {
+        float4* o = f.dd32 + (bpos * 4 + a) * 3 * nb + j;
+        for (int k = 0; k < 3; ++k)
+            o[k * nb] = make_float4((float)u[4 * k], (float)u[4 * k + 1], (float)u[4 * k + 2], (float)u[4 * k + 3]);
     }
 }
 
@@ -180,7 +186,7 @@ int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eox, bool eo3
     if (!eo16) t.eo16 = nullptr;
     if (!dd64) t.dd64 = nullptr;
     if (!dd32) t.dd32 = nullptr;
-    DD_KLAUNCH(h, format_gauge_kernel<<<grid_for(h->g.V, 128), 128, 0, h->stream>>>(h->g, U, t));
+    DD_KLAUNCH(h, format_gauge_kernel<<<dim3(grid_for(h->g.V, 128), 4), 128, 0, h->stream>>>(h->g, U, aligned16(U), t));
     DD_LAUNCH_CHECK(h, "format_gauge_kernel");
     return DD_OK;
 }
