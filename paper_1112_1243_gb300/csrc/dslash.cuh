@@ -193,107 +193,113 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
 // FP64 hop on the two-limb integers of xfix.cuh (in: SpinorX, links: LinkX).
 // SOut = SpinorX: out = hops; SOut = SpinorF64: out = (has_x ? xin : 0) + b *
 // hops, or rhat - (xin + b * hops) with resid, and |out|^2 to A.red.
+//
+// A block of four warps takes 32 sites: warp w makes the two hops along axis
+// w (a lane a site), leaves their sum and difference in shared memory, and
+// all threads add up the axes (four lanes a site, one spin each).  A site is
+// a chain of 4000 instructions: with all hops in one lane (128 registers, 16
+// warps an SM) 2^20 sites took 537 us, 128 sites 21 us; here 508 and 10 us
+// (8 x 16384 sites: 28 -> 15 us).  Two lanes a site with one spin each took
+// 2.5 times the instructions and 830 us.  At 2^20 sites what is left is
+// latency: 20 warps an SM (96 registers), DRAM at 45%, issue slots at 32%.
 template <class SX, class SOut, int MASK>
-__global__ void __launch_bounds__(128, 4) hop_x_kernel(HopArgs<SpinorX, SX, SOut, LinkX> A) {
+__global__ void __launch_bounds__(128, 5) hop_x_kernel(HopArgs<SpinorX, SX, SOut, LinkX> A) {
+    __shared__ long long part[4][24][X_PAD];  // axis; sum (0..11) and difference (12..23) of its hops
+    __shared__ int ex[4][X_TILE], hs[X_TILE];
     const int rhs = blockIdx.y;
     if (A.st && !A.st[rhs].active) return;
     const Geo& g = A.g;
     const long long Vh = g.Vh;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (A.sites && threadIdx.x == 0)
-        atomicAdd(A.sites, (unsigned long long)min((long long)blockDim.x, A.S.n - (long long)blockIdx.x * blockDim.x));
-    double nrm = 0.0;
-    if (t < A.S.n) {
+    const int lane = threadIdx.x & 31, a = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);  // uniform in the warp
+    const long long base = (long long)blockIdx.x * X_TILE;
+    if (A.sites && threadIdx.x == 0) atomicAdd(A.sites, (unsigned long long)min((long long)X_TILE, A.S.n - base));
+    auto site = [&](int i, int x[4]) -> int {  // even-odd index and coordinates of site i of the tile
+        const long long t = min(base + i, A.S.n - 1);
+        if (A.S.colour >= 0) return colour_site(g, A.S.colour, (int)t, A.p, x);
+        const int h = (int)A.S.at(t);
+        eo_coords(g, A.p, h, x);
+        return h;
+    };
+    {
         int x[4];
-        int h;
-        if (A.S.colour >= 0) {
-            h = colour_site(g, A.S.colour, (int)t, A.p, x);
-        } else {
-            h = (int)A.S.at(t);
-            eo_coords(g, A.p, h, x);
-        }
+        const int h = site(lane, x);
         const int s = canon_index(g, x);
         const SpinorX in = at_rhs(A.in, rhs);
         const int4* lk = A.lk.p + (long long)rhs * A.lk_rhs_stride;
         const int* le = LinkX{lk, A.lk.stride}.exps();
-        // neighbour d = 2 a (forward) or 2 a + 1 (backward): its index, the
-        // index and parity of the link; false when the hop is dropped
-        auto hop_at = [&](int d, int& yh, long long& lrow) {
-            const int a = d >> 1;
-            const bool fwd = !(d & 1);
-            const int xa = a == 0 ? x[0] : a == 1 ? x[1] : a == 2 ? x[2] : x[3];
-            const int La = g.L[a];
-            const bool edge = xa == (fwd ? La - 1 : 0);
-            const int step = edge ? -(La - 1) * g.st[a] : g.st[a];
-            yh = (fwd ? s + step : s - step) >> 1;
-            lrow = (long long)((fwd ? A.p : 1 - A.p) * 4 + a);
-            if (MASK) {
-                const int loc = xa - fast_div(xa, g.b[a], g.mb[a]) * g.b[a];
-                const bool face = loc == (fwd ? g.b[a] - 1 : 0);
-                if (MASK == 1 ? face : !face) return false;
-            }
-            return true;
-        };
-        int eout = 2 * X_ZERO;
-#pragma unroll 4
-        for (int d = 0; d < 8; ++d) {
-            int yh;
-            long long lrow;
-            if (hop_at(d, yh, lrow)) eout = max(eout, in.e[yh] + le[lrow * Vh + ((d & 1) ? yh : h)]);
+        const int xa = a == 0 ? x[0] : a == 1 ? x[1] : a == 2 ? x[2] : x[3];
+        const int La = g.L[a], sa = g.st[a];
+        const bool top = xa == La - 1, bottom = xa == 0;
+        const int yf = (top ? s - (La - 1) * sa : s + sa) >> 1, yb = (bottom ? s + (La - 1) * sa : s - sa) >> 1;
+        const long long rf = (long long)(A.p * 4 + a) * Vh + h, rb = (long long)((1 - A.p) * 4 + a) * Vh + yb;
+        bool okf = true, okb = true;
+        if (MASK) {
+            const int loc = xa - fast_div(xa, g.b[a], g.mb[a]) * g.b[a];
+            const bool ff = loc == g.b[a] - 1, fb = loc == 0;
+            okf = MASK == 1 ? !ff : ff;
+            okb = MASK == 1 ? !fb : fb;
         }
-        xacc acc[12];
-#pragma unroll
-        for (int k = 0; k < 12; ++k) acc[k].x = acc[k].y = 0;
-#pragma unroll 1
-        for (int d = 0; d < 8; ++d) {
-            int yh;
-            long long lrow;
-            if (!hop_at(d, yh, lrow)) continue;
-            const int a = d >> 1;
-            const bool fwd = !(d & 1);
-            const int lh = fwd ? h : yh;
-            const int shift = min(eout - (in.e[yh] + le[lrow * Vh + lh]), 62);
-            const bool flip = a == 3 && g.bc < 0 && x[3] == (fwd ? g.L[3] - 1 : 0);
-            x_hop(a, fwd, A.g5in ? -1 : 0, flip, shift, in, yh, lk + lrow * 9 * Vh + lh, Vh, acc);
-        }
-        if constexpr (std::is_same<SOut, SpinorX>::value) {
-            x_store_acc(at_rhs(A.out, rhs), h, acc, eout);
-        } else {
-            const bool bad = eout >= X_BAD_MIN;
-            double sc = 0.0;
-            const bool one = x_scale(eout, A.b, sc);
-            const bool none = eout <= X_ZERO / 2;
-            auto value = [&](long long v) -> double {
-                if (one) return (double)v;
-                if (bad) return __longlong_as_double(0x7ff8000000000000ll);
-                return none ? 0.0 : scalbn((double)v, eout - 56) * A.b;  // far from the exponents of one multiplier
-            };
-            if (!one) sc = 1.0;
-            const bool zeroed = A.colour_mask != 3 && !((A.colour_mask >> block_colour_of(g, x)) & 1);
-            const double sg = A.g5out ? -sc : sc;
-            Spinor<double> res;
-            if (A.has_x)
-                at_rhs(A.xin, rhs).load(h, res);
-            else
-                zero(res);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                const double f = k < 6 ? sc : sg;
-                res.c[k].x = fma(f, value(acc[k].x), res.c[k].x);
-                res.c[k].y = fma(f, value(acc[k].y), res.c[k].y);
-            }
-            if (A.resid) {
-                Spinor<double> bv;
-                at_rhs(A.rhat, rhs).load(h, bv);
-#pragma unroll
-                for (int k = 0; k < 12; ++k) res.c[k] = bv.c[k] - res.c[k];
-            }
-            if (zeroed) zero(res);
-            at_rhs(A.out, rhs).store(h, res);
-            if (A.red.op != FIN_NONE) nrm = snorm2(res);
-        }
+        const int ef = okf ? in.e[yf] + le[rf] : 2 * X_ZERO, eb = okb ? in.e[yb] + le[rb] : 2 * X_ZERO;
+        ex[a][lane] = max(ef, eb);
+        __syncthreads();
+        const int eout = max(max(ex[0][lane], ex[1][lane]), max(ex[2][lane], ex[3][lane]));
+        if (a == 0) hs[lane] = h;
+        const bool phase = a == 3 && g.bc < 0;
+        x_axis(a, A.g5in != 0, okf, eout - ef, in.p, in.stride, (unsigned)yf * 16u, lk + (long long)(A.p * 4 + a) * 9 * Vh,
+               (unsigned)h * 16u, phase && top, okb, eout - eb, (unsigned)yb * 16u,
+               lk + (long long)((1 - A.p) * 4 + a) * 9 * Vh, (unsigned)yb * 16u, phase && bottom, Vh, part[a], lane);
     }
-    if constexpr (!std::is_same<SOut, SpinorX>::value) {
+    __syncthreads();
+    const int i = 8 * a + (lane & 7), q = lane >> 3;  // spin q of site i
+    const bool valid = base + i < A.S.n;
+    const int h = hs[i];
+    const int eout = max(max(ex[0][i], ex[1][i]), max(ex[2][i], ex[3][i]));
+    xacc v[3];
+    x_gather(part, i, q, v);
+    if constexpr (std::is_same<SOut, SpinorX>::value) {
+        unsigned long long any = x_mag(v[0]) | x_mag(v[1]) | x_mag(v[2]);
+        any |= __shfl_xor_sync(0xffffffffu, any, 8);
+        any |= __shfl_xor_sync(0xffffffffu, any, 16);
+        if (valid) {
+            const SpinorX out = at_rhs(A.out, rhs);
+            const int sh = x_norm_shift(any);
+            if (q == 0) out.e[h] = x_norm_exponent(any, eout, sh);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) out.p[(3 * q + c) * out.stride + h] = x_normalise(v[c], sh);
+        }
+    } else {
+        double nrm = 0.0;
+        if (valid) {
+            bool zeroed = false;
+            if (A.colour_mask != 3) {
+                int x[4];
+                site(i, x);
+                zeroed = !((A.colour_mask >> block_colour_of(g, x)) & 1);
+            }
+            const SX xin = at_rhs(A.xin, rhs), bv = at_rhs(A.rhat, rhs);
+            const SOut out = at_rhs(A.out, rhs);
+            // sums times 2^(eout - 56) b: one multiplier where it is a normal
+            // number (conversion and FMA run on the FP64 pipe beside the
+            // integer pipes: 30 clocks a site)
+            const double f0 = (q > 1 && A.g5out) ? -A.b : A.b;
+            const bool usual = abs(eout) < 900;
+            const double f = usual ? __hiloint2double((eout - 56 + 1023) << 20, 0) * f0 : f0;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const long long k = (3 * q + c) * out.stride + h;
+                const double2 w = A.has_x ? xin.p[k] : make_double2(0.0, 0.0);
+                double2 z = make_double2((double)v[c].x, (double)v[c].y);
+                if (!usual) z = make_double2(x_to_double_any(v[c].x, eout), x_to_double_any(v[c].y, eout));
+                z = make_double2(fma(f, z.x, w.x), fma(f, z.y, w.y));
+                if (A.resid) {
+                    const double2 w = bv.p[k];
+                    z = make_double2(w.x - z.x, w.y - z.y);
+                }
+                if (zeroed) z = make_double2(0.0, 0.0);
+                out.p[k] = z;
+                if (A.red.op != FIN_NONE) nrm = fma(z.x, z.x, fma(z.y, z.y, nrm));
+            }
+        }
         if (A.red.op != FIN_NONE) grid_reduce(A.red, rhs, nrm);
     }
 }
@@ -315,12 +321,9 @@ inline void launch_hop(const HopArgs<SIn, SX, SOut, LK>& A, int nrhs, dd_handle*
     // which keeps the grid within the reduction partials)
     constexpr bool f64 = std::is_same<SIn, SpinorX>::value;
     int tpb = std::min(f64 ? h->tune.hop64_tpb : h->tune.hop_tpb, 128);  // the kernels' launch bound
-    // one warp per thread block while that leaves SMs without work (the FP64
-    // hop of one site is about 4000 instructions long)
-    if (f64)
-        while (tpb > 32 && (long long)grid_for(B.S.n, tpb) * nrhs < h->num_sms) tpb >>= 1;
+    if (f64) tpb = 128;  // four warps (hop_x_kernel)
     const int spt = (!f64 && h->tune.hop_spt == 2) ? 2 : 1;
-    dim3 grid(grid_for(B.S.n, (long long)tpb * spt), nrhs);
+    dim3 grid(grid_for(B.S.n, f64 ? X_TILE : (long long)tpb * spt), nrhs);
     constexpr int kind0 = hop_kind<SIn, SOut>();
     // whole-lattice hops keep kinds 0-2; Dirichlet hops are timed as 4 (FP64),
     // 5, 6 (one block colour's sites) or 8, 9 (every site)

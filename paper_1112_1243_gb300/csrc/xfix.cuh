@@ -20,11 +20,6 @@
 // Entries that are not finite mark their site or link (X_BAD): every result
 // they enter is NaN.  Subnormal entries count as zero.
 //
-// hop_x_kernel, one thread per output site, is bound by HBM (links 1184,
-// spinors 196 + 192 bytes a site) and the 1728 multiply-adds (27 clocks a
-// site of one SM at 64 lanes).  A runtime loop over the hops keeps it inside
-// the instruction cache; exponents are read twice (the second time from L1)
-// so that every hop is shifted to the largest exponent of the eight.
 #pragma once
 
 #include "dd_common.cuh"
@@ -56,15 +51,6 @@ DD_DEV int x_exponent(int maxhi, int& E) {
     E = maxhi >> 20;
     return E == 0x7ff ? X_BAD : (E == 0 ? X_ZERO : E - 1022);
 }
-// acc 2^(e - 56) scaled by b: the multiplier where it is a normal number
-// (one rounding), else false
-DD_DEV bool x_scale(int e, double b, double& sc) {
-    const int k = e - 56;
-    if (k < -900 || k > 900) return false;
-    sc = __hiloint2double((k + 1023) << 20, 0) * b;
-    return true;
-}
-
 // Spinor in limbs: chunk k (spin * 3 + colour) of site i at p[k * stride + i]
 // as (re.hi, re.lo, im.hi, im.lo), its exponent at e[i]
 struct SpinorX {
@@ -103,23 +89,26 @@ struct LinkX {
     static long long field_chunks(long long Vh) { return 72 * Vh + 2 * Vh; }
     DD_HD const int* exps() const { return reinterpret_cast<const int*>(p + 72 * stride); }
 };
-// one link, entries u[0..8] (re, im), into the formatted field
-DD_DEV void x_store_link(int4* p, long long stride, int par, int a, long long h, const double* u) {
+// one link, entries u[0..8] (re, im): entry k at p[k * stride], exponent at *e
+DD_DEV void x_store_entries(int4* p, long long stride, int* e, const double* u) {
     int m = 0;
 #pragma unroll
     for (int k = 0; k < 18; ++k) m = max(m, __double2hiint(u[k]) & 0x7fffffff);
     int E;
-    reinterpret_cast<int*>(p + 72 * stride)[(long long)(par * 4 + a) * stride + h] = x_exponent(m, E);
-    int4* o = p + (long long)(par * 4 + a) * 9 * stride + h;
+    *e = x_exponent(m, E);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         const int2 x = x_split(x_from_double(u[2 * k], E, 59)), y = x_split(x_from_double(u[2 * k + 1], E, 59));
-        o[k * stride] = make_int4(x.x, x.y, y.x, y.y);
+        p[k * stride] = make_int4(x.x, x.y, y.x, y.y);
     }
 }
+// ... of a field in the layout of LinkX
+DD_DEV void x_store_link(int4* p, long long stride, int par, int a, long long h, const double* u) {
+    x_store_entries(p + (long long)(par * 4 + a) * 9 * stride + h, stride,
+                    reinterpret_cast<int*>(p + 72 * stride) + (long long)(par * 4 + a) * stride + h, u);
+}
 
-// complex numbers of the hop: limbs of one projected component, and a
-// 64-bit result
+// ------------------------------------------------------------ one hop
 struct xlimb {
     int rh, rl, ih, il;
 };
@@ -128,158 +117,186 @@ struct xacc {
 };
 DD_DEV long long x_neg_if(long long v, long long m) { return (v ^ m) - m; }  // m = 0 or -1
 
-// a + s b limb by limb (m = 0: s = +1, m = -1: s = -1)
-DD_DEV xlimb x_add(int4 a, int br_h, int br_l, int mr, int bi_h, int bi_l, int mi) {
-    xlimb o;
-    o.rh = a.x + (br_h ^ mr) - mr;
-    o.rl = a.y + (br_l ^ mr) - mr;
-    o.ih = a.z + (bi_h ^ mi) - mi;
-    o.il = a.w + (bi_l ^ mi) - mi;
-    return o;
+// line of three projected components: u + l or u - l (NEG), ROT: u +- i l
+// with i z = (-z.y, z.x)
+template <bool ROT>
+DD_DEV void x_line(bool neg, const int4* u, const int4* l, xlimb* h) {
+    if (neg) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            h[c] = ROT ? xlimb{u[c].x + l[c].z, u[c].y + l[c].w, u[c].z - l[c].x, u[c].w - l[c].y}
+                       : xlimb{u[c].x - l[c].x, u[c].y - l[c].y, u[c].z - l[c].z, u[c].w - l[c].w};
+    } else {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            h[c] = ROT ? xlimb{u[c].x - l[c].z, u[c].y - l[c].w, u[c].z + l[c].x, u[c].w + l[c].y}
+                       : xlimb{u[c].x + l[c].x, u[c].y + l[c].y, u[c].z + l[c].z, u[c].w + l[c].w};
+    }
 }
-// (i sigma_a v) for a = 0, 1, 2 acts on the spin pair by a swap of spins
-// (a = 0, 1), a factor i (a = 0, 2) and signs; the time direction (a = 3)
-// has the identity.  fac: spin 0 gets f0, spin 1 gets f1 = f0 or -f0.
-//   a = 0: (i v1, i v0)   a = 1: (v1, -v0)   a = 2: (i v0, -i v1)   a = 3: (v0, v1)
+// entry k of a field of entries 16 bytes wide: a uniform base plus a 32-bit
+// lane offset (a parity has less than 2^28 sites), one address register a lane
+DD_DEV int4 x_load(const int4* base, long long k, unsigned off) {
+    return *reinterpret_cast<const int4*>(reinterpret_cast<const char*>(base + k) + off);
+}
+// (i sigma_a v) is, for a = 0: (i v1, i v0), 1: (v1, -v0), 2: (i v0, -i v1);
+// the time direction (a = 3) has the identity: (v0, v1).
 
-// h = upper + sg (i sigma_a lower) (a = 3: upper + sg lower), m = 0 / -1 for sg = +1 / -1
-DD_DEV void x_project(int a, int m, const SpinorX& in, long long y, xlimb* h) {
-    const int4* p = in.p + y;
-    const long long cs = in.stride;
-    const int s0 = (a < 2) ? 9 : 6, s1 = 15 - s0;    // lower chunks that meet spin 0 and spin 1
-    const int m1 = (a == 1 || a == 2) ? ~m : m;      // sign of the spin-1 line
+// h = upper + sg (i sigma_a lower) (a = 3: upper + sg lower), neg: sg = -1;
+// entry k of the source spinor is x_load(base, k * cs, off).  a and neg are
+// uniform in a warp.
+DD_DEV void x_project(int a, bool neg, const int4* base, long long cs, unsigned off, xlimb* h) {
+    const int s0 = (a < 2) ? 9 : 6, s1 = 15 - s0;            // lower entries that meet spin 0 and spin 1
+    const bool neg1 = (a == 1 || a == 2) ? !neg : neg;       // sign of the spin-1 line
     int4 u[6], l[6];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        u[c] = p[c * cs];
-        u[3 + c] = p[(3 + c) * cs];
-        l[c] = p[(s0 + c) * cs];
-        l[3 + c] = p[(s1 + c) * cs];
+        u[c] = x_load(base, c * cs, off);
+        u[3 + c] = x_load(base, (3 + c) * cs, off);
+        l[c] = x_load(base, (s0 + c) * cs, off);
+        l[3 + c] = x_load(base, (s1 + c) * cs, off);
     }
-    if (a == 0 || a == 2) {  // + sg i z: (-z.y, z.x)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            h[c] = x_add(u[c], l[c].z, l[c].w, ~m, l[c].x, l[c].y, m);
-            h[3 + c] = x_add(u[3 + c], l[3 + c].z, l[3 + c].w, ~m1, l[3 + c].x, l[3 + c].y, m1);
-        }
+    if (a & 1) {
+        x_line<false>(neg, u, l, h);
+        x_line<false>(neg1, u + 3, l + 3, h + 3);
     } else {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            h[c] = x_add(u[c], l[c].x, l[c].y, m, l[c].z, l[c].w, m);
-            h[3 + c] = x_add(u[3 + c], l[3 + c].x, l[3 + c].y, m1, l[3 + c].z, l[3 + c].w, m1);
-        }
+        x_line<true>(neg, u, l, h);
+        x_line<true>(neg1, u + 3, l + 3, h + 3);
     }
 }
 
-// acc += v on the upper spins, and the lower spins that belong to it:
-// a = 3: + sg v, else - sg i sigma_a v
-DD_DEV void x_accumulate(int a, long long m, const xacc* v, xacc* acc) {
+// One row of the product of a link with one spin of h, in units of
+// 2^(e_out - 56), e_out = shift + the exponents of link and source (shift
+// 0..62).  u: the row's three entries; f, q: h's partners of the imaginary
+// part in the real and imaginary sums, (-im, re) for U and (im, -re) for its
+// adjoint; half = 2^(shift - 1): the shift rounds to nearest (|sums| < 2^61).
+DD_DEV xacc x_row(const int4* u, const xlimb* h, const int2* f, const int2* q, long long half, int shift) {
+    long long hr = half, hi = half, cr = 1 << 29, ci = 1 << 29;  // cross sums rounded to nearest
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        hr += (long long)u[j].x * h[j].rh;
+        hi += (long long)u[j].x * h[j].ih;
+        cr += (long long)u[j].x * h[j].rl;
+        ci += (long long)u[j].x * h[j].il;
+        hr += (long long)u[j].z * f[j].x;
+        hi += (long long)u[j].z * q[j].x;
+        cr += (long long)u[j].y * h[j].rh;
+        ci += (long long)u[j].y * h[j].ih;
+        cr += (long long)u[j].z * f[j].y;
+        ci += (long long)u[j].z * q[j].y;
+        cr += (long long)u[j].w * f[j].x;
+        ci += (long long)u[j].w * q[j].x;
+    }
+    xacc v;
+    v.x = (hr + (cr >> 30)) >> shift;
+    v.y = (hi + (ci >> 30)) >> shift;
+    return v;
+}
+// v = U h (FWD) or U^dag h; entry(k) = entry k of the link; put(k, value)
+// receives entry k = 3 spin + colour
+template <bool FWD, class Entry, class Put>
+DD_DEV void x_multiply(int shift, const xlimb* h, Entry entry, Put put) {
+    const long long half = (1ll << shift) >> 1;
+    int2 f[6], q[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-        acc[k].x += v[k].x;
-        acc[k].y += v[k].y;
+        f[k] = FWD ? make_int2(-h[k].ih, -h[k].il) : make_int2(h[k].ih, h[k].il);
+        q[k] = FWD ? make_int2(h[k].rh, h[k].rl) : make_int2(-h[k].rh, -h[k].rl);
     }
-    if (a == 3) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            acc[6 + k].x += x_neg_if(v[k].x, m);
-            acc[6 + k].y += x_neg_if(v[k].y, m);
-        }
-    } else if (a == 1) {  // -sg (v1, -v0)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            acc[6 + c].x += x_neg_if(v[3 + c].x, ~m);
-            acc[6 + c].y += x_neg_if(v[3 + c].y, ~m);
-            acc[9 + c].x += x_neg_if(v[c].x, m);
-            acc[9 + c].y += x_neg_if(v[c].y, m);
-        }
-    } else if (a == 0) {  // -sg (i v1, i v0), i z = (-z.y, z.x)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            acc[6 + c].x += x_neg_if(v[3 + c].y, m);
-            acc[6 + c].y += x_neg_if(v[3 + c].x, ~m);
-            acc[9 + c].x += x_neg_if(v[c].y, m);
-            acc[9 + c].y += x_neg_if(v[c].x, ~m);
-        }
-    } else {  // -sg (i v0, -i v1)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            acc[6 + c].x += x_neg_if(v[c].y, m);
-            acc[6 + c].y += x_neg_if(v[c].x, ~m);
-            acc[9 + c].x += x_neg_if(v[3 + c].y, ~m);
-            acc[9 + c].y += x_neg_if(v[3 + c].x, m);
-        }
-    }
-}
-
-// One hop onto acc (24 integers in units of 2^(e_out - 56)).  lp: the link's
-// first entry, cs its chunk stride; fwd: U h, else U^dag h; mg5: -1 when the
-// input is taken with gamma5; flip: the hop carries the fermion phase -1;
-// shift = e_out - (exponents of the link and the site).
-DD_DEV void x_hop(int a, bool fwd, int mg5, bool flip, int shift, const SpinorX& in, long long y, const int4* lp,
-                  long long cs, xacc* acc) {
-    const int m = fwd ? 0 : -1;
-    xlimb h[6];
-    x_project(a, m ^ mg5, in, y, h);
-    xacc v[6];
-    const long long half = (1ll << shift) >> 1;  // the shift rounds to nearest (shift <= 62, |sums| < 2^61)
-    const int mre = ~m, mim = m;  // signs of the link's imaginary part in the real and imaginary sums
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        xlimb u[3];
+        int4 u[3];
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const int4 w = lp[(fwd ? 3 * i + j : 3 * j + i) * cs];
-            u[j] = xlimb{w.x, w.y, w.z, w.w};
-        }
+        for (int j = 0; j < 3; ++j) u[j] = entry(FWD ? 3 * i + j : 3 * j + i);
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            long long hr = half, hi = half, cr = 1 << 29, ci = 1 << 29;  // cross sums rounded to nearest
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const xlimb w = h[3 * s + j];
-                const int rih = (u[j].ih ^ mre) - mre, ril = (u[j].il ^ mre) - mre;
-                const int iih = (u[j].ih ^ mim) - mim, iil = (u[j].il ^ mim) - mim;
-                hr += (long long)u[j].rh * w.rh;
-                hr += (long long)rih * w.ih;
-                cr += (long long)u[j].rh * w.rl;
-                cr += (long long)u[j].rl * w.rh;
-                cr += (long long)rih * w.il;
-                cr += (long long)ril * w.ih;
-                hi += (long long)u[j].rh * w.ih;
-                hi += (long long)iih * w.rh;
-                ci += (long long)u[j].rh * w.il;
-                ci += (long long)u[j].rl * w.ih;
-                ci += (long long)iih * w.rl;
-                ci += (long long)iil * w.rh;
-            }
-            v[3 * s + i].x = (hr + (cr >> 30)) >> shift;
-            v[3 * s + i].y = (hi + (ci >> 30)) >> shift;
-        }
+        for (int s = 0; s < 2; ++s) put(3 * s + i, x_row(u, h + 3 * s, f + 3 * s, q + 3 * s, half, shift));
     }
-    if (flip) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            v[k].x = -v[k].x;
-            v[k].y = -v[k].y;
-        }
-    }
-    x_accumulate(a, m, v, acc);
 }
 
-// acc 2^(e - 56) -> limbs and exponent of an output spinor
-DD_DEV void x_store_acc(const SpinorX& out, long long i, const xacc* acc, int e) {
-    unsigned long long any = 0;
+// The forward and backward hop along axis a of one site, a lane each site:
+// sum (entries 0..11) and difference (12..23) of the products to part.  yf,
+// yb: byte offsets of the neighbours in entry 0 of the source; kf, kb: of the
+// links in entry 0 of the fields lf, lb; sf, sb: shifts (0 or more); flip:
+// the hop carries the fermion phase -1.
+constexpr int X_TILE = 32, X_PAD = 36;  // sites of a tile; padded row (two spins' reads meet different banks)
+DD_DEV void x_axis(int a, bool g5, bool okf, int sf, const int4* src, long long cs, unsigned yf, const int4* lf,
+                   unsigned kf, bool flipf, bool okb, int sb, unsigned yb, const int4* lb, unsigned kb, bool flipb,
+                   long long cl, long long (*part)[X_PAD], int lane) {
+    xacc vf[6];
 #pragma unroll
-    for (int k = 0; k < 12; ++k)
-        any |= (unsigned long long)(acc[k].x ^ (acc[k].x >> 63)) | (unsigned long long)(acc[k].y ^ (acc[k].y >> 63));
-    const int sh = any ? 7 - __clzll((long long)any) : 0;  // bits above 57
-    const int r = max(sh, 0), l = max(-sh, 0);
-    const long long half = r ? 1ll << (r - 1) : 0;
-    out.e[i] = e >= X_BAD_MIN ? X_BAD : (any == 0 ? X_ZERO : e + 1 + sh);
+    for (int k = 0; k < 6; ++k) vf[k].x = vf[k].y = 0;
+    if (okf) {
+        xlimb h[6];
+        x_project(a, g5, src, cs, yf, h);
+        x_multiply<true>(min(sf, 62), h, [&](int k) { return x_load(lf, k * cl, kf); },
+                         [&](int k, xacc v) { vf[k] = v; });
+        if (flipf) {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const int2 x = x_split(((acc[k].x + half) >> r) << l), y = x_split(((acc[k].y + half) >> r) << l);
-        out.p[k * out.stride + i] = make_int4(x.x, x.y, y.x, y.y);
+            for (int k = 0; k < 6; ++k) {
+                vf[k].x = -vf[k].x;
+                vf[k].y = -vf[k].y;
+            }
+        }
     }
+    // a backward hop with the phase enters with the opposite sign: sum and
+    // difference trade places
+    const int ks = flipb ? 12 : 0, kd = 12 - ks;
+    if (okb) {
+        xlimb h[6];
+        x_project(a, !g5, src, cs, yb, h);
+        x_multiply<false>(min(sb, 62), h, [&](int k) { return x_load(lb, k * cl, kb); }, [&](int k, xacc v) {
+            part[ks + 2 * k][lane] = vf[k].x + v.x;
+            part[ks + 2 * k + 1][lane] = vf[k].y + v.y;
+            part[kd + 2 * k][lane] = vf[k].x - v.x;
+            part[kd + 2 * k + 1][lane] = vf[k].y - v.y;
+        });
+    } else {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            part[2 * k][lane] = part[12 + 2 * k][lane] = vf[k].x;
+            part[2 * k + 1][lane] = part[13 + 2 * k][lane] = vf[k].y;
+        }
+    }
+}
+// spin q of site i from the four axes: the sums of the hops' upper spins, and
+// what they give to the lower ones, - i sigma_a (forward - backward), time:
+// + the difference
+DD_DEV void x_gather(const long long (*part)[24][X_PAD], int i, int q, xacc* v) {
+    const int r = q & 1;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const int own = 2 * (3 * r + c), other = 2 * (3 * (1 - r) + c);
+        if (q < 2) {
+            v[c].x = part[0][own][i] + part[1][own][i] + part[2][own][i] + part[3][own][i];
+            v[c].y = part[0][own + 1][i] + part[1][own + 1][i] + part[2][own + 1][i] + part[3][own + 1][i];
+        } else {
+            const long long (*d0)[X_PAD] = part[0] + 12, (*d1)[X_PAD] = part[1] + 12, (*d2)[X_PAD] = part[2] + 12,
+                            (*d3)[X_PAD] = part[3] + 12;
+            const long long m = r ? -1 : 0;
+            v[c].x = d0[other + 1][i] + x_neg_if(d1[other][i], ~m) + x_neg_if(d2[own + 1][i], m) + d3[own][i];
+            v[c].y = -d0[other][i] + x_neg_if(d1[other + 1][i], ~m) + x_neg_if(d2[own][i], ~m) + d3[own + 1][i];
+        }
+    }
+}
+
+// magnitude bits of a set of sums: OR of these, then x_bits
+DD_DEV unsigned long long x_mag(xacc v) {
+    return (unsigned long long)(v.x ^ (v.x >> 63)) | (unsigned long long)(v.y ^ (v.y >> 63));
+}
+// right (> 0) or left shift that brings sums with magnitude bits `any` to 57 bits
+DD_DEV int x_norm_shift(unsigned long long any) { return any ? 7 - __clzll((long long)any) : 0; }
+DD_DEV int x_norm_exponent(unsigned long long any, int e, int sh) {
+    return e >= X_BAD_MIN ? X_BAD : (any == 0 ? X_ZERO : e + 1 + sh);
+}
+DD_DEV int4 x_normalise(xacc v, int sh) {
+    const int r = max(sh, 0), l = max(-sh, 0);
+    const long long half = (1ll << r) >> 1;
+    const int2 x = x_split(((v.x + half) >> r) << l), y = x_split(((v.y + half) >> r) << l);
+    return make_int4(x.x, x.y, y.x, y.y);
+}
+
+// v 2^(e - 56) for any exponent: subnormal results, and NaN where a source or
+// link was not finite
+static __device__ __noinline__ double x_to_double_any(long long v, int e) {
+    if (e >= X_BAD_MIN) return __longlong_as_double(0x7ff8000000000000ll);
+    return e <= X_ZERO / 2 ? 0.0 : scalbn((double)v, e - 56);
 }

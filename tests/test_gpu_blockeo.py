@@ -1,0 +1,64 @@
+"""The persistent block solver in even-odd form (block_eo_kernel) against the
+oracle: block shapes with odd extents along any axis (vectors kept at full
+length for an odd extent along axis 0), one- and two-site extents, more and
+fewer sites than threads, every thread-block size, unchanged blocks."""
+import numpy as np
+import pytest
+
+from gpu_util import dev, host, lib_api
+from oracle import estimator, geometry, heatbath
+from oracle.interp import interpolate
+from paper_1112_1243_gb300 import synthetic
+
+pytestmark = pytest.mark.gpu
+KAPPA = 0.12
+
+
+@pytest.fixture(scope="module")
+def api():
+    return lib_api()
+
+
+def reference(U, Up, lat, n, seed, ctr):
+    """ln_b of the oracle (solves to 1e-14) and the error that a relative
+    residual of 1e-12 leaves: |delta ln| <= 2 (|eta| + |d|) |D_b^-1| 1e-12 |b|
+    per factor, |D_b^-1| <= 1 / (1 - 8 kappa) for unitary links."""
+    ln, tol = np.zeros(lat.nblocks), np.zeros(lat.nblocks)
+    for i in range(n):
+        Pi = estimator.Pieces(interpolate(U, Up, i / n, lat.active), lat, KAPPA)
+        Pj = estimator.Pieces(interpolate(U, Up, (i + 1) / n, lat.active), lat, KAPPA)
+        eta = estimator.block_noise(lat, i, seed, ctr)
+        b = Pi.dirichlet(eta) - Pj.dirichlet(eta)
+        d = Pj.dirichlet_solve(b)
+        per = lambda v: np.bincount(lat.block_id, weights=v, minlength=lat.nblocks)
+        sq = lambda v: np.sqrt(per(np.sum(np.abs(v) ** 2, axis=(1, 2))))
+        ln += per(-(2 * np.sum(np.conj(eta) * d, axis=(1, 2)).real + np.sum(np.abs(d) ** 2, axis=(1, 2))))
+        tol += 2 * (sq(eta) + sq(d)) / (1 - 8 * KAPPA) * 1e-12 * sq(b)
+    return ln, tol + 1e-12
+
+
+@pytest.mark.parametrize("dims,block,tpb", [
+    ((6, 6, 6, 6), (3, 3, 3, 3), 256),
+    ((6, 4, 4, 10), (3, 2, 2, 5), 64),
+    ((4, 6, 10, 6), (2, 3, 5, 3), 128),
+    ((8, 8, 8, 8), (4, 4, 4, 4), 256),
+    ((8, 8, 8, 8), (4, 4, 4, 4), 64),
+    ((12, 8, 4, 8), (6, 4, 2, 4), 256),
+    ((2, 4, 4, 4), (1, 2, 2, 2), 256),
+    ((20, 8, 8, 8), (5, 4, 4, 4), 128),
+])
+def test_block_shapes(api, dims, block, tpb):
+    n = 2
+    lat = geometry.Lattice(dims, block)
+    U = synthetic.random_gauge(dims, 0.3, 4)
+    cm = 1 if lat.active_mode == "intra" else 3
+    Up, _ = heatbath.gauge_update(U, lat, 5.3, 1, 0, 21, 4, colour_mask=cm)
+    h = api.dd_init(dims, block, KAPPA, max_rhs=n)
+    api.dd_set_tuning(h, block_tpb=tpb, block_ctas_per_sm=2)
+    ref, tol = reference(U, Up, lat, n, 9, 3)
+    got = host(api.dd_block_ratios_range(h, dev(U), dev(Up), 0, lat.nblocks, n, 9, 3))
+    assert np.all(np.abs(got - ref) <= tol)
+    assert api.dd_status(h)[0] == 0
+    # nothing proposed: exactly zero
+    got = host(api.dd_block_ratios_range(h, dev(U), dev(U), 0, lat.nblocks, n, 9, 3))
+    assert np.all(got == 0)
