@@ -23,9 +23,26 @@
 // block has 128 sites a parity and fills 256 threads.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include "blocksolve.cuh"
 #include "dfhop.cuh"
 #include "dslash.cuh"
+
+// The thread blocks that work on one item: one, or the whole cluster of a
+// large block (X_COOP_SITES).  Warps are numbered through the team.
+struct EoTeam {
+    int rank, size;
+    DD_DEV int warp() const { return rank * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5); }
+    DD_DEV int warps() const { return size * (int)(blockDim.x >> 5); }
+    // barrier of the team; writes before it, also to global memory, are visible after it
+    DD_DEV void sync() const {
+        if (size > 1)
+            cooperative_groups::this_cluster().sync();
+        else
+            __syncthreads();
+    }
+};
 
 struct EoSite {
     int l[4];
@@ -133,12 +150,12 @@ struct EoSums {
 };
 
 // out = Dtilde in (th: odd temporary); with ALL all six sums, else the first
-// two.  Every thread of the block calls this; in is complete, out is written
+// two.  Every thread of the team calls this; in is complete, out is written
 // by the lanes that own its entries (no barrier at the end).
-__device__ __noinline__ void eo_dtilde(const EoCtx c, const float2* in, float2* th, float2* out, const float2* lk,
+__device__ __noinline__ void eo_dtilde(const EoCtx c, const EoTeam T, const float2* in, float2* th, float2* out, const float2* lk,
                                        const float2* rhat, bool all, EoSums& S) {
-    const int lane = threadIdx.x & 31, sp = lane >> 4, step = 16 * (blockDim.x >> 5);
-    const int first = 16 * (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31, sp = lane >> 4, step = 16 * T.warps();
+    const int first = 16 * T.warp();
     for (int t0 = first; t0 < c.count; t0 += step) {
         EoSite s;
         const bool ok = eo_site(c, 1, t0 + (lane & 15), s);
@@ -148,7 +165,7 @@ __device__ __noinline__ void eo_dtilde(const EoCtx c, const float2* in, float2* 
 #pragma unroll
             for (int k = 0; k < 6; ++k) th[lane_comp(sp, k) * c.half + s.idx] = make_float2(r[k].x, r[k].y);
     }
-    __syncthreads();
+    T.sync();
 #pragma unroll
     for (int k = 0; k < 6; ++k) S.v[k] = dfl{0.f, 0.f};
     for (int t0 = first; t0 < c.count; t0 += step) {
@@ -175,15 +192,35 @@ __device__ __noinline__ void eo_dtilde(const EoCtx c, const float2* in, float2* 
     }
 }
 
-// block-wide sums of n pairs in FP64, valid in every thread
+constexpr int EO_CLUSTER = 8;  // thread blocks of a team
 struct EoShared {
     dfl part[6][8];
     double tot[6];
+    double all[EO_CLUSTER][6];  // the team's totals, by rank
     double sh[34];
     int ex[2][4][X_TILE], hs[2][X_TILE];
     int item;
 };
-DD_DEV void eo_total(EoShared& M, const EoSums& S, int n, double* out) {
+// totals of the team from every thread block's M.tot (n values, set by the
+// first threads), in a fixed order; valid in every thread
+DD_DEV void eo_team_total(EoShared& M, const EoTeam& T, int n, double* out) {
+    if (T.size > 1) {
+        auto cl = cooperative_groups::this_cluster();
+        for (int k = threadIdx.x; k < n * T.size; k += blockDim.x)
+            cl.map_shared_rank(&M, k / n)->all[T.rank][k % n] = M.tot[k % n];
+        cl.sync();
+        for (int k = 0; k < n; ++k) {
+            double t = 0.0;
+            for (int r = 0; r < T.size; ++r) t += M.all[r][k];
+            out[k] = t;
+        }
+        cl.sync();  // every rank has read before the next totals arrive
+    } else {
+        for (int k = 0; k < n; ++k) out[k] = M.tot[k];
+    }
+}
+// sums of n pairs over the team, in FP64
+DD_DEV void eo_total(EoShared& M, const EoTeam& T, const EoSums& S, int n, double* out) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int k = 0; k < n; ++k) {
         dfl a = S.v[k];
@@ -201,7 +238,16 @@ DD_DEV void eo_total(EoShared& M, const EoSums& S, int n, double* out) {
         M.tot[threadIdx.x] = t;
     }
     __syncthreads();
-    for (int k = 0; k < n; ++k) out[k] = M.tot[k];
+    eo_team_total(M, T, n, out);
+}
+// sum of one FP64 value a thread over the team
+DD_DEV double eo_sum(EoShared& M, const EoTeam& T, double v) {
+    v = block_sum(v, M.sh);
+    if (T.size == 1) return v;
+    if (threadIdx.x == 0) M.tot[0] = v;
+    __syncthreads();
+    eo_team_total(M, T, 1, &v);
+    return v;
 }
 
 // ------------------------------------------------ BiCGStab on Dtilde (FP32)
@@ -215,19 +261,19 @@ struct EoVecs {
     float2 *x, *r, *rhat, *p, *v, *s, *t, *th;
 };
 template <class F>
-DD_DEV void eo_each(const EoCtx& c, F f) {  // f(offset of a component of an even site owned by this lane)
-    const int lane = threadIdx.x & 31, sp = lane >> 4, step = 16 * (blockDim.x >> 5);
-    for (int t0 = 16 * (threadIdx.x >> 5); t0 < c.count; t0 += step) {
+DD_DEV void eo_each(const EoCtx& c, const EoTeam& T, F f) {  // f(offset of a component of an even site owned by this lane)
+    const int lane = threadIdx.x & 31, sp = lane >> 4, step = 16 * T.warps();
+    for (int t0 = 16 * T.warp(); t0 < c.count; t0 += step) {
         EoSite s;
         if (!eo_site(c, 0, t0 + (lane & 15), s)) continue;
 #pragma unroll
         for (int k = 0; k < 6; ++k) f(lane_comp(sp, k) * c.half + s.idx);
     }
 }
-DD_DEV int eo_bicgstab(const EoCtx& c, EoShared& M, const EoVecs& V, const float2* lk, double tol2rel, int maxit) {
+DD_DEV int eo_bicgstab(const EoCtx& c, const EoTeam& T, EoShared& M, const EoVecs& V, const float2* lk, double tol2rel, int maxit) {
     EoSums S;
     dfl rr0{0.f, 0.f};
-    eo_each(c, [&](int at) {
+    eo_each(c, T, [&](int at) {
         const float2 r = V.r[at];
         V.x[at] = make_float2(0.f, 0.f);
         V.rhat[at] = V.p[at] = r;
@@ -235,26 +281,27 @@ DD_DEV int eo_bicgstab(const EoCtx& c, EoShared& M, const EoVecs& V, const float
     });
     S.v[0] = rr0;
     double d[6];
-    eo_total(M, S, 1, d);  // barriers: p complete
+    eo_total(M, T, S, 1, d);
     if (!(d[0] > 0.0)) return 0;
+    T.sync();  // p complete
     const double target = tol2rel * d[0];
     cpx<double> rho = mk<double>(d[0], 0.0);
     int it = 0;
     while (it < maxit) {
-        eo_dtilde(c, V.p, V.th, V.v, lk, V.rhat, false, S);
-        eo_total(M, S, 2, d);
+        eo_dtilde(c, T, V.p, V.th, V.v, lk, V.rhat, false, S);
+        eo_total(M, T, S, 2, d);
         const cpx<double> rv = mk<double>(d[0], d[1]);
         if (!(norm2(rv) > 0.0)) break;
         const cpx<double> alpha = (1.0 / norm2(rv)) * cmul(rho, conj(rv));
         const cpx<float> aR = mk<float>((float)alpha.x, (float)alpha.y);
-        eo_each(c, [&](int at) {
+        eo_each(c, T, [&](int at) {
             const float2 r = V.r[at], v = V.v[at];
             const cpx<float> w = mk<float>(r.x, r.y) - cmul(aR, mk<float>(v.x, v.y));
             V.s[at] = make_float2(w.x, w.y);
         });
-        __syncthreads();
-        eo_dtilde(c, V.s, V.th, V.t, lk, V.rhat, true, S);
-        eo_total(M, S, 6, d);
+        T.sync();
+        eo_dtilde(c, T, V.s, V.th, V.t, lk, V.rhat, true, S);
+        eo_total(M, T, S, 6, d);
         ++it;
         const cpx<double> rt = mk<double>(d[0], d[1]), ts = mk<double>(d[2], d[3]);
         const double tt = d[4], ss = d[5];
@@ -272,7 +319,7 @@ DD_DEV int eo_bicgstab(const EoCtx& c, EoShared& M, const EoVecs& V, const float
             last = !isfinite(beta.x) || !isfinite(beta.y);
         }
         const cpx<float> bR = mk<float>((float)beta.x, (float)beta.y);
-        eo_each(c, [&](int at) {
+        eo_each(c, T, [&](int at) {
             const float2 x2 = V.x[at], p2 = V.p[at], s2 = V.s[at];
             const cpx<float> p = mk<float>(p2.x, p2.y), s = mk<float>(s2.x, s2.y);
             const cpx<float> x = mk<float>(x2.x, x2.y) + cmul(aR, p) + cmul(wR, s);
@@ -286,7 +333,7 @@ DD_DEV int eo_bicgstab(const EoCtx& c, EoShared& M, const EoVecs& V, const float
         });
         if (last) break;
         rho = rho_new;
-        __syncthreads();
+        T.sync();
     }
     return it;
 }
@@ -299,16 +346,16 @@ struct EoX {
 // hops of in (parity 1 - par) onto the sites of parity par, four warps a tile
 // of 32 sites (as hop_x_kernel): to limbs (xo.p given), or out = b1 - b2 +
 // coef * hops (b2 may be null).  lx: links of the block, entries [a][9][nb],
-// le: exponents [a][nb].  Barriers: in complete on entry, out complete on return.
+// le: exponents [a][nb].  In is complete on entry, out on return (team barrier).
 typedef long long EoPart[4][24][X_PAD];
-__device__ __noinline__ void eo_xhop(const EoCtx c, EoShared& M, EoPart* part, int par, EoX in, const int4* lx,
+__device__ __noinline__ void eo_xhop(const EoCtx c, const EoTeam T, EoShared& M, EoPart* part, int par, EoX in, const int4* lx,
                                      const int* le, EoX xo, double2* out, const double2* b1, const double2* b2,
                                      double coef) {
     const int lane = threadIdx.x & 31, wid = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), a = wid & 3;
-    const int grp = wid >> 2, ngrp = blockDim.x >> 7;
+    const int grp = wid >> 2, grp0 = T.rank * (blockDim.x >> 7), ngrp = T.size * (blockDim.x >> 7);
     const int ntile = (c.count + X_TILE - 1) / X_TILE;
     for (int tile0 = 0; tile0 < ntile; tile0 += ngrp) {
-        const int tile = tile0 + grp;
+        const int tile = tile0 + grp0 + grp;
         EoSite s;
         const bool ok = eo_site(c, par, tile * X_TILE + lane, s);
         const int la = a == 0 ? s.l[0] : a == 1 ? s.l[1] : a == 2 ? s.l[2] : s.l[3];
@@ -358,6 +405,7 @@ __device__ __noinline__ void eo_xhop(const EoCtx c, EoShared& M, EoPart* part, i
         }
         __syncthreads();
     }
+    T.sync();
 }
 
 // limbs of a spinor held by a lane pair (6 components each); every lane of
@@ -538,14 +586,31 @@ __global__ void __launch_bounds__(256, 2) block_eo_kernel(BlockArgs A) {
     __shared__ EoShared M;
     extern __shared__ long long dyn[];
     EoPart* part = reinterpret_cast<EoPart*>(dyn);
-    const int lane = threadIdx.x & 31, sp = lane >> 4, wid = threadIdx.x >> 5, step = 16 * (blockDim.x >> 5);
-    char* base = A.scratch + (long long)blockIdx.x * A.slot_bytes;
+    const int lane = threadIdx.x & 31, sp = lane >> 4;
+    auto cluster = cooperative_groups::this_cluster();
+    const int rank = (int)cluster.block_rank(), csize = (int)cluster.num_blocks();
+    bool coop = A.nbig > 0;  // the items of the large blocks come first
     for (;;) {
-        if (threadIdx.x == 0) M.item = atomicAdd(A.queue, 1);
-        __syncthreads();
+        if (coop) {
+            if (rank == 0 && threadIdx.x == 0) {
+                const int u = atomicAdd(A.queue, 1);
+                for (int r = 0; r < csize; ++r) cluster.map_shared_rank(&M, r)->item = u;
+            }
+            cluster.sync();
+        } else {
+            if (threadIdx.x == 0) M.item = A.nbig + atomicAdd(A.queue + 1, 1);
+            __syncthreads();
+        }
         const int item = M.item;
-        __syncthreads();
+        const EoTeam T{coop ? rank : 0, coop ? csize : 1};
+        T.sync();
+        if (coop && item >= A.nbig) {
+            coop = false;  // the same decision in every block of the cluster
+            continue;
+        }
         if (item >= A.nitems) break;
+        const int wid = T.warp(), step = 16 * T.warps();
+        char* base = A.scratch + (long long)(coop ? (int)blockIdx.x - rank : (int)blockIdx.x) * A.slot_bytes;
         const BlockItem it = BATCH ? A.items[item]
                                    : BlockItem{A.item_pos0 + item / A.item_n, item % A.item_n, item % A.item_n + 1,
                                                item % A.item_n, 0};
@@ -615,7 +680,7 @@ __global__ void __launch_bounds__(256, 2) block_eo_kernel(BlockArgs A) {
                 }
                 eo_store_limbs(ex, (int)nb, at, sp, ok, v);
             }
-        __syncthreads();
+        T.sync();
         // ---- b = -kappa (H[src] - H[sol]) eta, |b|^2
         double bb = 0.0;
         for (int par = 0; par < 2; ++par)
@@ -635,28 +700,29 @@ __global__ void __launch_bounds__(256, 2) block_eo_kernel(BlockArgs A) {
                 }
                 if (par) SpinorX{tx.p, tx.e, half}.store(s.idx, sv);
             }
-        bb = block_sum(bb, M.sh);
+        bb = eo_sum(M, T, bb);
+        T.sync();  // bt, bo and tx complete
         // ---- b~ = b_e + kappa H_eo b_o; x = 0, r = b~
-        eo_xhop(c, M, part, 0, tx, lx, le, EoX{nullptr, nullptr}, bt, bt, nullptr, c.kappa);
+        eo_xhop(c, T, M, part, 0, tx, lx, le, EoX{nullptr, nullptr}, bt, bt, nullptr, c.kappa);
         double rr = 0.0;
-        eo_each(c, [&](int at) {
+        eo_each(c, T, [&](int at) {
             const double2 v = bt[at];
             r64[at] = v;
             x64[at] = make_double2(0.0, 0.0);
             rr = fma(v.x, v.x, fma(v.y, v.y, rr));
         });
-        for (int i = threadIdx.x; i < half; i += blockDim.x) px.e[i] = X_ZERO;
-        rr = block_sum(rr, M.sh);
+        for (int i = T.rank * (int)blockDim.x + threadIdx.x; i < half; i += T.size * (int)blockDim.x) px.e[i] = X_ZERO;
+        rr = eo_sum(M, T, rr);
         int outer = 0;
         long long inner_its = 0;
         while (rr > A.tol2 * bb && outer < A.max_outer) {
             // inner right-hand side: the residual, normalised to unit norm
             const double rn = sqrt(rr), rinv = 1.0 / rn;
-            eo_each(c, [&](int at) {
+            eo_each(c, T, [&](int at) {
                 const double2 v = r64[at];
                 V.r[at] = make_float2((float)(rinv * v.x), (float)(rinv * v.y));
             });
-            inner_its += eo_bicgstab(c, M, V, l32, A.tol2_inner, A.maxit_inner);
+            inner_its += eo_bicgstab(c, T, M, V, l32, A.tol2_inner, A.maxit_inner);
             // x += |r| e; r = b~ - Dtilde x
             for (int t0 = 16 * wid; t0 < c.count; t0 += step) {
                 EoSite s;
@@ -673,18 +739,18 @@ __global__ void __launch_bounds__(256, 2) block_eo_kernel(BlockArgs A) {
                     }
                 eo_store_limbs(px, (int)half, s.idx, sp, ok, v);
             }
-            __syncthreads();
-            eo_xhop(c, M, part, 1, px, lx, le, tx, nullptr, nullptr, nullptr, 0.0);
-            eo_xhop(c, M, part, 0, tx, lx, le, EoX{nullptr, nullptr}, r64, bt, x64, c.kappa * c.kappa);
+            T.sync();
+            eo_xhop(c, T, M, part, 1, px, lx, le, tx, nullptr, nullptr, nullptr, 0.0);
+            eo_xhop(c, T, M, part, 0, tx, lx, le, EoX{nullptr, nullptr}, r64, bt, x64, c.kappa * c.kappa);
             rr = 0.0;
-            eo_each(c, [&](int at) {
+            eo_each(c, T, [&](int at) {
                 const double2 v = r64[at];
                 rr = fma(v.x, v.x, fma(v.y, v.y, rr));
             });
-            rr = block_sum(rr, M.sh);
+            rr = eo_sum(M, T, rr);
             ++outer;
         }
-        if (threadIdx.x == 0) {
+        if (T.rank == 0 && threadIdx.x == 0) {
             if (rr > A.tol2 * bb) raise_status(A.status, DD_ERR_NOT_CONVERGED);
             if (!isfinite(rr)) raise_status(A.status, DD_ERR_NUMERIC);
             if (A.stats) {
@@ -696,11 +762,11 @@ __global__ void __launch_bounds__(256, 2) block_eo_kernel(BlockArgs A) {
         }
         // ---- x_o = b_o + kappa H_oe x_e, and the result
         if (bb == 0.0) {  // an unchanged block: d = 0
-            if (threadIdx.x == 0) L.item_out[item] = -0.0;
-            __syncthreads();
+            if (T.rank == 0 && threadIdx.x == 0) L.item_out[item] = 0.0;
+            T.sync();
             continue;
         }
-        eo_xhop(c, M, part, 1, px, lx, le, EoX{nullptr, nullptr}, bt, bo, nullptr, c.kappa);
+        eo_xhop(c, T, M, part, 1, px, lx, le, EoX{nullptr, nullptr}, bt, bo, nullptr, c.kappa);
         double sum = 0.0;
         for (int par = 0; par < 2; ++par)
             for (int t0 = 16 * wid; t0 < c.count; t0 += step) {
@@ -714,9 +780,9 @@ __global__ void __launch_bounds__(256, 2) block_eo_kernel(BlockArgs A) {
                     sum += 2.0 * (e.x * v.x + e.y * v.y) + (v.x * v.x + v.y * v.y);
                 }
             }
-        sum = block_sum(sum, M.sh);
-        if (threadIdx.x == 0) L.item_out[item] = -sum;
-        __syncthreads();
+        sum = eo_sum(M, T, sum);
+        if (T.rank == 0 && threadIdx.x == 0) L.item_out[item] = -sum;
+        T.sync();
     }
 }
 
@@ -728,7 +794,7 @@ __global__ void __launch_bounds__(256, 2) block_solve64_kernel(BlockArgs A) {
     // scratch slot of this thread block: vectors eta, b, x, r and the inner x, r, p, q, z
     char* base = A.scratch + (long long)blockIdx.x * A.slot_bytes;
     for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(A.queue, 1);
+        if (threadIdx.x == 0) s_item = atomicAdd(A.queue, 1);  // one queue
         __syncthreads();
         const int item = s_item;
         __syncthreads();

@@ -1,18 +1,17 @@
-// Batched Dirichlet block solves in one persistent launch (Eq. 4step step 1
-// and the block inverses A^{-1}, E^{-1} of the Schur complement, Eq. ddfactor).
+// Block-local Dirichlet operator and the persistent launch of the block filter
+// (Eq. 4step step 1): its items, lattices and arguments, and CG on the
+// normal equations of one block.  The launches are in blockeo.cuh.
 //
 // Every thread block of the grid takes work items (block, factor) from an
 // atomic queue and runs a complete solve of D_b x = src for that item with
-// the whole thread block: FP64 defect correction around an inner CG on the
-// block's normal equations (FP32 arithmetic on FP32 storage, or FP64), all
-// vectors in a per-thread-block scratch slot laid out block-local and
-// chunk-major (coalesced, L2-resident for blocks up to 8^4 sites).
+// the whole thread block, all vectors in a per-thread-block scratch slot.
 //
 // D_b = 1 - kappa * H restricted to hops with both ends in block b (Dirichlet
 // boundary: hops leaving the block are dropped).  Blocks never straddle the
 // time edge (at least two blocks per direction), so no boundary phase occurs
 // inside a block.  Block data (links, vectors) are stored in block order:
-// position q = block_pos * bsites + local index, local index lexicographic.
+// block position, then sites of the block (FP64 vectors lexicographic; links
+// by parity, then lexicographic, see format_gauge_kernel).
 #pragma once
 
 #include <type_traits>
@@ -191,211 +190,51 @@ DD_DEV int block_cgnr(const BlockCtx& c, const S& x, const S& r, const S& p, con
     return it;
 }
 
-// N block-wide sums at once (two barriers for all of them); every thread
-// gets the sums.  shn: at least 32 * N doubles of shared memory.
-template <int N>
-DD_DEV void block_sum_n(double* v, double* shn) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-#pragma unroll
-    for (int k = 0; k < N; ++k) v[k] = warp_sum(v[k]);
-    __syncthreads();  // earlier readers of shn are done
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < N; ++k) shn[wid * N + k] = v[k];
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-        double t = 0.0;
-        for (int w = 0; w < nw; ++w) t += shn[w * N + k];
-        v[k] = t;
-    }
-}
-
-// Inner BiCGStab (van der Vorst) on D_b itself: x = 0, r holds r0 on entry;
-// rhat = r0 is the shadow residual; block-local complex scalars.  Stops when
-// |r|^2 <= tol2rel |r0|^2, after maxit iterations or at a breakdown (the
-// FP64 refinement around it restarts from the true residual).
-template <class R, class S, class LK>
-DD_DEV int block_bicgstab(const BlockCtx& c, const S& x, const S& r, const S& rhat, const S& p, const S& v,
-                          const S& s, const S& t, const LK& lk, double tol2rel, int maxit, double* sh) {
-    double rr0 = 0.0;
-    for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-        Spinor<R> z, a;
-        zero(z);
-        x.store(j, z);
-        p.store(j, z);
-        v.store(j, z);
-        r.load(j, a);
-        rhat.store(j, a);
-        rr0 += (double)snorm2(a);
-    }
-    rr0 = block_sum(rr0, sh);  // barrier: x, p, v, rhat complete
-    if (!(rr0 > 0.0)) return 0;
-    __shared__ double shn[32 * 3];
-    const double target = tol2rel * rr0;
-    cpx<double> rho_old = mk<double>(1.0, 0.0), alpha = mk<double>(1.0, 0.0), omega = mk<double>(1.0, 0.0);
-    int it = 0;
-    while (it < maxit) {
-        // rho = <rhat, r>
-        double d0 = 0.0, d1 = 0.0;
-        for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-            Spinor<R> a, b;
-            rhat.load(j, a);
-            r.load(j, b);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                d0 += (double)(a.c[k].x * b.c[k].x + a.c[k].y * b.c[k].y);
-                d1 += (double)(a.c[k].x * b.c[k].y - a.c[k].y * b.c[k].x);
-            }
-        }
-        double red[3] = {d0, d1, 0.0};
-        block_sum_n<2>(red, shn);
-        const cpx<double> rho = mk<double>(red[0], red[1]);
-        if (!(norm2(rho) > 0.0)) break;
-        const double den = norm2(rho_old) * norm2(omega);
-        if (!(den > 0.0)) break;
-        // beta = (rho / rho_old) (alpha / omega)
-        const cpx<double> beta = (1.0 / den) * cmul(cmul(rho, conj(rho_old)), cmul(alpha, conj(omega)));
-        const cpx<R> bR = mk<R>((R)beta.x, (R)beta.y), oR = mk<R>((R)omega.x, (R)omega.y);
-        for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-            Spinor<R> pp, rr, vv;
-            p.load(j, pp);
-            r.load(j, rr);
-            v.load(j, vv);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) pp.c[k] = rr.c[k] + cmul(bR, pp.c[k] - cmul(oR, vv.c[k]));
-            p.store(j, pp);
-        }
-        __syncthreads();
-        dirichlet_apply<R>(c, p, v, lk, 0);
-        __syncthreads();
-        d0 = d1 = 0.0;
-        for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-            Spinor<R> a, b;
-            rhat.load(j, a);
-            v.load(j, b);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                d0 += (double)(a.c[k].x * b.c[k].x + a.c[k].y * b.c[k].y);
-                d1 += (double)(a.c[k].x * b.c[k].y - a.c[k].y * b.c[k].x);
-            }
-        }
-        red[0] = d0;
-        red[1] = d1;
-        block_sum_n<2>(red, shn);
-        const cpx<double> rv = mk<double>(red[0], red[1]);
-        if (!(norm2(rv) > 0.0)) break;
-        alpha = (1.0 / norm2(rv)) * cmul(rho, conj(rv));
-        const cpx<R> aR = mk<R>((R)alpha.x, (R)alpha.y);
-        double ss = 0.0;
-        for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-            Spinor<R> rr, vv;
-            r.load(j, rr);
-            v.load(j, vv);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) rr.c[k] = rr.c[k] - cmul(aR, vv.c[k]);
-            s.store(j, rr);
-            ss += (double)snorm2(rr);
-        }
-        ss = block_sum(ss, sh);  // barrier: s complete
-        ++it;
-        if (ss <= target) {
-            for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-                Spinor<R> xx, pp;
-                x.load(j, xx);
-                p.load(j, pp);
-#pragma unroll
-                for (int k = 0; k < 12; ++k) xx.c[k] = xx.c[k] + cmul(aR, pp.c[k]);
-                x.store(j, xx);
-            }
-            __syncthreads();
-            break;
-        }
-        dirichlet_apply<R>(c, s, t, lk, 0);
-        __syncthreads();
-        double ts0 = 0.0, ts1 = 0.0, tt = 0.0;
-        for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-            Spinor<R> a, b;
-            t.load(j, a);
-            s.load(j, b);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                ts0 += (double)(a.c[k].x * b.c[k].x + a.c[k].y * b.c[k].y);
-                ts1 += (double)(a.c[k].x * b.c[k].y - a.c[k].y * b.c[k].x);
-            }
-            tt += (double)snorm2(a);
-        }
-        red[0] = ts0;
-        red[1] = ts1;
-        red[2] = tt;
-        block_sum_n<3>(red, shn);
-        const cpx<double> ts = mk<double>(red[0], red[1]);
-        tt = red[2];
-        if (!(tt > 0.0)) break;
-        omega = (1.0 / tt) * ts;
-        const cpx<R> wR = mk<R>((R)omega.x, (R)omega.y);
-        double rr = 0.0;
-        for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-            Spinor<R> xx, pp, sv, tv;
-            x.load(j, xx);
-            p.load(j, pp);
-            s.load(j, sv);
-            t.load(j, tv);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                xx.c[k] = xx.c[k] + cmul(aR, pp.c[k]) + cmul(wR, sv.c[k]);
-                sv.c[k] = sv.c[k] - cmul(wR, tv.c[k]);
-            }
-            x.store(j, xx);
-            r.store(j, sv);
-            rr += (double)snorm2(sv);
-        }
-        rr = block_sum(rr, sh);  // barrier: x and r complete
-        rho_old = rho;
-        if (rr <= target || !(norm2(omega) > 0.0)) break;
-    }
-    return it;
-}
-
 // ----------------------------------------------------------- the launch
-enum BlockMode { BLOCK_FILTER = 0, BLOCK_SOLVE = 1 };
-
 struct BlockItem {
     int block_pos;  // position of the block in block order
-    int f_src;      // field slot of the source operator (filter) / unused
+    int f_src;      // field slot of the source operator
     int f_sol;      // field slot of the solve
-    int vec;        // factor index (noise sub) / vector index in the banks
+    int vec;        // factor index (noise sub)
     int lat;        // lattice of the item in a multi-lattice launch (0 otherwise)
 };
 
-// one lattice of a multi-lattice launch (blocks of different shapes)
+// block shape of the even-odd solver (blockeo.cuh)
+struct EoCtx {
+    int bd[4], st[4];
+    int nb;     // sites of the block
+    int half;   // stride of one parity's vectors: nb / 2, or nb for an odd extent along axis 0
+    int sh;     // storage index of local site j: j >> sh
+    int count;  // sites to visit for one parity (an odd extent along axis 0: all, the wrong parity skipped)
+    int d0;     // extent along axis 0 in visited sites
+    unsigned m0, m1, m2;
+    float kappa2;
+    double kappa;
+};
+
+// one lattice of a launch (blocks of different shapes)
 struct LatDesc {
     Geo g;
     BlockCtx c;
-    const double2* dd64;
-    long long dd64_fs;
-    const float4* dd32;
+    EoCtx eo;
+    const double* canon;  // canonical FP64 links, field slot 0
+    long long canon_fs;   // doubles between consecutive slots
+    const int4* ddx;      // links in limbs, block order
+    long long ddx_fs;
+    const float2* dd32;
     long long dd32_fs;
+    const uint8_t* active;  // active links [V * 4]
     double* item_out;
 };
 
 struct BlockArgs {
-    const LatDesc* lats;  // multi-lattice launch: per-item lattice (null: the fields below)
-    Geo g;
-    BlockCtx c;
-    int mode;
+    const LatDesc* lats;  // multi-lattice launch: per-item lattice
+    LatDesc lat;          // single-lattice launch (lats null)
     const BlockItem* items;  // null: block-filter items k -> (block position item_pos0 + k / item_n, vector k % item_n)
     int nitems;
+    int nbig;  // leading items of large blocks, each solved by a cluster of thread blocks (block_eo_kernel)
     int item_pos0, item_n;
-    int* queue;
-    const double2* dd64;  // field slot 0, FP64 links in block order
-    long long dd64_fs;    // elements between consecutive field slots
-    const float4* dd32;
-    long long dd32_fs;
-    const double2* in_bank;  // BLOCK_SOLVE right-hand sides (block order, FP64)
-    double2* out_bank;       // BLOCK_SOLVE solutions
-    long long bank_vs;       // elements between consecutive vectors of a bank
-    double* item_out;        // BLOCK_FILTER: -(2 Re<eta, d> + |d|^2) per item
+    int* queue;  // heads of the two queues: large items, the others
     char* scratch;
     long long slot_bytes;
     uint64_t seed, ctr;
@@ -431,188 +270,19 @@ DD_DEV void block_origin(const Geo& g, int id, int o[4]) {
     o[3] = (r / g.nbk[2]) * g.b[3];
 }
 
-template <class LK>
-DD_DEV LK make_inner_links(const LatDesc& L, int f, int pos);
-template <>
-DD_DEV LinkF32 make_inner_links<LinkF32>(const LatDesc& L, int f, int pos) {
-    return LinkF32{L.dd32 + (long long)f * L.dd32_fs + (long long)pos * 4 * 3 * L.c.nb, L.c.nb};
-}
-template <>
-DD_DEV LinkF64 make_inner_links<LinkF64>(const LatDesc& L, int f, int pos) {
-    return LinkF64{L.dd64 + (long long)f * L.dd64_fs + (long long)pos * 4 * 9 * L.c.nb, L.c.nb};
-}
-template <class S>
-DD_DEV S scratch_spinor(char* base, int index, long long nb);
-template <>
-DD_DEV SpinorF32 scratch_spinor<SpinorF32>(char* base, int index, long long nb) {
-    return SpinorF32{(float4*)base + (long long)index * 6 * nb, nb};
-}
-template <>
-DD_DEV SpinorF64 scratch_spinor<SpinorF64>(char* base, int index, long long nb) {
-    return SpinorF64{(double2*)base + (long long)index * 12 * nb, nb};
-}
-
-template <class RI, class SI, class LKI>
-__global__ void __launch_bounds__(256, 2) block_solve_kernel(BlockArgs A) {
-    __shared__ double sh[34];
-    __shared__ int s_item;
-    // scratch slot of this thread block: FP64 vectors eta, b, x, r; inner vectors x, r, p, q, z
-    char* base = A.scratch + (long long)blockIdx.x * A.slot_bytes;
-    for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(A.queue, 1);
-        __syncthreads();
-        const int item = s_item;
-        __syncthreads();
-        if (item >= A.nitems) break;
-        const BlockItem it = A.items ? A.items[item]
-                                     : BlockItem{A.item_pos0 + item / A.item_n, item % A.item_n,
-                                                 item % A.item_n + 1, item % A.item_n, 0};
-        LatDesc L;
-        if (A.lats) {
-            L = A.lats[it.lat];
-        } else {
-            L.g = A.g;
-            L.c = A.c;
-            L.dd64 = A.dd64;
-            L.dd64_fs = A.dd64_fs;
-            L.dd32 = A.dd32;
-            L.dd32_fs = A.dd32_fs;
-            L.item_out = A.item_out;
-        }
-        const BlockCtx& c = L.c;
-        const long long nb = c.nb;
-        SpinorF64 eta{(double2*)base, nb};
-        SpinorF64 bv{(double2*)base + 12 * nb, nb};
-        SpinorF64 xv{(double2*)base + 24 * nb, nb};
-        SpinorF64 rv{(double2*)base + 36 * nb, nb};
-        char* ib = base + 48 * nb * sizeof(double2);
-        SI xi = scratch_spinor<SI>(ib, 0, nb), ri = scratch_spinor<SI>(ib, 1, nb),
-           pi = scratch_spinor<SI>(ib, 2, nb), qi = scratch_spinor<SI>(ib, 3, nb), zi = scratch_spinor<SI>(ib, 4, nb);
-        LinkF64 lsol{L.dd64 + (long long)it.f_sol * L.dd64_fs + (long long)it.block_pos * 4 * 9 * nb, nb};
-        LKI lsoli = make_inner_links<LKI>(L, it.f_sol, it.block_pos);
-        int colour;
-        int id = block_id_at(L.g, it.block_pos, &colour);
-        int org[4];
-        block_origin(L.g, id, org);
-        // ---- right-hand side
-        if (A.mode == BLOCK_FILTER) {
-            LinkF64 lsrc{L.dd64 + (long long)it.f_src * L.dd64_fs + (long long)it.block_pos * 4 * 9 * nb, nb};
-            for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-                int l[4];
-                local_coords(c, j, l);
-                int x[4] = {org[0] + l[0], org[1] + l[1], org[2] + l[2], org[3] + l[3]};
-                uint32_t s = (uint32_t)canon_index(L.g, x);
-                Spinor<double> e;
+// links of one block, read from a canonical FP64 field (V x 4 x 3 x 3 complex)
+struct LinkCanonF64 {
+    const double* U;
+    Geo g;
+    BlockCtx c;
+    int org[4];
+    template <class R>
+    DD_DEV void load(long long j, int a, Link<R>& u) const {
+        int l[4];
+        local_coords(c, (int)j, l);
+        int x[4] = {org[0] + l[0], org[1] + l[1], org[2] + l[2], org[3] + l[3]};
+        const double* p = U + ((long long)canon_index(g, x) * 4 + a) * 18;
 #pragma unroll
-                for (int k = 0; k < 12; ++k)
-                    e.c[k] = gaussian(s * 12u + k, (uint32_t)A.purpose, (uint32_t)it.vec, A.seed, stream_ctr(A.ctr, A.ctr_off));
-                eta.store(j, e);
-            }
-            __syncthreads();
-            // b = (D_b[src] - D_b[sol]) eta = -kappa (H[src] - H[sol]) eta
-            for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-                Spinor<double> h1;
-                dirichlet_hop_diff(c, j, eta, lsrc, lsol, h1);
-#pragma unroll
-                for (int k = 0; k < 12; ++k) h1.c[k] = (-c.kappa) * h1.c[k];
-                bv.store(j, h1);
-            }
-        } else {
-            SpinorF64 src{(double2*)A.in_bank + (long long)it.vec * A.bank_vs + (long long)it.block_pos * 12 * nb, nb};
-            for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-                Spinor<double> v;
-                src.load(j, v);
-                bv.store(j, v);
-            }
-        }
-        // ---- x = 0, r = b
-        double bb = 0.0;
-        for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-            Spinor<double> v, z;
-            bv.load(j, v);
-            rv.store(j, v);
-            zero(z);
-            xv.store(j, z);
-            bb += snorm2(v);
-        }
-        bb = block_sum(bb, sh);
-        double rr = bb;
-        int outer = 0;
-        long long inner_its = 0;
-        while (rr > A.tol2 * bb && outer < A.max_outer) {
-            // inner right-hand side: the FP64 residual, normalised to unit norm
-            const double rn = sqrt(rr), rinv = 1.0 / rn;
-            for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-                Spinor<double> v;
-                rv.load(j, v);
-#pragma unroll
-                for (int k = 0; k < 12; ++k) v.c[k] = rinv * v.c[k];
-                ri.store(j, v);
-            }
-            __syncthreads();
-            if constexpr (std::is_same<RI, float>::value) {
-                // FP32 inner vectors are half the size of the slot's FP64 ones:
-                // room for the seven BiCGStab vectors
-                SI hi = scratch_spinor<SI>(ib, 5, nb), si = scratch_spinor<SI>(ib, 6, nb),
-                   ti = scratch_spinor<SI>(ib, 7, nb);
-                inner_its += block_bicgstab<RI>(c, xi, ri, hi, pi, qi, si, ti, lsoli, A.tol2_inner, A.maxit_inner, sh);
-            } else {
-                inner_its += block_cgnr<RI>(c, xi, ri, pi, qi, zi, lsoli, A.tol2_inner, A.maxit_inner, sh);
-            }
-            // x += |r| e; r = b - D_b x (FP64)
-            for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-                Spinor<double> a;
-                Spinor<RI> e;
-                xv.load(j, a);
-                xi.load(j, e);
-#pragma unroll
-                for (int k = 0; k < 12; ++k)
-                    a.c[k] = a.c[k] + rn * mk<double>((double)e.c[k].x, (double)e.c[k].y);
-                xv.store(j, a);
-            }
-            __syncthreads();
-            rr = 0.0;
-            for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-                Spinor<double> acc, v, b;
-                dirichlet_hop<double>(c, j, xv, lsol, 0, acc);
-                xv.load(j, v);
-                bv.load(j, b);
-#pragma unroll
-                for (int k = 0; k < 12; ++k) b.c[k] = b.c[k] - (v.c[k] + (-c.kappa) * acc.c[k]);
-                rv.store(j, b);
-                rr += snorm2(b);
-            }
-            rr = block_sum(rr, sh);
-            ++outer;
-        }
-        if (rr > A.tol2 * bb && threadIdx.x == 0) raise_status(A.status, DD_ERR_NOT_CONVERGED);
-        if (A.stats && threadIdx.x == 0) {
-            atomicAdd(A.stats, 1ull);
-            atomicAdd(A.stats + 1, (unsigned long long)inner_its);
-            atomicAdd(A.stats + 2, (unsigned long long)outer);
-            atomicAdd(A.stats + 3, (unsigned long long)inner_its * (unsigned long long)nb);
-        }
-        if (!isfinite(rr) && threadIdx.x == 0) raise_status(A.status, DD_ERR_NUMERIC);
-        // ---- results
-        if (A.mode == BLOCK_FILTER) {
-            double s = 0.0;
-            for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-                Spinor<double> e, d;
-                eta.load(j, e);
-                xv.load(j, d);
-#pragma unroll
-                for (int k = 0; k < 12; ++k) s += 2.0 * (e.c[k].x * d.c[k].x + e.c[k].y * d.c[k].y) + norm2(d.c[k]);
-            }
-            s = block_sum(s, sh);
-            if (threadIdx.x == 0) L.item_out[item] = -s;
-        } else {
-            SpinorF64 dst{A.out_bank + (long long)it.vec * A.bank_vs + (long long)it.block_pos * 12 * nb, nb};
-            for (int j = threadIdx.x; j < c.nb; j += blockDim.x) {
-                Spinor<double> v;
-                xv.load(j, v);
-                dst.store(j, v);
-            }
-        }
-        __syncthreads();
+        for (int k = 0; k < 9; ++k) u.m[k / 3][k % 3] = mk<R>((R)p[2 * k], (R)p[2 * k + 1]);
     }
-}
+};

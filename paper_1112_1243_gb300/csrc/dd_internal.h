@@ -57,8 +57,8 @@ struct FieldSlot {
     int4* eox;       // eo layout, two-limb integers (LinkX, FP64 accuracy): [parity][dir][9][Vh], then exponents
     float4* eo32;    // eo layout, FP32 rows 0-1, 3 chunks
     uint2* eo16;     // eo layout, FP16 rows 0-1, 3 chunks
-    double2* dd64;   // block order, FP64 [blockpos][dir][chunk][bsites]
-    float4* dd32;    // block order, FP32 rows 0-1
+    int4* ddx;       // block order, two-limb integers [blockpos][dir][9][bsites], then exponents [blockpos][dir][bsites]
+    float2* dd32;    // block order, FP32 [blockpos][dir][9][bsites]
     double2* canon;  // canonical FP64 copy (interpolated fields)
     float4* eodf;    // eo layout, double-float (hi, lo) pairs, 9 chunks (outer_prec DD_PREC_DF64 only)
 };
@@ -329,11 +329,15 @@ inline int dd_require_feature(dd_handle* h, bool planned, const char* what) {
 // exact block log-determinant ratios of the block filter (lu.cu)
 int block_filter_exact(dd_handle* h, const double* U_old, const double* U_new, int colour_mask, double* ln_b);
 
+// bytes of a scratch slot of the persistent block solver for blocks of nb
+// sites (an odd extent along axis 0 keeps one parity's vectors at full length)
+inline size_t block_slot_bytes(long long nb) { return ((size_t)nb * 2240 + 8192 + 255) & ~(size_t)255; }
+
 // shared launch helpers (defined in lattice.cu / solver.cu)
 inline int grid_for(long long n, int threads) { return (int)((n + threads - 1) / threads); }
 
 // field formatting (lattice.cu)
-int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eox, bool eo32, bool eo16, bool dd64, bool dd32);
+int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eox, bool eo32, bool eo16, bool dd);
 // spinor packing between canonical FP64 and eo FP64 (lattice.cu)
 void launch_pack_spinor_eo(dd_handle* h, const double* in, double2* out, int parity, int nrhs, long long in_rhs_stride);
 void launch_unpack_spinor_eo(dd_handle* h, const double2* in, double* out, int parity, int nrhs, long long out_rhs_stride);

@@ -18,8 +18,10 @@
 //   ln r_b = sum_i -(2 Re<eta, d> + |d|^2), accept iff ln u_b < ln r_b.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
+#include "blockeo.cuh"
 #include "blocksolve.cuh"
 #include "dslash.cuh"
 #include "solver.h"
@@ -127,7 +129,7 @@ __global__ void inter_hop_kernel(Geo g, BlockCtx c, const double2* in_bank, doub
 
 // out = v - D_b[field] a on black sites, 0 on white (block order)
 __global__ void schur_source_kernel(Geo g, BlockCtx c, const double2* v_bank, const double2* a_bank,
-                                    double2* out_bank, long long vs, const double2* dd64, long long fs, int f0,
+                                    double2* out_bank, long long vs, const double* canon0, long long canon_fs, int f0,
                                     int fstep) {
     long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     int i = blockIdx.y;
@@ -139,7 +141,9 @@ __global__ void schur_source_kernel(Geo g, BlockCtx c, const double2* v_bank, co
     if (pos < g.nblocks / 2) {
         SpinorF64 av{(double2*)a_bank + (long long)i * vs + pos * 12 * c.nb, c.nb};
         SpinorF64 vv{(double2*)v_bank + (long long)i * vs + pos * 12 * c.nb, c.nb};
-        LinkF64 lk{dd64 + (long long)(f0 + i * fstep) * fs + pos * 4 * 9 * c.nb, c.nb};
+        int colour, org[4];
+        block_origin(g, block_id_at(g, (int)pos, &colour), org);
+        const LinkCanonF64 lk{canon0 + (long long)(f0 + i * fstep) * canon_fs, g, c, {org[0], org[1], org[2], org[3]}};
         Spinor<double> acc, a;
         dirichlet_hop<double>(c, j, av, lk, 0, acc);
         av.load(j, a);
@@ -275,6 +279,85 @@ static BlockCtx block_ctx(dd_handle* h) {
     return c;
 }
 
+static EoCtx eo_ctx(dd_handle* h) {
+    const Geo& g = h->g;
+    EoCtx c;
+    std::memset(&c, 0, sizeof(c));
+    int st = 1;
+    for (int a = 0; a < 4; ++a) {
+        c.bd[a] = g.b[a];
+        c.st[a] = st;
+        st *= g.b[a];
+    }
+    c.nb = g.bsites;
+    c.sh = (g.b[0] & 1) ? 0 : 1;
+    c.half = c.count = c.sh ? c.nb / 2 : c.nb;
+    c.d0 = c.sh ? g.b[0] / 2 : g.b[0];
+    auto magic = [&](int d) -> unsigned {  // see geo_finish; dividends are below nb
+        if (d <= 1 || (unsigned long long)c.nb * (unsigned long long)d >= (1ull << 32)) return 0u;
+        return (unsigned)(((1ull << 32) + d - 1) / d);
+    };
+    c.m0 = magic(c.d0);
+    c.m1 = magic(c.bd[1]);
+    c.m2 = magic(c.bd[2]);
+    c.kappa = h->prm.kappa;
+    c.kappa2 = (float)(h->prm.kappa * h->prm.kappa);
+    return c;
+}
+// the handle's lattice and field slots as a launch sees them
+static void fill_lat(dd_handle* h, LatDesc& L, double* item_out) {
+    L.g = h->g;
+    L.c = block_ctx(h);
+    L.eo = eo_ctx(h);
+    L.canon = (const double*)h->fields[0].canon;
+    L.canon_fs = (long long)(h->fields[1].canon - h->fields[0].canon) * 2;
+    L.ddx = h->fields[0].ddx;
+    L.ddx_fs = (long long)(h->fields[1].ddx - h->fields[0].ddx);
+    L.dd32 = h->fields[0].dd32;
+    L.dd32_fs = (long long)(h->fields[1].dd32 - h->fields[0].dd32);
+    L.active = h->d_active_mask;
+    L.item_out = item_out;
+}
+// blocks above this size are solved by a cluster of EO_CLUSTER thread blocks
+// each: one thread block of 256 threads is latency bound there (8^4: 29 ms an
+// item on its SM, IPC 0.35), and 304 items of 2.8 MB do not fit the L2 cache
+// while 38 do; 4^4 blocks fill a thread block of 256 threads exactly
+constexpr int EO_COOP_SITES = 1024;
+
+// the persistent launch on at most `slots` thread blocks (one scratch slot
+// each); A.nbig leading items belong to large blocks
+static int run_blocks(dd_handle* h, const BlockArgs& A, int slots, cudaStream_t s) {
+    if (A.inner_f64) {
+        DD_KLAUNCH(h, block_solve64_kernel<<<std::min(slots, A.nitems), h->tune.block_tpb, 0, s>>>(A));
+    } else {
+        // groups of four warps (eo_xhop): 128 threads at least
+        const int tpb = std::max(h->tune.block_tpb, 128);
+        const int csize = (A.nbig > 0 && slots >= EO_CLUSTER) ? EO_CLUSTER : 1;
+        BlockArgs B = A;
+        if (csize == 1) B.nbig = 0;
+        const long long want = (long long)B.nbig * csize + (A.nitems - B.nbig);
+        int grid = (int)std::min<long long>(slots, want);
+        grid = std::max(csize, grid / csize * csize);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(tpb);
+        cfg.dynamicSmemBytes = (size_t)(tpb / 128) * sizeof(EoPart);
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = csize;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        auto* kern = A.lats ? block_eo_kernel<true> : block_eo_kernel<false>;
+        DD_CUDA(h, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
+        DD_CUDA(h, cudaLaunchKernelEx(&cfg, kern, B));
+        ++h->launches;
+    }
+    DD_LAUNCH_CHECK(h, "persistent block solver");
+    return DD_OK;
+}
+
 // format slots 0..nslots-1 from interpolated (or copied) fields
 static int prepare_fields(dd_handle* h, const double* U_old, const double* U_new, int n, bool factors, bool eo,
                           bool all_links = false) {
@@ -289,7 +372,7 @@ static int prepare_fields(dd_handle* h, const double* U_old, const double* U_new
         FieldSlot& f = h->fields[k];
         bool need_eo = eo;  // old and new fields both enter even-odd solves
         rc = format_field(h, (const double*)f.canon, f, need_eo, need_eo && ip == DD_PREC_F32,
-                          need_eo && ip == DD_PREC_F16, true, true);
+                          need_eo && ip == DD_PREC_F16, true);
         if (rc) return rc;
     }
     return DD_OK;
@@ -315,28 +398,18 @@ static void block_timer_end(dd_handle* h, int nitems) {
 
 // block-filter items of the blocks at positions pos0 .. pos0 + nitems / n - 1,
 // n noise vectors each, in one persistent launch
-static int launch_blocks(dd_handle* h, int mode, int pos0, int n, int nitems, const double2* in_bank,
-                         double2* out_bank, uint64_t seed, uint64_t ctr) {
+static int launch_blocks(dd_handle* h, int pos0, int n, int nitems, uint64_t seed, uint64_t ctr) {
     if (nitems <= 0) return DD_OK;
-    DD_CUDA(h, cudaMemsetAsync(h->d_queue, 0, sizeof(int), h->stream));
+    DD_CUDA(h, cudaMemsetAsync(h->d_queue, 0, 2 * sizeof(int), h->stream));
     BlockArgs A;
     A.lats = nullptr;
-    A.g = h->g;
-    A.c = block_ctx(h);
-    A.mode = mode;
+    fill_lat(h, A.lat, h->d_item_out);
     A.items = nullptr;
     A.nitems = nitems;
+    A.nbig = h->g.bsites > EO_COOP_SITES ? nitems : 0;
     A.item_pos0 = pos0;
     A.item_n = n;
     A.queue = h->d_queue;
-    A.dd64 = h->fields[0].dd64;
-    A.dd64_fs = (long long)(h->fields[1].dd64 - h->fields[0].dd64);
-    A.dd32 = h->fields[0].dd32;
-    A.dd32_fs = (long long)(h->fields[1].dd32 - h->fields[0].dd32);
-    A.in_bank = in_bank;
-    A.out_bank = out_bank;
-    A.bank_vs = 12LL * h->g.V;
-    A.item_out = h->d_item_out;
     A.scratch = h->block_scratch;
     A.slot_bytes = (long long)h->block_slot_bytes;
     A.seed = seed;
@@ -350,17 +423,12 @@ static int launch_blocks(dd_handle* h, int mode, int pos0, int n, int nitems, co
     A.max_outer = A.inner_f64 ? 3 : 12;
     A.status = h->d_status;
     A.stats = h->d_sites + DD_TIMER_KINDS;
-    const int grid = std::min(nitems, std::min(h->block_slots, std::max(1, h->num_sms) * h->tune.block_ctas_per_sm));
-    const int tpb = h->tune.block_tpb;
+    const int slots = std::min(h->block_slots, std::max(1, h->num_sms) * h->tune.block_ctas_per_sm);
     const bool timed = block_timer_begin(h);
     ++h->block_launches;
-    if (A.inner_f64)
-        DD_KLAUNCH(h, block_solve_kernel<double, SpinorF64, LinkF64><<<grid, tpb, 0, h->stream>>>(A));
-    else
-        DD_KLAUNCH(h, block_solve_kernel<float, SpinorF32, LinkF32><<<grid, tpb, 0, h->stream>>>(A));
+    const int rc = run_blocks(h, A, slots, h->stream);
     if (timed) block_timer_end(h, nitems);
-    DD_LAUNCH_CHECK(h, "block_solve_kernel");
-    return DD_OK;
+    return rc;
 }
 
 // autotuner probe: one block-filter pass (one noise vector per block, every
@@ -375,9 +443,9 @@ int tune_block_filter(dd_handle* h, const double* U_old, const double* U_new, in
         cudaEventDestroy(e0);
         return dd_fail(h, DD_ERR_CUDA, "cudaEventCreate");
     }
-    rc = launch_blocks(h, BLOCK_FILTER, 0, 1, h->g.nblocks, nullptr, nullptr, 1, 0);
+    rc = launch_blocks(h, 0, 1, h->g.nblocks, 1, 0);
     cudaEventRecord(e0, h->stream);
-    for (int r = 0; r < reps && !rc; ++r) rc = launch_blocks(h, BLOCK_FILTER, 0, 1, h->g.nblocks, nullptr, nullptr, 1, 0);
+    for (int r = 0; r < reps && !rc; ++r) rc = launch_blocks(h, 0, 1, h->g.nblocks, 1, 0);
     cudaEventRecord(e1, h->stream);
     float t = -1.f;
     if (!rc && cudaEventSynchronize(e1) == cudaSuccess) {
@@ -648,7 +716,7 @@ extern "C" int dd_block_filter(dd_t h, const void* U_old, void* U_new, int colou
         const int half = g.nblocks / 2;
         const int pos0 = colour_mask == 2 ? half : 0;
         const int nb = colour_mask == 3 ? g.nblocks : half;
-        rc = launch_blocks(h, BLOCK_FILTER, pos0, n, nb * n, nullptr, nullptr, seed, ctr);
+        rc = launch_blocks(h, pos0, n, nb * n, seed, ctr);
         if (rc) return rc;
         DD_KLAUNCH(h, sum_items_kernel<<<grid_for(g.nblocks, 128), 128, 0, h->stream>>>(g, nullptr, colour_mask, pos0, n,
                                                                                        h->d_item_out, ln_b));
@@ -691,7 +759,7 @@ extern "C" int dd_block_ratios_range(dd_t h, const void* U_old, const void* U_ne
         return dd_fail(h, DD_ERR_INVALID_ARG, "dd_block_ratios_range: bad arguments");
     rc = prepare_fields(h, (const double*)U_old, (const double*)U_new, n, true, false);
     if (rc) return rc;
-    rc = launch_blocks(h, BLOCK_FILTER, pos0, n, npos * n, nullptr, nullptr, seed, ctr);
+    rc = launch_blocks(h, pos0, n, npos * n, seed, ctr);
     if (rc) return rc;
     DD_KLAUNCH(h, sum_range_kernel<<<grid_for(g.nblocks, 128), 128, 0, h->stream>>>(g, pos0, npos, n, h->d_item_out,
                                                                                    ln_b));
@@ -732,7 +800,7 @@ BatchPlan batch_plan(int nh, dd_handle* const* hs, int n) {
         nblk += hs[k]->g.nblocks;
     }
     p.nitems = nitems;
-    p.slot_bytes = (long long)((((size_t)nbmax * (4 * 192 + 5 * 192)) + 4096 + 255) & ~(size_t)255);
+    p.slot_bytes = (long long)block_slot_bytes(nbmax);
     p.slots = std::max(1, hs[0]->num_sms) * hs[0]->tune.block_ctas_per_sm;
     size_t off = 0;
     p.lats = off;
@@ -834,14 +902,7 @@ extern "C" int dd_block_filter_batch(int nh, const dd_t* hs_, const void* const*
     items.reserve(P.nitems);
     for (int k = 0; k < nh; ++k) {
         dd_handle* h = hs[k];
-        LatDesc& L = lats[k];
-        L.g = h->g;
-        L.c = block_ctx(h);
-        L.dd64 = h->fields[0].dd64;
-        L.dd64_fs = (long long)(h->fields[1].dd64 - h->fields[0].dd64);
-        L.dd32 = h->fields[0].dd32;
-        L.dd32_fs = (long long)(h->fields[1].dd32 - h->fields[0].dd32);
-        L.item_out = d_out;
+        fill_lat(h, lats[k], d_out);
     }
     std::vector<std::vector<int>> per_base(nh);
     for (int oi = 0; oi < nh; ++oi) {
@@ -874,26 +935,17 @@ extern "C" int dd_block_filter_batch(int nh, const dd_t* hs_, const void* const*
     if (!rc && !items.empty()) rc = upload_cached(h0, 1, d_items, items.data(), sizeof(BlockItem) * items.size());
     if (!rc) rc = upload_cached(h0, 2, d_bases, bases.data(), sizeof(int) * bases.size());
     if (rc) return rc;
-    DD_CUDA(h0, cudaMemsetAsync(d_queue, 0, sizeof(int), s));
+    DD_CUDA(h0, cudaMemsetAsync(d_queue, 0, 2 * sizeof(int), s));
     if (!items.empty()) {
         BlockArgs A;
         A.lats = d_lats;
-        A.g = h0->g;
-        A.c = block_ctx(h0);
-        A.mode = BLOCK_FILTER;
         A.items = d_items;
         A.nitems = (int)items.size();
+        A.nbig = 0;
+        for (const BlockItem& i : items) A.nbig += hs[i.lat]->g.bsites > EO_COOP_SITES;
         A.item_pos0 = 0;
         A.item_n = n;
         A.queue = d_queue;
-        A.dd64 = h0->fields[0].dd64;
-        A.dd64_fs = 0;
-        A.dd32 = h0->fields[0].dd32;
-        A.dd32_fs = 0;
-        A.in_bank = nullptr;
-        A.out_bank = nullptr;
-        A.bank_vs = 0;
-        A.item_out = d_out;
         A.scratch = w + P.scratch;
         A.slot_bytes = P.slot_bytes;
         A.seed = seed;
@@ -907,16 +959,11 @@ extern "C" int dd_block_filter_batch(int nh, const dd_t* hs_, const void* const*
         A.max_outer = A.inner_f64 ? 3 : 12;
         A.status = h0->d_status;
         A.stats = h0->d_sites + DD_TIMER_KINDS;
-        const int grid = std::min((int)items.size(), P.slots);
-        const int tpb = h0->tune.block_tpb;
         const bool timed = block_timer_begin(h0);
         ++h0->block_launches;
-        if (A.inner_f64)
-            DD_KLAUNCH(h0, block_solve_kernel<double, SpinorF64, LinkF64><<<grid, tpb, 0, s>>>(A));
-        else
-            DD_KLAUNCH(h0, block_solve_kernel<float, SpinorF32, LinkF32><<<grid, tpb, 0, s>>>(A));
+        rc = run_blocks(h0, A, P.slots, s);
         if (timed) block_timer_end(h0, (int)items.size());
-        DD_LAUNCH_CHECK(h0, "block_solve_kernel (batch)");
+        if (rc) return rc;
     }
     for (int k = 0; k < nh; ++k) {
         dd_handle* h = hs[k];
@@ -956,7 +1003,6 @@ extern "C" int dd_det_ratio_estimate(dd_t h, const void* U_old, const void* U_ne
     // field slot of the old / new operator of factor i: fs * i + {0, 1}
     const int fs = factors ? 1 : 0;
     const long long canon_fs = (long long)(h->fields[1].canon - h->fields[0].canon) * 2;  // doubles
-    const long long dd64_fs = (long long)(h->fields[1].dd64 - h->fields[0].dd64);
     dim3 gv(grid_for(g.V, 128), n);
     // 1. eta on black sites
     const int4 no_outer = make_int4(0, 0, 0, 0);
@@ -980,7 +1026,7 @@ extern "C" int dd_det_ratio_estimate(dd_t h, const void* U_old, const void* U_ne
     rc = dirichlet_solve_bank(h, bank[1], bank[5], n, 0, fs, 0);
     if (rc) return rc;
     // 6. s = v' - A' a  -> bank 3
-    DD_KLAUNCH(h, schur_source_kernel<<<gv, 128, 0, h->stream>>>(g, c, bank[2], bank[5], bank[3], vs, h->fields[0].dd64, dd64_fs, 1, fs));
+    DD_KLAUNCH(h, schur_source_kernel<<<gv, 128, 0, h->stream>>>(g, c, bank[2], bank[5], bank[3], vs, (const double*)h->fields[0].canon, canon_fs, 1, fs));
     // 7. global solve D' y = (s, 0)
     SolverVecs& v = h->vecs[0];
     DD_KLAUNCH(h, dd_to_eo_kernel<<<gv, 128, 0, h->stream>>>(g, c, bank[3], vs, v.be, v.bo));
@@ -1067,7 +1113,6 @@ extern "C" int dd_block_schur_filter(dd_t h, const void* U_old, void* U_new, int
         rc = prepare_fields(h, (const double*)U_old, (const double*)U_new, n, true, true);
         if (rc) return rc;
         const long long canon_fs = (long long)(h->fields[1].canon - h->fields[0].canon) * 2;
-        const long long dd64_fs = (long long)(h->fields[1].dd64 - h->fields[0].dd64);
         dim3 gv(grid_for(g2.V, 128), n);
         // 1. eta on the black sub-blocks of the selected blocks
         DD_KLAUNCH(h, noise_black_kernel<<<gv, 128, 0, h->stream>>>(g2, c2, bank[0], vs, DD_PURPOSE_BLOCK_SCHUR_NOISE, seed,
@@ -1089,7 +1134,7 @@ extern "C" int dd_block_schur_filter(dd_t h, const void* U_old, void* U_new, int
         rc = dirichlet_solve_bank(h, bank[1], bank[5], n, 0, 1, 0);
         if (rc) return rc;
         // 6. s = v' - A' a
-        DD_KLAUNCH(h, schur_source_kernel<<<gv, 128, 0, h->stream>>>(g2, c2, bank[2], bank[5], bank[3], vs, h->fields[0].dd64, dd64_fs, 1, 1));
+        DD_KLAUNCH(h, schur_source_kernel<<<gv, 128, 0, h->stream>>>(g2, c2, bank[2], bank[5], bank[3], vs, (const double*)h->fields[0].canon, canon_fs, 1, 1));
         DD_KLAUNCH(h, dd_to_eo_kernel<<<gv, 128, 0, h->stream>>>(g2, c2, bank[3], vs, v.be, v.bo));
         DD_LAUNCH_CHECK(h, "block schur stage 5-6");
     }

@@ -168,24 +168,31 @@ __global__ void __launch_bounds__(128) format_gauge_kernel(Geo g, const double* 
             o[k * Vh] = v;
         }
     }
-    if (f.dd64) {
-        double2* o = f.dd64 + (bpos * 4 + a) * 9 * nb + j;
-        for (int k = 0; k < 9; ++k) o[k * nb] = make_double2(u[2 * k], u[2 * k + 1]);
-    }
-    if (f.dd32) {
-        float4* o = f.dd32 + (bpos * 4 + a) * 3 * nb + j;
-        for (int k = 0; k < 3; ++k)
-            o[k * nb] = make_float4((float)u[4 * k], (float)u[4 * k + 1], (float)u[4 * k + 2], (float)u[4 * k + 3]);
+    if (f.ddx || f.dd32) {
+        // place in the block: by local parity, then lexicographic (even
+        // extent along axis 0), so that a solver on one parity reads
+        // consecutive links; lexicographic for an odd extent
+        int par_b = 0;
+#pragma unroll
+        for (int d = 0; d < 4; ++d) par_b ^= (x[d] % g.b[d]) & 1;
+        const long long at = (g.b[0] & 1) ? j : par_b * (nb / 2) + (j >> 1), row = bpos * 4 + a;
+        if (f.ddx) x_store_entries(f.ddx + row * 9 * nb + at, nb, reinterpret_cast<int*>(f.ddx + 36LL * g.V) + row * nb + at, u);
+        if (f.dd32) {
+            float2* o = f.dd32 + row * 9 * nb + at;
+            for (int k = 0; k < 9; ++k) o[k * nb] = make_float2((float)u[2 * k], (float)u[2 * k + 1]);
+        }
     }
 }
 
-int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eox, bool eo32, bool eo16, bool dd64, bool dd32) {
+int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eox, bool eo32, bool eo16, bool dd) {
     FieldSlot t = f;
     if (!eox) t.eox = nullptr;
     if (!eo32) t.eo32 = nullptr;
     if (!eo16) t.eo16 = nullptr;
-    if (!dd64) t.dd64 = nullptr;
-    if (!dd32) t.dd32 = nullptr;
+    if (!dd) {
+        t.ddx = nullptr;
+        t.dd32 = nullptr;
+    }
     DD_KLAUNCH(h, format_gauge_kernel<<<dim3(grid_for(h->g.V, 128), 4), 128, 0, h->stream>>>(h->g, U, aligned16(U), t));
     DD_LAUNCH_CHECK(h, "format_gauge_kernel");
     return DD_OK;
@@ -350,8 +357,8 @@ void plan(dd_handle* h, char* base) {
         f.eo16 = c.take<uint2>((size_t)2 * 4 * 3 * Vh);
         f.eodf = h->prm.outer_prec == DD_PREC_DF64 ? c.take<float4>((size_t)2 * 4 * 9 * Vh) : nullptr;
         if (est) {
-            f.dd64 = c.take<double2>((size_t)4 * 9 * V);
-            f.dd32 = c.take<float4>((size_t)4 * 3 * V);
+            f.ddx = c.take<int4>((size_t)37 * V);
+            f.dd32 = c.take<float2>((size_t)4 * 9 * V);
             f.canon = c.take<double2>((size_t)4 * 9 * V);
         }
     }
@@ -421,8 +428,7 @@ void plan(dd_handle* h, char* base) {
     h->d_scalars = c.take<double>((size_t)64 * (R + 2));
     // persistent block-solver slots
     const long long nb = h->g.bsites;
-    // 4 FP64 vectors + 5 inner vectors (FP64 at most) of one block
-    h->block_slot_bytes = ((size_t)nb * (4 * 192 + 5 * 192) + 4096 + 255) & ~(size_t)255;
+    h->block_slot_bytes = block_slot_bytes(nb);
     h->block_slots = std::max(1, h->num_sms) * DD_BLOCK_CTAS_MAX;
     h->block_scratch = c.take<char>(est ? h->block_slot_bytes * h->block_slots : 0);
     h->items_cap = std::max(h->g.nblocks, h->has_sub ? h->g2.nblocks : 0) * 2 * R + 64;
@@ -872,7 +878,7 @@ static int apply_common(dd_handle* h, void* out, const void* in, const void* U, 
     const Geo& g = h->g;
     const long long Vh = g.Vh;
     FieldSlot& f = h->fields[0];
-    rc = format_field(h, (const double*)U, f, prec == DD_PREC_F64, prec == DD_PREC_F32, prec == DD_PREC_F16, false, false);
+    rc = format_field(h, (const double*)U, f, prec == DD_PREC_F64, prec == DD_PREC_F32, prec == DD_PREC_F16, false);
     if (rc) return rc;
     SolverVecs& v = h->vecs[0];
     const bool even_in = (op == DD_OP_DTILDE || op == DD_OP_DTILDE_DAG);

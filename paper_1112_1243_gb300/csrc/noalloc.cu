@@ -29,22 +29,6 @@ constexpr double kNoallocInnerTol = 1e-10;   // relative target of one FP32 CG s
 constexpr int kNoallocInnerMaxit = 2000;     // iterations of one FP32 CG solve
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
 
-// links of one block, read from a canonical FP64 field (V x 4 x 3 x 3 complex)
-struct LinkCanonF64 {
-    const double* U;
-    Geo g;
-    BlockCtx c;
-    int org[4];
-    template <class R>
-    DD_DEV void load(long long j, int a, Link<R>& u) const {
-        int l[4];
-        local_coords(c, (int)j, l);
-        int x[4] = {org[0] + l[0], org[1] + l[1], org[2] + l[2], org[3] + l[3]};
-        const double* p = U + ((long long)canon_index(g, x) * 4 + a) * 18;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) u.m[k / 3][k % 3] = mk<R>((R)p[2 * k], (R)p[2 * k + 1]);
-    }
-};
 // the same links rounded to FP32, rows 0-1 stored, row 2 rebuilt (as LinkF32)
 struct LinkCanonF32 {
     const double* U;

@@ -1148,7 +1148,7 @@ extern "C" int dd_solve(dd_t h, void* x, const void* b, const void* U, int nrhs,
     if (!x || !b || !U || nrhs < 1 || nrhs > h->prm.max_rhs) return dd_fail(h, DD_ERR_INVALID_ARG, "dd_solve: bad arguments");
     if (prec < DD_PREC_F64 || prec > DD_PREC_F16) return dd_fail(h, DD_ERR_INVALID_ARG, "dd_solve: unknown precision");
     const long long V = h->g.V;
-    rc = format_field(h, (const double*)U, h->fields[0], true, prec == DD_PREC_F32, prec == DD_PREC_F16, false, false);
+    rc = format_field(h, (const double*)U, h->fields[0], true, prec == DD_PREC_F32, prec == DD_PREC_F16, false);
     if (rc) return rc;
     SolverVecs& v = h->vecs[0];
     launch_pack_spinor_eo(h, (const double*)b, v.be, 0, nrhs, 24 * V);
@@ -1178,7 +1178,7 @@ extern "C" int dd_sap_apply(dd_t h, void* out, const void* in, const void* U, in
     if (!h->d_colour_sites[0] || !h->d_colour_sites[1])
         return dd_fail(h, DD_ERR_UNSUPPORTED, "dd_sap_apply: needs an even block extent along axis 0");
     const long long V = h->g.V, Vh = h->g.Vh;
-    rc = format_field(h, (const double*)U, h->fields[0], true, prec == DD_PREC_F32, prec == DD_PREC_F16, false, false);
+    rc = format_field(h, (const double*)U, h->fields[0], true, prec == DD_PREC_F32, prec == DD_PREC_F16, false);
     if (rc) return rc;
     SolverVecs& v = h->vecs[0];
     launch_pack_spinor_eo(h, (const double*)in, v.be, 0, nrhs, 24 * V);

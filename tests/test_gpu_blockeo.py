@@ -1,7 +1,8 @@
 """The persistent block solver in even-odd form (block_eo_kernel) against the
 oracle: block shapes with odd extents along any axis (vectors kept at full
 length for an odd extent along axis 0), one- and two-site extents, more and
-fewer sites than threads, every thread-block size, unchanged blocks."""
+fewer sites than threads, every thread-block size, blocks large enough for a
+cluster of thread blocks, unchanged blocks."""
 import numpy as np
 import pytest
 
@@ -46,6 +47,8 @@ def reference(U, Up, lat, n, seed, ctr):
     ((12, 8, 4, 8), (6, 4, 2, 4), 256),
     ((2, 4, 4, 4), (1, 2, 2, 2), 256),
     ((20, 8, 8, 8), (5, 4, 4, 4), 128),
+    ((12, 12, 12, 12), (6, 6, 6, 6), 256),
+    ((14, 12, 12, 12), (7, 6, 6, 6), 128),
 ])
 def test_block_shapes(api, dims, block, tpb):
     n = 2
