@@ -69,26 +69,28 @@ DD_DEV int eo_full(const EoCtx& c, int par, int idx) { return c.sh ? par * c.hal
 // ---------------------------------------------------------------- FP32 hops
 // one hop of lane sp onto its sums: up (upper spin sp), lo / cross (lower
 // spin 2 + sp of this line / of the other lane's line); see xfix.cuh for the
-// spin structure
+// spin structure.  Entries are read at a uniform base plus a 32-bit lane
+// offset (bytes): ou / ol of the first upper / lower component, om of the
+// link's first entry.
+DD_DEV cpx<float> load32(const float2* base, int k, unsigned off) {
+    const float2 v = *reinterpret_cast<const float2*>(reinterpret_cast<const char*>(base + k) + off);
+    return mk<float>(v.x, v.y);
+}
 template <int AXIS, bool FWD>
-DD_DEV void hop32_lane(int sp, const float2* in, int n, const float2* lk, int nb, cpx<float>* up, cpx<float>* lo,
-                       cpx<float>* cross) {
+DD_DEV void hop32_lane(int sp, const float2* in, int n, unsigned ou, unsigned ol, const float2* lk, int nb, unsigned om,
+                       cpx<float>* up, cpx<float>* lo, cpx<float>* cross) {
     constexpr bool swap = AXIS < 2, rot = !(AXIS & 1);
     const float sg = FWD ? 1.f : -1.f;
     const float s1 = (AXIS == 1 || AXIS == 2) ? (sp ? -sg : sg) : sg;
-    const int lb = 3 * (swap ? 3 - sp : 2 + sp);
     cpx<float> h[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const float2 u = in[(3 * sp + c) * n], l = in[(lb + c) * n];
+        const cpx<float> u = load32(in, c * n, ou), l = load32(in, c * n, ol);
         h[c] = rot ? mk<float>(fmaf(-s1, l.y, u.x), fmaf(s1, l.x, u.y)) : mk<float>(fmaf(s1, l.x, u.x), fmaf(s1, l.y, u.y));
     }
     cpx<float> m[3][3];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const float2 v = lk[k * nb];
-        m[k / 3][k % 3] = mk<float>(v.x, v.y);
-    }
+    for (int k = 0; k < 9; ++k) m[k / 3][k % 3] = load32(lk, (AXIS * 9 + k) * nb, om);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         cpx<float> v = mk<float>(0.f, 0.f);
@@ -114,15 +116,19 @@ DD_DEV void hops32(const EoCtx& c, bool ok, int par, const EoSite& s, int sp, co
     cpx<float> cross[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) res[i] = res[3 + i] = cross[i] = mk<float>(0.f, 0.f);
-    const float2* own = lk + eo_full(c, par, s.idx);
-#define DD_HOP32(AXIS)                                                                                             \
-    if (ok && s.l[AXIS] < c.bd[AXIS] - 1)                                                                          \
-        hop32_lane<AXIS, true>(sp, in + ((s.j + c.st[AXIS]) >> c.sh), c.half, own + (long long)AXIS * 9 * c.nb, c.nb, \
-                               res, res + 3, cross);                                                               \
-    if (ok && s.l[AXIS] > 0) {                                                                                     \
-        const int y = (s.j - c.st[AXIS]) >> c.sh;                                                                  \
-        hop32_lane<AXIS, false>(sp, in + y, c.half, lk + (long long)AXIS * 9 * c.nb + eo_full(c, 1 - par, y), c.nb, \
-                                res, res + 3, cross);                                                              \
+    const unsigned row = (unsigned)c.half * 8u;
+    const unsigned up0 = 3u * sp * row, lo0 = 3u * (3 - sp) * row, lo1 = 3u * (2 + sp) * row;  // swapped, straight
+    const unsigned own = (unsigned)eo_full(c, par, s.idx) * 8u, other = (unsigned)eo_full(c, 1 - par, 0) * 8u;
+#define DD_HOP32(AXIS)                                                                                               \
+    if (ok && s.l[AXIS] < c.bd[AXIS] - 1) {                                                                          \
+        const unsigned y = (unsigned)((s.j + c.st[AXIS]) >> c.sh) * 8u;                                              \
+        hop32_lane<AXIS, true>(sp, in, c.half, up0 + y, (AXIS < 2 ? lo0 : lo1) + y, lk, c.nb, own, res, res + 3,     \
+                               cross);                                                                               \
+    }                                                                                                                \
+    if (ok && s.l[AXIS] > 0) {                                                                                       \
+        const unsigned y = (unsigned)((s.j - c.st[AXIS]) >> c.sh) * 8u;                                              \
+        hop32_lane<AXIS, false>(sp, in, c.half, up0 + y, (AXIS < 2 ? lo0 : lo1) + y, lk, c.nb, other + y, res,       \
+                                res + 3, cross);                                                                     \
     }
     DD_HOP32(0)
     DD_HOP32(1)
@@ -152,7 +158,7 @@ struct EoSums {
 // out = Dtilde in (th: odd temporary); with ALL all six sums, else the first
 // two.  Every thread of the team calls this; in is complete, out is written
 // by the lanes that own its entries (no barrier at the end).
-__device__ __noinline__ void eo_dtilde(const EoCtx c, const EoTeam T, const float2* in, float2* th, float2* out, const float2* lk,
+DD_DEV void eo_dtilde(const EoCtx& c, const EoTeam& T, const float2* in, float2* th, float2* out, const float2* lk,
                                        const float2* rhat, bool all, EoSums& S) {
     const int lane = threadIdx.x & 31, sp = lane >> 4, step = 16 * T.warps();
     const int first = 16 * T.warp();
@@ -285,23 +291,28 @@ DD_DEV int eo_bicgstab(const EoCtx& c, const EoTeam& T, EoShared& M, const EoVec
     if (!(d[0] > 0.0)) return 0;
     T.sync();  // p complete
     const double target = tol2rel * d[0];
-    cpx<double> rho = mk<double>(d[0], 0.0);
+    cpx<double> rho = mk<double>(d[0], 0.0), alpha = mk<double>(0.0, 0.0), rv = alpha;
+    cpx<float> aR = mk<float>(0.f, 0.f);
     int it = 0;
-    while (it < maxit) {
-        eo_dtilde(c, T, V.p, V.th, V.v, lk, V.rhat, false, S);
-        eo_total(M, T, S, 2, d);
-        const cpx<double> rv = mk<double>(d[0], d[1]);
-        if (!(norm2(rv) > 0.0)) break;
-        const cpx<double> alpha = (1.0 / norm2(rv)) * cmul(rho, conj(rv));
-        const cpx<float> aR = mk<float>((float)alpha.x, (float)alpha.y);
-        eo_each(c, T, [&](int at) {
-            const float2 r = V.r[at], v = V.v[at];
-            const cpx<float> w = mk<float>(r.x, r.y) - cmul(aR, mk<float>(v.x, v.y));
-            V.s[at] = make_float2(w.x, w.y);
-        });
-        T.sync();
-        eo_dtilde(c, T, V.s, V.th, V.t, lk, V.rhat, true, S);
-        eo_total(M, T, S, 6, d);
+    // two passes an iteration, v = Dtilde p and t = Dtilde s, with one copy
+    // of the operator in the code
+#pragma unroll 1
+    for (bool second = false; second || it < maxit; second = !second) {
+        eo_dtilde(c, T, second ? V.s : V.p, V.th, second ? V.t : V.v, lk, V.rhat, second, S);
+        eo_total(M, T, S, second ? 6 : 2, d);
+        if (!second) {
+            rv = mk<double>(d[0], d[1]);
+            if (!(norm2(rv) > 0.0)) break;
+            alpha = (1.0 / norm2(rv)) * cmul(rho, conj(rv));
+            aR = mk<float>((float)alpha.x, (float)alpha.y);
+            eo_each(c, T, [&](int at) {
+                const float2 r = V.r[at], v = V.v[at];
+                const cpx<float> w = mk<float>(r.x, r.y) - cmul(aR, mk<float>(v.x, v.y));
+                V.s[at] = make_float2(w.x, w.y);
+            });
+            T.sync();
+            continue;
+        }
         ++it;
         const cpx<double> rt = mk<double>(d[0], d[1]), ts = mk<double>(d[2], d[3]);
         const double tt = d[4], ss = d[5];
