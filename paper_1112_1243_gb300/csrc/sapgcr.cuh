@@ -376,16 +376,7 @@ struct SapGcr {
         hop<SpinorF32, SpinorF32, 0>(Ss, 0, in.o, in.e, out.e, 1.0, -k);
         hop<SpinorF32, SpinorF32, 0>(Ss, 1, in.e, in.o, out.o, 1.0, -k);
     }
-    Reduce store_red(double* out) const {
-        Reduce R_;
-        R_.partials = h->d_partials;
-        R_.counters = h->d_counters;
-        R_.st = nullptr;
-        R_.out = out;
-        R_.op = FIN_STORE;
-        R_.status = h->d_status;
-        return R_;
-    }
+    Reduce store_red(double* out) const { return dd_reduce(h, FIN_STORE, nullptr, out); }
 
     // z = SAP(rho), ncy cycles
     int precondition(FullF32 rho, FullF32 z) {
