@@ -25,7 +25,8 @@ struct CGState {
     int maxit;     // cap
     int flags;     // bit 0: hit maxit, bit 1: non-finite
     // complex scalars of BiCGStab
-    double rho_re, rho_im, al_re, al_im, om_re, om_im, be_re, be_im;
+    double rho_re, rho_im, al_re, al_im, om_re, om_im, be_re, be_im, rv_re, rv_im;
+    int last;      // the solve ended with x += alpha p + omega s still to be done
 };
 
 // reduction finishers run by the last thread block of a reduction
@@ -36,9 +37,10 @@ enum FinOp {
     FIN_RR = 3,
     FIN_BETA = 4,
     FIN_ZZ_INIT = 5,
-    FIN_BI_RHO = 6,    // three values
-    FIN_BI_ALPHA = 7,  // three values (third unused)
-    FIN_BI_OMEGA = 8   // three values
+    FIN_BI_RHO = 6,    // three values: <rh, r>, |r|^2 of the first residual
+    FIN_BI_ALPHA = 7,  // two values: <rh, v>
+    FIN_BI_OMEGA = 8,  // six values: <t, s>, |t|^2, <rh, t>, |s|^2
+    FIN_OUTER = 9      // |true residual|^2: stored, and the outer state updated
 };
 
 struct Reduce {

@@ -48,11 +48,14 @@ struct HopArgs {
     const CGState* st;        // per-rhs activity (may be null)
     Reduce red;               // |out|^2 reduction (red.op == FIN_NONE: off)
     unsigned long long* sites;  // timed launches: output sites processed (may be null)
-    // three-value reductions (BiCGStab): 0 off; 1: <rhat, out>; 2: <out, xin> and |out|^2
+    // BiCGStab's sums: 0 off; 1: <rhat, out>; 2: <out, xin>, |out|^2, <rh2, out> and |xin|^2
     int red3 = 0;
+    SIn rh2;                    // red3 == 2: the shadow residual (hop storage)
     SX rhat;                    // red3 == 1: the shadow residual; resid: the right-hand side
     SiteSet S = {nullptr, -1};  // output sites (n < 0: all Vh sites of parity p)
     int resid = 0;              // FP64 hops: out = rhat - (xin + b * hops)
+    int has2 = 0;               // FP64 hops: a second copy of out
+    SOut out2;
 };
 
 template <class LK>
@@ -120,7 +123,7 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
     const long long tile = (long long)blockDim.x * SPT;
     if (A.sites && threadIdx.x == 0)
         atomicAdd(A.sites, (unsigned long long)min(tile, A.S.n - (long long)blockIdx.x * tile));
-    double v3[3] = {0.0, 0.0, 0.0};
+    double v3[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     double nrm = 0.0;
 #pragma unroll
     for (int pass = 0; pass < SPT; ++pass) {
@@ -170,21 +173,28 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
             v3[0] += (double)d0;
             v3[1] += (double)d1;
         } else if (RED3 == 2) {
-            R d0 = 0, d1 = 0;
+            Spinor<R> rv;
+            at_rhs(A.rh2, rhs).load(h, rv);
+            R d0 = 0, d1 = 0, d2 = 0, d3 = 0;
 #pragma unroll
             for (int k = 0; k < 12; ++k) {
                 d0 += res.c[k].x * xv.c[k].x + res.c[k].y * xv.c[k].y;
                 d1 += res.c[k].x * xv.c[k].y - res.c[k].y * xv.c[k].x;
+                d2 += rv.c[k].x * res.c[k].x + rv.c[k].y * res.c[k].y;
+                d3 += rv.c[k].x * res.c[k].y - rv.c[k].y * res.c[k].x;
             }
             v3[0] += (double)d0;
             v3[1] += (double)d1;
             v3[2] += (double)snorm2(res);
+            v3[3] += (double)d2;
+            v3[4] += (double)d3;
+            v3[5] += (double)snorm2(xv);
         } else {
             nrm += (double)snorm2(res);
         }
     }
     if (RED3) {
-        grid_reduce3(A.red, rhs, v3);
+        grid_reduce_bi<RED3 == 1 ? 2 : 6>(A.red, rhs, v3);
     } else if (A.red.op != FIN_NONE) {
         grid_reduce(A.red, rhs, nrm);
     }
@@ -297,6 +307,7 @@ __global__ void __launch_bounds__(128, 5) hop_x_kernel(HopArgs<SpinorX, SX, SOut
                 }
                 if (zeroed) z = make_double2(0.0, 0.0);
                 out.p[k] = z;
+                if (A.has2) at_rhs(A.out2, rhs).p[k] = z;
                 if (A.red.op != FIN_NONE) nrm = fma(z.x, z.x, fma(z.y, z.y, nrm));
             }
         }

@@ -11,6 +11,20 @@ DD_DEV void finish(const Reduce& R, int rhs, double s) {
         case FIN_STORE:
             R.out[rhs] = s;
             break;
+        case FIN_OUTER: {  // defect correction: active while |r|^2 > tol2
+            // a non-finite true residual ends the system and is reported as NUMERIC
+            CGState& c = R.st[rhs];
+            R.out[rhs] = s;
+            c.rr = s;
+            if (!isfinite(s)) {
+                c.active = 0;
+                c.flags |= 2;
+                raise_status(R.status, DD_ERR_NUMERIC);
+            } else {
+                c.active = c.active && s > c.tol2;
+            }
+            break;
+        }
         case FIN_ALPHA: {  // alpha = zz / |A p|^2
             CGState& c = R.st[rhs];
             c.qq = s;
@@ -59,7 +73,7 @@ DD_DEV void finish(const Reduce& R, int rhs, double s) {
     }
 }
 
-// BiCGStab finishers on three sums (v0, v1, v2); complex scalars z = (re, im)
+// BiCGStab finishers on two, three or six sums; complex scalars z = (re, im)
 DD_DEV void cdiv(double ar, double ai, double br, double bi, double& cr, double& ci) {
     double d = br * br + bi * bi;
     cr = (ar * br + ai * bi) / d;
@@ -79,31 +93,21 @@ DD_DEV void bicg_fail(const Reduce& R, CGState& c, bool numeric = false) {
 DD_DEV void finish3(const Reduce& R, int rhs, const double* s) {
     CGState& c = R.st[rhs];
     switch (R.op) {
-        case FIN_BI_RHO: {  // s = (Re<rh,r>, Im<rh,r>, |r|^2): convergence, then beta
+        case FIN_BI_RHO: {  // s = (Re<rh,r>, Im<rh,r>, |r|^2) of the start; counts as the first iteration
             c.rr = s[2];
             c.iters += 1;
-            if (!isfinite(s[2]) || !isfinite(s[0]) || !isfinite(s[1])) {
-                bicg_fail(R, c, true);
-                break;
-            }
-            if (s[2] <= c.tol2) {
-                c.active = 0;
-                break;
-            }
-            if (c.iters >= c.maxit) {
-                c.active = 0;
-                c.flags |= 1;
-                break;
-            }
-            // beta = (rho_new / rho) (alpha / omega)
-            double qr, qi, wr, wi;
-            cdiv(s[0], s[1], c.rho_re, c.rho_im, qr, qi);
-            cdiv(c.al_re, c.al_im, c.om_re, c.om_im, wr, wi);
-            c.be_re = qr * wr - qi * wi;
-            c.be_im = qr * wi + qi * wr;
             c.rho_re = s[0];
             c.rho_im = s[1];
-            if (!(s[0] * s[0] + s[1] * s[1] > 0.0) || !isfinite(c.be_re) || !isfinite(c.be_im)) bicg_fail(R, c);
+            if (!isfinite(s[2]) || !isfinite(s[0]) || !isfinite(s[1])) {
+                bicg_fail(R, c, true);
+            } else if (s[2] <= c.tol2) {
+                c.active = 0;
+            } else if (c.iters >= c.maxit) {
+                c.active = 0;
+                c.flags |= 1;
+            } else if (!(s[0] * s[0] + s[1] * s[1] > 0.0)) {
+                bicg_fail(R, c);
+            }
             break;
         }
         case FIN_BI_ALPHA: {  // s = (Re<rh,v>, Im<rh,v>): alpha = rho / <rh,v>
@@ -117,23 +121,63 @@ DD_DEV void finish3(const Reduce& R, int rhs, const double* s) {
                 break;
             }
             cdiv(c.rho_re, c.rho_im, s[0], s[1], ar, ai);
+            c.rv_re = s[0];
+            c.rv_im = s[1];
             c.al_re = ar;
             c.al_im = ai;
             if (!isfinite(ar) || !isfinite(ai)) bicg_fail(R, c);
             break;
         }
-        case FIN_BI_OMEGA: {  // s = (Re<t,s>, Im<t,s>, |t|^2): omega = <t,s> / |t|^2
-            if (!isfinite(s[0]) || !isfinite(s[1]) || !isfinite(s[2])) {
-                bicg_fail(R, c, true);
-                break;
-            }
+        // omega = <t,s> / |t|^2, then everything of the next iteration that
+        // the vector updates x += alpha p + omega s, r = s - omega t, p = r +
+        // beta (p - omega v) need: |r|^2 = |s|^2 - 2 Re(conj(omega) <t,s>) +
+        // |omega|^2 |t|^2 and rho' = <rh,s> - omega <rh,t>, <rh,s> = rho -
+        // alpha <rh,v>, with alpha and omega as the updates take them
+        // (rounded to FP32).  The updates then need no sums of their own.
+        case FIN_BI_OMEGA: {
+            for (int k = 0; k < 6; ++k)
+                if (!isfinite(s[k])) {
+                    bicg_fail(R, c, true);
+                    return;
+                }
             if (!(s[2] > 0.0)) {
                 bicg_fail(R, c);
                 break;
             }
             c.om_re = s[0] / s[2];
             c.om_im = s[1] / s[2];
-            if (!isfinite(c.om_re) || !isfinite(c.om_im)) bicg_fail(R, c);
+            if (!isfinite(c.om_re) || !isfinite(c.om_im)) {
+                bicg_fail(R, c);
+                break;
+            }
+            const double ar = (double)(float)c.al_re, ai = (double)(float)c.al_im;
+            const double wr = (double)(float)c.om_re, wi = (double)(float)c.om_im;
+            c.rr = s[5] - 2.0 * (wr * s[0] + wi * s[1]) + (wr * wr + wi * wi) * s[2];
+            c.iters += 1;
+            c.last = 1;
+            if (c.rr <= c.tol2) {
+                c.active = 0;
+                break;
+            }
+            if (c.iters >= c.maxit) {
+                c.active = 0;
+                c.flags |= 1;
+                break;
+            }
+            const double nr = c.rho_re - (ar * c.rv_re - ai * c.rv_im) - (wr * s[3] - wi * s[4]);
+            const double ni = c.rho_im - (ar * c.rv_im + ai * c.rv_re) - (wr * s[4] + wi * s[3]);
+            // beta = (rho' / rho) (alpha / omega)
+            double qr, qi, er, ei;
+            cdiv(nr, ni, c.rho_re, c.rho_im, qr, qi);
+            cdiv(c.al_re, c.al_im, c.om_re, c.om_im, er, ei);
+            c.be_re = qr * er - qi * ei;
+            c.be_im = qr * ei + qi * er;
+            c.rho_re = nr;
+            c.rho_im = ni;
+            if (!(nr * nr + ni * ni > 0.0) || !isfinite(c.be_re) || !isfinite(c.be_im))
+                bicg_fail(R, c);
+            else
+                c.last = 0;
             break;
         }
         default:
@@ -219,5 +263,6 @@ DD_DEV void grid_reduce_n(const Reduce& R, int rhs, const double* v, void (*fin)
 }
 
 DD_DEV void finish1(const Reduce& R, int rhs, const double* s) { finish(R, rhs, s[0]); }
-DD_DEV void grid_reduce3(const Reduce& R, int rhs, const double* v) { grid_reduce_n<3>(R, rhs, v, finish3); }
+template <int N>
+DD_DEV void grid_reduce_bi(const Reduce& R, int rhs, const double* v) { grid_reduce_n<N>(R, rhs, v, finish3); }
 DD_DEV void grid_reduce(const Reduce& R, int rhs, double v) { grid_reduce_n<1>(R, rhs, &v, finish1); }

@@ -317,6 +317,7 @@ inline double* sap_rr(dd_handle* h) { return h->sap.sc + (2 * (DD_SAP_MAX_NKV + 
 
 template <class SH, class LK>
 struct SapGcr {
+    static constexpr bool takes_residual = false;
     dd_handle* h;
     int nrhs;
     SpinorF32 x, r;     // even parts: the correction (out) and the right-hand side (in, overwritten)

@@ -99,7 +99,10 @@ __global__ void cg_arm_kernel(int nrhs, CGState* st, const CGState* outer, const
     if (r >= nrhs) return;
     CGState c;
     c.zz = c.qq = c.alpha = c.beta = 0.0;
-    c.rr = rr0[r];
+    const double r0 = rr0 ? rr0[r] : 1.0;  // null: a right-hand side of unit norm
+    c.rr = r0;
+    c.rho_re = c.rho_im = c.al_re = c.al_im = c.om_re = c.om_im = c.be_re = c.be_im = c.rv_re = c.rv_im = 0.0;
+    c.last = 0;
     // relative target tol^2 |r0|^2, or a fraction of the outer absolute target.
     // A mixed inner solve is asked for no more than the outer loop still
     // needs: when ||r_outer|| is within 1/tol_inner of the outer target, the
@@ -108,8 +111,8 @@ __global__ void cg_arm_kernel(int nrhs, CGState* st, const CGState* outer, const
     double rel2 = tol * tol;
     if (abs_fac < 0.0 && outer && outer[r].rr > 0.0)
         rel2 = fmin(fmax(rel2, 0.09 * outer[r].tol2 / outer[r].rr), 0.01);
-    c.tol2 = (abs_fac > 0.0 && outer) ? abs_fac * outer[r].tol2 : rel2 * rr0[r];
-    c.active = (outer ? outer[r].active : 1) && rr0[r] > 0.0;
+    c.tol2 = (abs_fac > 0.0 && outer) ? abs_fac * outer[r].tol2 : rel2 * r0;
+    c.active = (outer ? outer[r].active : 1) && r0 > 0.0;
     c.iters = 0;
     c.maxit = maxit;
     c.flags = 0;
@@ -142,6 +145,26 @@ __global__ void outer_arm_kernel(int nrhs, CGState* outer, const double* bb, dou
     c.maxit = 0;
     c.flags = 0;
     outer[r] = c;
+}
+// |b|^2 over both parities, b_o in limbs for the hop of b~, x = 0
+__global__ void __launch_bounds__(128) solve_start_kernel(SiteSet S, SpinorF64 be, SpinorF64 bo, SpinorX box,
+                                                          SpinorF64 x, int* pxe, Reduce red) {
+    const int rhs = blockIdx.y;
+    const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    double nrm = 0.0;
+    if (ti < S.n) {
+        const long long i = S.at(ti);
+        Spinor<double> a;
+        at_rhs(be, rhs).load(i, a);
+        nrm = snorm2(a);
+        at_rhs(bo, rhs).load(i, a);
+        nrm += snorm2(a);
+        at_rhs(box, rhs).store(i, a);
+        zero(a);
+        at_rhs(x, rhs).store(i, a);
+        pxe[(long long)rhs * x.stride + i] = X_ZERO;
+    }
+    grid_reduce(red, rhs, nrm);
 }
 
 // x64 += scale * e (any storage; scale = |r_outer| when the inner system was
@@ -221,7 +244,9 @@ __global__ void zero64_kernel(SiteSet S, SpinorF64 v, int* pxe) {
 // ------------------------------------------------------------ CGNR runner
 template <class R, class SM, class SH, class LK, int MASK = 0>
 struct NormalCG {
+    static constexpr bool takes_residual = false;
     dd_handle* h;
+    int hint = 0;  // iterations of the longest system of the last run (eager)
     int nrhs;
     SM x, r, p, q, z;
     SH ph, rh, th;
@@ -278,8 +303,11 @@ struct NormalCG {
         std::vector<CGState> hs(nrhs);
         int done_iters = 0;
         bool polled = false;
+        // eager polls as in BiCGStab::run
+        int cur = maxit <= chunk ? chunk : hint > 0 ? hint : 8;
+        if (dd_stream_capturing(h)) cur = chunk;
         auto body = [&]() -> int {
-            for (int it = 0; it < chunk; ++it) {
+            for (int it = 0; it < cur; ++it) {
                 apply_p();
                 DD_KLAUNCH(h, cg_xr_kernel<R, SM, SH><<<grid, 128, 0, h->stream>>>(S, x, r, p, q, rh, copies, st, red(FIN_RR)));
                 apply_dag_r(FIN_BETA);
@@ -289,7 +317,8 @@ struct NormalCG {
         };
         // eager: poll the states every chunk iterations
         auto more = [&](bool& m) -> int {
-            done_iters += chunk;
+            done_iters += cur;
+            cur = 4;
             if (cudaMemcpyAsync(hs.data(), st, sizeof(CGState) * nrhs, cudaMemcpyDeviceToHost, h->stream) !=
                 cudaSuccess)
                 return DD_ERR_CUDA;
@@ -309,6 +338,8 @@ struct NormalCG {
             flags |= hs[k].flags;
         }
         if (iters_out) *iters_out += tot;
+        hint = 0;
+        for (int k = 0; k < nrhs; ++k) hint = std::max(hint, hs[k].iters);
         if (flags & 2) return DD_ERR_NUMERIC;
         return DD_OK;
     }
@@ -328,80 +359,56 @@ DD_DEV cpx<R> cscal(double re, double im) {
 // p and rhat live only in the hop storage SH: the rounded p is the one that
 // both v = Dtilde p and x += alpha p use, and rhat (any fixed vector) is the
 // rounded r0.
-template <class R, class SM, class SH>
-__global__ void bicg_start_kernel(SiteSet S, SM x, SM r, SH rhat, SH p, SM v, const CGState* outer) {
-    const int rhs = blockIdx.y;
-    if (outer && !outer[rhs].active) return;
-    const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (ti >= S.n) return;
-    const long long i = S.at(ti);
-    Spinor<R> z, a;
-    zero(z);
-    at_rhs(x, rhs).store(i, z);
-    at_rhs(p, rhs).store(i, z);
-    at_rhs(v, rhs).store(i, z);
-    at_rhs(r, rhs).load(i, a);
-    at_rhs(rhat, rhs).store(i, a);
-}
 
-__global__ void bicg_arm_kernel(int nrhs, CGState* st) {
-    int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= nrhs) return;
-    CGState& c = st[r];
-    c.rho_re = c.al_re = c.om_re = 1.0;
-    c.rho_im = c.al_im = c.om_im = 0.0;
-    c.be_re = c.be_im = 0.0;
-}
-
+// x = 0, r = r0 (with re: re / sqrt(rr), the FP64 residual at unit norm, so
+// that FP32 squares neither underflow nor overflow), rhat = p = r0, and the
+// sums of FIN_BI_RHO
 template <class R, class SM, class SH>
-__global__ void __launch_bounds__(128) bicg_rho_kernel(SiteSet S, SH rhat, SM r, const CGState* st, Reduce red) {
+__global__ void __launch_bounds__(128) bicg_start_kernel(SiteSet S, SM x, SM r, SH rhat, SH p, SpinorF64 re,
+                                                         const double* rr, const CGState* st, Reduce red) {
     const int rhs = blockIdx.y;
     if (!st[rhs].active) return;
     const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     double v[3] = {0.0, 0.0, 0.0};
     if (ti < S.n) {
         const long long i = S.at(ti);
-        Spinor<R> a, b;
-        at_rhs(rhat, rhs).load(i, a);
-        at_rhs(r, rhs).load(i, b);
+        Spinor<R> z, a, b;
+        zero(z);
+        at_rhs(x, rhs).store(i, z);
+        if (rr) {
+            const double inv = rr[rhs] > 0.0 ? 1.0 / sqrt(rr[rhs]) : 0.0;
+            Spinor<double> d;
+            at_rhs(re, rhs).load(i, d);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) a.c[k] = mk<R>((R)(inv * d.c[k].x), (R)(inv * d.c[k].y));
+            at_rhs(r, rhs).store(i, a);
+        } else {
+            at_rhs(r, rhs).load(i, a);
+        }
+        at_rhs(p, rhs).store(i, a);
+        at_rhs(rhat, rhs).store(i, a);
+        at_rhs(rhat, rhs).load(i, b);  // as rounded
         R d0 = 0, d1 = 0;
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            d0 += a.c[k].x * b.c[k].x + a.c[k].y * b.c[k].y;
-            d1 += a.c[k].x * b.c[k].y - a.c[k].y * b.c[k].x;
+            d0 += b.c[k].x * a.c[k].x + b.c[k].y * a.c[k].y;
+            d1 += b.c[k].x * a.c[k].y - b.c[k].y * a.c[k].x;
         }
         v[0] = (double)d0;
         v[1] = (double)d1;
-        v[2] = (double)snorm2(b);
+        v[2] = (double)snorm2(a);
     }
-    grid_reduce3(red, rhs, v);
+    grid_reduce_bi<3>(red, rhs, v);
 }
 
-// p = r + beta (p - omega v)
+// s = r - alpha v, hop copy of s; closes the update of a solve that ended
 template <class R, class SM, class SH>
-__global__ void __launch_bounds__(128) bicg_p_kernel(SiteSet S, SH p, SM r, SM v, const CGState* st) {
+__global__ void __launch_bounds__(128) bicg_s_kernel(SiteSet S, SM s, SM r, SM v, SH shop, int copy, CGState* st) {
     const int rhs = blockIdx.y;
-    if (!st[rhs].active) return;
-    const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (ti >= S.n) return;
-    const long long i = S.at(ti);
-    const CGState& c = st[rhs];
-    const cpx<R> be = cscal<R>(c.be_re, c.be_im), om = cscal<R>(c.om_re, c.om_im);
-    Spinor<R> pp, rr, vv;
-    at_rhs(p, rhs).load(i, pp);
-    at_rhs(r, rhs).load(i, rr);
-    at_rhs(v, rhs).load(i, vv);
-#pragma unroll
-    for (int k = 0; k < 12; ++k) pp.c[k] = rr.c[k] + cmul(be, pp.c[k] - cmul(om, vv.c[k]));
-    at_rhs(p, rhs).store(i, pp);
-}
-
-// s = r - alpha v, hop copy of s
-template <class R, class SM, class SH>
-__global__ void __launch_bounds__(128) bicg_s_kernel(SiteSet S, SM s, SM r, SM v, SH shop, int copy,
-                                                     const CGState* st) {
-    const int rhs = blockIdx.y;
-    if (!st[rhs].active) return;
+    if (!st[rhs].active) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) st[rhs].last = 0;
+        return;
+    }
     const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (ti >= S.n) return;
     const long long i = S.at(ti);
@@ -416,46 +423,45 @@ __global__ void __launch_bounds__(128) bicg_s_kernel(SiteSet S, SM s, SM r, SM v
     if (copy) at_rhs(shop, rhs).store(i, rr);
 }
 
-// x += alpha p + omega s, r = s - omega t; <rh, r>, |r|^2 -> FIN_BI_RHO
+// x += alpha p + omega s, r = s - omega t, p = r + beta (p - omega v): one
+// pass and no sums (FIN_BI_OMEGA has them), 680 bytes a site in FP16 storage
+// where p apart and x, r with three sums moved 880
 template <class R, class SM, class SH>
-__global__ void __launch_bounds__(128) bicg_xr_kernel(SiteSet S, SM x, SM r, SH p, SM s, SM t, SH rhat,
-                                                      const CGState* st, Reduce red) {
+__global__ void __launch_bounds__(128) bicg_xrp_kernel(SiteSet S, SM x, SM r, SH p, SM s, SM t, SM v,
+                                                       const CGState* st) {
     const int rhs = blockIdx.y;
-    if (!st[rhs].active) return;
+    const CGState& c = st[rhs];
+    if (!c.active && !c.last) return;
     const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    double v[3] = {0.0, 0.0, 0.0};
-    if (ti < S.n) {
-        const long long i = S.at(ti);
-        const CGState& c = st[rhs];
-        const cpx<R> al = cscal<R>(c.al_re, c.al_im), om = cscal<R>(c.om_re, c.om_im);
-        Spinor<R> xx, pp, ss, tt, rh;
-        at_rhs(x, rhs).load(i, xx);
-        at_rhs(p, rhs).load(i, pp);
-        at_rhs(s, rhs).load(i, ss);
+    if (ti >= S.n) return;
+    const long long i = S.at(ti);
+    const cpx<R> al = cscal<R>(c.al_re, c.al_im), om = cscal<R>(c.om_re, c.om_im);
+    Spinor<R> xx, pp, ss;
+    at_rhs(x, rhs).load(i, xx);
+    at_rhs(p, rhs).load(i, pp);
+    at_rhs(s, rhs).load(i, ss);
 #pragma unroll
-        for (int k = 0; k < 12; ++k) xx.c[k] = xx.c[k] + cmul(al, pp.c[k]) + cmul(om, ss.c[k]);
-        at_rhs(x, rhs).store(i, xx);
-        at_rhs(t, rhs).load(i, tt);
+    for (int k = 0; k < 12; ++k) xx.c[k] = xx.c[k] + cmul(al, pp.c[k]) + cmul(om, ss.c[k]);
+    at_rhs(x, rhs).store(i, xx);
+    if (!c.active) return;
+    const cpx<R> be = cscal<R>(c.be_re, c.be_im);
+    Spinor<R> vv;
+    at_rhs(t, rhs).load(i, xx);
+    at_rhs(v, rhs).load(i, vv);
 #pragma unroll
-        for (int k = 0; k < 12; ++k) ss.c[k] = ss.c[k] - cmul(om, tt.c[k]);
-        at_rhs(r, rhs).store(i, ss);
-        at_rhs(rhat, rhs).load(i, rh);
-        R d0 = 0, d1 = 0;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            d0 += rh.c[k].x * ss.c[k].x + rh.c[k].y * ss.c[k].y;
-            d1 += rh.c[k].x * ss.c[k].y - rh.c[k].y * ss.c[k].x;
-        }
-        v[0] = (double)d0;
-        v[1] = (double)d1;
-        v[2] = (double)snorm2(ss);
+    for (int k = 0; k < 12; ++k) {
+        ss.c[k] = ss.c[k] - cmul(om, xx.c[k]);
+        pp.c[k] = ss.c[k] + cmul(be, pp.c[k] - cmul(om, vv.c[k]));
     }
-    grid_reduce3(red, rhs, v);
+    at_rhs(r, rhs).store(i, ss);
+    at_rhs(p, rhs).store(i, pp);
 }
 
 template <class R, class SM, class SH, class LK, int MASK = 0>
 struct BiCGStab {
+    static constexpr bool takes_residual = true;  // the start kernel normalises the FP64 residual
     dd_handle* h;
+    int hint = 0;  // iterations of the longest system of the last run (eager)
     int nrhs;
     SM x, r, v, s, t;
     SH p, rhat, shop, th;  // p and rhat only in hop storage; shop: hop copy of s
@@ -487,6 +493,7 @@ struct BiCGStab {
         A.st = st;
         A.red = red(op);
         A.red3 = red3;
+        A.rh2 = rhat;
         if constexpr (std::is_same<SX, SH>::value)
             A.rhat = rhat;  // read by the red3 == 1 form only
         else
@@ -501,30 +508,36 @@ struct BiCGStab {
         launch_hop<R, SH, SM, SH, LK, MASK>(args(1, in_h, v, th, 0.0, 1.0, 0, FIN_NONE, 0), nrhs, h);
         launch_hop<R, SH, SX, SM, LK, MASK>(args(0, th, in_m, out, 1.0, -k2, 1, op, red3), nrhs, h);
     }
-    // solve Dtilde x = r (r holds the right-hand side; x starts at 0)
-    int run(const double* rr0, double tol, double abs_fac, int maxit, int chunk, int* iters_out) {
+    // solve Dtilde x = r (r holds the right-hand side of squared norm rr0, or,
+    // with re, becomes re / sqrt(rre); x starts at 0)
+    int run(const double* rr0, double tol, double abs_fac, int maxit, int chunk, int* iters_out,
+            const SpinorF64* re = nullptr, const double* rre = nullptr) {
         dim3 grid(grid_for(S.n, 128), nrhs);
         if (maxit < 1) maxit = 1;
-        DD_KLAUNCH(h, cg_arm_kernel<<<1, 64, 0, h->stream>>>(nrhs, st, outer, rr0, tol, abs_fac, maxit));
-        DD_KLAUNCH(h, bicg_arm_kernel<<<1, 64, 0, h->stream>>>(nrhs, st));
-        DD_KLAUNCH(h, bicg_start_kernel<R, SM, SH><<<grid, 128, 0, h->stream>>>(S, x, r, rhat, p, v, outer));
-        DD_KLAUNCH(h, bicg_rho_kernel<R, SM, SH><<<grid, 128, 0, h->stream>>>(S, rhat, r, st, red(FIN_BI_RHO)));
+        DD_KLAUNCH(h, cg_arm_kernel<<<1, 64, 0, h->stream>>>(nrhs, st, outer, re ? nullptr : rr0, tol, abs_fac, maxit));
+        DD_KLAUNCH(h, bicg_start_kernel<R, SM, SH><<<grid, 128, 0, h->stream>>>(
+                          S, x, r, rhat, p, re ? *re : SpinorF64{nullptr, 0}, re ? rre : nullptr, st, red(FIN_BI_RHO)));
         std::vector<CGState> hs(nrhs);
         int done = 0;
         bool polled = false;
+        // eager: the first poll comes after as many iterations as the last run
+        // took (a defect cycle takes about as many as the one before), further
+        // ones every 4: with a poll every 16 an 8^4 solve of 8 iterations a
+        // cycle launched half of its kernels for nothing
+        int cur = maxit <= chunk ? chunk : hint > 0 ? hint : 8;
+        if (dd_stream_capturing(h)) cur = chunk;
         auto body = [&]() -> int {
-            for (int it = 0; it < chunk; ++it) {
-                DD_KLAUNCH(h, bicg_p_kernel<R, SM, SH><<<grid, 128, 0, h->stream>>>(S, p, r, v, st));
+            for (int it = 0; it < cur; ++it) {
                 apply(p, p, v, FIN_BI_ALPHA, 1);
                 DD_KLAUNCH(h, bicg_s_kernel<R, SM, SH><<<grid, 128, 0, h->stream>>>(S, s, r, v, shop, copies, st));
                 apply(shop, s, t, FIN_BI_OMEGA, 2);
-                DD_KLAUNCH(h, bicg_xr_kernel<R, SM, SH><<<grid, 128, 0, h->stream>>>(S, x, r, p, s, t, rhat, st,
-                                                                                     red(FIN_BI_RHO)));
+                DD_KLAUNCH(h, bicg_xrp_kernel<R, SM, SH><<<grid, 128, 0, h->stream>>>(S, x, r, p, s, t, v, st));
             }
             return cudaGetLastError() == cudaSuccess ? DD_OK : DD_ERR_CUDA;
         };
         auto more = [&](bool& m) -> int {
-            done += chunk;
+            done += cur;
+            cur = 4;
             if (cudaMemcpyAsync(hs.data(), st, sizeof(CGState) * nrhs, cudaMemcpyDeviceToHost, h->stream) !=
                 cudaSuccess)
                 return DD_ERR_CUDA;
@@ -545,6 +558,9 @@ struct BiCGStab {
             flags |= hs[k].flags;
         }
         if (iters_out) *iters_out += tot;
+        hint = 0;
+        for (int k = 0; k < nrhs; ++k)
+            if (hs[k].iters > 1) hint = std::max(hint, hs[k].iters - 1);
         // a breakdown only ends this inner solve; the outer FP64 loop restarts from the true residual
         (void)flags;
         return DD_OK;
@@ -578,7 +594,8 @@ Reduce store_reduce(dd_handle* h, double* out) { return dd_reduce(h, FIN_STORE, 
 // bvec - that with resid (SOut SpinorF64), or the hops alone (SOut SpinorX)
 template <int MASK, class SOut>
 void hop64(dd_handle* h, SiteSet S, int nrhs, int par, SpinorX in, SpinorF64 xin, SOut out, double b, int hasx,
-           LinkX lk, long long lk_rs, const CGState* st, Reduce red, const SpinorF64* bvec = nullptr) {
+           LinkX lk, long long lk_rs, const CGState* st, Reduce red, const SpinorF64* bvec = nullptr,
+           const SOut* out2 = nullptr) {
     HopArgs<SpinorX, SpinorF64, SOut, LinkX> A;
     A.g = h->g;
     A.p = par;
@@ -598,6 +615,8 @@ void hop64(dd_handle* h, SiteSet S, int nrhs, int par, SpinorX in, SpinorF64 xin
     A.S = S;
     A.rhat = bvec ? *bvec : xin;
     A.resid = bvec != nullptr;
+    A.has2 = out2 != nullptr;
+    A.out2 = out2 ? *out2 : out;
     launch_hop<double, SpinorX, SpinorF64, SOut, LinkX, MASK>(A, nrhs, h);
 }
 
@@ -639,46 +658,43 @@ int defect_correction(dd_handle* h, int nrhs, int field0, int step, Inner& cg, b
     const long long rs64 = field_stride<LinkX>(h, step);
     CGState* outer = h->d_cg + h->prm.max_rhs;
     double* bb = h->d_scalars;
-    double* tmp = h->d_scalars + nrhs;
     double* rr = h->d_scalars + 2 * nrhs;
     double* ones = h->d_scalars + 3 * nrhs;
     Reduce none;
     none.op = FIN_NONE;
-    // |b|^2 over both parities, then b~ = b_e + kappa H_eo b_o (in place)
-    DD_KLAUNCH(h, norm2_kernel<SpinorF64><<<grid, 128, 0, h->stream>>>(S, be, store_reduce(h, bb)));
-    DD_KLAUNCH(h, norm2_kernel<SpinorF64><<<grid, 128, 0, h->stream>>>(S, bo, store_reduce(h, tmp)));
-    DD_KLAUNCH(h, add_scalars_kernel<<<1, 64, 0, h->stream>>>(nrhs, bb, tmp));
-    DD_KLAUNCH(h, copy_kernel<SpinorF64, SpinorX><<<grid, 128, 0, h->stream>>>(S, bo, box, nullptr));
-    hop64<MASK>(h, S, nrhs, 0, box, be, be, kappa, 1, lk64, rs64, nullptr, none);
+    // |b|^2 over both parities, then b~ = b_e + kappa H_eo b_o (in place; also
+    // the first residual, with |b~|^2 to the outer states)
+    DD_KLAUNCH(h, solve_start_kernel<<<grid, 128, 0, h->stream>>>(S, be, bo, box, xe, v.pxe, store_reduce(h, bb)));
     DD_KLAUNCH(h, outer_arm_kernel<<<1, 64, 0, h->stream>>>(nrhs, outer, bb, tol));
-    DD_KLAUNCH(h, zero64_kernel<<<grid, 128, 0, h->stream>>>(S, xe, v.pxe));
-    DD_KLAUNCH(h, copy_kernel<SpinorF64, SpinorF64><<<grid, 128, 0, h->stream>>>(S, be, re, nullptr));
-    DD_KLAUNCH(h, norm2_kernel<SpinorF64><<<grid, 128, 0, h->stream>>>(S, re, store_reduce(h, rr)));
-    DD_KLAUNCH(h, outer_update_kernel<<<1, 64, 0, h->stream>>>(nrhs, outer, rr, h->d_status));
+    hop64<MASK>(h, S, nrhs, 0, box, be, be, kappa, 1, lk64, rs64, nullptr, dd_reduce(h, FIN_OUTER, outer, rr), nullptr, &re);
     if (cudaGetLastError() != cudaSuccess) return DD_ERR_CUDA;
     const double tol_inner = fp64_inner ? 0.0 : h->prm.tol_inner;
     int total = 0, cycles = 0;
     bool polled = false;
     std::vector<CGState> hs(nrhs);
     auto body = [&]() -> int {
-        // inner right-hand side: the current FP64 residual
-        // (the mixed inner system is normalised to |r| = 1)
-        if (!fp64_inner) {
-            DD_KLAUNCH(h, normalised_copy_kernel<SM><<<grid, 128, 0, h->stream>>>(S, re, cg.r, rr, outer));
-            DD_KLAUNCH(h, fill_kernel<<<1, 64, 0, h->stream>>>(nrhs, ones, 1.0));
+        // inner right-hand side: the current FP64 residual (the mixed inner
+        // system is normalised to |r| = 1); inner stopping rule: FP64 inner
+        // aims at the outer target directly (with margin), the mixed inner at
+        // a relative reduction tol_inner
+        int it = 0, rc = DD_OK;
+        if constexpr (Inner::takes_residual) {
+            rc = cg.run(nullptr, tol_inner, -1.0, maxit - total, 16, &it, &re, rr);
+        } else {
+            if (!fp64_inner) {
+                DD_KLAUNCH(h, normalised_copy_kernel<SM><<<grid, 128, 0, h->stream>>>(S, re, cg.r, rr, outer));
+                DD_KLAUNCH(h, fill_kernel<<<1, 64, 0, h->stream>>>(nrhs, ones, 1.0));
+            }
+            rc = cg.run(fp64_inner ? rr : ones, tol_inner, fp64_inner ? 0.25 : -1.0, maxit - total, 16, &it);
         }
-        // inner stopping rule: FP64 inner aims at the outer target directly
-        // (with margin), the mixed inner at a relative reduction tol_inner
-        int it = 0;
-        int rc = cg.run(fp64_inner ? rr : ones, tol_inner, fp64_inner ? 0.25 : -1.0, maxit - total, 16, &it);
         total += it;
         if (rc) return rc;
         DD_KLAUNCH(h, add_correction_kernel<SM><<<grid, 128, 0, h->stream>>>(S, xe, px, cg.x,
                                                                           fp64_inner ? nullptr : rr, outer));
         // true residual r = b~ - Dtilde x (FP64)
         hop64<MASK>(h, S, nrhs, 1, px, xe, tx, 1.0, 0, lk64, rs64, outer, none);
-        hop64<MASK>(h, S, nrhs, 0, tx, xe, re, -kappa * kappa, 1, lk64, rs64, outer, store_reduce(h, rr), &be);
-        DD_KLAUNCH(h, outer_update_kernel<<<1, 64, 0, h->stream>>>(nrhs, outer, rr, h->d_status));
+        hop64<MASK>(h, S, nrhs, 0, tx, xe, re, -kappa * kappa, 1, lk64, rs64, outer,
+                    dd_reduce(h, FIN_OUTER, outer, rr), &be);
         return cudaGetLastError() == cudaSuccess ? DD_OK : DD_ERR_CUDA;
     };
     auto more = [&](bool& m) -> int {
