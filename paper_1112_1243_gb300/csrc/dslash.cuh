@@ -32,6 +32,20 @@ DD_DEV SpinorF16 at_rhs(SpinorF16 s, int r) {
     return s;
 }
 
+// canonical FP64 spinors of the caller (16-byte aligned), V sites a rhs
+struct SpinorC {
+    double2* p;
+    long long stride;
+};
+DD_DEV SpinorC at_rhs(SpinorC s, int r) {
+    s.p += (long long)r * 12 * s.stride;
+    return s;
+}
+// entry k of the site with even-odd index h and canonical index s
+DD_DEV long long entry_at(const SpinorF64& f, int k, int h, int s) { return k * f.stride + h; }
+DD_DEV long long entry_at(const SpinorC& f, int k, int h, int s) { return (long long)s * 12 + k; }
+DD_DEV long long entry_at(const SpinorX& f, int k, int h, int s) { return k * f.stride + h; }
+
 template <class SIn, class SX, class SOut, class LK>
 struct HopArgs {
     Geo g;
@@ -56,6 +70,10 @@ struct HopArgs {
     int resid = 0;              // FP64 hops: out = rhat - (xin + b * hops)
     int has2 = 0;               // FP64 hops: a second copy of out
     SOut out2;
+    int both = 0;               // FP64 hops: both output parities in one launch (blockIdx.z), in2: the input of parity 1
+    SIn in2;
+    int ob[4] = {0, 0, 0, 0};   // MASK 2: hops that leave a block of these extents are dropped too (0: none)
+    const double* U = nullptr;  // FP64 hops on canonical fields: the links, for sites with non-finite neighbours
 };
 
 template <class LK>
@@ -212,11 +230,55 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
 // (8 x 16384 sites: 28 -> 15 us).  Two lanes a site with one spin each took
 // 2.5 times the instructions and 830 us.  At 2^20 sites what is left is
 // latency: 20 warps an SM (96 registers), DRAM at 45%, issue slots at 32%.
+
+// The hops onto one site in FP64 arithmetic on the caller's fields (x: its
+// coordinates): the integer form marks whole sites and links that hold a
+// number that is not finite; this keeps what such a number does to each
+// component.
+template <int MASK>
+__device__ __noinline__ void hop_canonical(const Geo& g, const int* x, const double* U, const double2* in, int g5in,
+                                           Spinor<double>& acc) {
+    zero(acc);
+    const int s = canon_index(g, x);
+    const bool al16 = (reinterpret_cast<uintptr_t>(U) & 15) == 0;
+#pragma unroll 1
+    for (int a = 0; a < 4; ++a) {
+        const int loc = x[a] % g.b[a];
+#pragma unroll 1
+        for (int dir = 1; dir >= -1; dir -= 2) {
+            const bool face = loc == (dir > 0 ? g.b[a] - 1 : 0);
+            if (MASK && (MASK == 1 ? face : !face)) continue;
+            const int y = shift_index(g, x, a, dir);
+            Spinor<double> v;
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {
+                const double2 w = in[(long long)y * 12 + k];
+                v.c[k] = mk<double>(w.x, w.y);
+            }
+            if (g5in) gamma5(v);
+            Half<double> h, uh;
+            project<double>(a, dir, v, h);
+            Link<double> u;
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                const double2 w = load_c(U, ((long long)(dir > 0 ? s : y) * 4 + a) * 9 + k, al16);
+                u.m[k / 3][k % 3] = mk<double>(w.x, w.y);
+            }
+            if (dir > 0)
+                mul_link(u, h, uh);
+            else
+                mul_link_dag(u, h, uh);
+            const bool wrap = a == 3 && x[3] == (dir > 0 ? g.L[3] - 1 : 0);
+            accumulate<double>(a, dir, uh, wrap ? (double)g.bc : 1.0, acc);
+        }
+    }
+}
+
 template <class SX, class SOut, int MASK>
 __global__ void __launch_bounds__(128, 5) hop_x_kernel(HopArgs<SpinorX, SX, SOut, LinkX> A) {
     __shared__ long long part[4][24][X_PAD];  // axis; sum (0..11) and difference (12..23) of its hops
-    __shared__ int ex[4][X_TILE], hs[X_TILE];
-    const int rhs = blockIdx.y;
+    __shared__ int ex[4][X_TILE], hs[X_TILE], ss[X_TILE];
+    const int rhs = blockIdx.y, par = A.both ? (int)blockIdx.z : A.p;
     if (A.st && !A.st[rhs].active) return;
     const Geo& g = A.g;
     const long long Vh = g.Vh;
@@ -225,44 +287,52 @@ __global__ void __launch_bounds__(128, 5) hop_x_kernel(HopArgs<SpinorX, SX, SOut
     if (A.sites && threadIdx.x == 0) atomicAdd(A.sites, (unsigned long long)min((long long)X_TILE, A.S.n - base));
     auto site = [&](int i, int x[4]) -> int {  // even-odd index and coordinates of site i of the tile
         const long long t = min(base + i, A.S.n - 1);
-        if (A.S.colour >= 0) return colour_site(g, A.S.colour, (int)t, A.p, x);
+        if (A.S.colour >= 0) return colour_site(g, A.S.colour, (int)t, par, x);
         const int h = (int)A.S.at(t);
-        eo_coords(g, A.p, h, x);
+        eo_coords(g, par, h, x);
         return h;
     };
     {
         int x[4];
         const int h = site(lane, x);
         const int s = canon_index(g, x);
-        const SpinorX in = at_rhs(A.in, rhs);
+        const SpinorX in = at_rhs((A.both && par) ? A.in2 : A.in, rhs);
         const int4* lk = A.lk.p + (long long)rhs * A.lk_rhs_stride;
         const int* le = LinkX{lk, A.lk.stride}.exps();
         const int xa = a == 0 ? x[0] : a == 1 ? x[1] : a == 2 ? x[2] : x[3];
         const int La = g.L[a], sa = g.st[a];
         const bool top = xa == La - 1, bottom = xa == 0;
         const int yf = (top ? s - (La - 1) * sa : s + sa) >> 1, yb = (bottom ? s + (La - 1) * sa : s - sa) >> 1;
-        const long long rf = (long long)(A.p * 4 + a) * Vh + h, rb = (long long)((1 - A.p) * 4 + a) * Vh + yb;
+        const long long rf = (long long)(par * 4 + a) * Vh + h, rb = (long long)((1 - par) * 4 + a) * Vh + yb;
         bool okf = true, okb = true;
         if (MASK) {
             const int loc = xa - fast_div(xa, g.b[a], g.mb[a]) * g.b[a];
             const bool ff = loc == g.b[a] - 1, fb = loc == 0;
             okf = MASK == 1 ? !ff : ff;
             okb = MASK == 1 ? !fb : fb;
+            if (MASK == 2 && A.ob[a]) {
+                const int lo = xa % A.ob[a];
+                okf = okf && lo != A.ob[a] - 1;
+                okb = okb && lo != 0;
+            }
         }
         const int ef = okf ? in.e[yf] + le[rf] : 2 * X_ZERO, eb = okb ? in.e[yb] + le[rb] : 2 * X_ZERO;
         ex[a][lane] = max(ef, eb);
+        if (a == 0) {
+            hs[lane] = h;
+            ss[lane] = s;
+        }
         __syncthreads();
         const int eout = max(max(ex[0][lane], ex[1][lane]), max(ex[2][lane], ex[3][lane]));
-        if (a == 0) hs[lane] = h;
         const bool phase = a == 3 && g.bc < 0;
-        x_axis(a, A.g5in != 0, okf, eout - ef, in.p, in.stride, (unsigned)yf * 16u, lk + (long long)(A.p * 4 + a) * 9 * Vh,
+        x_axis(a, A.g5in != 0, okf, eout - ef, in.p, in.stride, (unsigned)yf * 16u, lk + (long long)(par * 4 + a) * 9 * Vh,
                (unsigned)h * 16u, phase && top, okb, eout - eb, (unsigned)yb * 16u,
-               lk + (long long)((1 - A.p) * 4 + a) * 9 * Vh, (unsigned)yb * 16u, phase && bottom, Vh, part[a], lane);
+               lk + (long long)((1 - par) * 4 + a) * 9 * Vh, (unsigned)yb * 16u, phase && bottom, Vh, part[a], lane);
     }
     __syncthreads();
     const int i = 8 * a + (lane & 7), q = lane >> 3;  // spin q of site i
     const bool valid = base + i < A.S.n;
-    const int h = hs[i];
+    const int h = hs[i], s = ss[i];
     const int eout = max(max(ex[0][i], ex[1][i]), max(ex[2][i], ex[3][i]));
     xacc v[3];
     x_gather(part, i, q, v);
@@ -292,14 +362,33 @@ __global__ void __launch_bounds__(128, 5) hop_x_kernel(HopArgs<SpinorX, SX, SOut
             // number (conversion and FMA run on the FP64 pipe beside the
             // integer pipes: 30 clocks a site)
             const double f0 = (q > 1 && A.g5out) ? -A.b : A.b;
-            const bool usual = abs(eout) < 900;
+            bool usual = abs(eout) < 900;
+            double2 other[3];
+            if (!usual) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    other[c] = make_double2(x_to_double_any(v[c].x, eout), x_to_double_any(v[c].y, eout));
+                if constexpr (std::is_same<SX, SpinorC>::value) {
+                    if (eout >= X_BAD_MIN) {
+                        int x[4];
+                        site(i, x);
+                        Spinor<double> acc;
+                        hop_canonical<MASK>(g, x, A.U, xin.p, A.g5in, acc);
+#pragma unroll
+                        for (int c = 0; c < 3; ++c)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                if (e == q) other[c] = make_double2(acc.c[3 * e + c].x, acc.c[3 * e + c].y);
+                    }
+                }
+            }
             const double f = usual ? __hiloint2double((eout - 56 + 1023) << 20, 0) * f0 : f0;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const long long k = (3 * q + c) * out.stride + h;
+                const long long k = entry_at(out, 3 * q + c, h, s);
                 const double2 w = A.has_x ? xin.p[k] : make_double2(0.0, 0.0);
                 double2 z = make_double2((double)v[c].x, (double)v[c].y);
-                if (!usual) z = make_double2(x_to_double_any(v[c].x, eout), x_to_double_any(v[c].y, eout));
+                if (!usual) z = other[c];
                 z = make_double2(fma(f, z.x, w.x), fma(f, z.y, w.y));
                 if (A.resid) {
                     const double2 w = bv.p[k];
@@ -334,7 +423,7 @@ inline void launch_hop(const HopArgs<SIn, SX, SOut, LK>& A, int nrhs, dd_handle*
     int tpb = std::min(f64 ? h->tune.hop64_tpb : h->tune.hop_tpb, 128);  // the kernels' launch bound
     if (f64) tpb = 128;  // four warps (hop_x_kernel)
     const int spt = (!f64 && h->tune.hop_spt == 2) ? 2 : 1;
-    dim3 grid(grid_for(B.S.n, f64 ? X_TILE : (long long)tpb * spt), nrhs);
+    dim3 grid(grid_for(B.S.n, f64 ? X_TILE : (long long)tpb * spt), nrhs, f64 && A.both ? 2 : 1);
     constexpr int kind0 = hop_kind<SIn, SOut>();
     // whole-lattice hops keep kinds 0-2; Dirichlet hops are timed as 4 (FP64),
     // 5, 6 (one block colour's sites) or 8, 9 (every site)

@@ -866,6 +866,65 @@ int apply_eo_ops(dd_handle* h, int op, SH in_e, SH in_o, SS x_e, SS x_o, SH th, 
 
 }  // namespace
 
+// canonical spinors -> limbs, both parities (one thread a site)
+__global__ void __launch_bounds__(128) pack_x_kernel(Geo g, const double* __restrict__ in, bool al16, SpinorX even,
+                                                     SpinorX odd) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+    if (s >= g.V) return;
+    int x[4];
+    canon_coords(g, s, x);
+    Spinor<double> v;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const double2 w = load_c(in, ((long long)r * g.V + s) * 12 + k, al16);
+        v.c[k] = mk<double>(w.x, w.y);
+    }
+    at_rhs(((x[0] + x[1] + x[2] + x[3]) & 1) ? odd : even, r).store(s >> 1, v);
+}
+
+// D, D^dag, the block operators or the hops between blocks in FP64, straight
+// between the caller's fields: links and spinors into limbs, then one launch
+// for both parities (three launches; packing to FP64 vectors, two hops and
+// unpacking made nine: 48 us on 4^4 and 0.6 of 2.2 ms at 32^3 x 64).  Taken
+// when both spinor fields start on 16-byte boundaries.
+static int apply_canonical(dd_handle* h, void* out, const void* in, const void* U, int op, int nrhs, int colour_mask,
+                           int mask_mode) {
+    const Geo& g = h->g;
+    const long long Vh = g.Vh;
+    SolverVecs& v = h->vecs[0];
+    const SpinorX even{v.px, v.pxe, Vh}, odd{reinterpret_cast<int4*>(v.re), v.rxe, Vh};
+    DD_KLAUNCH(h, pack_x_kernel<<<dim3(grid_for(g.V, 128), nrhs), 128, 0, h->stream>>>(g, (const double*)in, true, even,
+                                                                                      odd));
+    HopArgs<SpinorX, SpinorC, SpinorC, LinkX> A;
+    A.g = g;
+    A.p = 0;
+    A.both = 1;
+    A.in = odd;
+    A.in2 = even;
+    A.xin = SpinorC{(double2*)in, g.V};
+    A.out = SpinorC{(double2*)out, g.V};
+    A.rhat = A.xin;
+    A.out2 = A.out;
+    A.lk = LinkX{h->fields[0].eox, Vh};
+    A.lk_rhs_stride = 0;
+    A.a = 1.0;
+    A.b = -h->prm.kappa;
+    A.has_x = op != DD_OP_INTER;
+    A.g5in = A.g5out = op == DD_OP_DDAG;
+    A.colour_mask = colour_mask;
+    A.st = nullptr;
+    A.red.op = FIN_NONE;
+    A.U = (const double*)U;
+    if (op == DD_OP_INTER)
+        launch_hop<double, SpinorX, SpinorC, SpinorC, LinkX, 2>(A, nrhs, h);
+    else if (mask_mode == 1)
+        launch_hop<double, SpinorX, SpinorC, SpinorC, LinkX, 1>(A, nrhs, h);
+    else
+        launch_hop<double, SpinorX, SpinorC, SpinorC, LinkX, 0>(A, nrhs, h);
+    DD_LAUNCH_CHECK(h, "apply");
+    return DD_OK;
+}
+
 static int apply_common(dd_handle* h, void* out, const void* in, const void* U, int op, int prec, int nrhs,
                         int colour_mask, int mask_mode) {
     int rc = dd_require_ws(h);
@@ -884,6 +943,8 @@ static int apply_common(dd_handle* h, void* out, const void* in, const void* U, 
     const bool even_in = (op == DD_OP_DTILDE || op == DD_OP_DTILDE_DAG);
     const bool odd_in = (op == DD_OP_HEO);
     const bool sub_out = even_in || odd_in;
+    if (prec == DD_PREC_F64 && !sub_out && aligned16(in) && aligned16(out))
+        return apply_canonical(h, out, in, U, op, nrhs, colour_mask, mask_mode);
     // input parities in FP64 eo chunks
     if (even_in) {
         launch_pack_spinor_sub(h, (const double*)in, v.be, nrhs);

@@ -85,3 +85,51 @@ def test_scales_far_from_one(api):
     out = dev(np.ones_like(psi))
     api.dd_apply_D(h, out, dev(0 * psi), dev(U), api.DD_OP_D, api.DD_PREC_F64, 1)
     assert np.all(host(out) == 0)
+
+
+def test_non_finite_numbers_stay_in_their_components(api):
+    """An infinity or NaN in a spinor or link entry reaches exactly the
+    components that the FP64 stencil takes it to."""
+    dims, block, kappa = (4, 4, 6, 4), (2, 2, 3, 2), 0.13
+    lat = geometry.Lattice(dims, block)
+    U, psi = synthetic.random_gauge(dims, 0.4, 2), synthetic.random_spinor(dims, 5)
+    psi[17, 2, 1] = np.inf
+    U[200, 3, 1, 2] = np.nan
+    h = api.dd_init(dims, block, kappa)
+    out = dev(np.zeros_like(psi))
+    api.dd_apply_D(h, out, dev(psi), dev(U), api.DD_OP_D, api.DD_PREC_F64, 1)
+    got = host(out)
+    # sites next to neither are finite, and equal to those of the clean fields
+    touched = {17, 200, int(lat.fwd[200, 3])} | {int(n[17, a]) for n in (lat.fwd, lat.bwd) for a in range(4)}
+    clean = np.array([s not in touched for s in range(lat.V)])
+    assert np.all(np.isfinite(got[clean]))
+    bad = ~np.isfinite(got)
+    # the link's row 1 (forward, at its site) and column 2 (backward, at its far end); the rest stays finite
+    assert bad[200, :, 1].all() and not bad[200, :, 0].any() and not bad[200, :, 2].any()
+    far = int(lat.fwd[200, 3])
+    assert bad[far, :, 2].all() and not bad[far, :, 0].any() and not bad[far, :, 1].any()
+    # a spinor component: its own at its site; two of the four spins of every neighbour, all colours
+    assert bad[17].sum() == 1 and bad[17, 2, 1]
+    for n in touched - {17, 200, far}:
+        assert bad[n].all(axis=1).sum() >= 2
+
+
+@pytest.mark.parametrize("shift", [0, 8])
+def test_fields_on_8_byte_boundaries(api, shift):
+    """The C ABI asks for the alignment of a double: the same numbers through
+    the paths for 16-byte and for 8-byte boundaries."""
+    import torch
+    dims, block = (4, 4, 4, 6), (2, 2, 2, 3)
+    U, psi = synthetic.random_gauge(dims, 0.4, 2), synthetic.random_spinor(dims, 5, nrhs=2)
+    h = api.dd_init(dims, block, 0.13, max_rhs=2)
+    ref = dev(np.zeros_like(psi))
+    api.dd_apply_D(h, ref, dev(psi), dev(U), api.DD_OP_DDAG, api.DD_PREC_F64, 2)
+
+    def at(a):
+        flat = torch.zeros(2 * a.size + 2, dtype=torch.float64, device="cuda")
+        flat[shift // 8:shift // 8 + 2 * a.size] = dev(a).view(torch.float64).reshape(-1)
+        return flat, flat.data_ptr() + shift
+    bufs = [at(np.zeros_like(psi)), at(psi), at(U)]
+    api.dd_apply_D(h, bufs[0][1], bufs[1][1], bufs[2][1], api.DD_OP_DDAG, api.DD_PREC_F64, 2)
+    got = host(bufs[0][0])[shift // 8:shift // 8 + 2 * psi.size].view(np.complex128).reshape(psi.shape)
+    assert np.array_equal(got, host(ref))
