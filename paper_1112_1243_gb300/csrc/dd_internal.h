@@ -157,7 +157,8 @@ struct dd_handle {
     size_t ws_needed = 0;
     std::vector<FieldSlot> fields;   // max_rhs + 1 slots
     std::vector<SolverVecs> vecs;    // max_rhs systems
-    double2* dd_vec = nullptr;       // block-ordered FP64 vectors: [6][max_rhs][12][V]
+    double2* dd_vec = nullptr;       // even-odd vectors of the estimator: [3][parity][max_rhs][12][Vh]
+    int* d_xexp = nullptr;           // exponents of the one in limbs: [parity][max_rhs][Vh]
     CGState* d_cg = nullptr;         // [3 * max_rhs + 2]: inner, outer, SAP block-solver states
     SapVecs sap;                     // SAP-preconditioned GCR (krylov DD_KRYLOV_SAP_GCR)
     double* d_partials = nullptr;    // reduction partials

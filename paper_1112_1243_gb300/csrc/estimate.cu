@@ -43,137 +43,50 @@ DD_DEV void dd_coords(const Geo& g, const BlockCtx& c, long long q, int x[4], in
     for (int a = 0; a < 4; ++a) x[a] = o[a] + l[a];
 }
 
-// extents of the enclosing blocks of a two-level decomposition (x = 0: none)
-DD_DEV bool same_outer_block(int4 ob, const int x[4], const int y[4]) {
-    return ob.x == 0 || (x[0] / ob.x == y[0] / ob.x && x[1] / ob.y == y[1] / ob.y && x[2] / ob.z == y[2] / ob.z &&
-                         x[3] / ob.w == y[3] / ob.w);
-}
+// colour of the enclosing block of extents ob
 DD_DEV int outer_colour(int4 ob, const int x[4]) { return (x[0] / ob.x + x[1] / ob.y + x[2] / ob.z + x[3] / ob.w) & 1; }
 
-// eta on the black sites (purpose / sub), 0 on white; block order.  With
-// enclosing blocks (ob.x > 0) only inside the enclosing blocks whose colour
-// is in outer_mask.
-__global__ void noise_black_kernel(Geo g, BlockCtx c, double2* bank, long long vs, int purpose, uint64_t seed,
-                                   uint64_t ctr0, const unsigned long long* ctr_off, int4 ob, int outer_mask) {
+// eta on the black sites (purpose / sub), in FP64 and in limbs; the white
+// sites are not written (no kernel reads them).  With enclosing blocks (ob.x
+// > 0) 0 outside the enclosing blocks whose colour is in outer_mask.  Threads
+// in block order: the black sites come first, so no warp holds white ones.
+__global__ void __launch_bounds__(128) noise_black_kernel(Geo g, BlockCtx c, double2* eta, SpinorX ee, SpinorX eo,
+                                                          long long parity_stride, int purpose, uint64_t seed,
+                                                          uint64_t ctr0, const unsigned long long* ctr_off, int4 ob,
+                                                          int outer_mask) {
     const uint64_t ctr = stream_ctr(ctr0, ctr_off);
-    long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    int i = blockIdx.y;
-    if (q >= g.V) return;
+    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.y;
+    if (q >= g.V / 2) return;
     int x[4], col;
     dd_coords(g, c, q, x, &col);
-    long long pos = q / c.nb, j = q % c.nb;
-    SpinorF64 out{bank + (long long)i * vs + pos * 12 * c.nb, c.nb};
+    const uint32_t s = (uint32_t)canon_index(g, x);
+    const int par = (x[0] + x[1] + x[2] + x[3]) & 1;
     Spinor<double> e;
-    uint32_t s = (uint32_t)canon_index(g, x);
-    if (col == 0 && (ob.x == 0 || ((outer_mask >> outer_colour(ob, x)) & 1))) {
+    if (ob.x == 0 || ((outer_mask >> outer_colour(ob, x)) & 1)) {
         for (int k = 0; k < 12; ++k) e.c[k] = gaussian(s * 12u + k, (uint32_t)purpose, (uint32_t)i, seed, ctr);
     } else {
         zero(e);
     }
-    out.store(j, e);
+    at_rhs(SpinorF64{eta + par * parity_stride, g.Vh}, i).store(s >> 1, e);
+    at_rhs(par ? eo : ee, i).store(s >> 1, e);
 }
 
-// out = -kappa * (hops that cross block faces) in, on the sites of colour
-// `target` (0 elsewhere).  Links from the canonical FP64 copy of the field
-// of slot f0 + i * fstep for right-hand side i.  With enclosing blocks
-// (ob.x > 0), hops that leave the enclosing block are dropped as well.
-__global__ void inter_hop_kernel(Geo g, BlockCtx c, const double2* in_bank, double2* out_bank, long long vs,
-                                 const double* canon0, long long canon_fs, int f0, int fstep, int target,
-                                 int4 ob) {
-    long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    int i = blockIdx.y;
-    if (q >= g.V) return;
-    const double* U = canon0 + (long long)(f0 + i * fstep) * canon_fs;
-    int x[4], col;
-    dd_coords(g, c, q, x, &col);
-    long long pos = q / c.nb, j = q % c.nb;
-    Spinor<double> acc;
-    zero(acc);
-    if (col == target) {
-        const int s = canon_index(g, x);
-        for (int a = 0; a < 4; ++a) {
-            // a hop crosses a block face iff x sits on that face (two or more blocks per direction)
-            const int loc = x[a] % g.b[a];
-            for (int dir = +1; dir >= -1; dir -= 2) {
-                if (dir > 0 ? loc != g.b[a] - 1 : loc != 0) continue;
-                int y[4] = {x[0], x[1], x[2], x[3]};
-                y[a] += dir;
-                if (y[a] == g.L[a]) y[a] = 0;
-                if (y[a] < 0) y[a] = g.L[a] - 1;
-                if (!same_outer_block(ob, x, y)) continue;
-                long long qy = dd_position(g, y);
-                SpinorF64 src{(double2*)in_bank + (long long)i * vs + (qy / c.nb) * 12 * c.nb, c.nb};
-                Spinor<double> sp;
-                src.load(qy % c.nb, sp);
-                Half<double> hf, uh;
-                project<double>(a, dir, sp, hf);
-                Link<double> u;
-                const int ys = canon_index(g, y);
-                const double* lp = U + ((long long)(dir > 0 ? s : ys) * 4 + a) * 18;
-                for (int k = 0; k < 9; ++k) u.m[k / 3][k % 3] = mk<double>(lp[2 * k], lp[2 * k + 1]);
-                if (dir > 0)
-                    mul_link(u, hf, uh);
-                else
-                    mul_link_dag(u, hf, uh);
-                double sc = 1.0;
-                if (a == 3 && ((dir > 0 && x[3] == g.L[3] - 1) || (dir < 0 && x[3] == 0))) sc = g.bc;
-                accumulate<double>(a, dir, uh, sc, acc);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 12; ++k) acc.c[k] = (-c.kappa) * acc.c[k];
-    }
-    SpinorF64 dst{out_bank + (long long)i * vs + pos * 12 * c.nb, c.nb};
-    dst.store(j, acc);
-}
-
-// out = v - D_b[field] a on black sites, 0 on white (block order)
-__global__ void schur_source_kernel(Geo g, BlockCtx c, const double2* v_bank, const double2* a_bank,
-                                    double2* out_bank, long long vs, const double* canon0, long long canon_fs, int f0,
-                                    int fstep) {
-    long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    int i = blockIdx.y;
-    if (q >= g.V) return;
-    long long pos = q / c.nb;
-    int j = (int)(q % c.nb);
-    SpinorF64 dst{out_bank + (long long)i * vs + pos * 12 * c.nb, c.nb};
-    Spinor<double> r;
-    if (pos < g.nblocks / 2) {
-        SpinorF64 av{(double2*)a_bank + (long long)i * vs + pos * 12 * c.nb, c.nb};
-        SpinorF64 vv{(double2*)v_bank + (long long)i * vs + pos * 12 * c.nb, c.nb};
-        int colour, org[4];
-        block_origin(g, block_id_at(g, (int)pos, &colour), org);
-        const LinkCanonF64 lk{canon0 + (long long)(f0 + i * fstep) * canon_fs, g, c, {org[0], org[1], org[2], org[3]}};
-        Spinor<double> acc, a;
-        dirichlet_hop<double>(c, j, av, lk, 0, acc);
-        av.load(j, a);
-        vv.load(j, r);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) r.c[k] = r.c[k] - (a.c[k] + (-c.kappa) * acc.c[k]);
-    } else {
-        zero(r);
-    }
-    dst.store(j, r);
-}
-
-// block order (FP64) -> eo FP64 chunks of the global solver
-__global__ void dd_to_eo_kernel(Geo g, BlockCtx c, const double2* bank, long long vs, double2* be, double2* bo) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    int i = blockIdx.y;
-    if (s >= g.V) return;
-    int x[4];
-    canon_coords(g, s, x);
-    long long q = dd_position(g, x);
-    SpinorF64 src{(double2*)bank + (long long)i * vs + (q / c.nb) * 12 * c.nb, c.nb};
+// limbs of an even-odd solution (both parities)
+__global__ void __launch_bounds__(128) limbs_kernel(SiteSet S, SpinorF64 xe, SpinorF64 xo, SpinorX le, SpinorX lo) {
+    const int rhs = blockIdx.y;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= S.n) return;
+    const long long i = S.at(t);
     Spinor<double> v;
-    src.load(q % c.nb, v);
-    const int par = (x[0] + x[1] + x[2] + x[3]) & 1;
-    SpinorF64 dst{(par ? bo : be) + (long long)i * 12 * g.Vh, g.Vh};
-    dst.store(s >> 1, v);
+    at_rhs(xe, rhs).load(i, v);
+    at_rhs(le, rhs).store(i, v);
+    at_rhs(xo, rhs).load(i, v);
+    at_rhs(lo, rhs).store(i, v);
 }
 
-// ln_i = -sum_black (2 Re<eta, d> + |d|^2), d from the eo solution
-__global__ void __launch_bounds__(128) estimate_kernel(Geo g, BlockCtx c, const double2* eta_bank, long long vs,
+// ln_i = -sum_black (2 Re<eta, d> + |d|^2)
+__global__ void __launch_bounds__(128) estimate_kernel(Geo g, BlockCtx c, const double2* eta, long long parity_stride,
                                                        const double2* xe, const double2* xo, Reduce red) {
     long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     int i = blockIdx.y;
@@ -181,11 +94,10 @@ __global__ void __launch_bounds__(128) estimate_kernel(Geo g, BlockCtx c, const 
     if (q < g.V / 2) {  // black sites come first in block order
         int x[4], col;
         dd_coords(g, c, q, x, &col);
-        SpinorF64 es{(double2*)eta_bank + (long long)i * vs + (q / c.nb) * 12 * c.nb, c.nb};
         Spinor<double> e, d;
-        es.load(q % c.nb, e);
         const int s = canon_index(g, x);
         const int par = (x[0] + x[1] + x[2] + x[3]) & 1;
+        at_rhs(SpinorF64{(double2*)eta + par * parity_stride, g.Vh}, i).load(s >> 1, e);
         SpinorF64 ds{(double2*)(par ? xo : xe) + (long long)i * 12 * g.Vh, g.Vh};
         ds.load(s >> 1, d);
 #pragma unroll
@@ -359,6 +271,7 @@ static int run_blocks(dd_handle* h, const BlockArgs& A, int slots, cudaStream_t 
 }
 
 // format slots 0..nslots-1 from interpolated (or copied) fields
+// (eo: for even-odd solves, else in block order for the persistent solver)
 static int prepare_fields(dd_handle* h, const double* U_old, const double* U_new, int n, bool factors, bool eo,
                           bool all_links = false) {
     const int nslots = factors ? n + 1 : 2;
@@ -372,7 +285,7 @@ static int prepare_fields(dd_handle* h, const double* U_old, const double* U_new
         FieldSlot& f = h->fields[k];
         bool need_eo = eo;  // old and new fields both enter even-odd solves
         rc = format_field(h, (const double*)f.canon, f, need_eo, need_eo && ip == DD_PREC_F32,
-                          need_eo && ip == DD_PREC_F16, true);
+                          need_eo && ip == DD_PREC_F16, !need_eo);
         if (rc) return rc;
     }
     return DD_OK;
@@ -465,49 +378,95 @@ static void raise_status_host(dd_handle* h, int code) {
     DD_KLAUNCH(h, set_status_kernel<<<1, 1, 0, h->stream>>>(h->d_status, code));
 }
 
-// eo FP64 chunks of the global solver -> block order (FP64); sites of
-// blocks whose colour is not in colour_mask are written as zero
-__global__ void eo_to_dd_kernel(Geo g, BlockCtx c, const double2* xe, const double2* xo, double2* bank,
-                                long long vs, int colour_mask) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    int i = blockIdx.y;
-    if (s >= g.V) return;
-    int x[4];
-    canon_coords(g, s, x);
-    long long q = dd_position(g, x);
-    const int par = (x[0] + x[1] + x[2] + x[3]) & 1;
-    SpinorF64 src{(double2*)(par ? xo : xe) + (long long)i * 12 * g.Vh, g.Vh};
-    Spinor<double> v;
-    if ((colour_mask >> block_colour_of(g, x)) & 1)
-        src.load(s >> 1, v);
-    else
-        zero(v);
-    SpinorF64 dst{bank + (long long)i * vs + (q / c.nb) * 12 * c.nb, c.nb};
-    dst.store(q % c.nb, v);
-}
-
-// out_bank[i] = (D_bb + D_ww)^{-1} in_bank[i] for i < n, with the gauge field
-// of slot field0 + i * step: every Dirichlet block solve of every factor in
-// one batched even-odd Krylov solve (inner precision of the handle, FP64
-// defect correction to tol_block relative to the whole right-hand side).
-// The right-hand sides live on the blocks of one colour (0 black, 1 white);
-// only that colour's sites are visited, the other colour of out_bank is 0.
-static int dirichlet_solve_bank(dd_handle* h, const double2* in_bank, double2* out_bank, int n, int field0,
-                                int step, int colour) {
+// ------------------------------------------------------ the Schur pieces
+// The source s of the global solve (or, on the sub-block level, of the block
+// solve) of every factor i (fields f = fs * i and f + 1), left in the
+// solver's right-hand side (white sites 0).  All vectors stay in the even-odd
+// layout of the solver and the hops between and inside blocks are those of
+// hop_x_kernel; one batched even-odd Dirichlet solve per inverse (inner
+// precision of the handle, FP64 accuracy to tol_block relative to the whole
+// right-hand side) visits the sites of one colour only.  With vectors in
+// block order and FP64 stencils on canonical links the hops between blocks,
+// A' and the reordering took 6.2 of 125 ms of a step at 16^3 x 32; they take 2.2.
+static int schur_source(dd_handle* h, int n, int fs, int purpose, uint64_t seed, uint64_t ctr, int4 ob,
+                        int outer_mask) {
     const Geo& g = h->g;
     const BlockCtx c = block_ctx(h);
-    const long long vs = 12LL * g.V;
+    const long long Vh = g.Vh, ps = (long long)h->prm.max_rhs * 12 * Vh;  // entries between the parities of a bank
     SolverVecs& v = h->vecs[0];
-    dim3 gv(grid_for(g.V, 128), n);
-    DD_KLAUNCH(h, dd_to_eo_kernel<<<gv, 128, 0, h->stream>>>(g, c, in_bank, vs, v.be, v.bo));
-    DD_LAUNCH_CHECK(h, "dd_to_eo_kernel");
-    int it = 0;
-    int rc = solve_packed(h, n, field0, step, h->prm.inner_prec, h->prm.tol_block, h->prm.maxit, &it, nullptr, 1,
-                          colour);
-    if (rc && rc != DD_ERR_NOT_CONVERGED) return dd_fail(h, rc, "Dirichlet block solves failed");
-    if (rc == DD_ERR_NOT_CONVERGED) raise_status_host(h, DD_ERR_NOT_CONVERGED);
-    DD_KLAUNCH(h, eo_to_dd_kernel<<<gv, 128, 0, h->stream>>>(g, c, v.xe, v.xo, out_bank, vs, 1 << colour));
-    DD_LAUNCH_CHECK(h, "eo_to_dd_kernel");
+    double2* eta = h->dd_vec;
+    int4* etax = reinterpret_cast<int4*>(h->dd_vec + 2 * ps);
+    double2* vp = h->dd_vec + 4 * ps;
+    const SpinorX ex[2] = {{etax, h->d_xexp, Vh}, {etax + ps, h->d_xexp + (long long)h->prm.max_rhs * Vh, Vh}};
+    const SpinorX zx[2] = {{v.px, v.pxe, Vh}, {v.tx, v.txe, Vh}};
+    const SpinorF64 b[2] = {{v.be, Vh}, {v.bo, Vh}}, x[2] = {{v.xe, Vh}, {v.xo, Vh}},
+                    p[2] = {{vp, Vh}, {vp + ps, Vh}};
+    const long long rs = fs ? (long long)(h->fields[1].eox - h->fields[0].eox) : 0;
+    auto sites = [&](int colour) {
+        return h->d_colour_sites[colour] ? SiteSet{h->d_colour_sites[colour], Vh / 2, colour} : SiteSet{nullptr, Vh};
+    };
+    auto args = [&](int colour, int f, const SpinorX* in, const SpinorF64* out, int par) {
+        HopArgs<SpinorX, SpinorF64, SpinorF64, LinkX> A;
+        A.g = g;
+        A.p = par;
+        A.in = in[1 - par];
+        A.xin = A.out = A.rhat = A.out2 = out[par];
+        A.lk = LinkX{h->fields[f].eox, Vh};
+        A.lk_rhs_stride = rs;
+        A.a = 1.0;
+        A.b = -h->prm.kappa;
+        A.has_x = A.g5in = A.g5out = 0;
+        A.colour_mask = h->d_colour_sites[colour] ? 3 : 1 << colour;
+        A.st = nullptr;
+        A.red.op = FIN_NONE;
+        A.S = sites(colour);
+        A.ob[0] = ob.x;
+        A.ob[1] = ob.y;
+        A.ob[2] = ob.z;
+        A.ob[3] = ob.w;
+        return A;
+    };
+    // hops across block faces onto the sites of one colour
+    auto inter = [&](int colour, int f, const SpinorX* in, const SpinorF64* out) {
+        for (int par = 0; par < 2; ++par)
+            launch_hop<double, SpinorX, SpinorF64, SpinorF64, LinkX, 2>(args(colour, f, in, out, par), n, h);
+    };
+    // x = D_b^{-1} b on the blocks of one colour, and its limbs
+    auto solve = [&](int colour, int f) -> int {
+        int it = 0;
+        const int rc = solve_packed(h, n, f, fs, h->prm.inner_prec, h->prm.tol_block, h->prm.maxit, &it, nullptr, 1, colour);
+        if (rc && rc != DD_ERR_NOT_CONVERGED) return dd_fail(h, rc, "Dirichlet block solves failed");
+        if (rc == DD_ERR_NOT_CONVERGED) raise_status_host(h, DD_ERR_NOT_CONVERGED);
+        const SiteSet S = sites(colour);
+        DD_KLAUNCH(h, limbs_kernel<<<dim3(grid_for(S.n, 128), n), 128, 0, h->stream>>>(S, x[0], x[1], zx[0], zx[1]));
+        return DD_OK;
+    };
+    // 1. eta on the black sites
+    DD_KLAUNCH(h, noise_black_kernel<<<dim3(grid_for(g.V / 2, 128), n), 128, 0, h->stream>>>(
+                      g, c, eta, ex[0], ex[1], ps, purpose, seed, ctr, h->d_ctr_off, ob, outer_mask));
+    // 2. v' = B' E'^{-1} C' eta
+    inter(1, 1, ex, b);
+    int rc = solve(1, 1);
+    if (rc) return rc;
+    inter(0, 1, zx, p);
+    // 3. v = B E^{-1} C eta, a = A^{-1} v
+    inter(1, 0, ex, b);
+    rc = solve(1, 0);
+    if (rc) return rc;
+    inter(0, 0, zx, b);
+    rc = solve(0, 0);
+    if (rc) return rc;
+    // 4. s = v' - A' a on the black sites
+    for (int par = 0; par < 2; ++par) {
+        DD_CUDA(h, cudaMemsetAsync(b[par].p, 0, sizeof(double2) * 12 * Vh * n, h->stream));
+        auto A = args(0, 1, zx, b, par);
+        A.xin = x[par];
+        A.has_x = 1;
+        A.rhat = p[par];
+        A.resid = 1;
+        launch_hop<double, SpinorX, SpinorF64, SpinorF64, LinkX, 1>(A, n, h);
+    }
+    DD_LAUNCH_CHECK(h, "Schur pieces");
     return DD_OK;
 }
 
@@ -996,49 +955,20 @@ extern "C" int dd_det_ratio_estimate(dd_t h, const void* U_old, const void* U_ne
     if (rc) return rc;
     const Geo& g = h->g;
     const BlockCtx c = block_ctx(h);
-    const int R = h->prm.max_rhs;
-    const long long vs = 12LL * g.V;
-    double2* bank[6];
-    for (int k = 0; k < 6; ++k) bank[k] = h->dd_vec + (long long)k * R * vs;
     // field slot of the old / new operator of factor i: fs * i + {0, 1}
     const int fs = factors ? 1 : 0;
-    const long long canon_fs = (long long)(h->fields[1].canon - h->fields[0].canon) * 2;  // doubles
-    dim3 gv(grid_for(g.V, 128), n);
-    // 1. eta on black sites
-    const int4 no_outer = make_int4(0, 0, 0, 0);
-    DD_KLAUNCH(h, noise_black_kernel<<<gv, 128, 0, h->stream>>>(g, c, bank[0], vs, DD_PURPOSE_GLOBAL_NOISE, seed, ctr,
-                                                               h->d_ctr_off, no_outer, 3));
-    // 2. w = C eta, w' = C' eta (onto white sites)
-    DD_KLAUNCH(h, inter_hop_kernel<<<gv, 128, 0, h->stream>>>(g, c, bank[0], bank[1], vs, (const double*)h->fields[0].canon, canon_fs, 0, fs, 1, no_outer));
-    DD_KLAUNCH(h, inter_hop_kernel<<<gv, 128, 0, h->stream>>>(g, c, bank[0], bank[2], vs, (const double*)h->fields[0].canon, canon_fs, 1, fs, 1, no_outer));
-    DD_LAUNCH_CHECK(h, "schur stage 1-2");
-    // 3. z = E^{-1} w, z' = E'^{-1} w': all white-block solves of all factors
-    //    as one batched even-odd CG on the Dirichlet operator
-    rc = dirichlet_solve_bank(h, bank[1], bank[3], n, 0, fs, 1);
+    rc = schur_source(h, n, fs, DD_PURPOSE_GLOBAL_NOISE, seed, ctr, make_int4(0, 0, 0, 0), 3);
     if (rc) return rc;
-    rc = dirichlet_solve_bank(h, bank[2], bank[4], n, 1, fs, 1);
-    if (rc) return rc;
-    // 4. v = B z, v' = B' z' (onto black sites)
-    DD_KLAUNCH(h, inter_hop_kernel<<<gv, 128, 0, h->stream>>>(g, c, bank[3], bank[1], vs, (const double*)h->fields[0].canon, canon_fs, 0, fs, 0, no_outer));
-    DD_KLAUNCH(h, inter_hop_kernel<<<gv, 128, 0, h->stream>>>(g, c, bank[4], bank[2], vs, (const double*)h->fields[0].canon, canon_fs, 1, fs, 0, no_outer));
-    DD_LAUNCH_CHECK(h, "schur stage 4");
-    // 5. a = A^{-1} v (black-block solves)
-    rc = dirichlet_solve_bank(h, bank[1], bank[5], n, 0, fs, 0);
-    if (rc) return rc;
-    // 6. s = v' - A' a  -> bank 3
-    DD_KLAUNCH(h, schur_source_kernel<<<gv, 128, 0, h->stream>>>(g, c, bank[2], bank[5], bank[3], vs, (const double*)h->fields[0].canon, canon_fs, 1, fs));
-    // 7. global solve D' y = (s, 0)
+    // the global solve D' y = (s, 0)
     SolverVecs& v = h->vecs[0];
-    DD_KLAUNCH(h, dd_to_eo_kernel<<<gv, 128, 0, h->stream>>>(g, c, bank[3], vs, v.be, v.bo));
-    DD_LAUNCH_CHECK(h, "schur stage 6-7");
     int iters = 0;
     rc = solve_packed(h, n, 1, fs, h->prm.inner_prec, h->prm.tol_global, h->prm.maxit, &iters,
                       nullptr);
     if (rc && rc != DD_ERR_NOT_CONVERGED) return dd_fail(h, rc, "dd_det_ratio_estimate: global solve failed");
-    // 8. ln r_i
     const Reduce red = dd_reduce(h, FIN_STORE, nullptr, ln_out);
     dim3 gb(grid_for(g.V / 2, 128), n);
-    DD_KLAUNCH(h, estimate_kernel<<<gb, 128, 0, h->stream>>>(g, c, bank[0], vs, v.xe, v.xo, red));
+    DD_KLAUNCH(h, estimate_kernel<<<gb, 128, 0, h->stream>>>(
+                      g, c, h->dd_vec, (long long)h->prm.max_rhs * 12 * g.Vh, v.xe, v.xo, red));
     DD_LAUNCH_CHECK(h, "estimate_kernel");
     if (rc == DD_ERR_NOT_CONVERGED) return dd_fail(h, rc, "dd_det_ratio_estimate: global solve hit maxit");
     return DD_OK;
@@ -1048,10 +978,10 @@ extern "C" int dd_det_ratio_estimate(dd_t h, const void* U_old, const void* U_ne
 // ln_b[b] = -sum_i sum_{x in b, black sub-block} (2 Re<eta_i, d_i>_x + |d_i|_x^2)
 // for every block b of g1 with colour in colour_mask (0 for the others): one
 // thread block per block b, a fixed summation order (deterministic).  eta in
-// the block order of the sub-blocks (g2, c2), d in even-odd FP64 chunks.
-__global__ void __launch_bounds__(256) estimate_blocks_kernel(Geo g1, Geo g2, BlockCtx c2, const double2* eta_bank,
-                                                              long long vs, const double2* xe, const double2* xo,
-                                                              int n, int colour_mask, double* ln_b) {
+// even-odd FP64 chunks as d.
+__global__ void __launch_bounds__(256) estimate_blocks_kernel(Geo g1, Geo g2, const double2* eta,
+                                                              long long parity_stride, const double2* xe,
+                                                              const double2* xo, int n, int colour_mask, double* ln_b) {
     __shared__ double sh[34];
     const int b = blockIdx.x;
     int o[4];
@@ -1068,12 +998,10 @@ __global__ void __launch_bounds__(256) estimate_blocks_kernel(Geo g1, Geo g2, Bl
                         j / (g1.b[0] * g1.b[1] * g1.b[2])};
             int x[4] = {o[0] + l[0], o[1] + l[1], o[2] + l[2], o[3] + l[3]};
             if (block_colour_of(g2, x)) continue;  // white sub-block: eta = 0
-            const long long q = dd_position(g2, x);
-            SpinorF64 es{(double2*)eta_bank + (long long)i * vs + (q / c2.nb) * 12 * c2.nb, c2.nb};
             Spinor<double> e, d;
-            es.load(q % c2.nb, e);
             const int s = canon_index(g1, x);
             const int par = (x[0] + x[1] + x[2] + x[3]) & 1;
+            at_rhs(SpinorF64{(double2*)eta + par * parity_stride, g1.Vh}, i).load(s >> 1, e);
             SpinorF64 ds{(double2*)(par ? xo : xe) + (long long)i * 12 * g1.Vh, g1.Vh};
             ds.load(s >> 1, d);
             double t = 0.0;
@@ -1096,56 +1024,29 @@ extern "C" int dd_block_schur_filter(dd_t h, const void* U_old, void* U_new, int
     if (!U_old || !U_new || !ln_b || !accept || n < 1 || n > h->prm.max_rhs || colour_mask < 1 || colour_mask > 3)
         return dd_fail(h, DD_ERR_INVALID_ARG, "dd_block_schur_filter: bad arguments");
     const Geo g1 = h->g;
-    const int R = h->prm.max_rhs;
-    const long long vs = 12LL * g1.V;
-    double2* bank[6];
-    for (int k = 0; k < 6; ++k) bank[k] = h->dd_vec + (long long)k * R * vs;
     const int4 ob = make_int4(g1.b[0], g1.b[1], g1.b[2], g1.b[3]);
     SolverVecs& v = h->vecs[0];
     Geo g2;
-    BlockCtx c2;
     {
-        // Schur pieces of the sub-block decomposition inside every block:
-        // block order, Dirichlet solves and colour tables of the sub-blocks
+        // Schur pieces of the sub-block decomposition inside every block (hops
+        // across sub-block faces stay inside their block), eta on the black
+        // sub-blocks of the selected blocks
         LevelScope level(h, true);
         g2 = h->g;
-        c2 = block_ctx(h);
         rc = prepare_fields(h, (const double*)U_old, (const double*)U_new, n, true, true);
         if (rc) return rc;
-        const long long canon_fs = (long long)(h->fields[1].canon - h->fields[0].canon) * 2;
-        dim3 gv(grid_for(g2.V, 128), n);
-        // 1. eta on the black sub-blocks of the selected blocks
-        DD_KLAUNCH(h, noise_black_kernel<<<gv, 128, 0, h->stream>>>(g2, c2, bank[0], vs, DD_PURPOSE_BLOCK_SCHUR_NOISE, seed,
-                                                                   ctr, h->d_ctr_off, ob, colour_mask));
-        // 2. w = C eta, w' = C' eta (hops across sub-block faces inside a block)
-        DD_KLAUNCH(h, inter_hop_kernel<<<gv, 128, 0, h->stream>>>(g2, c2, bank[0], bank[1], vs, (const double*)h->fields[0].canon, canon_fs, 0, 1, 1, ob));
-        DD_KLAUNCH(h, inter_hop_kernel<<<gv, 128, 0, h->stream>>>(g2, c2, bank[0], bank[2], vs, (const double*)h->fields[0].canon, canon_fs, 1, 1, 1, ob));
-        DD_LAUNCH_CHECK(h, "block schur stage 1-2");
-        // 3. z = E^{-1} w, z' = E'^{-1} w' (white sub-blocks)
-        rc = dirichlet_solve_bank(h, bank[1], bank[3], n, 0, 1, 1);
+        rc = schur_source(h, n, 1, DD_PURPOSE_BLOCK_SCHUR_NOISE, seed, ctr, ob, colour_mask);
         if (rc) return rc;
-        rc = dirichlet_solve_bank(h, bank[2], bank[4], n, 1, 1, 1);
-        if (rc) return rc;
-        // 4. v = B z, v' = B' z'
-        DD_KLAUNCH(h, inter_hop_kernel<<<gv, 128, 0, h->stream>>>(g2, c2, bank[3], bank[1], vs, (const double*)h->fields[0].canon, canon_fs, 0, 1, 0, ob));
-        DD_KLAUNCH(h, inter_hop_kernel<<<gv, 128, 0, h->stream>>>(g2, c2, bank[4], bank[2], vs, (const double*)h->fields[0].canon, canon_fs, 1, 1, 0, ob));
-        DD_LAUNCH_CHECK(h, "block schur stage 4");
-        // 5. a = A^{-1} v (black sub-blocks)
-        rc = dirichlet_solve_bank(h, bank[1], bank[5], n, 0, 1, 0);
-        if (rc) return rc;
-        // 6. s = v' - A' a
-        DD_KLAUNCH(h, schur_source_kernel<<<gv, 128, 0, h->stream>>>(g2, c2, bank[2], bank[5], bank[3], vs, (const double*)h->fields[0].canon, canon_fs, 1, 1));
-        DD_KLAUNCH(h, dd_to_eo_kernel<<<gv, 128, 0, h->stream>>>(g2, c2, bank[3], vs, v.be, v.bo));
-        DD_LAUNCH_CHECK(h, "block schur stage 5-6");
     }
-    // 7. D1' y = (s, 0): the Dirichlet operator of the blocks plays the part
+    // D1' y = (s, 0): the Dirichlet operator of the blocks plays the part
     //    of D in the global step (even-odd formats do not depend on blocks)
     int iters = 0;
     rc = solve_packed(h, n, 1, 1, h->prm.inner_prec, h->prm.tol_global, h->prm.maxit, &iters, nullptr, 1);
     if (rc && rc != DD_ERR_NOT_CONVERGED) return dd_fail(h, rc, "dd_block_schur_filter: block solve failed");
     if (rc == DD_ERR_NOT_CONVERGED) raise_status_host(h, DD_ERR_NOT_CONVERGED);
-    // 8. per-block log-ratios, decisions, restore
-    DD_KLAUNCH(h, estimate_blocks_kernel<<<g1.nblocks, 256, 0, h->stream>>>(g1, g2, c2, bank[0], vs, v.xe, v.xo, n,
+    // per-block log-ratios, decisions, restore
+    DD_KLAUNCH(h, estimate_blocks_kernel<<<g1.nblocks, 256, 0, h->stream>>>(g1, g2, h->dd_vec,
+                                                                          (long long)h->prm.max_rhs * 12 * g1.Vh, v.xe, v.xo, n,
                                                                           colour_mask, ln_b));
     DD_KLAUNCH(h, block_accept_kernel<<<grid_for(g1.nblocks, 128), 128, 0, h->stream>>>(
                       g1, colour_mask, ln_b, accept, seed, ctr, h->d_ctr_off, DD_PURPOSE_BLOCK_SCHUR_ACCEPT));

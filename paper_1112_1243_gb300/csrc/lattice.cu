@@ -402,8 +402,10 @@ void plan(dd_handle* h, char* base) {
     v.q16 = c.take<uint4>((size_t)R * 3 * Vh);
     v.q16n = c.take<float>((size_t)R * Vh);
     }
-    // block-ordered FP64 vectors: 6 banks of R vectors (estimator)
-    h->dd_vec = c.take<double2>(est ? (size_t)6 * R * 12 * V : 0);
+    // even-odd vectors of the estimator, 3 banks of R vectors (both parities):
+    // eta in FP64, eta in limbs, v' in FP64
+    h->dd_vec = c.take<double2>(est ? (size_t)3 * R * 12 * V : 0);
+    h->d_xexp = c.take<int>(est ? (size_t)R * V : 0);
     h->d_cg = c.take<CGState>((size_t)3 * R + 2);
     // SAP-preconditioned GCR (global solves): full FP32 vectors (even, odd
     // halves of R systems each) and the block solver's vectors
