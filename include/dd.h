@@ -347,10 +347,10 @@ int dd_global_accept(dd_t h, void* U, const void* U_old, const double* ln_r, int
  * or of the domain Schur complement Dhat (which = 2, out[0] = ln|det Dhat|,
  * at most 512 sites).  out: device doubles.  Blocked LU (panels of 32
  * columns); panels of matrices above 384 rows are factorised by one
- * cooperative launch whose thread blocks meet at a bounded grid barrier.
+ * cooperative launch whose thread blocks wait, boundedly, for one another's
+ * pivot candidates.
  * Device status (dd_status): DD_ERR_NUMERIC for a zero pivot,
- * DD_ERR_TIMEOUT if a grid barrier gave up waiting (the results are then
- * invalid). */
+ * DD_ERR_TIMEOUT if such a wait gave up (the results are then invalid). */
 int dd_logdet_exact(dd_t h, const void* U, int which, double* out);
 
 /* Trailing update of the dense LU of dd_logdet_exact (matrices above 384
@@ -367,14 +367,14 @@ int dd_logdet_exact(dd_t h, const void* U, int which, double* out);
  * slices.  Errors: DD_ERR_INVALID_ARG (on not 0 or 1). */
 int dd_lu_tensor_cores(dd_t h, int on);
 
-/* Check of the bounded wait in the grid barrier of the LU panel launch (the
+/* Check of the bounded wait of the LU panel launch (the
  * paper has no counterpart: failure detection of the only kernel of the
  * library that waits on other thread blocks).  Runs a cooperative launch of
- * up to 8 thread blocks through three grid barriers; with missing > 0 the
- * last barrier waits for that many arrivals that never come, gives up after
+ * up to 8 thread blocks through three exchanges of messages; with missing > 0
+ * the last one also waits for that many that never come, gives up after
  * its poll limit (a few seconds), raises DD_ERR_TIMEOUT in the device status
  * word (dd_status) and returns.  *passed = 1 when every block passed all
- * barriers, else 0.  Synchronises the handle's stream; needs the exact-path
+ * exchanges, else 0.  Synchronises the handle's stream; needs the exact-path
  * workspace (DD_FEAT_EXACT).  Errors: DD_ERR_INVALID_ARG (passed NULL,
  * missing outside 0..64), DD_ERR_UNSUPPORTED, DD_ERR_CUDA. */
 int dd_barrier_check(dd_t h, int missing, int* passed);

@@ -337,7 +337,7 @@ def dd_lu_tensor_cores(h, on=True):
 
 
 def dd_barrier_check(h, missing=0):
-    """Grid barrier of the LU panel launch with `missing` arrivals that never
+    """Message exchange of the LU panel launch with `missing` messages that never
     come: True when every thread block passed (the bounded wait raises
     DD_ERR_TIMEOUT in the device status word otherwise)."""
     out = ctypes.c_int()

@@ -106,13 +106,14 @@ __global__ void zero_kernel(long long n, double2* p) {
 //   3. A22 -= L21 U12, a complex FP64 GEMM (zgemm_tile_kernel).
 // Panels of matrices up to LU_SINGLE_MAX rows live in the shared memory of
 // one thread block.  Larger panels are split into slices of LU_PR rows over
-// the thread blocks of one cooperative launch, which meet once per column at
-// a grid barrier: every block publishes its best pivot candidate (value,
-// row, and the row's panel entries) and the owner of row k publishes that
-// row; after the barrier every block picks the same winner and swaps inside
-// its own slice.  The published buffers alternate between two copies by
-// column parity, so a block never overwrites a copy that a slower block may
-// still read.
+// the thread blocks of one cooperative launch, which exchange tagged messages
+// once per column: every block publishes its best pivot candidate (value and
+// row, then the row's panel entries) and the owner of row k publishes that
+// row; every block reads all candidates, picks the same winner and swaps
+// inside its own slice.  The messages alternate between two copies by column
+// parity: a block that has read all candidates of column j knows that every
+// other block is done with those of column j - 1, so its messages of column
+// j + 1 overwrite nothing that is still read.
 constexpr int LU_NB = 32;
 constexpr int LU_PR = 32;
 constexpr int LU_SINGLE_MAX = 384;
@@ -120,6 +121,12 @@ constexpr int LU_THREADS = 256;
 constexpr int LU_LD = LU_NB + 1;  // padded row of a panel slice in shared memory
 constexpr long long LU_SPIN_LIMIT = 1ll << 22;
 
+// |a|^2 for the pivot search; NaN counts as the largest, so that every column
+// has a pivot row (a NaN pivot then raises DD_ERR_NUMERIC)
+DD_DEV double pivot_size(double2 a) {
+    const double v = a.x * a.x + a.y * a.y;
+    return v >= 0.0 ? v : __longlong_as_double(0x7ff0000000000000ll);
+}
 DD_DEV void argmax_merge(double& v, int& i, double ov, int oi) {
     if (ov > v || (ov == v && oi < i)) {
         v = ov;
@@ -127,15 +134,23 @@ DD_DEV void argmax_merge(double& v, int& i, double ov, int oi) {
     }
 }
 
+// A message of two doubles: each 32-bit half travels with the tag in one
+// 64-bit word, so a reader that finds the tag in all four words has the value,
+// and needs neither a barrier nor a fence.  Tags differ for every column of a
+// factorisation, 0 (the buffers' start) is none.
+struct LuMsg {
+    ulonglong2 re, im;
+};
 struct LuAux {
     int* ipiv;      // [batch][n]: row swapped with row k at step k
-    double* part;   // [2][chunk][ctas][2]: (|a|^2, row) of each block's candidate
-    double2* prow;  // [2][chunk][ctas][LU_NB]: that candidate's panel row
-    double2* rowk;  // [2][chunk][LU_NB]: panel row k before the swap
-    unsigned* bar;  // arrivals at the grid barrier (zeroed before each launch)
+    LuMsg* cand;    // [2][chunk][ctas]: (|a|^2, row) of each block's candidate
+    LuMsg* prow;    // [2][chunk][ctas][LU_NB]: that candidate's panel row
+    LuMsg* rowk;    // [2][chunk][LU_NB]: panel row k before the swap
+    unsigned tag0;  // column k0 + j has the tag tag0 + j
     int* perm;      // [batch][4 LU_NB + 1]: the panel's row swaps as one permutation
                     // (destination rows, source rows, count)
 };
+static_assert(LU_NB == 32, "a panel's pivots are one a lane");
 static_assert(LU_PR >= LU_NB, "the first thread block of a panel must own all its pivot rows");
 
 // (value, row) pair of the largest value, lowest row on ties, over the
@@ -160,62 +175,89 @@ DD_DEV void block_argmax(double best, int bi, double* sv, int* si) {
     __syncthreads();
 }
 
-// grid barrier of a cooperative launch; false (and DD_ERR_TIMEOUT in the
-// status word) when the other blocks did not arrive within LU_SPIN_LIMIT polls
-DD_DEV bool lu_grid_barrier(unsigned* bar, unsigned target, int* status, int* s_ok) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // the arrival releases the block's writes before the barrier (ordered
-        // after them by __syncthreads); the acquiring load of the count
-        // orders the block's later reads after the other blocks' writes
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-        int ok = 1;
-        for (long long spin = 0;; ++spin) {
-            unsigned v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if (v >= target) break;
-            if (spin >= LU_SPIN_LIMIT) {
-                ok = 0;
-                raise_status(status, DD_ERR_TIMEOUT);
-                break;
-            }
-            __nanosleep(16);
+DD_DEV ulonglong2 lu_tagged(double v, unsigned tag) {
+    const unsigned long long t = (unsigned long long)tag << 32;
+    return make_ulonglong2(t | (unsigned)__double2loint(v), t | (unsigned)__double2hiint(v));
+}
+DD_DEV void lu_send(LuMsg* p, double re, double im, unsigned tag) {
+    const ulonglong2 a = lu_tagged(re, tag), b = lu_tagged(im, tag);
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(&p->re), "l"(a.x), "l"(a.y) : "memory");
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(&p->im), "l"(b.x), "l"(b.y) : "memory");
+}
+DD_DEV LuMsg lu_peek(const LuMsg* p) {
+    LuMsg m;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(m.re.x), "=l"(m.re.y) : "l"(&p->re) : "memory");
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(m.im.x), "=l"(m.im.y) : "l"(&p->im) : "memory");
+    return m;
+}
+DD_DEV bool lu_has(const LuMsg& m, unsigned tag) {
+    return (unsigned)(m.re.x >> 32) == tag && (unsigned)(m.re.y >> 32) == tag && (unsigned)(m.im.x >> 32) == tag &&
+           (unsigned)(m.im.y >> 32) == tag;
+}
+DD_DEV double2 lu_value(const LuMsg& m) {
+    return make_double2(__hiloint2double((int)(unsigned)m.re.y, (int)(unsigned)m.re.x),
+                        __hiloint2double((int)(unsigned)m.im.y, (int)(unsigned)m.im.x));
+}
+// N messages a lane (of a full warp); false (and DD_ERR_TIMEOUT in the status
+// word) when one of them did not come within LU_SPIN_LIMIT polls
+template <int N>
+DD_DEV bool lu_receive(const LuMsg* const* from, unsigned tag, double2* v, int* status) {
+    for (long long spin = 0;; ++spin) {
+        LuMsg m[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) m[i] = lu_peek(from[i]);
+        bool all = true;
+#pragma unroll
+        for (int i = 0; i < N; ++i) all = all && lu_has(m[i], tag);
+        if (__all_sync(0xffffffffu, all)) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) v[i] = lu_value(m[i]);
+            return true;
         }
-        *s_ok = ok;
+        if (spin >= LU_SPIN_LIMIT) {
+            if ((threadIdx.x & 31) == 0) raise_status(status, DD_ERR_TIMEOUT);
+            return false;
+        }
     }
-    __syncthreads();
-    return *s_ok != 0;
 }
 
 // the panel's swaps as one permutation of the rows they touch (the first
 // thread block owns rows k0.. and wrote their pivots): position i of the
-// list receives the value that row src[i] held before the panel
+// list receives the value that row src[i] held before the panel.  One warp:
+// positions lane and 32 + lane of the list live in lane's registers, a row is
+// looked up by ballot (one thread with the list in local memory and 32
+// dependent loads of the pivots was a tail on every panel).
 DD_DEV void lu_panel_permutation(const LuAux& aux, int m, int n, int k0, int nbe) {
-    int rows[2 * LU_NB], src[2 * LU_NB];
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int piv = lane < nbe ? aux.ipiv[(long long)m * n + k0 + lane] : -1;
+    int ra = lane < nbe ? k0 + lane : -2, sa = ra, rb = -2, sb = -2;
     int nrow = nbe;
-    for (int t = 0; t < nbe; ++t) rows[t] = src[t] = k0 + t;
     for (int t = 0; t < nbe; ++t) {
-        const int p = aux.ipiv[(long long)m * n + k0 + t];
-        int q = -1;
-        for (int i = 0; i < nrow; ++i)
-            if (rows[i] == p) {
-                q = i;
-                break;
-            }
-        if (q < 0) {
-            q = nrow++;
-            rows[q] = src[q] = p;
+        const int p = __shfl_sync(full, piv, t);
+        const unsigned ina = __ballot_sync(full, ra == p), inb = __ballot_sync(full, rb == p);
+        int q = ina ? __ffs(ina) - 1 : inb ? 31 + __ffs(inb) : nrow;
+        if (q == nrow) {
+            if (q == lane) ra = sa = p;
+            if (q == lane + 32) rb = sb = p;
+            ++nrow;
         }
-        const int tmp = src[t];
-        src[t] = src[q];
-        src[q] = tmp;
+        const int st = __shfl_sync(full, sa, t);
+        const int qa = __shfl_sync(full, sa, q & 31), qb = __shfl_sync(full, sb, q & 31);
+        if (t == lane) sa = q < 32 ? qa : qb;
+        if (q == lane) sa = st;
+        if (q == lane + 32) sb = st;
     }
     int* pm = aux.perm + (long long)m * (4 * LU_NB + 1);
-    for (int i = 0; i < nrow; ++i) {
-        pm[i] = rows[i];
-        pm[2 * LU_NB + i] = src[i];
+    if (lane < nrow) {
+        pm[lane] = ra;
+        pm[2 * LU_NB + lane] = sa;
     }
-    pm[4 * LU_NB] = nrow;
+    if (lane + 32 < nrow) {
+        pm[lane + 32] = rb;
+        pm[2 * LU_NB + lane + 32] = sb;
+    }
+    if (lane == 0) pm[4 * LU_NB] = nrow;
 }
 
 // panel factorisation, step 1, of matrices up to LU_SINGLE_MAX rows: one
@@ -241,8 +283,7 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_kernel(double2* M, long l
         double best = -1.0;
         int bi = INT_MAX;
         for (int r = max(0, k - r0) + tid; r < nr; r += blockDim.x) {
-            const double2 v = pan[r * LU_LD + j];
-            argmax_merge(best, bi, v.x * v.x + v.y * v.y, r0 + r);
+            argmax_merge(best, bi, pivot_size(pan[r * LU_LD + j]), r0 + r);
         }
         block_argmax(best, bi, sv, si);
         const bool own_k = k >= r0 && k < r0 + nr;
@@ -283,7 +324,7 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_kernel(double2* M, long l
         const int r = e % nr, j = e / nr;
         A[(r0 + r) + (long long)(k0 + j) * n] = pan[r * LU_LD + j];
     }
-    if (c == 0 && tid == 0) lu_panel_permutation(aux, m, n, k0, nbe);
+    if (c == 0 && tid < 32) lu_panel_permutation(aux, m, n, k0, nbe);
 }
 
 // Panel factorisation of matrices above LU_SINGLE_MAX rows: thread block b of
@@ -293,7 +334,14 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_kernel(double2* M, long l
 // multipliers go to Lm, not into the column being read, so the update needs
 // no extra barrier; a row that moves carries its multipliers (Lm, columns
 // left of j) and its remaining entries (pan, columns from j on).
+//
+// Bound by the latency of a column's chain, not by its work: update of one
+// column, candidate to L2, all candidates from L2, winner's row from L2.  Warp
+// 0 updates column j + 1 first and publishes its candidate while the others
+// still update.  With a grid barrier a
+// column instead of messages ln|det D| at 3072^2 took 40.8 ms, now 37.4.
 static_assert(LU_PR == 32, "one panel row per lane");
+constexpr int LU_POLL = 4;  // candidates a lane reads at once
 __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, long long mstride, int n, int k0,
                                                                     int nbe, LuAux aux, double* logdet, int* status) {
     __shared__ double2 pan[LU_PR][LU_LD];
@@ -301,7 +349,7 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
     __shared__ double2 urow[LU_NB];
     __shared__ double2 s_inv;     // 1 / pivot of the current column
     __shared__ double s_pm[LU_NB];  // |pivot|^2 per column (their logs are summed at the end)
-    __shared__ int s_p, s_ok;
+    __shared__ int s_p;             // pivot row; -1: a message did not come
     const int m = blockIdx.y, c = blockIdx.x, ctas = gridDim.x, tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     double2* A = M + (long long)m * mstride;
@@ -312,78 +360,98 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
         pan[r][j] = A[(r0 + r) + (long long)(k0 + j) * n];
     }
     __syncthreads();
+    int bi = INT_MAX;  // warp 0: the block's candidate row of the current column
+    auto candidate = [&](int j) {
+        double best = -1.0;
+        bi = INT_MAX;
+        if (lane < nr && r0 + lane >= k0 + j) {
+            best = pivot_size(pan[lane][j]);
+            bi = r0 + lane;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            argmax_merge(best, bi, __shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, bi, o));
+        if (lane == 0)
+            lu_send(aux.cand + ((long long)(j & 1) * gridDim.y + m) * ctas + c, best, (double)bi, aux.tag0 + j);
+    };
+    if (warp == 0) candidate(0);
     for (int j = 0; j < nbe; ++j) {
         const int k = k0 + j;
         const bool own_k = k >= r0 && k < r0 + nr;
         const long long mc = (long long)(j & 1) * gridDim.y + m;
+        const unsigned tag = aux.tag0 + j;
         if (warp == 0) {
-            double best = -1.0;
-            int bi = INT_MAX;
-            if (lane < nr && r0 + lane >= k) {
-                const double2 v = pan[lane][j];
-                best = v.x * v.x + v.y * v.y;
-                bi = r0 + lane;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-                argmax_merge(best, bi, __shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, bi, o));
-            if (lane == 0) {
-                aux.part[(mc * ctas + c) * 2] = best;
-                aux.part[(mc * ctas + c) * 2 + 1] = (double)bi;
-            }
             if (lane < nbe) {
-                if (best >= 0.0) {
-                    const int rb = bi - r0;
-                    aux.prow[(mc * ctas + c) * LU_NB + lane] = lane < j ? Lm[rb][lane] : pan[rb][lane];
+                if (bi != INT_MAX) {
+                    const double2 u = lane < j ? Lm[bi - r0][lane] : pan[bi - r0][lane];
+                    lu_send(aux.prow + (mc * ctas + c) * LU_NB + lane, u.x, u.y, tag);
                 }
-                if (own_k) aux.rowk[mc * LU_NB + lane] = lane < j ? Lm[k - r0][lane] : pan[k - r0][lane];
+                if (own_k) {
+                    const double2 u = lane < j ? Lm[k - r0][lane] : pan[k - r0][lane];
+                    lu_send(aux.rowk + mc * LU_NB + lane, u.x, u.y, tag);
+                }
             }
-        }
-        if (!lu_grid_barrier(aux.bar, (unsigned)(j + 1) * ctas * gridDim.y, status, &s_ok)) return;
-        if (warp == 0) {
             double bv = -1.0;
             int bidx = INT_MAX;
-            for (int q = lane; q < ctas; q += 32)
-                argmax_merge(bv, bidx, __ldcg(aux.part + (mc * ctas + q) * 2),
-                             (int)__ldcg(aux.part + (mc * ctas + q) * 2 + 1));
+            bool ok = true;
+            for (int q0 = lane; ok && q0 - lane < ctas; q0 += 32 * LU_POLL) {
+                const LuMsg* from[LU_POLL];
+                double2 v[LU_POLL];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-                argmax_merge(bv, bidx, __shfl_xor_sync(0xffffffffu, bv, o), __shfl_xor_sync(0xffffffffu, bidx, o));
-            const int bc = (bidx - k0) / LU_PR;
-            if (lane < nbe) {
-                const double2 u = __ldcg(aux.prow + (mc * ctas + bc) * LU_NB + lane);
-                const double2 old = __ldcg(aux.rowk + mc * LU_NB + lane);
-                urow[lane] = u;
-                if (lane == j) {  // the pivot: its reciprocal once for the block
-                    const double pm = u.x * u.x + u.y * u.y;
-                    s_pm[j] = pm;
-                    s_inv = pm > 0.0 ? make_double2(u.x / pm, -u.y / pm) : make_double2(0.0, 0.0);
-                }
-                if (own_k) (lane < j ? Lm[k - r0][lane] : pan[k - r0][lane]) = u;
-                if (bidx != k && bidx >= r0 && bidx < r0 + nr) (lane < j ? Lm[bidx - r0][lane] : pan[bidx - r0][lane]) = old;
+                for (int i = 0; i < LU_POLL; ++i) from[i] = aux.cand + mc * ctas + min(q0 + 32 * i, ctas - 1);
+                ok = lu_receive<LU_POLL>(from, tag, v, status);
+#pragma unroll
+                for (int i = 0; i < LU_POLL; ++i)
+                    if (ok) argmax_merge(bv, bidx, v[i].x, (int)v[i].y);
             }
-            if (lane == 0) s_p = bidx;
+            if (ok) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+                    argmax_merge(bv, bidx, __shfl_xor_sync(0xffffffffu, bv, o), __shfl_xor_sync(0xffffffffu, bidx, o));
+                const int bc = (bidx - k0) / LU_PR, at = min(lane, nbe - 1);
+                const LuMsg* from[2] = {aux.prow + (mc * ctas + bc) * LU_NB + at, aux.rowk + mc * LU_NB + at};
+                double2 v[2];
+                ok = lu_receive<2>(from, tag, v, status);
+                if (ok && lane < nbe) {
+                    const double2 u = v[0], old = v[1];
+                    urow[lane] = u;
+                    if (lane == j) {  // the pivot: its reciprocal once for the block
+                        const double pm = u.x * u.x + u.y * u.y;
+                        s_pm[j] = pm;
+                        s_inv = pm > 0.0 ? make_double2(u.x / pm, -u.y / pm) : make_double2(0.0, 0.0);
+                    }
+                    if (own_k) (lane < j ? Lm[k - r0][lane] : pan[k - r0][lane]) = u;
+                    if (bidx != k && bidx >= r0 && bidx < r0 + nr) (lane < j ? Lm[bidx - r0][lane] : pan[bidx - r0][lane]) = old;
+                }
+            }
+            if (lane == 0) s_p = ok ? bidx : -1;
         }
         __syncthreads();
+        if (s_p < 0) return;
         const double pm = s_pm[j];
         if (tid == 0 && own_k) {
             aux.ipiv[(long long)m * n + k] = s_p;
             if (!(pm > 0.0)) raise_status(status, DD_ERR_NUMERIC);
         }
         const int r = lane;
-        if (r < nr && r0 + r > k) {
+        const bool below = r < nr && r0 + r > k;
+        cpx<double> l = mk<double>(0.0, 0.0);
+        if (below) {
             const double2 a = pan[r][j];
-            if (pm > 0.0) {
-                const cpx<double> l = cmul(mk<double>(a.x, a.y), mk<double>(s_inv.x, s_inv.y));
-                if (warp == 0) Lm[r][j] = make_double2(l.x, l.y);
-                for (int jj = j + 1 + warp; jj < nbe; jj += nwarps) {
-                    const double2 u = urow[jj];
-                    double2& t = pan[r][jj];
-                    t.x -= l.x * u.x - l.y * u.y;
-                    t.y -= l.x * u.y + l.y * u.x;
-                }
-            } else if (warp == 0) {
-                Lm[r][j] = a;  // zero pivot: column left as it is (DD_ERR_NUMERIC raised)
+            l = pm > 0.0 ? cmul(mk<double>(a.x, a.y), mk<double>(s_inv.x, s_inv.y)) : mk<double>(a.x, a.y);
+            // zero pivot: column left as it is (DD_ERR_NUMERIC raised)
+            if (warp == 0) Lm[r][j] = make_double2(l.x, l.y);
+        }
+        for (int jj = j + 1 + warp; jj < nbe; jj += nwarps) {
+            if (below && pm > 0.0) {
+                const double2 u = urow[jj];
+                double2& t = pan[r][jj];
+                t.x -= l.x * u.x - l.y * u.y;
+                t.y -= l.x * u.y + l.y * u.x;
+            }
+            if (jj == j + 1) {  // warp 0
+                __syncwarp();
+                candidate(j + 1);
             }
         }
         __syncthreads();
@@ -399,7 +467,7 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
         for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
         if (lane == 0) logdet[m] += l;
     }
-    if (c == 0 && tid == 0) lu_panel_permutation(aux, m, n, k0, nbe);
+    if (c == 0 && tid < 32) lu_panel_permutation(aux, m, n, k0, nbe);
 }
 
 // step 2: one warp per column right of the panel: the panel's row
@@ -774,21 +842,21 @@ static int lu_batched(dd_handle* h, double2* M, long long mstride, int batch, in
         chunk = (int)std::min<long long>(batch, resident / ctas0);
     }
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    size_t o = 0;
+    size_t o = 0, msg_off = 0, msg_end = 0;
     LuAux aux{};
     aux.ipiv = (int*)(scr + o);
     o += up((size_t)batch * n * sizeof(int));
     aux.perm = (int*)(scr + o);
     o += up((size_t)batch * (4 * LU_NB + 1) * sizeof(int));
     if (!single) {
-        aux.part = (double*)(scr + o);
-        o += up((size_t)2 * chunk * ctas0 * 2 * sizeof(double));
-        aux.prow = (double2*)(scr + o);
-        o += up((size_t)2 * chunk * ctas0 * LU_NB * sizeof(double2));
-        aux.rowk = (double2*)(scr + o);
-        o += up((size_t)2 * chunk * LU_NB * sizeof(double2));
-        aux.bar = (unsigned*)(scr + o);
-        o += 256;
+        msg_off = o;
+        aux.cand = (LuMsg*)(scr + o);
+        o += up((size_t)2 * chunk * ctas0 * sizeof(LuMsg));
+        aux.prow = (LuMsg*)(scr + o);
+        o += up((size_t)2 * chunk * ctas0 * LU_NB * sizeof(LuMsg));
+        aux.rowk = (LuMsg*)(scr + o);
+        o += up((size_t)2 * chunk * LU_NB * sizeof(LuMsg));
+        msg_end = o;
     }
     if (o > cap) return dd_fail(h, DD_ERR_UNSUPPORTED, "dense LU: no room for the pivot scratch");
     // slices of the tensor-core trailing update (matrices above LU_SINGLE_MAX rows)
@@ -816,6 +884,10 @@ static int lu_batched(dd_handle* h, double2* M, long long mstride, int batch, in
         }
     }
     DD_KLAUNCH(h, zero_doubles_kernel<<<grid_for(batch, 64), 64, 0, h->stream>>>(batch, logdet));
+    if (!single) {
+        cudaError_t e = cudaMemsetAsync(scr + msg_off, 0, msg_end - msg_off, h->stream);  // no tags yet
+        if (e != cudaSuccess) return dd_cuda_check(h, e, "lu message reset");
+    }
     for (int k0 = 0; k0 < n; k0 += LU_NB) {
         const int nbe = std::min(LU_NB, n - k0);
         if (single) {
@@ -827,19 +899,18 @@ static int lu_batched(dd_handle* h, double2* M, long long mstride, int batch, in
             const int ctas = grid_for(n - k0, LU_PR);
             for (int m0 = 0; m0 < batch; m0 += chunk) {
                 const int mb = std::min(chunk, batch - m0);
-                cudaError_t e = cudaMemsetAsync(aux.bar, 0, sizeof(unsigned), h->stream);
-                if (e != cudaSuccess) return dd_cuda_check(h, e, "lu barrier reset");
                 double2* Mc = M + (long long)m0 * mstride;
                 double* ldc = logdet + m0;
                 LuAux ac = aux;
                 ac.ipiv = aux.ipiv + (long long)m0 * n;
                 ac.perm = aux.perm + (long long)m0 * (4 * LU_NB + 1);
+                ac.tag0 = (unsigned)(m0 / chunk) * (unsigned)n + (unsigned)k0 + 1u;
                 int nn = n, kk0 = k0, nb_ = nbe;
                 long long ms = mstride;
                 int* st = h->d_status;
                 void* args[] = {&Mc, &ms, &nn, &kk0, &nb_, &ac, &ldc, &st};
-                e = cudaLaunchCooperativeKernel((const void*)lu_panel_multi_kernel, dim3(ctas, mb), dim3(LU_THREADS), args,
-                                                0, h->stream);
+                cudaError_t e = cudaLaunchCooperativeKernel((const void*)lu_panel_multi_kernel, dim3(ctas, mb), dim3(LU_THREADS),
+                                                            args, 0, h->stream);
                 ++h->launches;
                 if (e != cudaSuccess) return dd_cuda_check(h, e, "lu_panel_kernel (cooperative launch)");
             }
@@ -1014,13 +1085,19 @@ int block_filter_exact(dd_handle* h, const double* U_old, const double* U_new, i
     return DD_OK;
 }
 
-// check of the bounded wait of the grid barrier: `rounds` barriers of all
-// thread blocks; the last one waits for `missing` arrivals that never come
-__global__ void barrier_check_kernel(unsigned* bar, int rounds, int missing, int* status, int* passed) {
-    __shared__ int s_ok;
-    for (int r = 1; r <= rounds; ++r) {
-        const unsigned target = (unsigned)r * gridDim.x + (r == rounds ? (unsigned)missing : 0u);
-        if (!lu_grid_barrier(bar, target, status, &s_ok)) return;
+// check of the bounded wait of the panel launch: `rounds` exchanges of all
+// thread blocks; the last one also waits for `missing` messages that never come
+__global__ void barrier_check_kernel(LuMsg* msg, int slots, int rounds, int missing, int* status, int* passed) {
+    for (int r = 0; r < rounds; ++r) {
+        LuMsg* at = msg + (r & 1) * slots;
+        const unsigned tag = (unsigned)r + 1u;
+        if (threadIdx.x == 0) lu_send(at + blockIdx.x, (double)r, 0.0, tag);
+        const int count = gridDim.x + (r == rounds - 1 ? missing : 0);
+        for (int q = threadIdx.x; q - (int)threadIdx.x < count; q += 32) {
+            const LuMsg* from[1] = {at + min(q, count - 1)};
+            double2 v[1];
+            if (!lu_receive<1>(from, tag, v, status)) return;
+        }
     }
     if (threadIdx.x == 0) atomicAdd(passed, 1);
 }
@@ -1033,15 +1110,16 @@ extern "C" int dd_barrier_check(dd_t h, int missing, int* passed) {
     if (!passed || missing < 0 || missing > 64) return dd_fail(h, DD_ERR_INVALID_ARG, "dd_barrier_check: bad arguments");
     size_t cap = 0;
     char* scr = lu_scratch(h, &cap);
-    if (cap < 256) return dd_fail(h, DD_ERR_UNSUPPORTED, "dd_barrier_check: no scratch");
-    unsigned* bar = (unsigned*)scr;
-    int* dpassed = (int*)(scr + 128);
-    DD_CUDA(h, cudaMemsetAsync(scr, 0, 256, h->stream));
     const int ctas = std::max(1, std::min(8, h->num_sms));
-    int rounds = 3;
-    void* args[] = {&bar, &rounds, &missing, &h->d_status, &dpassed};
-    cudaError_t e = cudaLaunchCooperativeKernel((const void*)barrier_check_kernel, dim3(ctas), dim3(LU_THREADS), args,
-                                                0, h->stream);
+    int slots = ctas + missing, rounds = 3;
+    const size_t bytes = 256 + (size_t)2 * slots * sizeof(LuMsg);
+    if (cap < bytes) return dd_fail(h, DD_ERR_UNSUPPORTED, "dd_barrier_check: no scratch");
+    int* dpassed = (int*)scr;
+    LuMsg* msg = (LuMsg*)(scr + 256);
+    DD_CUDA(h, cudaMemsetAsync(scr, 0, bytes, h->stream));
+    void* args[] = {&msg, &slots, &rounds, &missing, &h->d_status, &dpassed};
+    cudaError_t e = cudaLaunchCooperativeKernel((const void*)barrier_check_kernel, dim3(ctas), dim3(32), args, 0,
+                                                h->stream);
     ++h->launches;
     if (e != cudaSuccess) return dd_cuda_check(h, e, "barrier_check_kernel (cooperative launch)");
     int np = 0;
