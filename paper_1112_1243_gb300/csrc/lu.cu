@@ -121,13 +121,15 @@ constexpr int LU_THREADS = 256;
 constexpr int LU_LD = LU_NB + 1;  // padded row of a panel slice in shared memory
 constexpr long long LU_SPIN_LIMIT = 1ll << 22;
 
-// |a|^2 for the pivot search; NaN counts as the largest, so that every column
-// has a pivot row (a NaN pivot then raises DD_ERR_NUMERIC)
-DD_DEV double pivot_size(double2 a) {
-    const double v = a.x * a.x + a.y * a.y;
-    return v >= 0.0 ? v : __longlong_as_double(0x7ff0000000000000ll);
+// |a|^2 for the pivot search as an integer of the same order (no candidate:
+// -1): comparisons stay off the FP64 pipe, 2 lanes wide, which a column's chain
+// waits for.  NaN counts as the largest, so that every column has a pivot row
+// (a NaN pivot then raises DD_ERR_NUMERIC).
+DD_DEV long long pivot_size(double2 a) {
+    const long long v = __double_as_longlong(a.x * a.x + a.y * a.y);
+    return v < 0 || v > 0x7ff0000000000000ll ? 0x7ff0000000000000ll : v;
 }
-DD_DEV void argmax_merge(double& v, int& i, double ov, int oi) {
+DD_DEV void argmax_merge(long long& v, int& i, long long ov, int oi) {
     if (ov > v || (ov == v && oi < i)) {
         v = ov;
         i = oi;
@@ -155,10 +157,10 @@ static_assert(LU_PR >= LU_NB, "the first thread block of a panel must own all it
 
 // (value, row) pair of the largest value, lowest row on ties, over the
 // thread block; the result is in sv[0], si[0] for every thread
-DD_DEV void block_argmax(double best, int bi, double* sv, int* si) {
+DD_DEV void block_argmax(long long best, int bi, long long* sv, int* si) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+        const long long ov = __shfl_xor_sync(0xffffffffu, best, o);
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         argmax_merge(best, bi, ov, oi);
     }
@@ -266,7 +268,7 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_kernel(double2* M, long l
                                                               int rows_per, LuAux aux, double* logdet, int* status) {
     extern __shared__ double2 pan[];  // [rows_per][LU_LD]
     __shared__ double2 urow[LU_NB];
-    __shared__ double sv[LU_THREADS / 32];
+    __shared__ long long sv[LU_THREADS / 32];
     __shared__ int si[LU_THREADS / 32];
     __shared__ int s_p;
     const int m = blockIdx.y, c = blockIdx.x, tid = threadIdx.x;
@@ -280,7 +282,7 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_kernel(double2* M, long l
     __syncthreads();
     for (int j = 0; j < nbe; ++j) {
         const int k = k0 + j;
-        double best = -1.0;
+        long long best = -1;
         int bi = INT_MAX;
         for (int r = max(0, k - r0) + tid; r < nr; r += blockDim.x) {
             argmax_merge(best, bi, pivot_size(pan[r * LU_LD + j]), r0 + r);
@@ -338,8 +340,9 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_kernel(double2* M, long l
 // Bound by the latency of a column's chain, not by its work: update of one
 // column, candidate to L2, all candidates from L2, winner's row from L2.  Warp
 // 0 updates column j + 1 first and publishes its candidate while the others
-// still update.  With a grid barrier a
-// column instead of messages ln|det D| at 3072^2 took 40.8 ms, now 37.4.
+// still update; it alone forms the multipliers (every warp did, on the FP64
+// pipe).  ln|det D| at 3072^2: 40.8 ms with a grid barrier a column, 37.4 with
+// messages, 33.2 with the chain's comparisons and multipliers off the pipe.
 static_assert(LU_PR == 32, "one panel row per lane");
 constexpr int LU_POLL = 4;  // candidates a lane reads at once
 __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, long long mstride, int n, int k0,
@@ -347,7 +350,6 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
     __shared__ double2 pan[LU_PR][LU_LD];
     __shared__ double2 Lm[LU_PR][LU_LD];
     __shared__ double2 urow[LU_NB];
-    __shared__ double2 s_inv;     // 1 / pivot of the current column
     __shared__ double s_pm[LU_NB];  // |pivot|^2 per column (their logs are summed at the end)
     __shared__ int s_p;             // pivot row; -1: a message did not come
     const int m = blockIdx.y, c = blockIdx.x, ctas = gridDim.x, tid = threadIdx.x;
@@ -362,7 +364,7 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
     __syncthreads();
     int bi = INT_MAX;  // warp 0: the block's candidate row of the current column
     auto candidate = [&](int j) {
-        double best = -1.0;
+        long long best = -1;
         bi = INT_MAX;
         if (lane < nr && r0 + lane >= k0 + j) {
             best = pivot_size(pan[lane][j]);
@@ -372,7 +374,8 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
         for (int o = 16; o > 0; o >>= 1)
             argmax_merge(best, bi, __shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, bi, o));
         if (lane == 0)
-            lu_send(aux.cand + ((long long)(j & 1) * gridDim.y + m) * ctas + c, best, (double)bi, aux.tag0 + j);
+            lu_send(aux.cand + ((long long)(j & 1) * gridDim.y + m) * ctas + c, __longlong_as_double(best), __hiloint2double(0, bi),
+                    aux.tag0 + j);
     };
     if (warp == 0) candidate(0);
     for (int j = 0; j < nbe; ++j) {
@@ -391,7 +394,7 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
                     lu_send(aux.rowk + mc * LU_NB + lane, u.x, u.y, tag);
                 }
             }
-            double bv = -1.0;
+            long long bv = -1;
             int bidx = INT_MAX;
             bool ok = true;
             for (int q0 = lane; ok && q0 - lane < ctas; q0 += 32 * LU_POLL) {
@@ -402,7 +405,7 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
                 ok = lu_receive<LU_POLL>(from, tag, v, status);
 #pragma unroll
                 for (int i = 0; i < LU_POLL; ++i)
-                    if (ok) argmax_merge(bv, bidx, v[i].x, (int)v[i].y);
+                    if (ok) argmax_merge(bv, bidx, __double_as_longlong(v[i].x), __double2loint(v[i].y));
             }
             if (ok) {
 #pragma unroll
@@ -412,16 +415,29 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
                 const LuMsg* from[2] = {aux.prow + (mc * ctas + bc) * LU_NB + at, aux.rowk + mc * LU_NB + at};
                 double2 v[2];
                 ok = lu_receive<2>(from, tag, v, status);
-                if (ok && lane < nbe) {
+                if (ok) {
                     const double2 u = v[0], old = v[1];
-                    urow[lane] = u;
-                    if (lane == j) {  // the pivot: its reciprocal once for the block
-                        const double pm = u.x * u.x + u.y * u.y;
-                        s_pm[j] = pm;
-                        s_inv = pm > 0.0 ? make_double2(u.x / pm, -u.y / pm) : make_double2(0.0, 0.0);
+                    // the pivot's reciprocal, real part in even lanes, imaginary
+                    // part in odd ones: one division deep
+                    const double px = __shfl_sync(0xffffffffu, u.x, j), py = __shfl_sync(0xffffffffu, u.y, j);
+                    const double pm = px * px + py * py;
+                    const double part = (lane & 1 ? -py : px) / pm;
+                    const cpx<double> inv =
+                        mk<double>(__shfl_sync(0xffffffffu, part, 0), __shfl_sync(0xffffffffu, part, 1));
+                    if (lane == 0) s_pm[j] = pm;
+                    if (lane < nbe) {
+                        urow[lane] = u;
+                        if (own_k) (lane < j ? Lm[k - r0][lane] : pan[k - r0][lane]) = u;
+                        if (bidx != k && bidx >= r0 && bidx < r0 + nr) (lane < j ? Lm[bidx - r0][lane] : pan[bidx - r0][lane]) = old;
                     }
-                    if (own_k) (lane < j ? Lm[k - r0][lane] : pan[k - r0][lane]) = u;
-                    if (bidx != k && bidx >= r0 && bidx < r0 + nr) (lane < j ? Lm[bidx - r0][lane] : pan[bidx - r0][lane]) = old;
+                    __syncwarp();
+                    // the column's multipliers, once for the block; zero pivot:
+                    // column left as it is (DD_ERR_NUMERIC raised)
+                    if (lane < nr && r0 + lane > k) {
+                        const double2 a = pan[lane][j];
+                        const cpx<double> l = pm > 0.0 ? cmul(mk<double>(a.x, a.y), inv) : mk<double>(a.x, a.y);
+                        Lm[lane][j] = make_double2(l.x, l.y);
+                    }
                 }
             }
             if (lane == 0) s_p = ok ? bidx : -1;
@@ -435,13 +451,7 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
         }
         const int r = lane;
         const bool below = r < nr && r0 + r > k;
-        cpx<double> l = mk<double>(0.0, 0.0);
-        if (below) {
-            const double2 a = pan[r][j];
-            l = pm > 0.0 ? cmul(mk<double>(a.x, a.y), mk<double>(s_inv.x, s_inv.y)) : mk<double>(a.x, a.y);
-            // zero pivot: column left as it is (DD_ERR_NUMERIC raised)
-            if (warp == 0) Lm[r][j] = make_double2(l.x, l.y);
-        }
+        const double2 l = below ? Lm[r][j] : make_double2(0.0, 0.0);
         for (int jj = j + 1 + warp; jj < nbe; jj += nwarps) {
             if (below && pm > 0.0) {
                 const double2 u = urow[jj];
