@@ -362,19 +362,26 @@ DD_DEV cpx<R> cscal(double re, double im) {
 
 // x = 0, r = r0 (with re: re / sqrt(rr), the FP64 residual at unit norm, so
 // that FP32 squares neither underflow nor overflow), rhat = p = r0, and the
-// sums of FIN_BI_RHO
+// sums of FIN_BI_RHO.  A system that the outer solver still works on gets x = 0
+// also where there is nothing to solve (right-hand side zero: state inactive):
+// the caller uses x all the same.
 template <class R, class SM, class SH>
 __global__ void __launch_bounds__(128) bicg_start_kernel(SiteSet S, SM x, SM r, SH rhat, SH p, SpinorF64 re,
-                                                         const double* rr, const CGState* st, Reduce red) {
+                                                         const double* rr, const CGState* st, const CGState* outer,
+                                                         Reduce red) {
     const int rhs = blockIdx.y;
-    if (!st[rhs].active) return;
+    if (outer && !outer[rhs].active) return;
     const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (ti < S.n) {
+        Spinor<R> z;
+        zero(z);
+        at_rhs(x, rhs).store(S.at(ti), z);
+    }
+    if (!st[rhs].active) return;
     double v[3] = {0.0, 0.0, 0.0};
     if (ti < S.n) {
         const long long i = S.at(ti);
-        Spinor<R> z, a, b;
-        zero(z);
-        at_rhs(x, rhs).store(i, z);
+        Spinor<R> a, b;
         if (rr) {
             const double inv = rr[rhs] > 0.0 ? 1.0 / sqrt(rr[rhs]) : 0.0;
             Spinor<double> d;
@@ -516,7 +523,8 @@ struct BiCGStab {
         if (maxit < 1) maxit = 1;
         DD_KLAUNCH(h, cg_arm_kernel<<<1, 64, 0, h->stream>>>(nrhs, st, outer, re ? nullptr : rr0, tol, abs_fac, maxit));
         DD_KLAUNCH(h, bicg_start_kernel<R, SM, SH><<<grid, 128, 0, h->stream>>>(
-                          S, x, r, rhat, p, re ? *re : SpinorF64{nullptr, 0}, re ? rre : nullptr, st, red(FIN_BI_RHO)));
+                          S, x, r, rhat, p, re ? *re : SpinorF64{nullptr, 0}, re ? rre : nullptr, st, outer,
+                          red(FIN_BI_RHO)));
         std::vector<CGState> hs(nrhs);
         int done = 0;
         bool polled = false;
