@@ -602,6 +602,9 @@ __global__ void __launch_bounds__(256, 2) block_eo_kernel(BlockArgs A) {
     auto cluster = cooperative_groups::this_cluster();
     const int rank = (int)cluster.block_rank(), csize = (int)cluster.num_blocks();
     bool coop = A.nbig > 0;  // the items of the large blocks come first
+    // every thread block of the cluster runs before one writes into another's
+    // shared memory (the first item below)
+    if (coop) cluster.sync();
     for (;;) {
         if (coop) {
             if (rank == 0 && threadIdx.x == 0) {
