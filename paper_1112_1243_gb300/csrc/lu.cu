@@ -839,8 +839,9 @@ static int lu_batched(dd_handle* h, double2* M, long long mstride, int batch, in
     const int ctas0 = single ? 1 : grid_for(n, LU_PR);
     int chunk = batch;
     if (single) {
-        const size_t smem = (size_t)n * LU_LD * sizeof(double2);
-        cudaError_t e = cudaFuncSetAttribute(lu_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // the largest size for every n: the attribute belongs to the process
+        constexpr int smem_max = LU_SINGLE_MAX * LU_LD * (int)sizeof(double2);
+        cudaError_t e = cudaFuncSetAttribute(lu_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
         if (e != cudaSuccess) return dd_cuda_check(h, e, "lu_panel_kernel shared memory");
     } else {
         // one cooperative launch holds every thread block of its matrices
