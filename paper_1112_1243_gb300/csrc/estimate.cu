@@ -254,6 +254,9 @@ static int run_blocks(dd_handle* h, const BlockArgs& A, int slots, cudaStream_t 
         cfg.gridDim = dim3(grid);
         cfg.blockDim = dim3(tpb);
         cfg.dynamicSmemBytes = (size_t)(tpb / 128) * sizeof(EoPart);
+        // the attribute belongs to the process, not to this launch: always the
+        // largest block's size, so that threads with other shapes do not lower it
+        const int smem_max = 2 * (int)sizeof(EoPart);
         cfg.stream = s;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -262,7 +265,7 @@ static int run_blocks(dd_handle* h, const BlockArgs& A, int slots, cudaStream_t 
         cfg.attrs = at;
         cfg.numAttrs = 1;
         auto* kern = A.lats ? block_eo_kernel<true> : block_eo_kernel<false>;
-        DD_CUDA(h, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
+        DD_CUDA(h, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
         DD_CUDA(h, cudaLaunchKernelEx(&cfg, kern, B));
         ++h->launches;
     }

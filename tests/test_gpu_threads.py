@@ -49,6 +49,27 @@ def check(make, shapes, rounds):
         assert all(np.array_equal(r, w) for r in g)
 
 
+def test_block_solver_shapes_in_threads(api):
+    import torch
+    dims, block = (4, 4, 4, 4), (2, 2, 2, 2)
+    U = synthetic.random_gauge(dims, 0.3, 4)
+    Ud, Upd = dev(U), dev(U)
+    api.dd_gauge_update(api.dd_init(dims, block, 0.12), Upd, 1, 5.3, 1, 0, 21, 4)
+    torch.cuda.synchronize()
+
+    def make(tpb):
+        hs = {}
+
+        def job():
+            if not hs:
+                hs["h"] = api.dd_init(dims, block, 0.12)
+                api.dd_set_tuning(hs["h"], block_tpb=tpb, block_ctas_per_sm=2)
+            return api.dd_block_ratios_range(hs["h"], Ud, Upd, 0, 16, 1, 9, 3)
+        return job
+
+    check(make, [256, 128, 256, 128], 300)
+
+
 def test_exact_block_determinants_in_threads(api):
     import torch
     fields = {}
