@@ -379,6 +379,13 @@ int dd_lu_tensor_cores(dd_t h, int on);
  * missing outside 0..64), DD_ERR_UNSUPPORTED, DD_ERR_CUDA. */
 int dd_barrier_check(dd_t h, int missing, int* passed);
 
+/* Check of what follows such a wait (no counterpart in the paper): one panel
+ * and its row swaps with the factorisation marked as failed.  *untouched = 1
+ * when neither changed the matrix.  Synchronises the handle's stream, uses
+ * the exact-path workspace.  Errors: DD_ERR_INVALID_ARG (untouched NULL),
+ * DD_ERR_UNSUPPORTED, DD_ERR_CUDA. */
+int dd_lu_failure_check(dd_t h, int* untouched);
+
 /* Mean plaquette <Re tr U_P / 3> (device, 1 double). */
 int dd_plaquette(dd_t h, const void* U, double* out);
 

@@ -345,6 +345,14 @@ def dd_barrier_check(h, missing=0):
     return bool(out.value)
 
 
+def dd_lu_failure_check(h):
+    """One panel of the dense LU and its row swaps on a factorisation marked
+    as failed: True when they left the matrix as it was."""
+    out = ctypes.c_int()
+    _check(h, _lib.load().dd_lu_failure_check(h.ptr, ctypes.byref(out)))
+    return out.value == 1
+
+
 def dd_alu_peaks(stream=None):
     """Measured FP64 FMA, FP32 FMA and FP64 mma.sync throughput (TFLOP/s) of the current GPU."""
     out = (ctypes.c_double * 3)()

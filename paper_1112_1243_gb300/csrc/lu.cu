@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "dd_internal.h"
@@ -151,7 +152,12 @@ struct LuAux {
     unsigned tag0;  // column k0 + j has the tag tag0 + j
     int* perm;      // [batch][4 LU_NB + 1]: the panel's row swaps as one permutation
                     // (destination rows, source rows, count)
+    int* failed;    // set when a wait gave up: the rest of the factorisation is
+                    // left out (null: panels without waits)
 };
+// A panel that gave up leaves its pivots and its permutation unwritten: they
+// must not be used as row numbers, and later panels need not wait again.
+DD_DEV bool lu_failed(const int* failed) { return failed && *(const volatile int*)failed; }
 static_assert(LU_NB == 32, "a panel's pivots are one a lane");
 static_assert(LU_PR >= LU_NB, "the first thread block of a panel must own all its pivot rows");
 
@@ -354,6 +360,7 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
     __shared__ int s_p;             // pivot row; -1: a message did not come
     const int m = blockIdx.y, c = blockIdx.x, ctas = gridDim.x, tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const bool failed = lu_failed(aux.failed);
     double2* A = M + (long long)m * mstride;
     const int r0 = k0 + c * LU_PR;
     const int nr = min(LU_PR, n - r0);
@@ -361,7 +368,7 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
         const int r = e % nr, j = e / nr;
         pan[r][j] = A[(r0 + r) + (long long)(k0 + j) * n];
     }
-    __syncthreads();
+    if (__syncthreads_or(failed)) return;
     int bi = INT_MAX;  // warp 0: the block's candidate row of the current column
     auto candidate = [&](int j) {
         long long best = -1;
@@ -443,7 +450,10 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
             if (lane == 0) s_p = ok ? bidx : -1;
         }
         __syncthreads();
-        if (s_p < 0) return;
+        if (s_p < 0) {
+            if (tid == 0) *aux.failed = 1;
+            return;
+        }
         const double pm = s_pm[j];
         if (tid == 0 && own_k) {
             aux.ipiv[(long long)m * n + k] = s_p;
@@ -485,7 +495,8 @@ __global__ void __launch_bounds__(LU_THREADS) lu_panel_multi_kernel(double2* M, 
 // substitution with the unit lower triangle L11, lane r holding row k0 + r
 constexpr int LU_TRSM_WARPS = 4;
 __global__ void __launch_bounds__(32 * LU_TRSM_WARPS) lu_swap_trsm_kernel(double2* M, long long mstride, int n,
-                                                                         int ncols, int k0, int nbe, const int* perm) {
+                                                                         int ncols, int k0, int nbe, const int* perm,
+                                                                         const int* failed) {
     __shared__ double2 L[LU_NB][LU_LD];
     __shared__ int s_dst[2 * LU_NB], s_src[2 * LU_NB];
     __shared__ int s_np;
@@ -500,8 +511,12 @@ __global__ void __launch_bounds__(32 * LU_TRSM_WARPS) lu_swap_trsm_kernel(double
         s_dst[tid] = pm[tid];
         s_src[tid] = pm[2 * LU_NB + tid];
     }
-    if (tid == 0) s_np = pm[4 * LU_NB];
+    if (tid == 0) {
+        const int count = pm[4 * LU_NB];
+        s_np = lu_failed(failed) ? -1 : count;
+    }
     __syncthreads();
+    if (s_np < 0) return;
     const int j = k0 + nbe + blockIdx.x * LU_TRSM_WARPS + (tid >> 5);
     if (j >= ncols) return;  // uniform per warp
     double2* col = A + (long long)j * n;
@@ -858,9 +873,11 @@ static int lu_batched(dd_handle* h, double2* M, long long mstride, int batch, in
     aux.ipiv = (int*)(scr + o);
     o += up((size_t)batch * n * sizeof(int));
     aux.perm = (int*)(scr + o);
+    if (!single) msg_off = o;
     o += up((size_t)batch * (4 * LU_NB + 1) * sizeof(int));
     if (!single) {
-        msg_off = o;
+        aux.failed = (int*)(scr + o);
+        o += up(sizeof(int));
         aux.cand = (LuMsg*)(scr + o);
         o += up((size_t)2 * chunk * ctas0 * sizeof(LuMsg));
         aux.prow = (LuMsg*)(scr + o);
@@ -896,7 +913,8 @@ static int lu_batched(dd_handle* h, double2* M, long long mstride, int batch, in
     }
     DD_KLAUNCH(h, zero_doubles_kernel<<<grid_for(batch, 64), 64, 0, h->stream>>>(batch, logdet));
     if (!single) {
-        cudaError_t e = cudaMemsetAsync(scr + msg_off, 0, msg_end - msg_off, h->stream);  // no tags yet
+        // no swaps, not failed, no tags yet
+        cudaError_t e = cudaMemsetAsync(scr + msg_off, 0, msg_end - msg_off, h->stream);
         if (e != cudaSuccess) return dd_cuda_check(h, e, "lu message reset");
     }
     for (int k0 = 0; k0 < n; k0 += LU_NB) {
@@ -929,7 +947,7 @@ static int lu_batched(dd_handle* h, double2* M, long long mstride, int batch, in
         const int right = ncols - k0 - nbe;
         if (right > 0) {
             DD_KLAUNCH(h, lu_swap_trsm_kernel<<<dim3(grid_for(right, LU_TRSM_WARPS), batch), 32 * LU_TRSM_WARPS, 0,
-                                                h->stream>>>(M, mstride, n, ncols, k0, nbe, aux.perm));
+                                                h->stream>>>(M, mstride, n, ncols, k0, nbe, aux.perm, aux.failed));
             const int below = n - k0 - nbe;
             if (below > 0 && tensor) {
                 for (int mi = 0; mi < batch; ++mi) {
@@ -1137,6 +1155,65 @@ extern "C" int dd_barrier_check(dd_t h, int missing, int* passed) {
     DD_CUDA(h, cudaMemcpyAsync(&np, dpassed, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     DD_CUDA(h, cudaStreamSynchronize(h->stream));
     *passed = np == ctas ? 1 : 0;
+    return DD_OK;
+}
+
+// The launches after a wait that gave up, with the failure flag set by the
+// host: a panel and its row swaps on a matrix in the scratch of the exact path
+// (perm holds a valid swap of its rows 0 and 32, so a launch that went on
+// would stay in bounds and show).
+extern "C" int dd_lu_failure_check(dd_t h, int* untouched) {
+    int rc = dd_require_ws(h);
+    if (rc) return rc;
+    rc = dd_require_feature(h, h->feat_exact, "dd_lu_failure_check");
+    if (rc) return rc;
+    if (!untouched) return dd_fail(h, DD_ERR_INVALID_ARG, "dd_lu_failure_check: bad arguments");
+    constexpr int n = 2 * LU_NB, ctas = n / LU_PR;
+    std::vector<double2> want(n * n), got(n * n);
+    for (int k = 0; k < n * n; ++k) want[k] = make_double2(1.0 / (k + 1), k % n == k / n ? 4.0 : 0.5);
+    std::vector<int> perm(4 * LU_NB + 1, 0);
+    perm[0] = perm[2 * LU_NB + 1] = 0;
+    perm[1] = perm[2 * LU_NB] = LU_NB;
+    perm[4 * LU_NB] = 2;
+    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t bytes = up(want.size() * sizeof(double2)) + up(sizeof(double)) + up(n * sizeof(int)) +
+                         up(perm.size() * sizeof(int)) + up(sizeof(int)) +
+                         up((size_t)2 * ctas * sizeof(LuMsg)) + up((size_t)2 * ctas * LU_NB * sizeof(LuMsg)) +
+                         up((size_t)2 * LU_NB * sizeof(LuMsg));
+    if (h->lu_bytes < bytes) return dd_fail(h, DD_ERR_UNSUPPORTED, "dd_lu_failure_check: no scratch");
+    char* p = (char*)h->d_lu;
+    DD_CUDA(h, cudaMemsetAsync(p, 0, bytes, h->stream));
+    auto take = [&](size_t b) {
+        char* q = p;
+        p += up(b);
+        return q;
+    };
+    double2* M = (double2*)take(want.size() * sizeof(double2));
+    double* logdet = (double*)take(sizeof(double));
+    LuAux aux{};
+    aux.ipiv = (int*)take(n * sizeof(int));
+    aux.perm = (int*)take(perm.size() * sizeof(int));
+    aux.failed = (int*)take(sizeof(int));
+    aux.cand = (LuMsg*)take((size_t)2 * ctas * sizeof(LuMsg));
+    aux.prow = (LuMsg*)take((size_t)2 * ctas * LU_NB * sizeof(LuMsg));
+    aux.rowk = (LuMsg*)take((size_t)2 * LU_NB * sizeof(LuMsg));
+    aux.tag0 = 1;
+    const int one = 1;
+    DD_CUDA(h, cudaMemcpyAsync(M, want.data(), want.size() * sizeof(double2), cudaMemcpyHostToDevice, h->stream));
+    DD_CUDA(h, cudaMemcpyAsync(aux.perm, perm.data(), perm.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+    DD_CUDA(h, cudaMemcpyAsync(aux.failed, &one, sizeof(int), cudaMemcpyHostToDevice, h->stream));
+    long long ms = 0;
+    int nn = n, k0 = 0, nbe = LU_NB;
+    void* args[] = {&M, &ms, &nn, &k0, &nbe, &aux, &logdet, &h->d_status};
+    cudaError_t e = cudaLaunchCooperativeKernel((const void*)lu_panel_multi_kernel, dim3(ctas, 1), dim3(LU_THREADS), args, 0,
+                                                h->stream);
+    ++h->launches;
+    if (e != cudaSuccess) return dd_cuda_check(h, e, "lu_panel_kernel (cooperative launch)");
+    DD_KLAUNCH(h, lu_swap_trsm_kernel<<<dim3(grid_for(n - LU_NB, LU_TRSM_WARPS), 1), 32 * LU_TRSM_WARPS, 0, h->stream>>>(
+                      M, ms, n, n, 0, LU_NB, aux.perm, aux.failed));
+    DD_CUDA(h, cudaMemcpyAsync(got.data(), M, got.size() * sizeof(double2), cudaMemcpyDeviceToHost, h->stream));
+    DD_CUDA(h, cudaStreamSynchronize(h->stream));
+    *untouched = std::memcmp(got.data(), want.data(), got.size() * sizeof(double2)) == 0 ? 1 : 0;
     return DD_OK;
 }
 

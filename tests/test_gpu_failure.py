@@ -111,3 +111,16 @@ def test_grid_barrier_wait_is_bounded(api):
     assert api.dd_status(h)[0] == 0              # read and cleared
     assert float(host(api.dd_logdet_exact(h, U, 0))[0]) == ref
     assert api.dd_status(h)[0] == 0
+
+
+def test_a_failed_factorisation_is_left_alone(api):
+    """After a wait that gave up, pivots and the row permutation may be
+    unwritten: the launches that follow must not use them."""
+    dims, block = (4, 4, 4, 4), (2, 2, 2, 2)
+    h = api.dd_init(dims, block, 0.12)
+    U = dev(synthetic.random_gauge(dims, 0.4, 1))
+    ref = float(host(api.dd_logdet_exact(h, U, 0))[0])
+    assert api.dd_lu_failure_check(h) is True
+    assert api.dd_status(h)[0] == 0
+    assert float(host(api.dd_logdet_exact(h, U, 0))[0]) == ref  # the mark is of one factorisation
+    assert api.dd_status(h)[0] == 0
