@@ -32,18 +32,43 @@ DD_DEV SpinorF16 at_rhs(SpinorF16 s, int r) {
     return s;
 }
 
-// canonical FP64 spinors of the caller (16-byte aligned), V sites a rhs
+// canonical FP64 spinors of the caller, stride sites a rhs: the whole lattice,
+// or (half) the sites of one parity; AL: on 16-byte boundaries (the C ABI asks
+// only for those of a double)
+template <bool AL>
 struct SpinorC {
-    double2* p;
+    double* p;
     long long stride;
+    int half;
 };
-DD_DEV SpinorC at_rhs(SpinorC s, int r) {
-    s.p += (long long)r * 12 * s.stride;
+template <bool AL>
+DD_DEV SpinorC<AL> at_rhs(SpinorC<AL> s, int r) {
+    s.p += (long long)r * 24 * s.stride;
     return s;
 }
+DD_DEV double2 load_entry(const SpinorF64& f, long long i) { return f.p[i]; }
+DD_DEV void store_entry(const SpinorF64& f, long long i, double2 v) { f.p[i] = v; }
+template <bool AL>
+DD_DEV double2 load_entry(const SpinorC<AL>& f, long long i) {
+    return load_c(f.p, i, AL);
+}
+template <bool AL>
+DD_DEV void store_entry(const SpinorC<AL>& f, long long i, double2 v) {
+    if (AL) {
+        reinterpret_cast<double2*>(f.p)[i] = v;
+    } else {
+        f.p[2 * i] = v.x;
+        f.p[2 * i + 1] = v.y;
+    }
+}
+template <class S>
+struct is_canonical : std::false_type {};
+template <bool AL>
+struct is_canonical<SpinorC<AL>> : std::true_type {};
 // entry k of the site with even-odd index h and canonical index s
 DD_DEV long long entry_at(const SpinorF64& f, int k, int h, int s) { return k * f.stride + h; }
-DD_DEV long long entry_at(const SpinorC& f, int k, int h, int s) { return (long long)s * 12 + k; }
+template <bool AL>
+DD_DEV long long entry_at(const SpinorC<AL>& f, int k, int h, int s) { return (long long)(f.half ? h : s) * 12 + k; }
 DD_DEV long long entry_at(const SpinorX& f, int k, int h, int s) { return k * f.stride + h; }
 
 template <class SIn, class SX, class SOut, class LK>
@@ -73,7 +98,8 @@ struct HopArgs {
     int both = 0;               // FP64 hops: both output parities in one launch (blockIdx.z), in2: the input of parity 1
     SIn in2;
     int ob[4] = {0, 0, 0, 0};   // MASK 2: hops that leave a block of these extents are dropped too (0: none)
-    const double* U = nullptr;  // FP64 hops on canonical fields: the links, for sites with non-finite neighbours
+    const double* U = nullptr;  // FP64 hops on canonical fields: the caller's links and the hop's input, for sites
+    SX src;                     // with neighbours that are not finite (null: such a site is NaN as a whole)
 };
 
 template <class LK>
@@ -235,8 +261,8 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
 // coordinates): the integer form marks whole sites and links that hold a
 // number that is not finite; this keeps what such a number does to each
 // component.
-template <int MASK>
-__device__ __noinline__ void hop_canonical(const Geo& g, const int* x, const double* U, const double2* in, int g5in,
+template <int MASK, bool AL>
+__device__ __noinline__ void hop_canonical(const Geo& g, const int* x, const double* U, const SpinorC<AL>& in, int g5in,
                                            Spinor<double>& acc) {
     zero(acc);
     const int s = canon_index(g, x);
@@ -252,7 +278,7 @@ __device__ __noinline__ void hop_canonical(const Geo& g, const int* x, const dou
             Spinor<double> v;
 #pragma unroll
             for (int k = 0; k < 12; ++k) {
-                const double2 w = in[(long long)y * 12 + k];
+                const double2 w = load_entry(in, entry_at(in, k, y >> 1, y));
                 v.c[k] = mk<double>(w.x, w.y);
             }
             if (g5in) gamma5(v);
@@ -368,12 +394,12 @@ __global__ void __launch_bounds__(128, 5) hop_x_kernel(HopArgs<SpinorX, SX, SOut
 #pragma unroll
                 for (int c = 0; c < 3; ++c)
                     other[c] = make_double2(x_to_double_any(v[c].x, eout), x_to_double_any(v[c].y, eout));
-                if constexpr (std::is_same<SX, SpinorC>::value) {
-                    if (eout >= X_BAD_MIN) {
+                if constexpr (is_canonical<SX>::value) {
+                    if (eout >= X_BAD_MIN && A.U) {
                         int x[4];
                         site(i, x);
                         Spinor<double> acc;
-                        hop_canonical<MASK>(g, x, A.U, xin.p, A.g5in, acc);
+                        hop_canonical<MASK>(g, x, A.U, at_rhs(A.src, rhs), A.g5in, acc);
 #pragma unroll
                         for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -386,17 +412,17 @@ __global__ void __launch_bounds__(128, 5) hop_x_kernel(HopArgs<SpinorX, SX, SOut
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const long long k = entry_at(out, 3 * q + c, h, s);
-                const double2 w = A.has_x ? xin.p[k] : make_double2(0.0, 0.0);
+                const double2 w = A.has_x ? load_entry(xin, k) : make_double2(0.0, 0.0);
                 double2 z = make_double2((double)v[c].x, (double)v[c].y);
                 if (!usual) z = other[c];
                 z = make_double2(fma(f, z.x, w.x), fma(f, z.y, w.y));
                 if (A.resid) {
-                    const double2 w = bv.p[k];
+                    const double2 w = load_entry(bv, k);
                     z = make_double2(w.x - z.x, w.y - z.y);
                 }
                 if (zeroed) z = make_double2(0.0, 0.0);
-                out.p[k] = z;
-                if (A.has2) at_rhs(A.out2, rhs).p[k] = z;
+                store_entry(out, k, z);
+                if (A.has2) store_entry(at_rhs(A.out2, rhs), k, z);
                 if (A.red.op != FIN_NONE) nrm = fma(z.x, z.x, fma(z.y, z.y, nrm));
             }
         }

@@ -803,15 +803,14 @@ extern "C" int dd_finalize(dd_t h) {
 // ------------------------------------------------------ operator application
 namespace {
 
-// SH: storage of the hop inputs (in_e, in_o, th), SS: of the results and of
-// the terms that enter without a hop (x_e, x_o); the same for FP32 and FP16
-template <class R, class SH, class SS, class LK>
-int apply_eo_ops(dd_handle* h, int op, SH in_e, SH in_o, SS x_e, SS x_o, SH th, SS out_e, SS out_o, LK lk, int nrhs,
-                 int colour_mask, int mask_mode) {
+template <class SS, class LK>
+int apply_eo_ops(dd_handle* h, int op, SS in_e, SS in_o, SS out_e, SS out_o, LK lk, int nrhs, int colour_mask,
+                 int mask_mode) {
     const Geo& g = h->g;
     const double k = h->prm.kappa;
-    auto mk_args = [&](int p, SH in, SS x, auto out, double a, double b, int hasx, int g5) {
-        HopArgs<SH, SS, decltype(out), LK> A;
+    typedef typename SS::real R;
+    auto mk_args = [&](int p, SS in, SS x, SS out, double a, double b, int hasx, int g5) {
+        HopArgs<SS, SS, SS, LK> A;
         A.g = g;
         A.p = p;
         A.in = in;
@@ -832,34 +831,34 @@ int apply_eo_ops(dd_handle* h, int op, SH in_e, SH in_o, SS x_e, SS x_o, SH th, 
     cudaStream_t s = h->stream;
     if (op == DD_OP_D || op == DD_OP_DDAG) {
         int g5 = (op == DD_OP_DDAG);
-        auto A0 = mk_args(0, in_o, x_e, out_e, 1.0, -k, 1, g5);
-        auto A1 = mk_args(1, in_e, x_o, out_o, 1.0, -k, 1, g5);
+        auto A0 = mk_args(0, in_o, in_e, out_e, 1.0, -k, 1, g5);
+        auto A1 = mk_args(1, in_e, in_o, out_o, 1.0, -k, 1, g5);
         if (mask_mode == 1) {
-            launch_hop<R, SH, SS, SS, LK, 1>(A0, nrhs, h);
-            launch_hop<R, SH, SS, SS, LK, 1>(A1, nrhs, h);
+            launch_hop<R, SS, SS, SS, LK, 1>(A0, nrhs, h);
+            launch_hop<R, SS, SS, SS, LK, 1>(A1, nrhs, h);
         } else {
-            launch_hop<R, SH, SS, SS, LK, 0>(A0, nrhs, h);
-            launch_hop<R, SH, SS, SS, LK, 0>(A1, nrhs, h);
+            launch_hop<R, SS, SS, SS, LK, 0>(A0, nrhs, h);
+            launch_hop<R, SS, SS, SS, LK, 0>(A1, nrhs, h);
         }
     } else if (op == DD_OP_INTER) {
-        auto A0 = mk_args(0, in_o, x_e, out_e, 0.0, -k, 0, 0);
-        auto A1 = mk_args(1, in_e, x_o, out_o, 0.0, -k, 0, 0);
-        launch_hop<R, SH, SS, SS, LK, 2>(A0, nrhs, h);
-        launch_hop<R, SH, SS, SS, LK, 2>(A1, nrhs, h);
+        auto A0 = mk_args(0, in_o, in_e, out_e, 0.0, -k, 0, 0);
+        auto A1 = mk_args(1, in_e, in_o, out_o, 0.0, -k, 0, 0);
+        launch_hop<R, SS, SS, SS, LK, 2>(A0, nrhs, h);
+        launch_hop<R, SS, SS, SS, LK, 2>(A1, nrhs, h);
     } else if (op == DD_OP_DTILDE || op == DD_OP_DTILDE_DAG) {
-        // t = H_oe psi_e (odd temporary); out_e = psi_e - k^2 H_eo t
+        // t = H_oe psi_e (out_o: odd temporary); out_e = psi_e - k^2 H_eo t
         int g5 = (op == DD_OP_DTILDE_DAG);
-        auto A1 = mk_args(1, in_e, x_e, th, 0.0, 1.0, 0, 0);
+        auto A1 = mk_args(1, in_e, in_e, out_o, 0.0, 1.0, 0, 0);
         A1.g5in = g5;
         A1.g5out = 0;
-        auto A0 = mk_args(0, th, x_e, out_e, 1.0, -k * k, 1, 0);
+        auto A0 = mk_args(0, out_o, in_e, out_e, 1.0, -k * k, 1, 0);
         A0.g5in = 0;
         A0.g5out = g5;
-        launch_hop<R, SH, SS, SH, LK, 0>(A1, nrhs, h);
-        launch_hop<R, SH, SS, SS, LK, 0>(A0, nrhs, h);
+        launch_hop<R, SS, SS, SS, LK, 0>(A1, nrhs, h);
+        launch_hop<R, SS, SS, SS, LK, 0>(A0, nrhs, h);
     } else if (op == DD_OP_HEO) {
-        auto A0 = mk_args(0, in_o, x_e, out_e, 0.0, 1.0, 0, 0);
-        launch_hop<R, SH, SS, SS, LK, 0>(A0, nrhs, h);
+        auto A0 = mk_args(0, in_o, in_e, out_e, 0.0, 1.0, 0, 0);
+        launch_hop<R, SS, SS, SS, LK, 0>(A0, nrhs, h);
     } else {
         return DD_ERR_INVALID_ARG;
     }
@@ -868,61 +867,106 @@ int apply_eo_ops(dd_handle* h, int op, SH in_e, SH in_o, SS x_e, SS x_o, SH th, 
 
 }  // namespace
 
-// canonical spinors -> limbs, both parities (one thread a site)
-__global__ void __launch_bounds__(128) pack_x_kernel(Geo g, const double* __restrict__ in, bool al16, SpinorX even,
-                                                     SpinorX odd) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
-    if (s >= g.V) return;
-    int x[4];
-    canon_coords(g, s, x);
+// canonical spinors -> limbs (one thread a site): the whole lattice, or the
+// sites of one parity (half) to `even`
+__global__ void __launch_bounds__(128) pack_x_kernel(Geo g, const double* __restrict__ in, bool al16, bool half,
+                                                     SpinorX even, SpinorX odd) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y, n = half ? (int)g.Vh : (int)g.V;
+    if (s >= n) return;
     Spinor<double> v;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-        const double2 w = load_c(in, ((long long)r * g.V + s) * 12 + k, al16);
+        const double2 w = load_c(in, ((long long)r * n + s) * 12 + k, al16);
         v.c[k] = mk<double>(w.x, w.y);
     }
-    at_rhs(((x[0] + x[1] + x[2] + x[3]) & 1) ? odd : even, r).store(s >> 1, v);
+    if (half) {
+        at_rhs(even, r).store(s, v);
+    } else {
+        int x[4];
+        canon_coords(g, s, x);
+        at_rhs(((x[0] + x[1] + x[2] + x[3]) & 1) ? odd : even, r).store(s >> 1, v);
+    }
 }
 
-// D, D^dag, the block operators or the hops between blocks in FP64, straight
-// between the caller's fields: links and spinors into limbs, then one launch
-// for both parities (three launches; packing to FP64 vectors, two hops and
-// unpacking made nine: 48 us on 4^4 and 0.6 of 2.2 ms at 32^3 x 64).  Taken
-// when both spinor fields start on 16-byte boundaries.
+// Every operator in FP64, straight between the caller's fields: links and
+// spinors into limbs, then one launch for both parities (three launches;
+// packing to FP64 vectors, two hops and unpacking made nine: 48 us on 4^4 and
+// 0.6 of 2.2 ms at 32^3 x 64).  Dtilde = 1 - kappa^2 H_eo H_oe keeps H_oe psi in
+// FP64 between its two hops, so that a number that is not finite reaches the
+// components it belongs to.
+template <bool AL>
 static int apply_canonical(dd_handle* h, void* out, const void* in, const void* U, int op, int nrhs, int colour_mask,
                            int mask_mode) {
     const Geo& g = h->g;
     const long long Vh = g.Vh;
     SolverVecs& v = h->vecs[0];
+    const bool dtilde = op == DD_OP_DTILDE || op == DD_OP_DTILDE_DAG, half = dtilde || op == DD_OP_HEO;
     const SpinorX even{v.px, v.pxe, Vh}, odd{reinterpret_cast<int4*>(v.re), v.rxe, Vh};
-    DD_KLAUNCH(h, pack_x_kernel<<<dim3(grid_for(g.V, 128), nrhs), 128, 0, h->stream>>>(g, (const double*)in, true, even,
-                                                                                      odd));
-    HopArgs<SpinorX, SpinorC, SpinorC, LinkX> A;
+    typedef SpinorC<AL> SC;
+    auto canonical = [&](const void* p) { return SC{(double*)p, half ? Vh : g.V, half}; };
+    // an output over the input or the links (not promised, but it has always
+    // worked): the input is copied first, non-finite sites are NaN as a whole
+    const size_t bytes = (size_t)(half ? Vh : g.V) * nrhs * 192, ubytes = (size_t)g.V * 576;
+    auto overlap = [](const void* a, size_t na, const void* b, size_t nb) {
+        return (const char*)a < (const char*)b + nb && (const char*)b < (const char*)a + na;
+    };
+    if (overlap(out, bytes, in, bytes)) {
+        // be and bo lie one after the other (a parity's vectors are a multiple of 256 bytes)
+        DD_CUDA(h, cudaMemcpyAsync(v.be, in, bytes, cudaMemcpyDeviceToDevice, h->stream));
+        in = v.be;
+    }
+    HopArgs<SpinorX, SC, SC, LinkX> A;
     A.g = g;
     A.p = 0;
-    A.both = 1;
-    A.in = odd;
-    A.in2 = even;
-    A.xin = SpinorC{(double2*)in, g.V};
-    A.out = SpinorC{(double2*)out, g.V};
-    A.rhat = A.xin;
-    A.out2 = A.out;
+    A.xin = A.src = A.rhat = canonical(in);
+    A.out = A.out2 = canonical(out);
     A.lk = LinkX{h->fields[0].eox, Vh};
     A.lk_rhs_stride = 0;
     A.a = 1.0;
     A.b = -h->prm.kappa;
-    A.has_x = op != DD_OP_INTER;
+    A.has_x = !half && op != DD_OP_INTER;
     A.g5in = A.g5out = op == DD_OP_DDAG;
     A.colour_mask = colour_mask;
     A.st = nullptr;
     A.red.op = FIN_NONE;
-    A.U = (const double*)U;
-    if (op == DD_OP_INTER)
-        launch_hop<double, SpinorX, SpinorC, SpinorC, LinkX, 2>(A, nrhs, h);
-    else if (mask_mode == 1)
-        launch_hop<double, SpinorX, SpinorC, SpinorC, LinkX, 1>(A, nrhs, h);
-    else
-        launch_hop<double, SpinorX, SpinorC, SpinorC, LinkX, 0>(A, nrhs, h);
+    A.U = overlap(out, bytes, U, ubytes) ? nullptr : (const double*)U;
+    auto pack = [&](SC f, SpinorX e) {
+        DD_KLAUNCH(h, pack_x_kernel<<<dim3(grid_for(f.stride, 128), nrhs), 128, 0, h->stream>>>(g, f.p, AL, half, e, odd));
+    };
+    pack(A.src, even);
+    A.in = A.in2 = even;
+    if (op == DD_OP_HEO) {
+        A.b = 1.0;
+        launch_hop<double, SpinorX, SC, SC, LinkX, 0>(A, nrhs, h);
+    } else if (dtilde) {
+        const int g5 = op == DD_OP_DTILDE_DAG;
+        const SC t = canonical(v.xo);
+        const SpinorX tx{v.tx, v.txe, Vh};
+        A.p = 1;
+        A.b = 1.0;
+        A.g5in = g5;
+        A.out = A.out2 = t;
+        launch_hop<double, SpinorX, SC, SC, LinkX, 0>(A, nrhs, h);
+        pack(t, tx);
+        A.p = 0;
+        A.in = A.in2 = tx;
+        A.src = t;
+        A.b = -h->prm.kappa * h->prm.kappa;
+        A.has_x = 1;
+        A.g5in = 0;
+        A.g5out = g5;
+        A.out = A.out2 = canonical(out);
+        launch_hop<double, SpinorX, SC, SC, LinkX, 0>(A, nrhs, h);
+    } else {
+        A.both = 1;
+        A.in = odd;
+        if (op == DD_OP_INTER)
+            launch_hop<double, SpinorX, SC, SC, LinkX, 2>(A, nrhs, h);
+        else if (mask_mode == 1)
+            launch_hop<double, SpinorX, SC, SC, LinkX, 1>(A, nrhs, h);
+        else
+            launch_hop<double, SpinorX, SC, SC, LinkX, 0>(A, nrhs, h);
+    }
     DD_LAUNCH_CHECK(h, "apply");
     return DD_OK;
 }
@@ -945,8 +989,10 @@ static int apply_common(dd_handle* h, void* out, const void* in, const void* U, 
     const bool even_in = (op == DD_OP_DTILDE || op == DD_OP_DTILDE_DAG);
     const bool odd_in = (op == DD_OP_HEO);
     const bool sub_out = even_in || odd_in;
-    if (prec == DD_PREC_F64 && !sub_out && aligned16(in) && aligned16(out))
-        return apply_canonical(h, out, in, U, op, nrhs, colour_mask, mask_mode);
+    if (prec == DD_PREC_F64)
+        return aligned16(in) && aligned16(out)
+                   ? apply_canonical<true>(h, out, in, U, op, nrhs, colour_mask, mask_mode)
+                   : apply_canonical<false>(h, out, in, U, op, nrhs, colour_mask, mask_mode);
     // input parities in FP64 eo chunks
     if (even_in) {
         launch_pack_spinor_sub(h, (const double*)in, v.be, nrhs);
@@ -959,19 +1005,12 @@ static int apply_common(dd_handle* h, void* out, const void* in, const void* U, 
     DD_LAUNCH_CHECK(h, "pack");
     dim3 cg(grid_for(Vh, 128), nrhs);
     SpinorF64 be{v.be, Vh}, bo{v.bo, Vh}, xe{v.xe, Vh}, xo{v.xo, Vh};
-    if (prec == DD_PREC_F64) {
-        // hop inputs in limbs: even in px, odd in the buffer of re
-        const LinkX lk{f.eox, Vh};
-        const SpinorX ie{v.px, v.pxe, Vh}, io{reinterpret_cast<int4*>(v.re), v.rxe, Vh}, th{v.tx, v.txe, Vh};
-        if (!odd_in) DD_KLAUNCH(h, convert_from64_kernel<<<cg, 128, 0, h->stream>>>(Vh, be, ie));
-        if (!even_in) DD_KLAUNCH(h, convert_from64_kernel<<<cg, 128, 0, h->stream>>>(Vh, bo, io));
-        rc = apply_eo_ops<double>(h, op, ie, io, be, bo, th, xe, xo, lk, nrhs, colour_mask, mask_mode);
-    } else if (prec == DD_PREC_F32) {
+    if (prec == DD_PREC_F32) {
         SpinorF32 ie{v.r32, Vh}, io{v.t32, Vh}, oe{v.p32, Vh}, oo{v.q32, Vh};
         DD_KLAUNCH(h, convert_from64_kernel<<<cg, 128, 0, h->stream>>>(Vh, be, ie));
         DD_KLAUNCH(h, convert_from64_kernel<<<cg, 128, 0, h->stream>>>(Vh, bo, io));
         LinkF32 lk{f.eo32, Vh};
-        rc = apply_eo_ops<float>(h, op, ie, io, ie, io, oo, oe, oo, lk, nrhs, colour_mask, mask_mode);
+        rc = apply_eo_ops(h, op, ie, io, oe, oo, lk, nrhs, colour_mask, mask_mode);
         DD_KLAUNCH(h, convert_to64_kernel<<<cg, 128, 0, h->stream>>>(Vh, oe, xe));
         DD_KLAUNCH(h, convert_to64_kernel<<<cg, 128, 0, h->stream>>>(Vh, oo, xo));
     } else {
@@ -979,7 +1018,7 @@ static int apply_common(dd_handle* h, void* out, const void* in, const void* U, 
         DD_KLAUNCH(h, convert_from64_kernel<<<cg, 128, 0, h->stream>>>(Vh, be, ie));
         DD_KLAUNCH(h, convert_from64_kernel<<<cg, 128, 0, h->stream>>>(Vh, bo, io));
         LinkF16 lk{f.eo16, Vh};
-        rc = apply_eo_ops<float>(h, op, ie, io, ie, io, oo, oe, oo, lk, nrhs, colour_mask, mask_mode);
+        rc = apply_eo_ops(h, op, ie, io, oe, oo, lk, nrhs, colour_mask, mask_mode);
         DD_KLAUNCH(h, convert_to64_kernel<<<cg, 128, 0, h->stream>>>(Vh, oe, xe));
         DD_KLAUNCH(h, convert_to64_kernel<<<cg, 128, 0, h->stream>>>(Vh, oo, xo));
     }

@@ -133,3 +133,82 @@ def test_fields_on_8_byte_boundaries(api, shift):
     api.dd_apply_D(h, bufs[0][1], bufs[1][1], bufs[2][1], api.DD_OP_DDAG, api.DD_PREC_F64, 2)
     got = host(bufs[0][0])[shift // 8:shift // 8 + 2 * psi.size].view(np.complex128).reshape(psi.shape)
     assert np.array_equal(got, host(ref))
+
+
+def hop_bad(bad_u, bad_psi, lat):
+    """Which components of H psi a number that is not finite reaches: the projection joins two spins of a neighbour,
+    the link all colours whose entry or whose component is not finite."""
+    out = np.zeros_like(bad_psi)
+    for a in range(4):
+        pair = np.abs(GAMMA_AXIS[a]).argmax(1)
+        for y, links in ((lat.fwd[:, a], bad_u[:, a]), (lat.bwd[:, a], np.swapaxes(bad_u[lat.bwd[:, a], a], 1, 2))):
+            w = bad_psi[y]
+            w = w | w[:, pair]
+            out |= (links[:, None, :, :] | w[:, :, None, :]).any(3)
+    return out
+
+
+@pytest.mark.parametrize("shift", [0, 8])
+@pytest.mark.parametrize("op", ["D", "DDAG", "HEO", "DTILDE", "DTILDE_DAG"])
+def test_non_finite_numbers_of_every_operator(api, op, shift):
+    """The same components for every operator, on 16- and on 8-byte
+    boundaries; all others equal to those of the clean fields."""
+    import torch
+    dims, block = (4, 4, 6, 4), (2, 2, 3, 2)
+    lat = geometry.Lattice(dims, block)
+    parity = geometry_parity(lat)
+    sites = {"HEO": np.flatnonzero(parity == 1), "DTILDE": np.flatnonzero(parity == 0)}.get(op.split("_")[0],
+                                                                                           np.arange(lat.V))
+    U, psi = synthetic.random_gauge(dims, 0.4, 2), synthetic.random_spinor(dims, 5)
+    mask = np.zeros(lat.V, dtype=bool)
+    mask[sites] = True
+    psi[~mask] = 0
+    h = api.dd_init(dims, block, 0.13)
+
+    def at(a):
+        flat = torch.zeros(2 * a.size + 2, dtype=torch.float64, device="cuda")
+        flat[shift // 8:shift // 8 + 2 * a.size] = dev(a).view(torch.float64).reshape(-1)
+        return flat, flat.data_ptr() + shift
+
+    def apply(U, psi):
+        bufs = [at(np.zeros_like(psi[sites])), at(psi[sites]), at(U)]
+        api.dd_apply_D(h, bufs[0][1], bufs[1][1], bufs[2][1], getattr(api, "DD_OP_" + op), api.DD_PREC_F64, 1)
+        n = 2 * psi[sites].size
+        return host(bufs[0][0])[shift // 8:shift // 8 + n].view(np.complex128).reshape(psi[sites].shape)
+
+    clean = apply(U, psi)
+    U[200, 3, 1, 2] = np.nan
+    psi[sites[17], 2, 1] = np.inf
+    got = apply(U, psi)
+    bad_u, bad_psi = ~np.isfinite(U), ~np.isfinite(psi)
+    hop = hop_bad(bad_u, bad_psi, lat)
+    if op == "HEO":
+        want = hop[parity == 0]
+    elif op.startswith("DTILDE"):
+        hop[parity == 0] = False
+        want = (hop_bad(bad_u, hop, lat) | bad_psi)[parity == 0]
+    else:
+        want = hop | bad_psi
+    assert np.array_equal(~np.isfinite(got), want)
+    assert want.any() and not want.all()
+    ok = ~want
+    assert np.abs(got[ok] - clean[ok]).max() <= 1e-14 * np.abs(clean).max()
+
+
+@pytest.mark.parametrize("op", ["D", "HEO", "DTILDE"])
+def test_output_over_the_input(api, op):
+    """Not promised by the interface, but it works as it always has."""
+    dims, block = (4, 4, 4, 6), (2, 2, 2, 3)
+    U, psi = synthetic.random_gauge(dims, 0.4, 2), synthetic.random_spinor(dims, 5)
+    if op != "D":
+        psi = psi[: psi.shape[0] // 2]
+    h = api.dd_init(dims, block, 0.13)
+    ref, io, Ud = dev(np.zeros_like(psi)), dev(psi), dev(U)
+    api.dd_apply_D(h, ref, dev(psi), Ud, getattr(api, "DD_OP_" + op), api.DD_PREC_F64, 1)
+    api.dd_apply_D(h, io, io, Ud, getattr(api, "DD_OP_" + op), api.DD_PREC_F64, 1)
+    assert np.array_equal(host(io), host(ref))
+
+
+def geometry_parity(lat):
+    x = np.stack(np.meshgrid(*(np.arange(d) for d in lat.dims), indexing="ij"))
+    return x.sum(0).reshape(-1, order="F") % 2
