@@ -423,11 +423,14 @@ __device__ __noinline__ void eo_xhop(const EoCtx c, const EoTeam T, EoShared& M,
 // limbs of a spinor held by a lane pair (6 components each); every lane of
 // the warp calls this
 DD_DEV void eo_store_limbs(EoX x, int stride, int idx, int sp, bool ok, const cpx<double>* v) {
-    int m = 0;
+    XTop top;
     if (ok)
 #pragma unroll
-        for (int k = 0; k < 6; ++k)
-            m = max(m, max(__double2hiint(v[k].x) & 0x7fffffff, __double2hiint(v[k].y) & 0x7fffffff));
+        for (int k = 0; k < 6; ++k) {
+            top.add(v[k].x);
+            top.add(v[k].y);
+        }
+    int m = top.get();
     m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
     if (!ok) return;
     int E;

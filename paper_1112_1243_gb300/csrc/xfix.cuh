@@ -18,8 +18,7 @@
 // below 2^-55 of the largest entry around a site, FP64's own are about 2^-53
 // of the summed terms: the integer form is the more accurate one.
 // Entries that are not finite mark their site or link (X_BAD): every result
-// they enter is NaN.  Subnormal entries count as zero.
-//
+// they enter is NaN.
 #pragma once
 
 #include "dd_common.cuh"
@@ -34,22 +33,35 @@ DD_DEV int2 x_split(long long v) {
     return make_int2((int)((v - lo) >> 30), lo);
 }
 // v 2^(bits + 1022 - E) rounded to an integer; E: biased exponent of the
-// largest entry, so |result| <= 2^bits (53 <= bits <= 60)
+// largest entry, so |result| <= 2^bits (53 <= bits <= 60).  A subnormal number
+// has the exponent 1 and no leading bit; E is below 1 where all entries are.
 DD_DEV long long x_from_double(double v, int E, int bits) {
     const int hi = __double2hiint(v);
     const int ex = (hi >> 20) & 0x7ff;
     unsigned long long m =
-        ((unsigned long long)((unsigned)(hi & 0xfffff) | 0x100000u) << 32) | (unsigned)__double2loint(v);
-    const int d = E - ex;
-    m = (ex == 0 || d > 60) ? 0ull : (((m << (bits - 53)) + ((1ull << d) >> 1)) >> d);
+        ((unsigned long long)((unsigned)(hi & 0xfffff) | (ex ? 0x100000u : 0u)) << 32) | (unsigned)__double2loint(v);
+    const int d = max(E, 1) - max(ex, 1);
+    m = d > 60 ? 0ull : (((m << (bits - 53 + max(1 - E, 0))) + ((1ull << d) >> 1)) >> d);
     return hi < 0 ? -(long long)m : (long long)m;
 }
-// common exponent of n doubles from the OR-free maximum of their high words
-// (sign cleared): the biased exponent E (0: nothing but zeros and
-// subnormals) and the stored exponent
-DD_DEV int x_exponent(int maxhi, int& E) {
-    E = maxhi >> 20;
-    return E == 0x7ff ? X_BAD : (E == 0 ? X_ZERO : E - 1022);
+// Magnitude of the largest of a set of doubles: its high word (sign cleared);
+// where all high words are 0, -32..-1 by the leading bit of the low words;
+// X_NONE where every number is 0.  Larger values are larger numbers.
+constexpr int X_NONE = -(1 << 30);
+struct XTop {
+    int m = 0;
+    unsigned lo = 0;
+    DD_DEV void add(double v) {
+        m = max(m, __double2hiint(v) & 0x7fffffff);
+        lo |= (unsigned)__double2loint(v);
+    }
+    DD_DEV int get() const { return m ? m : (lo ? -1 - __clz((int)lo) : X_NONE); }
+};
+// biased exponent E of that magnitude (below 1: subnormal) and the stored exponent
+DD_DEV int x_exponent(int top, int& E) {
+    E = top >> 20;
+    if (E < 1) E = top > 0 ? 12 - __clz(top) : (top == X_NONE ? 1 : top - 19);
+    return E == 0x7ff ? X_BAD : (top == X_NONE ? X_ZERO : E - 1022);
 }
 // Spinor in limbs: chunk k (spin * 3 + colour) of site i at p[k * stride + i]
 // as (re.hi, re.lo, im.hi, im.lo), its exponent at e[i]
@@ -59,12 +71,14 @@ struct SpinorX {
     long long stride;
     typedef double real;
     DD_DEV void store(long long i, const Spinor<double>& s) const {
-        int m = 0;
+        XTop top;
 #pragma unroll
-        for (int k = 0; k < 12; ++k)
-            m = max(m, max(__double2hiint(s.c[k].x) & 0x7fffffff, __double2hiint(s.c[k].y) & 0x7fffffff));
+        for (int k = 0; k < 12; ++k) {
+            top.add(s.c[k].x);
+            top.add(s.c[k].y);
+        }
         int E;
-        e[i] = x_exponent(m, E);
+        e[i] = x_exponent(top.get(), E);
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
             const int2 a = x_split(x_from_double(s.c[k].x, E, 57)), b = x_split(x_from_double(s.c[k].y, E, 57));
@@ -91,11 +105,11 @@ struct LinkX {
 };
 // one link, entries u[0..8] (re, im): entry k at p[k * stride], exponent at *e
 DD_DEV void x_store_entries(int4* p, long long stride, int* e, const double* u) {
-    int m = 0;
+    XTop top;
 #pragma unroll
-    for (int k = 0; k < 18; ++k) m = max(m, __double2hiint(u[k]) & 0x7fffffff);
+    for (int k = 0; k < 18; ++k) top.add(u[k]);
     int E;
-    *e = x_exponent(m, E);
+    *e = x_exponent(top.get(), E);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         const int2 x = x_split(x_from_double(u[2 * k], E, 59)), y = x_split(x_from_double(u[2 * k + 1], E, 59));

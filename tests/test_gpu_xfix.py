@@ -212,3 +212,30 @@ def test_output_over_the_input(api, op):
 def geometry_parity(lat):
     x = np.stack(np.meshgrid(*(np.arange(d) for d in lat.dims), indexing="ij"))
     return x.sum(0).reshape(-1, order="F") % 2
+
+
+@pytest.mark.parametrize("kind", ["spinor", "spinor mixed", "link"])
+def test_subnormal_numbers(api, kind):
+    """Subnormal entries are numbers like all others: the hops between blocks
+    (their sum alone) against extended precision, to the bound above and half
+    a unit of the smallest number for a subnormal result."""
+    dims, block, kappa = (4, 4, 6, 4), (1, 1, 1, 1), 0.125
+    lat = geometry.Lattice(dims, block)
+    U, psi = synthetic.random_gauge(dims, 0.4, 2), synthetic.random_spinor(dims, 5)
+    if kind == "spinor":
+        psi = psi * 2.0 ** -1060
+    elif kind == "spinor mixed":  # largest entries normal, others below the normal range
+        psi = psi * 2.0 ** -1020
+        psi[:, 1::2] *= 2.0 ** -14
+    else:
+        U, psi = U * 2.0 ** -1050, psi * 2.0 ** 600
+    h = api.dd_init(dims, block, kappa)
+    out = dev(np.zeros_like(psi))
+    api.dd_apply_D(h, out, dev(psi), dev(U), api.DD_OP_INTER, api.DD_PREC_F64, 1)
+    got = host(out)
+    hop, mag = hop_extended(U, psi, lat)
+    ref = -LD(kappa) * hop
+    err = np.abs(got.astype(LD) - ref).max((1, 2)).astype(np.longdouble)
+    top = np.abs(ref).max((1, 2))
+    assert np.abs(ref).max() > 0 and np.all(err <= np.sqrt(2) * (2.0 ** -53 * top + kappa * 2.0 ** -54 * mag
+                                                               + np.longdouble(2.0) ** -1075 * 2))
