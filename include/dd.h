@@ -58,7 +58,11 @@ extern "C" {
 #define DD_ERR_NO_WORKSPACE (-7)
 
 /* arithmetic / storage precision of a kernel */
-#define DD_PREC_F64 0 /* FP64 storage and arithmetic */
+#define DD_PREC_F64 0 /* FP64 storage and accuracy.  dd_apply_D and dd_apply_D_block: every component to a few
+                         roundings (2^-53) of its own products, for any finite input, subnormal numbers included,
+                         and numbers that are not finite reach the components that FP64 arithmetic takes them to.
+                         Inside the solvers (residuals, the FP64 Krylov method, Schur pieces, block filter) hops
+                         are accurate to 8 x 2^-53 of the largest product around a site */
 #define DD_PREC_F32 1 /* FP32 storage (links: rows 1-2, third row rebuilt), FP32 arithmetic */
 #define DD_PREC_F16 2 /* FP16 storage (spinors with a per-site FP32 scale), FP32 arithmetic */
 #define DD_PREC_DF64 3 /* dd_params.outer_prec only: double-float (pairs of FP32, 48-bit significand)

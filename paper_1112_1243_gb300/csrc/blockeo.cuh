@@ -388,7 +388,7 @@ __device__ __noinline__ void eo_xhop(const EoCtx c, const EoTeam T, EoShared& M,
         const int i = 8 * a + (lane & 7), q = lane >> 3, idx = M.hs[grp][i];
         const int eout = max(max(M.ex[grp][0][i], M.ex[grp][1][i]), max(M.ex[grp][2][i], M.ex[grp][3][i]));
         xacc v[3];
-        x_gather(part[grp], i, q, v);
+        x_gather<false>(part[grp], i, q, v, nullptr);
         if (xo.p) {
             unsigned long long any = x_mag(v[0]) | x_mag(v[1]) | x_mag(v[2]);
             any |= __shfl_xor_sync(0xffffffffu, any, 8);

@@ -340,7 +340,9 @@ inline size_t block_slot_bytes(long long nb) { return ((size_t)nb * 2240 + 8192 
 inline int grid_for(long long n, int threads) { return (int)((n + threads - 1) / threads); }
 
 // field formatting (lattice.cu)
-int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eox, bool eo32, bool eo16, bool dd);
+// (wide: mark links of a wide range, for the FP64 operators)
+int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eox, bool eo32, bool eo16, bool dd,
+                 bool wide = false);
 // spinor packing between canonical FP64 and eo FP64 (lattice.cu)
 void launch_pack_spinor_eo(dd_handle* h, const double* in, double2* out, int parity, int nrhs, long long in_rhs_stride);
 void launch_unpack_spinor_eo(dd_handle* h, const double2* in, double* out, int parity, int nrhs, long long out_rhs_stride);

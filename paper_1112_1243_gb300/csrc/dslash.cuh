@@ -37,6 +37,7 @@ DD_DEV SpinorF16 at_rhs(SpinorF16 s, int r) {
 // only for those of a double)
 template <bool AL>
 struct SpinorC {
+    static constexpr bool aligned = AL;
     double* p;
     long long stride;
     int half;
@@ -257,53 +258,167 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
 // 2.5 times the instructions and 830 us.  At 2^20 sites what is left is
 // latency: 20 warps an SM (96 registers), DRAM at 45%, issue slots at 32%.
 
-// The hops onto one site in FP64 arithmetic on the caller's fields (x: its
-// coordinates): the integer form marks whole sites and links that hold a
-// number that is not finite; this keeps what such a number does to each
-// component.
-template <int MASK, bool AL>
+// sum kept as a pair of FP64 numbers
+struct Pair64 {
+    double hi, lo;
+    DD_DEV void add(double v, double err) {
+        const double s = hi + v, b = s - hi;
+        lo += (hi - (s - b)) + (v - b) + err;
+        hi = s;
+    }
+    // + a (h + e)
+    DD_DEV void mac(double a, double h, double e) {
+        const double p = a * h;
+        add(p, fma(a, e, fma(a, h, -p)));
+    }
+};
+// The hops onto spin q of one site in FP64 arithmetic on the caller's fields
+// (x: its coordinates).  The integer form has one exponent for a
+// neighbourhood: it marks whole sites and links that hold a number that is
+// not finite, and leaves few bits for entries far below the largest ones (a
+// colour or spin that the links do not mix with a larger one).  For those
+// this keeps what FP64 gives each component, of the colours in the bits of
+// few.  PAIRS: projections and sums as pairs of FP64 numbers, one rounding of
+// the result.
+template <int MASK, bool AL, bool PAIRS>
 __device__ __noinline__ void hop_canonical(const Geo& g, const int* x, const double* U, const SpinorC<AL>& in, int g5in,
-                                           Spinor<double>& acc) {
-    zero(acc);
+                                           int q, int few, double2* out) {
     const int s = canon_index(g, x);
     const bool al16 = (reinterpret_cast<uintptr_t>(U) & 15) == 0;
-#pragma unroll 1
-    for (int a = 0; a < 4; ++a) {
-        const int loc = x[a] % g.b[a];
-#pragma unroll 1
-        for (int dir = 1; dir >= -1; dir -= 2) {
-            const bool face = loc == (dir > 0 ? g.b[a] - 1 : 0);
-            if (MASK && (MASK == 1 ? face : !face)) continue;
-            const int y = shift_index(g, x, a, dir);
-            Spinor<double> v;
+    cpx<double> acc[3];
+    Pair64 pr[3], pi[3];
 #pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                const double2 w = load_entry(in, entry_at(in, k, y >> 1, y));
-                v.c[k] = mk<double>(w.x, w.y);
-            }
-            if (g5in) gamma5(v);
-            Half<double> h, uh;
-            project<double>(a, dir, v, h);
-            Link<double> u;
+    for (int c = 0; c < 3; ++c) {
+        acc[c] = mk<double>(0.0, 0.0);
+        pr[c] = pi[c] = Pair64{0.0, 0.0};
+    }
+#pragma unroll 1
+    for (int d = 0; d < 8; ++d) {
+        const int a = d >> 1, dir = (d & 1) ? -1 : 1;
+        const int loc = x[a] - fast_div(x[a], g.b[a], g.mb[a]) * g.b[a];
+        const bool face = loc == (dir > 0 ? g.b[a] - 1 : 0);
+        if (MASK && (MASK == 1 ? face : !face)) continue;
+        const int y = shift_index(g, x, a, dir);
+        // line r of the projection: upper spin r, and the lower spin that meets it
+        const int r = q < 2 ? q : (a < 2 ? 3 - q : q - 2), low = a < 2 ? 3 - r : 2 + r;
+        // sign of i sigma_a on that line (times i for a = 0, 2)
+        const bool rot = !(a & 1), neg = (a == 1 || a == 2) && r == 1;
+        const double sl = (neg != (dir < 0)) != (g5in != 0) ? -1.0 : 1.0;
+        cpx<double> h[3], e[3];
 #pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                const double2 w = load_c(U, ((long long)(dir > 0 ? s : y) * 4 + a) * 9 + k, al16);
-                u.m[k / 3][k % 3] = mk<double>(w.x, w.y);
+        for (int c = 0; c < 3; ++c) {
+            const double2 u = load_entry(in, entry_at(in, 3 * r + c, y >> 1, y)),
+                          l = load_entry(in, entry_at(in, 3 * low + c, y >> 1, y));
+            const double lx = rot ? -sl * l.y : sl * l.x, ly = rot ? sl * l.x : sl * l.y;
+            Pair64 hx{u.x, 0.0}, hy{u.y, 0.0};
+            hx.add(lx, 0.0);
+            hy.add(ly, 0.0);
+            h[c] = mk<double>(hx.hi, hy.hi);
+            e[c] = mk<double>(hx.lo, hy.lo);
+        }
+        const bool wrap = a == 3 && x[3] == (dir > 0 ? g.L[3] - 1 : 0);
+        double sc = wrap ? (double)g.bc : 1.0;
+        if (q > 1) {
+            // lower spin q: - dir i sigma_a of the product, time + dir
+            const bool lneg = (a == 1 || a == 2) && q == 3;
+            if ((a == 3) == (dir < 0)) sc = -sc;
+            if (lneg) sc = -sc;
+        }
+        const long long lk = ((long long)(dir > 0 ? s : y) * 4 + a) * 9;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            if (!((few >> i) & 1)) continue;
+            cpx<double> v = mk<double>(0.0, 0.0);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const double2 w = load_c(U, lk + (dir > 0 ? 3 * i + j : 3 * j + i), al16);
+                const cpx<double> m = mk<double>(w.x, dir > 0 ? w.y : -w.y);
+                if (PAIRS) {
+                    // sc m h, times i for a rotated lower spin
+                    const bool turn = q > 1 && rot;
+                    Pair64 &re = turn ? pi[i] : pr[i], &im = turn ? pr[i] : pi[i];
+                    const double si = turn ? -sc : sc;
+                    re.mac(sc * m.x, h[j].x, e[j].x);
+                    re.mac(-sc * m.y, h[j].y, e[j].y);
+                    im.mac(si * m.x, h[j].y, e[j].y);
+                    im.mac(si * m.y, h[j].x, e[j].x);
+                } else {
+                    v = cmac(v, m, h[j]);
+                }
             }
-            if (dir > 0)
-                mul_link(u, h, uh);
-            else
-                mul_link_dag(u, h, uh);
-            const bool wrap = a == 3 && x[3] == (dir > 0 ? g.L[3] - 1 : 0);
-            accumulate<double>(a, dir, uh, wrap ? (double)g.bc : 1.0, acc);
+            if (!PAIRS) {
+                if (q > 1 && rot) v = itimes(v);
+                acc[i] = acc[i] + sc * v;
+            }
         }
     }
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        if ((few >> c) & 1)
+            out[c] = PAIRS ? make_double2(pr[c].hi + pr[c].lo, pi[c].hi + pi[c].lo) : make_double2(acc[c].x, acc[c].y);
+}
+
+// Of the entries in the bits of few (hops all below 2^-3 of the largest
+// product): those whose products are, too.  The hops may also be small
+// because their products cancel, and then the integer form has the smaller
+// error.  Sums of |link| |projected spinor|
+// from the limbs in FP32, in units of the largest product 2^eout.  Bit 3 of
+// the result: some lie above 2^-8, where FP64 products and sums would lose
+// to the integer form in the error against the neighbourhood, and pairs of
+// FP64 numbers keep both.  Random fields: the hops of one axis alone (sites
+// at block corners, hops between blocks) get here, 1e-6 of the others.
+template <int MASK>
+__device__ __noinline__ int hop_few_bits(const Geo& g, const int* x, const SpinorX& in, const LinkX& lk, int par,
+                                         int g5in, int q, int eout, int few) {
+    const long long Vh = g.Vh;
+    const int s = canon_index(g, x);
+    const int* le = lk.exps();
+    float sum[3] = {0.f, 0.f, 0.f};
+    auto mag = [](int4 v) {
+        return fabsf(fmaf((float)v.x, 0x1p30f, (float)v.y)) + fabsf(fmaf((float)v.z, 0x1p30f, (float)v.w));
+    };
+#pragma unroll 1
+    for (int d = 0; d < 8; ++d) {
+        const int a = d >> 1, dir = (d & 1) ? -1 : 1;
+        const int loc = x[a] - fast_div(x[a], g.b[a], g.mb[a]) * g.b[a];
+        const bool face = loc == (dir > 0 ? g.b[a] - 1 : 0);
+        if (MASK && (MASK == 1 ? face : !face)) continue;
+        const int y = shift_index(g, x, a, dir) >> 1, row = (dir > 0 ? par : 1 - par) * 4 + a, at = dir > 0 ? s >> 1 : y;
+        int e = in.e[y] + le[row * Vh + at];
+        e -= x_wide_marks(e) * X_WIDE;
+        if (e <= X_ZERO / 2) continue;
+        const float scale = scalbnf(0x1p-116f, max(e - eout, -60) + 60);  // of limbs: 2^-57 2^-59, times 2^60
+        xlimb h[6];
+        x_project(a, (dir < 0) != (g5in != 0), in.p, in.stride, (unsigned)y * 16u, h);
+        const int r = q < 2 ? q : (a < 2 ? 3 - q : q - 2);
+        float hm[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const xlimb v = r ? h[3 + c] : h[c];
+            hm[c] = mag(make_int4(v.rh, v.rl, v.ih, v.il)) * scale;
+        }
+        for (int c = 0; c < 3; ++c)
+            if ((few >> c) & 1)
+                for (int j = 0; j < 3; ++j) {
+                    const int k = dir > 0 ? 3 * c + j : 3 * j + c;
+                    sum[c] = fmaf(mag(x_load(lk.p + (long long)row * 9 * Vh, k * Vh, (unsigned)at * 16u)), hm[j], sum[c]);
+                }
+    }
+    int found = 0;
+    for (int c = 0; c < 3; ++c) {
+        if (!((few >> c) & 1) || sum[c] >= 0x1p57f) continue;
+        found |= 1 << c;
+        if (sum[c] > 0x1p52f) found |= 8;
+    }
+    return found;
 }
 
 template <class SX, class SOut, int MASK>
 __global__ void __launch_bounds__(128, 5) hop_x_kernel(HopArgs<SpinorX, SX, SOut, LinkX> A) {
     __shared__ long long part[4][24][X_PAD];  // axis; sum (0..11) and difference (12..23) of its hops
     __shared__ int ex[4][X_TILE], hs[X_TILE], ss[X_TILE];
+    __shared__ unsigned char wide[4][X_TILE];  // X_WIDE marks of an axis
+    constexpr bool canonical = is_canonical<SX>::value;
     const int rhs = blockIdx.y, par = A.both ? (int)blockIdx.z : A.p;
     if (A.st && !A.st[rhs].active) return;
     const Geo& g = A.g;
@@ -342,7 +457,13 @@ __global__ void __launch_bounds__(128, 5) hop_x_kernel(HopArgs<SpinorX, SX, SOut
                 okb = okb && lo != 0;
             }
         }
-        const int ef = okf ? in.e[yf] + le[rf] : 2 * X_ZERO, eb = okb ? in.e[yb] + le[rb] : 2 * X_ZERO;
+        int ef = okf ? in.e[yf] + le[rf] : 2 * X_ZERO, eb = okb ? in.e[yb] + le[rb] : 2 * X_ZERO;
+        if (canonical) {
+            const int mf = x_wide_marks(ef), mb = x_wide_marks(eb);
+            ef -= mf * X_WIDE;
+            eb -= mb * X_WIDE;
+            wide[a][lane] = (unsigned char)(mf | mb);
+        }
         ex[a][lane] = max(ef, eb);
         if (a == 0) {
             hs[lane] = h;
@@ -361,7 +482,8 @@ __global__ void __launch_bounds__(128, 5) hop_x_kernel(HopArgs<SpinorX, SX, SOut
     const int h = hs[i], s = ss[i];
     const int eout = max(max(ex[0][i], ex[1][i]), max(ex[2][i], ex[3][i]));
     xacc v[3];
-    x_gather(part, i, q, v);
+    int mag[3];
+    x_gather<canonical>(part, i, q, v, mag);
     if constexpr (std::is_same<SOut, SpinorX>::value) {
         unsigned long long any = x_mag(v[0]) | x_mag(v[1]) | x_mag(v[2]);
         any |= __shfl_xor_sync(0xffffffffu, any, 8);
@@ -390,21 +512,36 @@ __global__ void __launch_bounds__(128, 5) hop_x_kernel(HopArgs<SpinorX, SX, SOut
             const double f0 = (q > 1 && A.g5out) ? -A.b : A.b;
             bool usual = abs(eout) < 900;
             double2 other[3];
+            int few = 0;
+            if constexpr (canonical) {
+                if (A.U) {
+                    if (eout >= X_BAD_MIN) {
+                        few = 7;
+                    } else if (min(min(mag[0], mag[1]), mag[2]) < X_SMALL && eout > X_ZERO / 2) {
+                        few = x_small(part, i, q, mag, (wide[0][i] | wide[1][i] | wide[2][i] | wide[3][i]) != 0);
+                        if (few) {
+                            int x[4];
+                            site(i, x);
+                            few = hop_few_bits<MASK>(g, x, at_rhs((A.both && par) ? A.in2 : A.in, rhs),
+                                                     LinkX{A.lk.p + (long long)rhs * A.lk_rhs_stride, A.lk.stride}, par,
+                                                     A.g5in, q, eout, few);
+                        }
+                    }
+                    usual = usual && !few;
+                }
+            }
             if (!usual) {
 #pragma unroll
                 for (int c = 0; c < 3; ++c)
                     other[c] = make_double2(x_to_double_any(v[c].x, eout), x_to_double_any(v[c].y, eout));
-                if constexpr (is_canonical<SX>::value) {
-                    if (eout >= X_BAD_MIN && A.U) {
+                if constexpr (canonical) {
+                    if (few) {
                         int x[4];
                         site(i, x);
-                        Spinor<double> acc;
-                        hop_canonical<MASK>(g, x, A.U, at_rhs(A.src, rhs), A.g5in, acc);
-#pragma unroll
-                        for (int c = 0; c < 3; ++c)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                if (e == q) other[c] = make_double2(acc.c[3 * e + c].x, acc.c[3 * e + c].y);
+                        if (few & 8)
+                            hop_canonical<MASK, SX::aligned, true>(g, x, A.U, at_rhs(A.src, rhs), A.g5in, q, few, other);
+                        else
+                            hop_canonical<MASK, SX::aligned, false>(g, x, A.U, at_rhs(A.src, rhs), A.g5in, q, few, other);
                     }
                 }
             }

@@ -126,7 +126,7 @@ std::vector<uint8_t> active_links(const HostGeo& G, int mode) {
 
 // --------------------------------------------------------- field formatting
 // one thread a link (blockIdx.y: its direction)
-__global__ void __launch_bounds__(128) format_gauge_kernel(Geo g, const double* __restrict__ U, bool al16,
+__global__ void __launch_bounds__(128) format_gauge_kernel(Geo g, const double* __restrict__ U, bool al16, bool wide,
                                                            FieldSlot f) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x, a = blockIdx.y;
     if (s >= g.V) return;
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(128) format_gauge_kernel(Geo g, const double* 
         u[2 * k] = v.x;
         u[2 * k + 1] = v.y;
     }
-    if (f.eox) x_store_link(f.eox, Vh, par, a, h, u);
+    if (f.eox) x_store_link(f.eox, Vh, par, a, h, u, wide);
     if (f.eox && f.eodf) {
         float4* o = f.eodf + ((long long)par * 4 + a) * 9 * Vh + h;
         for (int k = 0; k < 9; ++k) {
@@ -184,7 +184,8 @@ __global__ void __launch_bounds__(128) format_gauge_kernel(Geo g, const double* 
     }
 }
 
-int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eox, bool eo32, bool eo16, bool dd) {
+int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eox, bool eo32, bool eo16, bool dd,
+                 bool wide) {
     FieldSlot t = f;
     if (!eox) t.eox = nullptr;
     if (!eo32) t.eo32 = nullptr;
@@ -193,7 +194,7 @@ int format_field(dd_handle* h, const double* U, FieldSlot& f, bool eox, bool eo3
         t.ddx = nullptr;
         t.dd32 = nullptr;
     }
-    DD_KLAUNCH(h, format_gauge_kernel<<<dim3(grid_for(h->g.V, 128), 4), 128, 0, h->stream>>>(h->g, U, aligned16(U), t));
+    DD_KLAUNCH(h, format_gauge_kernel<<<dim3(grid_for(h->g.V, 128), 4), 128, 0, h->stream>>>(h->g, U, aligned16(U), wide, t));
     DD_LAUNCH_CHECK(h, "format_gauge_kernel");
     return DD_OK;
 }
@@ -880,11 +881,11 @@ __global__ void __launch_bounds__(128) pack_x_kernel(Geo g, const double* __rest
         v.c[k] = mk<double>(w.x, w.y);
     }
     if (half) {
-        at_rhs(even, r).store(s, v);
+        at_rhs(even, r).store<true>(s, v);
     } else {
         int x[4];
         canon_coords(g, s, x);
-        at_rhs(((x[0] + x[1] + x[2] + x[3]) & 1) ? odd : even, r).store(s >> 1, v);
+        at_rhs(((x[0] + x[1] + x[2] + x[3]) & 1) ? odd : even, r).store<true>(s >> 1, v);
     }
 }
 
@@ -983,7 +984,7 @@ static int apply_common(dd_handle* h, void* out, const void* in, const void* U, 
     const Geo& g = h->g;
     const long long Vh = g.Vh;
     FieldSlot& f = h->fields[0];
-    rc = format_field(h, (const double*)U, f, prec == DD_PREC_F64, prec == DD_PREC_F32, prec == DD_PREC_F16, false);
+    rc = format_field(h, (const double*)U, f, prec == DD_PREC_F64, prec == DD_PREC_F32, prec == DD_PREC_F16, false, true);
     if (rc) return rc;
     SolverVecs& v = h->vecs[0];
     const bool even_in = (op == DD_OP_DTILDE || op == DD_OP_DTILDE_DAG);

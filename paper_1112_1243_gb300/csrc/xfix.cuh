@@ -14,9 +14,17 @@
 // 64-bit sums are exact.  With the projection h = psi_upper +- psi_lower
 // (limb by limb, |h_hi| <= 2^28, |h_lo| <= 2^30) the six terms of a colour
 // sum stay below 6 x 2^57 (hi hi') and 7.5 x 2^59 (cross), and eight hops
-// below 8 x 6 x 2^57 < 2^63, for any links and spinors.  Rounding errors are
-// below 2^-55 of the largest entry around a site, FP64's own are about 2^-53
-// of the summed terms: the integer form is the more accurate one.
+// below 8 x 6 x 2^57 < 2^63, for any links and spinors.
+// Error, in units of 2^-56 of the largest product of a link and a spinor entry
+// around a site: a hop drops at most 3 (lo lo'), rounds 1 away and takes 3.75
+// from the rounding of its inputs, so eight hops stay below 62 units, 7.8 x
+// 2^-53, in the worst case.  Relative to a component's own products random
+// fields give at most 0.6 x 2^-53 (0.92 for the FP64 stencil).  This is a
+// bound against the neighbourhood's largest numbers; a component far below
+// them that the links do not mix with them has fewer bits.  The operators of
+// the interface find such components and take them from FP64 arithmetic
+// (hop_x_kernel, hop_canonical); inside the solvers, whose targets are norms,
+// the bound serves as it is.
 // Entries that are not finite mark their site or link (X_BAD): every result
 // they enter is NaN.
 #pragma once
@@ -26,6 +34,12 @@
 constexpr int X_BAD = 1 << 26;      // exponent of a non-finite site or link
 constexpr int X_BAD_MIN = 1 << 25;  // a sum of exponents with an X_BAD in it is above
 constexpr int X_ZERO = -(1 << 24);  // exponent of an all-zero site or link
+constexpr int X_WIDE = 1 << 20;     // added where entries lie far below the largest (fields of the FP64 operators)
+// marks in a sum of two exponents (0, 1 or 2), none in the special values
+DD_DEV int x_wide_marks(int e) {
+    const int k = (e + X_WIDE / 2) / X_WIDE;
+    return e > 0 && k <= 2 ? k : 0;
+}
 
 // 64-bit integer -> limbs (value = hi 2^30 + lo)
 DD_DEV int2 x_split(long long v) {
@@ -48,12 +62,23 @@ DD_DEV long long x_from_double(double v, int E, int bits) {
 // where all high words are 0, -32..-1 by the leading bit of the low words;
 // X_NONE where every number is 0.  Larger values are larger numbers.
 constexpr int X_NONE = -(1 << 30);
+constexpr int X_WIDE_BITS = 24;
 struct XTop {
     int m = 0;
     unsigned lo = 0;
+    unsigned least = ~0u;  // add_wide: smallest high word of a number that is not 0, less 1
     DD_DEV void add(double v) {
         m = max(m, __double2hiint(v) & 0x7fffffff);
         lo |= (unsigned)__double2loint(v);
+    }
+    DD_DEV void add_wide(double v) {
+        const unsigned hi = (unsigned)__double2hiint(v) & 0x7fffffffu;
+        least = min(least, (hi | min((unsigned)__double2loint(v), 1u)) - 1u);
+        add(v);
+    }
+    // entries that are not 0 far below the largest one: limbs of few bits, or 0
+    DD_DEV bool wide() const {
+        return least != ~0u && (least < (1u << 20) || (m >> 20) - (int)(least >> 20) > X_WIDE_BITS);
     }
     DD_DEV int get() const { return m ? m : (lo ? -1 - __clz((int)lo) : X_NONE); }
 };
@@ -70,15 +95,22 @@ struct SpinorX {
     int* e;
     long long stride;
     typedef double real;
+    // WIDE: mark a site with entries far below its largest (X_WIDE)
+    template <bool WIDE = false>
     DD_DEV void store(long long i, const Spinor<double>& s) const {
         XTop top;
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            top.add(s.c[k].x);
-            top.add(s.c[k].y);
+            if (WIDE) {
+                top.add_wide(s.c[k].x);
+                top.add_wide(s.c[k].y);
+            } else {
+                top.add(s.c[k].x);
+                top.add(s.c[k].y);
+            }
         }
         int E;
-        e[i] = x_exponent(top.get(), E);
+        e[i] = x_exponent(top.get(), E) + (WIDE && top.wide() ? X_WIDE : 0);
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
             const int2 a = x_split(x_from_double(s.c[k].x, E, 57)), b = x_split(x_from_double(s.c[k].y, E, 57));
@@ -104,12 +136,12 @@ struct LinkX {
     DD_HD const int* exps() const { return reinterpret_cast<const int*>(p + 72 * stride); }
 };
 // one link, entries u[0..8] (re, im): entry k at p[k * stride], exponent at *e
-DD_DEV void x_store_entries(int4* p, long long stride, int* e, const double* u) {
+DD_DEV void x_store_entries(int4* p, long long stride, int* e, const double* u, bool wide = false) {
     XTop top;
 #pragma unroll
-    for (int k = 0; k < 18; ++k) top.add(u[k]);
+    for (int k = 0; k < 18; ++k) top.add_wide(u[k]);
     int E;
-    *e = x_exponent(top.get(), E);
+    *e = x_exponent(top.get(), E) + (wide && top.wide() ? X_WIDE : 0);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         const int2 x = x_split(x_from_double(u[2 * k], E, 59)), y = x_split(x_from_double(u[2 * k + 1], E, 59));
@@ -117,9 +149,9 @@ DD_DEV void x_store_entries(int4* p, long long stride, int* e, const double* u) 
     }
 }
 // ... of a field in the layout of LinkX
-DD_DEV void x_store_link(int4* p, long long stride, int par, int a, long long h, const double* u) {
+DD_DEV void x_store_link(int4* p, long long stride, int par, int a, long long h, const double* u, bool wide) {
     x_store_entries(p + (long long)(par * 4 + a) * 9 * stride + h, stride,
-                    reinterpret_cast<int*>(p + 72 * stride) + (long long)(par * 4 + a) * stride + h, u);
+                    reinterpret_cast<int*>(p + 72 * stride) + (long long)(par * 4 + a) * stride + h, u, wide);
 }
 
 // ------------------------------------------------------------ one hop
@@ -271,25 +303,73 @@ DD_DEV void x_axis(int a, bool g5, bool okf, int sf, const int4* src, long long 
         }
     }
 }
+// high word of |v| (of -v - 1 for a negative one)
+DD_DEV int x_mag_hi(long long v) {
+    const int h = (int)(v >> 32);
+    return h ^ (h >> 31);
+}
 // spin q of site i from the four axes: the sums of the hops' upper spins, and
 // what they give to the lower ones, - i sigma_a (forward - backward), time:
-// + the difference
-DD_DEV void x_gather(const long long (*part)[24][X_PAD], int i, int q, xacc* v) {
+// + the difference.  MAG: mag[c] the OR of the high words of the numbers that
+// entry c is made of.
+template <bool MAG>
+DD_DEV void x_gather(const long long (*part)[24][X_PAD], int i, int q, xacc* v, int* mag) {
     const int r = q & 1;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const int own = 2 * (3 * r + c), other = 2 * (3 * (1 - r) + c);
         if (q < 2) {
-            v[c].x = part[0][own][i] + part[1][own][i] + part[2][own][i] + part[3][own][i];
-            v[c].y = part[0][own + 1][i] + part[1][own + 1][i] + part[2][own + 1][i] + part[3][own + 1][i];
+            xacc p[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) p[a] = xacc{part[a][own][i], part[a][own + 1][i]};
+            v[c].x = p[0].x + p[1].x + p[2].x + p[3].x;
+            v[c].y = p[0].y + p[1].y + p[2].y + p[3].y;
+            if (MAG) {
+                mag[c] = 0;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) mag[c] |= x_mag_hi(p[a].x) | x_mag_hi(p[a].y);
+            }
         } else {
             const long long (*d0)[X_PAD] = part[0] + 12, (*d1)[X_PAD] = part[1] + 12, (*d2)[X_PAD] = part[2] + 12,
                             (*d3)[X_PAD] = part[3] + 12;
             const long long m = r ? -1 : 0;
-            v[c].x = d0[other + 1][i] + x_neg_if(d1[other][i], ~m) + x_neg_if(d2[own + 1][i], m) + d3[own][i];
-            v[c].y = -d0[other][i] + x_neg_if(d1[other + 1][i], ~m) + x_neg_if(d2[own][i], ~m) + d3[own + 1][i];
+            const xacc p0{d0[other][i], d0[other + 1][i]}, p1{d1[other][i], d1[other + 1][i]},
+                p2{d2[own][i], d2[own + 1][i]}, p3{d3[own][i], d3[own + 1][i]};
+            v[c].x = p0.y + x_neg_if(p1.x, ~m) + x_neg_if(p2.y, m) + p3.x;
+            v[c].y = -p0.x + x_neg_if(p1.y, ~m) + x_neg_if(p2.x, ~m) + p3.y;
+            if (MAG)
+                mag[c] = x_mag_hi(p0.x) | x_mag_hi(p0.y) | x_mag_hi(p1.x) | x_mag_hi(p1.y) | x_mag_hi(p2.x) |
+                         x_mag_hi(p2.y) | x_mag_hi(p3.x) | x_mag_hi(p3.y);
         }
     }
+}
+// Entries (a bit each) that the common exponent of their neighbourhood leaves
+// few bits for: those whose hops are all below 2^53 in units of 2^-56 of the
+// largest product, 2^-3 of it (X_SMALL: the high word).  Above the line the
+// integer form's error is within a few units of 2^-53 of the entry's own
+// hops, as FP64's is.  The sums (upper spins) or differences (lower spins) of
+// forward and backward hops that x_gather reads may be small where the hops
+// are not, so this looks at both; rarely called (random fields: 4e-4 of the
+// sites).  Hops that are all 0 are just that, unless a number near them is so
+// far below the others that its limbs are 0 (wide).
+constexpr int X_SMALL = 1 << 21;
+static __device__ __noinline__ int x_small(const long long (*part)[24][X_PAD], int i, int q, const int* mag, bool wide) {
+    const int r = q & 1;
+    int found = 0;
+    for (int c = 0; c < 3; ++c) {
+        if (mag[c] >= X_SMALL) continue;
+        int m = 0;
+        long long any = 0;
+        for (int a = 0; a < 4; ++a) {
+            const int k = 2 * (3 * (q > 1 && a < 2 ? 1 - r : r) + c);
+            for (int e = 0; e < 2; ++e) {
+                m |= x_mag_hi(part[a][k + e][i]) | x_mag_hi(part[a][k + e + 12][i]);
+                any |= part[a][k + e][i] | part[a][k + e + 12][i];
+            }
+        }
+        if (m < X_SMALL && (any || wide)) found |= 1 << c;
+    }
+    return found;
 }
 
 // magnitude bits of a set of sums: OR of these, then x_bits

@@ -239,3 +239,73 @@ def test_subnormal_numbers(api, kind):
     top = np.abs(ref).max((1, 2))
     assert np.abs(ref).max() > 0 and np.all(err <= np.sqrt(2) * (2.0 ** -53 * top + kappa * 2.0 ** -54 * mag
                                                                + np.longdouble(2.0) ** -1075 * 2))
+
+
+def own_terms(U, psi, lat):
+    """Per component of H psi the sum of |link entry| (|upper| + |lower|) over its own products."""
+    out, U, psi = np.zeros(psi.shape, dtype=np.longdouble), np.abs(U.astype(LD)), np.abs(psi.astype(LD))
+    for a in range(4):
+        pair = np.abs(GAMMA_AXIS[a]).argmax(1)
+        for y, links in ((lat.fwd[:, a], U[:, a]), (lat.bwd[:, a], np.swapaxes(U[lat.bwd[:, a], a], 1, 2))):
+            w = psi[y]
+            out += np.einsum("sij,skj->ski", links, w + w[:, pair])
+    return out
+
+
+@pytest.mark.parametrize("op", ["D", "INTER", "HEO", "DTILDE"])
+@pytest.mark.parametrize("kind", ["colour 1e-6", "colour 1e-18", "colour 1e-200", "spin 1e-9", "links", "one spin",
+                                  "spread", "plain"])
+def test_each_component_keeps_the_accuracy_of_fp64(api, op, kind):
+    """Entries far below the largest of their site, where no link mixes them
+    with larger ones.  Per component, relative to its own terms: FP64 has one
+    rounding for the projection, six for a colour product and eight for the
+    hops; the integer form up to 8.5 units of 2^-56 of the largest product a
+    hop (3 dropped, 1 rounded, 4.5 of the inputs), eight hops, for a component
+    whose largest hop is above 2^-3 of it: 68 x 2^-53."""
+    dims, block, kappa = (4, 6, 4, 8), (2, 3, 2, 4), 0.125
+    lat = geometry.Lattice(dims, block)
+    parity = geometry_parity(lat)
+    rng = np.random.default_rng(3)
+    U, psi = synthetic.random_gauge(dims, 0.4, 2), synthetic.random_spinor(dims, 5)
+    if kind.startswith("colour") or kind == "spin 1e-9":
+        if kind.startswith("colour"):
+            U = np.where(np.eye(3, dtype=bool), np.exp(2j * np.pi * rng.random(U.shape[:2]))[..., None, None], 0)
+            psi[:, :, 1] *= float(kind.split()[1])
+        else:
+            psi[:, 2:] *= 1e-9
+    elif kind == "links":
+        U = U * np.exp(rng.uniform(-40, 0, U.shape)) + np.eye(3)
+        psi[:, :, 2] *= 1e-25
+    elif kind == "one spin":
+        psi[:, [0, 2, 3]] = 0
+    elif kind == "spread":
+        psi = psi * np.exp(12 * rng.standard_normal(psi.shape))
+    sites = {"HEO": parity == 1, "DTILDE": parity == 0}.get(op, parity >= 0)
+    psi[~sites] = 0
+    h = api.dd_init(dims, block, kappa)
+    out = dev(np.zeros_like(psi[sites]))
+    api.dd_apply_D(h, out, dev(psi[sites]), dev(U), getattr(api, "DD_OP_" + op), api.DD_PREC_F64, 1)
+    got, k = host(out), LD(kappa)
+    if op == "INTER":
+        # only the hops that cross block faces: those of the lattice without the ones inside
+        inside = api.dd_init(dims, block, kappa)
+        blk = dev(np.zeros_like(psi))
+        api.dd_apply_D_block(inside, blk, dev(psi), dev(U), 3, api.DD_PREC_F64, 1)
+        got = got + host(blk)
+        ref, terms = psi - k * hop_extended(U, psi, lat)[0], np.abs(psi) + kappa * own_terms(U, psi, lat)
+    else:
+        hop, terms = hop_extended(U, psi, lat)[0], own_terms(U, psi, lat)
+        if op == "D":
+            ref, terms = psi - k * hop, np.abs(psi) + kappa * terms
+        elif op == "HEO":
+            ref, terms = hop[parity == 0], terms[parity == 0]
+        else:
+            hop[parity == 0] = 0
+            terms[parity == 0] = 0
+            ref = (psi - k * k * hop_extended(U, hop, lat)[0])[parity == 0]
+            terms = (np.abs(psi) + 2 * kappa * kappa * own_terms(U, terms, lat))[parity == 0]
+    err = np.abs(got.astype(LD) - ref).astype(np.longdouble)
+    bound = np.sqrt(2) * (68 + 2) * np.longdouble(2.0) ** -53 * terms
+    print(op, kind, "largest error in units of 2^-53 of a component's own terms:",
+          float((err[terms > 0] / terms[terms > 0]).max() * 2.0 ** 53))
+    assert np.all(err <= bound), float((err[terms > 0] / terms[terms > 0]).max() * 2.0 ** 53)
