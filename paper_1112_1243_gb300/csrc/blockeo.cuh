@@ -445,59 +445,21 @@ DD_DEV void eo_store_limbs(EoX x, int stride, int idx, int sp, bool ok, const cp
 
 // ------------------------------------------------------------ the source
 // (H_b[U_src] - H_b[U_sol]) eta at one site: only hops whose links differ
-// contribute (the proposal changes active links only).  The difference of
-// the 59-bit links is exact and is brought back to 59 bits, so it keeps the
-// relative accuracy of the FP64 difference.  One lane a site.
-struct XDiff {  // difference of two links: entries (u1 << l1) - (u2 << l2) at a common scale, then << up
-    int e;      // exponent of the difference
-    int r1, r2, up;
-    bool any;
-};
-DD_DEV long long x_join(int h, int l) { return ((long long)h << 30) + l; }
-DD_DEV int4 x_diff_entry(const int4* p1, const int4* p2, long long k, const XDiff& d) {
-    const int4 a = p1[k], b = p2[k];
-    const long long x = ((x_join(a.x, a.y) >> d.r1) - (x_join(b.x, b.y) >> d.r2)) << d.up;
-    const long long y = ((x_join(a.z, a.w) >> d.r1) - (x_join(b.z, b.w) >> d.r2)) << d.up;
-    const int2 s = x_split(x), t = x_split(y);
-    return make_int4(s.x, s.y, t.x, t.y);
-}
-DD_DEV XDiff x_diff(const int4* p1, int e1, const int4* p2, int e2, long long cl) {
-    XDiff d;
-    const int e = max(e1, e2);
-    d.r1 = min(e - e1, 62);
-    d.r2 = min(e - e2, 62);
-    d.up = 0;
-    unsigned long long any = 0;
-    for (int k = 0; k < 9; ++k) {
-        const int4 a = p1[k * cl], b = p2[k * cl];
-        xacc v;
-        v.x = (x_join(a.x, a.y) >> d.r1) - (x_join(b.x, b.y) >> d.r2);
-        v.y = (x_join(a.z, a.w) >> d.r1) - (x_join(b.z, b.w) >> d.r2);
-        any |= x_mag(v);
-        any |= (unsigned long long)((v.x | v.y) < 0);  // -1 has no magnitude bits
-    }
-    d.any = any != 0 || e >= X_BAD_MIN;
-    // 59 bits: the difference of two 59-bit numbers may have 60
-    const int z = __clzll((long long)(any | 1ull));  // leading zeros of the largest magnitude
-    const int up = z - 5;                            // brings the leading bit to bit 58
-    if (up >= 0) {
-        d.up = up;
-        d.e = e - up;
-    } else {  // 60 bits: halve both
-        d.r1 += 1;
-        d.r2 += 1;
-        d.e = e + 1;
-    }
-    return d;
-}
-
+// contribute (the proposal changes active links only).  The difference of two
+// links is taken in FP64 from the canonical fields and then put into limbs of
+// its own scale: for a small rotation it lies far below the links, and limbs
+// of the links (59 bits of the largest entry) would have few bits of it.  One
+// lane a site.
 struct EoSource {
-    const int4 *l1, *l2;  // links of the block in the two fields, [a][9][nb]
-    const int *e1, *e2;   // their exponents, [a][nb]
-    const uint8_t* active;  // [V * 4]
+    const double2 *u1, *u2;  // the two fields, canonical
+    const uint8_t* active;   // [V * 4]
     Geo g;
     int org[4];
 };
+DD_DEV double2 link_diff(const EoSource& Q, long long k) {
+    const double2 a = Q.u1[k], b = Q.u2[k];
+    return make_double2(a.x - b.x, a.y - b.y);
+}
 __device__ __noinline__ void eo_source(const EoCtx c, const EoSource& Q, bool ok, int par, const EoSite& s, EoX eta,
                                        cpx<double>* b) {
     xacc acc[12];
@@ -507,52 +469,55 @@ __device__ __noinline__ void eo_source(const EoCtx c, const EoSource& Q, bool ok
 #pragma unroll
     for (int a = 0; a < 4; ++a) x[a] = Q.org[a] + s.l[a];
     const int site = ok ? canon_index(Q.g, x) : 0;
-    auto hop_at = [&](int d, int& y, int& lk) {  // eta index of the neighbour, index of the link
+    auto hop_at = [&](int d, int& y, long long& lk) {  // eta index of the neighbour, first entry of the link
         const int a = d >> 1;
         const int la = a == 0 ? s.l[0] : a == 1 ? s.l[1] : a == 2 ? s.l[2] : s.l[3];
         if ((d & 1) ? la == 0 : la == c.bd[a] - 1) return false;
-        if (!Q.active[(long long)((d & 1) ? site - Q.g.st[a] : site) * 4 + a]) return false;
+        const long long l = (long long)((d & 1) ? site - Q.g.st[a] : site) * 4 + a;
+        if (!Q.active[l]) return false;
         y = eo_full(c, 1 - par, ((d & 1) ? s.j - c.st[a] : s.j + c.st[a]) >> c.sh);
-        lk = (d & 1) ? y : eo_full(c, par, s.idx);
+        lk = l * 9;
         return true;
     };
     int eout = 2 * X_ZERO;
-    unsigned use = 0;
+    int de[8];  // exponents of the differences, X_ZERO: no hop
 #pragma unroll 1
     for (int d = 0; d < 8; ++d) {
-        int y, lk;
+        int y;
+        long long lk;
+        de[d] = X_ZERO;
         if (!ok || !hop_at(d, y, lk)) continue;
-        const long long o = (long long)(d >> 1) * 9 * c.nb + lk;
-        const int oe = (d >> 1) * c.nb + lk;
-        const XDiff D = x_diff(Q.l1 + o, Q.e1[oe], Q.l2 + o, Q.e2[oe], c.nb);
-        if (!D.any) continue;
-        use |= 1u << d;
-        eout = max(eout, D.e + eta.e[y]);
+        XTop top;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const double2 v = link_diff(Q, lk + k);
+            top.add(v.x);
+            top.add(v.y);
+        }
+        int E;
+        de[d] = x_exponent(top.get(), E);
+        if (de[d] != X_ZERO) eout = max(eout, de[d] + eta.e[y]);
     }
+    const bool use = eout != 2 * X_ZERO;
 #pragma unroll 1
     for (int d = 0; d < 8; ++d) {
-        int y, lk;
-        if (!((use >> d) & 1) || !hop_at(d, y, lk)) continue;
+        int y;
+        long long lk;
+        if (de[d] == X_ZERO || !hop_at(d, y, lk)) continue;
         const int a = d >> 1;
         const bool fwd = !(d & 1);
-        const long long o = (long long)a * 9 * c.nb + lk;
-        const int oe = a * c.nb + lk;
-        const XDiff D = x_diff(Q.l1 + o, Q.e1[oe], Q.l2 + o, Q.e2[oe], c.nb);
         xlimb h[6];
         x_project(a, !fwd, eta.p, c.nb, (unsigned)y * 16u, h);
-        const int shift = min(eout - (D.e + eta.e[y]), 62);
-        const int4 *p1 = Q.l1 + o, *p2 = Q.l2 + o;
+        const int shift = min(eout - (de[d] + eta.e[y]), 62), E = de[d] + 1022;
         xacc v[6];
         // one body for U h and U^dag h: the adjoint's entries, conjugated
         x_multiply<true>(
             shift, h,
             [&](int k) {
-                int4 u = x_diff_entry(p1, p2, (long long)(fwd ? k : 3 * (k % 3) + k / 3) * c.nb, D);
-                if (!fwd) {
-                    u.z = -u.z;
-                    u.w = -u.w;
-                }
-                return u;
+                const double2 v = link_diff(Q, lk + (fwd ? k : 3 * (k % 3) + k / 3));
+                const int2 re = x_split(x_from_double(v.x, E, 59));
+                const int2 im = x_split(x_from_double(fwd ? v.y : -v.y, E, 59));
+                return make_int4(re.x, re.y, im.x, im.y);
             },
             [&](int k, xacc w) { v[k] = w; });
         // upper spins, and the lower spins that belong to them (xfix.cuh)
@@ -664,10 +629,8 @@ __global__ void __launch_bounds__(256, 2) block_eo_kernel(BlockArgs A) {
         int colour;
         const int id = block_id_at(L.g, it.block_pos, &colour);
         EoSource Q;
-        Q.l1 = L.ddx + (long long)it.f_src * L.ddx_fs + lo;
-        Q.e1 = reinterpret_cast<const int*>(L.ddx + (long long)it.f_src * L.ddx_fs + 36LL * L.g.V) + leo;
-        Q.l2 = lx;
-        Q.e2 = le;
+        Q.u1 = reinterpret_cast<const double2*>(L.canon + (long long)it.f_src * L.canon_fs);
+        Q.u2 = reinterpret_cast<const double2*>(L.canon + (long long)it.f_sol * L.canon_fs);
         Q.active = L.active;
         Q.g = L.g;
         block_origin(L.g, id, Q.org);

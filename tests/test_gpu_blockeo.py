@@ -65,3 +65,38 @@ def test_block_shapes(api, dims, block, tpb):
     # nothing proposed: exactly zero
     got = host(api.dd_block_ratios_range(h, dev(U), dev(U), 0, lat.nblocks, n, 9, 3))
     assert np.all(got == 0)
+
+
+def test_source_of_small_rotations(api):
+    """Links that differ only in entries far below their largest one: diagonal
+    links with off-diagonal entries near 2^-26, of which the proposal changes
+    2^-10 parts.  The reference takes the difference of the links in FP64 and
+    scales it up before the operator adds it to the noise; what is left is
+    that of the solve (reference(), relative to |b|)."""
+    dims, block = (8, 4, 4, 8), (4, 2, 2, 4)
+    lat = geometry.Lattice(dims, block)
+    rng = np.random.default_rng(3)
+    V = int(np.prod(dims))
+    U = np.zeros((V, 4, 3, 3), dtype=np.complex128)
+    ph = rng.uniform(0, 2 * np.pi, (V, 4, 3))
+    ph[..., 2] = -ph[..., 0] - ph[..., 1]
+    for k in range(3):
+        U[..., k, k] = np.exp(1j * ph[..., k])
+    off = rng.standard_normal((2, V, 4, 3, 3))
+    off = (off[0] + 1j * off[1]) * (1 - np.eye(3)) * 2.0 ** -26
+    change = 1 + 2.0 ** -10 * rng.standard_normal((V, 4, 3, 3))
+    Up = U + off * np.where(lat.active[..., None, None], change, 1.0)
+    U = U + off
+    diff = (U - Up) * 2.0 ** 40  # exact differences, scaled to about 1
+    assert 0 < np.abs(U - Up).max() < 2.0 ** -30
+    eta = estimator.block_noise(lat, 0, 9, 3)
+    b = 2.0 ** -40 * (estimator.Pieces(diff, lat, KAPPA).dirichlet(eta) - eta)
+    d = estimator.Pieces(Up, lat, KAPPA).dirichlet_solve(b)
+    per = lambda v: np.bincount(lat.block_id, weights=v, minlength=lat.nblocks)
+    sq = lambda v: np.sqrt(per(np.sum(np.abs(v) ** 2, axis=(1, 2))))
+    ref = per(-(2 * np.sum(np.conj(eta) * d, axis=(1, 2)).real + np.sum(np.abs(d) ** 2, axis=(1, 2))))
+    tol = 2 * (sq(eta) + sq(d)) / (1 - 8 * KAPPA) * 1e-12 * sq(b)
+    h = api.dd_init(dims, block, KAPPA, max_rhs=1)
+    got = host(api.dd_block_ratios_range(h, dev(U), dev(Up), 0, lat.nblocks, 1, 9, 3))
+    assert np.all(np.abs(got - ref) <= tol)
+    assert api.dd_status(h)[0] == 0
