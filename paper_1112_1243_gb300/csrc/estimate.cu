@@ -46,24 +46,26 @@ DD_DEV void dd_coords(const Geo& g, const BlockCtx& c, long long q, int x[4], in
 // colour of the enclosing block of extents ob
 DD_DEV int outer_colour(int4 ob, const int x[4]) { return (x[0] / ob.x + x[1] / ob.y + x[2] / ob.z + x[3] / ob.w) & 1; }
 
-// eta on the black sites (purpose / sub), in FP64 and in limbs; the white
-// sites are not written (no kernel reads them).  With enclosing blocks (ob.x
-// > 0) 0 outside the enclosing blocks whose colour is in outer_mask.  Threads
-// in block order: the black sites come first, so no warp holds white ones.
+// eta on the black sites (purpose / sub), in FP64 and in limbs.  n: sites to
+// write, V / 2, or V where the hops visit the sites of both colours (no site
+// lists: odd extents along axis 0) and read the white ones, which are 0, for
+// results that are then dropped.  With enclosing blocks (ob.x > 0) 0 outside
+// the enclosing blocks whose colour is in outer_mask.  Threads in block order:
+// the black sites come first.
 __global__ void __launch_bounds__(128) noise_black_kernel(Geo g, BlockCtx c, double2* eta, SpinorX ee, SpinorX eo,
                                                           long long parity_stride, int purpose, uint64_t seed,
                                                           uint64_t ctr0, const unsigned long long* ctr_off, int4 ob,
-                                                          int outer_mask) {
+                                                          int outer_mask, long long n) {
     const uint64_t ctr = stream_ctr(ctr0, ctr_off);
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int i = blockIdx.y;
-    if (q >= g.V / 2) return;
+    if (q >= n) return;
     int x[4], col;
     dd_coords(g, c, q, x, &col);
     const uint32_t s = (uint32_t)canon_index(g, x);
     const int par = (x[0] + x[1] + x[2] + x[3]) & 1;
     Spinor<double> e;
-    if (ob.x == 0 || ((outer_mask >> outer_colour(ob, x)) & 1)) {
+    if (col == 0 && (ob.x == 0 || ((outer_mask >> outer_colour(ob, x)) & 1))) {
         for (int k = 0; k < 12; ++k) e.c[k] = gaussian(s * 12u + k, (uint32_t)purpose, (uint32_t)i, seed, ctr);
     } else {
         zero(e);
@@ -445,8 +447,9 @@ static int schur_source(dd_handle* h, int n, int fs, int purpose, uint64_t seed,
         return DD_OK;
     };
     // 1. eta on the black sites
-    DD_KLAUNCH(h, noise_black_kernel<<<dim3(grid_for(g.V / 2, 128), n), 128, 0, h->stream>>>(
-                      g, c, eta, ex[0], ex[1], ps, purpose, seed, ctr, h->d_ctr_off, ob, outer_mask));
+    const long long nnoise = h->d_colour_sites[0] ? g.V / 2 : g.V;
+    DD_KLAUNCH(h, noise_black_kernel<<<dim3(grid_for(nnoise, 128), n), 128, 0, h->stream>>>(
+                      g, c, eta, ex[0], ex[1], ps, purpose, seed, ctr, h->d_ctr_off, ob, outer_mask, nnoise));
     // 2. v' = B' E'^{-1} C' eta
     inter(1, 1, ex, b);
     int rc = solve(1, 1);

@@ -199,3 +199,29 @@ def test_global_accept(api):
         assert bool(host(acc)[0]) == ref_acc
         assert abs(float(host(margin)[0]) - (float(ln.sum()) - lu)) < 1e-15
         assert np.array_equal(host(Ud), U1 if ref_acc else U0)
+
+
+@pytest.mark.parametrize("dims,block", [((6, 4, 4, 4), (3, 2, 2, 2)), ((6, 6, 6, 6), (3, 3, 3, 3))])
+def test_odd_extents_do_not_read_the_workspace_as_found(api, dims, block):
+    """Odd extents along axis 0 have no site lists of a block colour: the hops
+    visit all sites and drop what they find on the wrong ones.  The estimate is
+    the same whatever the workspace held before."""
+    import torch
+    n = 2
+    U = dev(synthetic.random_gauge(dims, 0.3, 4))
+    lat = geometry.Lattice(dims, block)
+    Up = U.clone()
+    api.dd_gauge_update(api.dd_init(dims, block, 0.12), Up, 1 if lat.active_mode == "intra" else 3, 5.3, 1, 0, 21, 4)
+    size = api.dd_init(dims, block, 0.12, max_rhs=n).workspace.numel()
+    got = []
+    for byte in (0, 0x7f, 0xff):
+        found = torch.full((size,), byte, dtype=torch.uint8, device="cuda")
+        torch.cuda.synchronize()
+        where = found.data_ptr()
+        del found
+        h = api.dd_init(dims, block, 0.12, max_rhs=n)  # the allocator hands the same memory out again
+        assert h.workspace.data_ptr() == where
+        got.append(host(api.dd_det_ratio_estimate(h, U, Up, n, 9, 3)))
+        assert api.dd_status(h)[0] == 0
+        del h
+    assert np.all(np.isfinite(got[0])) and np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
