@@ -581,7 +581,8 @@ int dd_graph_destroy(dd_graph_t graph);
 
 /* Autotuner of the launch shapes (no counterpart in the paper).
  * what: DD_TUNE_HOP (thread-block size x sites per thread of the even-odd
- * hop kernels, FP16/FP32 storage and FP64 separately), DD_TUNE_BLOCK
+ * hop kernels in FP16/FP32 storage, and thread-block size of the
+ * double-float hop where outer_prec is DD_PREC_DF64), DD_TUNE_BLOCK
  * (thread-block size and thread blocks per SM of the persistent block
  * solver, at most 4 per SM, and whether the stochastic block filter runs
  * faster as that persistent launch or as batched whole-lattice Dirichlet
@@ -592,7 +593,7 @@ int dd_graph_destroy(dd_graph_t graph);
  * pass over the fields (U_old, U_new) (device gauge fields; required for
  * DD_TUNE_BLOCK, may be NULL otherwise).  The fastest shape is kept by the
  * handle and used by every later launch.  The result is cached per process
- * and per (device, lattice, blocks, inner precision, max_rhs); when the
+ * and per (device, lattice, blocks, precisions, max_rhs); when the
  * environment variable DD_TUNE_CACHE names a file, tuned shapes are
  * appended to it and read back by later processes.  report (host, may be
  * NULL) receives the chosen shapes and the average launch times (ms) of the
@@ -600,8 +601,10 @@ int dd_graph_destroy(dd_graph_t graph);
  * kernels and synchronises the stream; not allowed inside a capture.
  * dd_set_tuning sets the shapes directly (threads 64 or 128 and 1 or 2
  * sites per thread for the FP16/FP32 hops; 64 or 128 threads and 1 site per
- * thread for the FP64 hops; 64, 128 or 256 threads and 1..4 blocks per SM
- * for the block solver; filter_masked 0 = persistent block-filter launch,
+ * thread for the double-float hop (outer_prec DD_PREC_DF64; the FP64 hop has
+ * one shape, 128 threads a tile of 32 sites); 64, 128 or 256 threads and 1..4
+ * blocks per SM for the block solver, 64 taken as 128 unless block_prec is
+ * DD_PREC_F64; filter_masked 0 = persistent block-filter launch,
  * 1 = whole-lattice Dirichlet solves).
  * Changing the block-solver shape changes dd_block_filter_batch_workspace. */
 #define DD_TUNE_HOP 1

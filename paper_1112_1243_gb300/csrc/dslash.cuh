@@ -583,8 +583,8 @@ inline void launch_hop(const HopArgs<SIn, SX, SOut, LK>& A, int nrhs, dd_handle*
     // tile shape from the handle's tuning (threads x sites per thread >= 32,
     // which keeps the grid within the reduction partials)
     constexpr bool f64 = std::is_same<SIn, SpinorX>::value;
-    int tpb = std::min(f64 ? h->tune.hop64_tpb : h->tune.hop_tpb, 128);  // the kernels' launch bound
-    if (f64) tpb = 128;  // four warps (hop_x_kernel)
+    // four warps (hop_x_kernel), or the tuned shape within the kernels' launch bound
+    const int tpb = f64 ? 128 : std::min(h->tune.hop_tpb, 128);
     const int spt = (!f64 && h->tune.hop_spt == 2) ? 2 : 1;
     dim3 grid(grid_for(B.S.n, f64 ? X_TILE : (long long)tpb * spt), nrhs, f64 && A.both ? 2 : 1);
     constexpr int kind0 = hop_kind<SIn, SOut>();

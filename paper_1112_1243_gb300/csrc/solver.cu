@@ -1018,6 +1018,25 @@ int defect_correction_df(dd_handle* h, int nrhs, int field0, int step, Inner& cg
 
 }  // namespace
 
+void launch_tune_hop_df(dd_handle* h, int nrhs) {
+    SolverVecs& v = h->vecs[0];
+    const long long Vh = h->g.Vh;
+    DFHopArgs A;
+    A.g = h->g;
+    A.p = 0;
+    A.in = SpinorDF{reinterpret_cast<float4*>(v.x64), Vh};
+    A.xin = A.bin = SpinorDF{reinterpret_cast<float4*>(v.q64), Vh};
+    A.out = SpinorDF{reinterpret_cast<float4*>(v.p64), Vh};
+    A.lk = LinkDF{h->fields[0].eodf, Vh};
+    A.lk_rhs_stride = 0;
+    A.c = df_from_double(h->prm.kappa);
+    A.st = nullptr;
+    A.sig_exp = nullptr;
+    A.red.op = FIN_NONE;
+    A.S = SiteSet{nullptr, Vh};
+    hopdf<0, 1>(h, nrhs, A);
+}
+
 template <class B>
 static void fill_bicg(dd_handle* h, B& bi, long long Vh, CGState* inner, CGState* outer, int nrhs) {
     bi.nrhs = nrhs;

@@ -23,3 +23,8 @@
 // solution is left as it was).
 int solve_packed(dd_handle* h, int nrhs, int field0, int field_step, int prec, double tol, int maxit, int* iters,
                  double* relres, int mask = 0, int colour = -1);
+
+// One double-float hop over the whole lattice between the FP64 vectors of the
+// solver (x64, q64 -> p64), for the timing of its launch shapes; the handle
+// has outer_prec DD_PREC_DF64.
+void launch_tune_hop_df(dd_handle* h, int nrhs);

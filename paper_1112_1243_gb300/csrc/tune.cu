@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "dslash.cuh"
+#include "solver.h"
 
 int tune_block_filter(dd_handle* h, const double* U_old, const double* U_new, int reps, float* ms);
 int tune_block_filter_masked(dd_handle* h, const double* U_old, const double* U_new, int reps, float* ms);
@@ -34,6 +35,9 @@ std::string tune_key(dd_handle* h) {
                   h->g.L[0], h->g.L[1], h->g.L[2], h->g.L[3], h->g.b[0], h->g.b[1], h->g.b[2], h->g.b[3],
                   h->prm.inner_prec, h->prm.max_rhs);
     std::string k(buf);
+    // other candidates than on the default precisions
+    if (h->prm.outer_prec == DD_PREC_DF64) k += "|df";
+    if (h->prm.block_prec == DD_PREC_F64) k += "|b64";
     for (char& c : k)
         if (c == ' ') c = '_';
     return k;
@@ -101,8 +105,11 @@ struct Shape {
 // thread-block size x sites per thread >= 64 keeps every grid within the
 // reduction partials planned for 64-site tiles
 const Shape kHopShapes[] = {{128, 1}, {64, 1}, {128, 2}, {64, 2}};
+// of the double-float hop; the FP64 hop has one shape, four warps a tile of 32 sites
 const Shape kHop64Shapes[] = {{128, 1}, {64, 1}};
 const Shape kBlockShapes[] = {{256, 2}, {256, 1}, {128, 2}, {128, 4}, {64, 4}};
+// smallest thread block of the mixed block solver: groups of four warps (eo_xhop)
+constexpr int kBlockMixedMin = 128;
 
 }  // namespace
 
@@ -196,12 +203,21 @@ extern "C" int dd_autotune(dd_t h, int what, const void* U_old, const void* U_ne
             B.st = nullptr;
             B.red.op = FIN_NONE;
             B.sites = nullptr;
+            const bool df = h->prm.outer_prec == DD_PREC_DF64;
+            if (df) {
+                DD_CUDA(h, cudaMemsetAsync(v.x64, 0, sizeof(double2) * 12 * Vh * R, h->stream));
+                DD_CUDA(h, cudaMemsetAsync(v.q64, 0, sizeof(double2) * 12 * Vh * R, h->stream));
+            }
             best = 1e30f;
             for (const Shape& s : kHop64Shapes) {
+                if (!df && s.tpb != 128) continue;
                 h->tune.hop64_tpb = s.tpb;
                 h->tune.hop64_spt = s.spt;
                 float ms = time_launches(h, std::max(2, reps / 4), [&] {
-                    launch_hop<double, SpinorX, SpinorF64, SpinorF64, LinkX, 0>(B, R, h);
+                    if (df)
+                        launch_tune_hop_df(h, R);
+                    else
+                        launch_hop<double, SpinorX, SpinorF64, SpinorF64, LinkX, 0>(B, R, h);
                 });
                 if (ms < 0) return dd_fail(h, DD_ERR_CUDA, "dd_autotune: FP64 hop timing failed");
                 if (s.tpb == 128 && s.spt == 1) r.hop64_default_ms = ms;
@@ -219,6 +235,7 @@ extern "C" int dd_autotune(dd_t h, int what, const void* U_old, const void* U_ne
             float best = 1e30f;
             TuneConfig keep = h->tune;
             for (const Shape& s : kBlockShapes) {
+                if (h->prm.block_prec != DD_PREC_F64 && s.tpb < kBlockMixedMin) continue;
                 h->tune.block_tpb = s.tpb;
                 h->tune.block_ctas_per_sm = s.spt;
                 float ms = -1.f;

@@ -114,3 +114,33 @@ def test_instrumentation_counts_and_peaks():
     assert cnt2 >= 2                                   # FP64 residual hops of the defect correction
     api.dd_kernel_timer(h, 1, 0, 1)                    # reset
     assert api.dd_solver_stats(h, 0)["solves"] == 0
+
+
+def test_autotune_times_shapes_that_differ(api):
+    """The FP64 hop and the mixed block solver have no 64-thread form (the
+    choice would be noise): the tuner reports the shapes that run.  With a
+    double-float residual the hop64 shape is that hop's, and the solve meets
+    its target with either."""
+    dims, block, kappa = (8, 8, 8, 8), (4, 4, 4, 4), 0.13
+    lat = geometry.Lattice(dims, block)
+    U = synthetic.random_gauge(dims, 0.3, 2)
+    Ud = dev(U)
+    Up = Ud.clone()
+    h = api.dd_init(dims, block, kappa, max_rhs=2)
+    api.dd_gauge_update(h, Up, 3, 5.3, 1, 0, 7, 0)
+    for _ in range(12):
+        rep = api.dd_autotune(h, api.DD_TUNE_HOP | api.DD_TUNE_BLOCK | api.DD_TUNE_NO_CACHE, Ud, Up, reps=2)
+        assert rep["hop64_tpb"] == 128 and rep["hop64_ms"] == rep["hop64_default_ms"] > 0
+        assert rep["block_tpb"] >= 128
+    h = api.dd_init(dims, block, kappa, max_rhs=2, outer_prec=api.DD_PREC_DF64)
+    rep = api.dd_autotune(h, api.DD_TUNE_HOP | api.DD_TUNE_NO_CACHE, None, None, reps=4)
+    assert rep["hop64_tpb"] in (64, 128) and 0 < rep["hop64_ms"] <= rep["hop64_default_ms"]
+    b = synthetic.random_spinor(dims, 12, nrhs=2)
+    for tpb in (64, 128):
+        api.dd_set_tuning(h, rep["hop_tpb"], rep["hop_spt"], tpb, 1, 256, 2)
+        x = dev(np.zeros_like(b))
+        api.dd_solve(h, x, dev(b), Ud, 2, api.DD_PREC_F16)
+        for r in range(2):
+            true = np.linalg.norm(b[r] - dirac.apply_D(U, host(x)[r], lat, kappa)) / np.linalg.norm(b[r])
+            assert true <= 1e-10 * 1.01
+    assert api.dd_status(h)[0] == 0
