@@ -203,23 +203,6 @@ DD_DEV void reconstruct_row2(Link<R>& u) {
     u.m[2][2] = conj(cmul(u.m[0][0], u.m[1][1]) - cmul(u.m[0][1], u.m[1][0]));
 }
 
-// FP64 link, all 9 entries: 9 chunks of double2 per direction.
-// Link (site i, direction a) chunk k at p[(a*9 + k) * stride + i].
-struct LinkF64 {
-    const double2* p;
-    long long stride;
-    static constexpr int chunks = 9;
-    template <class R>
-    DD_DEV void load(long long i, int a, Link<R>& u) const {
-        const double2* q = p + (long long)a * 9 * stride + i;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            double2 v = q[k * stride];
-            u.m[k / 3][k % 3] = mk<R>((R)v.x, (R)v.y);
-        }
-    }
-};
-
 // FP32 link, rows 0-1 stored (3 chunks of float4), row 2 rebuilt.
 struct LinkF32 {
     const float4* p;

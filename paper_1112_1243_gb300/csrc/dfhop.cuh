@@ -113,13 +113,6 @@ DD_DEV void cdf_mac(cdf& acc, cdf u, cdf h) {
     df_mac(acc.im, u.re, h.im);
     df_mac(acc.im, u.im, h.re);
 }
-// acc += conj(u) * h
-DD_DEV void cdf_macc(cdf& acc, cdf u, cdf h) {
-    df_mac(acc.re, u.re, h.re);
-    df_mac(acc.re, u.im, h.im);
-    df_mac(acc.im, u.re, h.im);
-    df_mac(acc.im, df_neg(u.im), h.re);
-}
 
 struct DFHopArgs {
     Geo g;

@@ -81,7 +81,8 @@ struct HopArgs {
     SOut out;                 // output (parity p)
     LK lk;                    // gauge field, both parities: [parity][dir][chunk][Vh]
     long long lk_rhs_stride;  // elements between the fields of consecutive rhs (0: shared)
-    double a, b;
+    double a = 1.0;           // the FP64 hops take 1
+    double b;
     int has_x;
     int g5in, g5out;
     int colour_mask;          // 3 = every site; else zero the output outside these block colours

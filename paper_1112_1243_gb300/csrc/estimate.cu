@@ -418,7 +418,6 @@ static int schur_source(dd_handle* h, int n, int fs, int purpose, uint64_t seed,
         A.xin = A.out = A.rhat = A.out2 = out[par];
         A.lk = LinkX{h->fields[f].eox, Vh};
         A.lk_rhs_stride = rs;
-        A.a = 1.0;
         A.b = -h->prm.kappa;
         A.has_x = A.g5in = A.g5out = 0;
         A.colour_mask = h->d_colour_sites[colour] ? 3 : 1 << colour;

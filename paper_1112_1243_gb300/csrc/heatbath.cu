@@ -7,8 +7,8 @@
 // SU(2)-proportional part k V; the new element is R = X V^dag, X drawn from
 // exp(alpha x0) dX (alpha = 2 beta k / 3) by the Kennedy-Pendleton sampler
 // (at most 64 tries), direction of (x1, x2, x3) uniform; U <- R U.
-// Over-relaxation: R = (V^dag)^2.  One launch per (colour, direction, site
-// parity) group: links of one direction and one site parity share no
+// Over-relaxation: R = (V^dag)^2.  One launch per (direction, site parity), both
+// block colours together: links of one direction and one site parity share no
 // plaquette, so a group is updated in parallel.
 #include <algorithm>
 #include <cmath>
@@ -19,9 +19,6 @@
 
 namespace {
 
-struct Q4 {
-    double a0, a1, a2, a3;
-};
 // 2x2 SU(2) matrix in the parametrisation [[a0 + i a3, a2 + i a1], [-a2 + i a1, a0 - i a3]]
 struct M2 {
     cpx<double> m[2][2];

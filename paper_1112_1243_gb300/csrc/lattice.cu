@@ -923,7 +923,6 @@ static int apply_canonical(dd_handle* h, void* out, const void* in, const void* 
     A.out = A.out2 = canonical(out);
     A.lk = LinkX{h->fields[0].eox, Vh};
     A.lk_rhs_stride = 0;
-    A.a = 1.0;
     A.b = -h->prm.kappa;
     A.has_x = !half && op != DD_OP_INTER;
     A.g5in = A.g5out = op == DD_OP_DDAG;

@@ -229,8 +229,7 @@ __global__ void copy_kernel(SiteSet S, SIn in, SOut out, const CGState* outer) {
     at_rhs(in, rhs).load(i, a);
     at_rhs(out, rhs).store(i, a);
 }
-// v = 0, and (pxe given) the exponents of its copy in limbs
-__global__ void zero64_kernel(SiteSet S, SpinorF64 v, int* pxe) {
+__global__ void zero64_kernel(SiteSet S, SpinorF64 v) {
     const int rhs = blockIdx.y;
     const long long ti = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (ti >= S.n) return;
@@ -238,7 +237,6 @@ __global__ void zero64_kernel(SiteSet S, SpinorF64 v, int* pxe) {
     Spinor<double> z;
     zero(z);
     at_rhs(v, rhs).store(i, z);
-    if (pxe) pxe[(long long)rhs * v.stride + i] = X_ZERO;
 }
 
 // ------------------------------------------------------------ CGNR runner
@@ -612,7 +610,6 @@ void hop64(dd_handle* h, SiteSet S, int nrhs, int par, SpinorX in, SpinorF64 xin
     A.out = out;
     A.lk = lk;
     A.lk_rhs_stride = lk_rs;
-    A.a = 1.0;
     A.b = b;
     A.has_x = hasx;
     A.g5in = 0;
@@ -926,7 +923,7 @@ int defect_correction_df(dd_handle* h, int nrhs, int field0, int step, Inner& cg
     A.c = df_from_double(kappa);
     hopdf<MASK, 1>(h, nrhs, A);
     DD_KLAUNCH(h, outer_arm_kernel<<<1, 64, 0, h->stream>>>(nrhs, outer, bb, tol));
-    DD_KLAUNCH(h, zero64_kernel<<<grid, 128, 0, h->stream>>>(S, SpinorF64{v.x64, Vh}, nullptr));
+    DD_KLAUNCH(h, zero64_kernel<<<grid, 128, 0, h->stream>>>(S, SpinorF64{v.x64, Vh}));
     DD_KLAUNCH(h, df_round_kernel<<<grid, 128, 0, h->stream>>>(S, btd, r32, sig, store_reduce(h, rr)));
     DD_KLAUNCH(h, outer_update_kernel<<<1, 64, 0, h->stream>>>(nrhs, outer, rr, h->d_status));
     if (cudaGetLastError() != cudaSuccess) return DD_ERR_CUDA;

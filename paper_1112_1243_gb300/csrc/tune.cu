@@ -195,7 +195,6 @@ extern "C" int dd_autotune(dd_t h, int what, const void* U_old, const void* U_ne
             B.out = SpinorF64{v.xe, Vh};
             B.lk = LinkX{h->fields[0].eox, Vh};
             B.lk_rhs_stride = 0;
-            B.a = 1.0;
             B.b = -k2;
             B.has_x = 1;
             B.g5in = B.g5out = 0;

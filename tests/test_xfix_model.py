@@ -74,3 +74,33 @@ def test_colour_product_error():
         worst = max(worst, float(abs(got - exact) / Fraction(2) ** (eu + eh)))
     assert worst < 2.0 ** -55
     assert worst > 0.0
+
+
+@pytest.mark.parametrize("kind", ["worst", "random"])
+def test_hop_error_with_projected_operands(kind):
+    """One colour sum of a hop with h = upper +- lower limb by limb, in units of
+    2^-56 of the largest product of entries: 3 for the six products of low
+    limbs, 1 for the two roundings, 3.75 for the rounding of the inputs.
+    worst: every low limb -2^29, so that the dropped products add up."""
+    rng = np.random.default_rng(11)
+    worst = 0
+    for _ in range(200):
+        hh = cross = 0
+        exact = Fraction(0)
+        u, up, lo = rng.uniform(-1, 1, 6), rng.uniform(-1, 1, 6), rng.uniform(-1, 1, 6)
+        u[0] = up[0] = 1 - 2.0 ** -53  # exponent 0 for all
+        for a, p, l in zip(u, up, lo):
+            na, np_, nl = to_int(a, 0, LINK_BITS), to_int(p, 0, SPINOR_BITS), to_int(l, 0, SPINOR_BITS)
+            if kind == "worst":
+                na, np_, nl = ((n >> LIMB << LIMB) - (1 << (LIMB - 1)) for n in (na, np_, nl))
+                exact += Fraction(na * (np_ + nl)) / 2 ** (LINK_BITS + SPINOR_BITS)
+            else:
+                exact += Fraction(float(a)) * (Fraction(float(p)) + Fraction(float(l)))
+            (ah, al), (ph, pl), (lh, ll) = split(na), split(np_), split(nl)
+            hh += ah * (ph + lh)
+            cross += ah * (pl + ll) + al * (ph + lh)
+        units = abs(Fraction(hh + ((cross + (1 << 29)) >> LIMB)) - exact * 2 ** 56)
+        worst = max(worst, units)
+        assert units <= (4 if kind == "worst" else 7.75)
+    if kind == "worst":
+        assert worst > 2.5  # the dropped products are there
