@@ -279,10 +279,13 @@ def run_reference(args, cfg):
 # FP64 hop: 1320 flops per site for the stencil (165 per hop) + 48 for the xpay term
 FP64_HOP_FLOPS = 1368
 FLOPS_PER_HOP = 165
-# one BiCGStab iteration of the persistent block solver, per block site (FP32):
-# two Dirichlet applications (1368 flops each at most) + the vector updates and
-# inner products (about 960 flops over the 12 complex components)
-BLOCK_ITER_FLOPS = 2 * FP64_HOP_FLOPS + 960
+# one BiCGStab iteration of the persistent block solver (block_eo_kernel, even-odd),
+# per block site (FP32): two even-odd Dirichlet operators, whose two half hops are
+# together one hop of every site (1320 flops at most), and on every other site the
+# operator's own term, the vector updates (s 8, x 16, r 8, p 16 flops a complex
+# component) and the sums (<rhat, v>, <rhat, t>, <t, s> 8 each, |t|^2, |s|^2 4 each):
+# 12 x (2 x 4 + 48 + 32) / 2
+BLOCK_ITER_FLOPS = 2 * 1320 + 528
 # unit counts and clock (152 SMs, 2070 MHz): FP64 2 FMA per SM per cycle,
 # FP32 128 FMA per SM per cycle -- the fallback when the live probe fails
 DERIVED_PEAKS = {"fp64_fma": 152 * 2 * 2 * 2.07e9 / 1e12, "fp32_fma": 152 * 128 * 2 * 2.07e9 / 1e12}
@@ -309,7 +312,7 @@ def kernel_models(block):
             FLOPS_PER_HOP * k, "site"),
         6: ("hop_eo_kernel FP16 -> FP32 + xpay, Dirichlet blocks, one colour's sites", "hbm", 52 + 24 * k + 96 + 96,
             48 + FLOPS_PER_HOP * k, "site"),
-        7: ("block_solve_kernel (persistent, FP32 BiCGStab + FP64 refinement)", "fp32", None, BLOCK_ITER_FLOPS,
+        7: ("block_eo_kernel (persistent, even-odd FP32 BiCGStab + refinement on integers)", "fp32", None, BLOCK_ITER_FLOPS,
             "block site x inner iteration"),
         8: ("hop_eo_kernel FP16 -> FP16, Dirichlet blocks, every site", "hbm", 52 + 24 * k + 52, FLOPS_PER_HOP * k,
             "site"),
