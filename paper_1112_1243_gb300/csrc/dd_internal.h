@@ -25,7 +25,7 @@ struct CGState {
     int maxit;     // cap
     int flags;     // bit 0: hit maxit, bit 1: non-finite
     // complex scalars of BiCGStab
-    double rho_re, rho_im, al_re, al_im, om_re, om_im, be_re, be_im, rv_re, rv_im;
+    double rho_re, rho_im, al_re, al_im, om_re, om_im, be_re, be_im;
     int last;      // the solve ended with x += alpha p + omega s still to be done
 };
 
@@ -39,7 +39,7 @@ enum FinOp {
     FIN_ZZ_INIT = 5,
     FIN_BI_RHO = 6,    // three values: <rh, r>, |r|^2 of the first residual
     FIN_BI_ALPHA = 7,  // two values: <rh, v>
-    FIN_BI_OMEGA = 8,  // six values: <t, s>, |t|^2, <rh, t>, |s|^2
+    FIN_BI_OMEGA = 8,  // eight values: <t, s>, |t|^2, <rh, t>, |s|^2, <rh, s>
     FIN_OUTER = 9      // |true residual|^2: stored, and the outer state updated
 };
 

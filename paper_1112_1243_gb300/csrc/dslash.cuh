@@ -89,7 +89,7 @@ struct HopArgs {
     const CGState* st;        // per-rhs activity (may be null)
     Reduce red;               // |out|^2 reduction (red.op == FIN_NONE: off)
     unsigned long long* sites;  // timed launches: output sites processed (may be null)
-    // BiCGStab's sums: 0 off; 1: <rhat, out>; 2: <out, xin>, |out|^2, <rh2, out> and |xin|^2
+    // BiCGStab's sums: 0 off; 1: <rhat, out>; 2: <out, xin>, |out|^2, <rh2, out>, |xin|^2 and <rh2, xin>
     int red3 = 0;
     SIn rh2;                    // red3 == 2: the shadow residual (hop storage)
     SX rhat;                    // red3 == 1: the shadow residual; resid: the right-hand side
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
     const long long tile = (long long)blockDim.x * SPT;
     if (A.sites && threadIdx.x == 0)
         atomicAdd(A.sites, (unsigned long long)min(tile, A.S.n - (long long)blockIdx.x * tile));
-    double v3[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    double v3[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     double nrm = 0.0;
 #pragma unroll
     for (int pass = 0; pass < SPT; ++pass) {
@@ -221,13 +221,15 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
         } else if (RED3 == 2) {
             Spinor<R> rv;
             at_rhs(A.rh2, rhs).load(h, rv);
-            R d0 = 0, d1 = 0, d2 = 0, d3 = 0;
+            R d0 = 0, d1 = 0, d2 = 0, d3 = 0, d4 = 0, d5 = 0;
 #pragma unroll
             for (int k = 0; k < 12; ++k) {
                 d0 += res.c[k].x * xv.c[k].x + res.c[k].y * xv.c[k].y;
                 d1 += res.c[k].x * xv.c[k].y - res.c[k].y * xv.c[k].x;
                 d2 += rv.c[k].x * res.c[k].x + rv.c[k].y * res.c[k].y;
                 d3 += rv.c[k].x * res.c[k].y - rv.c[k].y * res.c[k].x;
+                d4 += rv.c[k].x * xv.c[k].x + rv.c[k].y * xv.c[k].y;
+                d5 += rv.c[k].x * xv.c[k].y - rv.c[k].y * xv.c[k].x;
             }
             v3[0] += (double)d0;
             v3[1] += (double)d1;
@@ -235,12 +237,14 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
             v3[3] += (double)d2;
             v3[4] += (double)d3;
             v3[5] += (double)snorm2(xv);
+            v3[6] += (double)d4;
+            v3[7] += (double)d5;
         } else {
             nrm += (double)snorm2(res);
         }
     }
     if (RED3) {
-        grid_reduce_bi<RED3 == 1 ? 2 : 6>(A.red, rhs, v3);
+        grid_reduce_bi<RED3 == 1 ? 2 : 8>(A.red, rhs, v3);
     } else if (A.red.op != FIN_NONE) {
         grid_reduce(A.red, rhs, nrm);
     }

@@ -423,8 +423,9 @@ void plan(dd_handle* h, char* base) {
         s.nblk = (int)nblk;
         s.sc = c.take<double>(on ? (size_t)R * 4 * (DD_SAP_MAX_NKV + 4) : 0);
     }
-    // partials of grid reductions with tiles of 64 sites of one parity or more (6 values per tile)
-    h->partials_cap = (size_t)(grid_for(std::max(Vh, V), 64) + 64) * (R + 1) * 4;
+    // partials of grid reductions with tiles of 64 sites of one parity or more
+    // (8 values per tile, and per group of DD_REDUCE_GROUP tiles; V = 2 Vh)
+    h->partials_cap = (size_t)(grid_for(std::max(Vh, V), 64) + 64) * (R + 1) * 5;
     h->d_partials = c.take<double>(h->partials_cap);
     h->reduce_gmax = (int)((grid_for(std::max(Vh, V), 64) + 64 + DD_REDUCE_GROUP - 1) / DD_REDUCE_GROUP);
     h->d_counters = c.take<unsigned>(dd_counter_count(h));

@@ -73,7 +73,7 @@ DD_DEV void finish(const Reduce& R, int rhs, double s) {
     }
 }
 
-// BiCGStab finishers on two, three or six sums; complex scalars z = (re, im)
+// BiCGStab finishers on two, three or eight sums; complex scalars z = (re, im)
 DD_DEV void cdiv(double ar, double ai, double br, double bi, double& cr, double& ci) {
     double d = br * br + bi * bi;
     cr = (ar * br + ai * bi) / d;
@@ -121,8 +121,6 @@ DD_DEV void finish3(const Reduce& R, int rhs, const double* s) {
                 break;
             }
             cdiv(c.rho_re, c.rho_im, s[0], s[1], ar, ai);
-            c.rv_re = s[0];
-            c.rv_im = s[1];
             c.al_re = ar;
             c.al_im = ai;
             if (!isfinite(ar) || !isfinite(ai)) bicg_fail(R, c);
@@ -131,11 +129,13 @@ DD_DEV void finish3(const Reduce& R, int rhs, const double* s) {
         // omega = <t,s> / |t|^2, then everything of the next iteration that
         // the vector updates x += alpha p + omega s, r = s - omega t, p = r +
         // beta (p - omega v) need: |r|^2 = |s|^2 - 2 Re(conj(omega) <t,s>) +
-        // |omega|^2 |t|^2 and rho' = <rh,s> - omega <rh,t>, <rh,s> = rho -
-        // alpha <rh,v>, with alpha and omega as the updates take them
-        // (rounded to FP32).  The updates then need no sums of their own.
+        // |omega|^2 |t|^2 and rho' = <rh,s> - omega <rh,t>, with omega as the
+        // updates take it (rounded to FP32).  The updates then need no sums of
+        // their own.  <rh,s> is a sum of the vectors, not rho - alpha <rh,v>:
+        // rho then kept the rounding of every iteration before, and solves
+        // asked for 1e-7 and less in one cycle did not end.
         case FIN_BI_OMEGA: {
-            for (int k = 0; k < 6; ++k)
+            for (int k = 0; k < 8; ++k)
                 if (!isfinite(s[k])) {
                     bicg_fail(R, c, true);
                     return;
@@ -150,7 +150,6 @@ DD_DEV void finish3(const Reduce& R, int rhs, const double* s) {
                 bicg_fail(R, c);
                 break;
             }
-            const double ar = (double)(float)c.al_re, ai = (double)(float)c.al_im;
             const double wr = (double)(float)c.om_re, wi = (double)(float)c.om_im;
             c.rr = s[5] - 2.0 * (wr * s[0] + wi * s[1]) + (wr * wr + wi * wi) * s[2];
             c.iters += 1;
@@ -164,8 +163,8 @@ DD_DEV void finish3(const Reduce& R, int rhs, const double* s) {
                 c.flags |= 1;
                 break;
             }
-            const double nr = c.rho_re - (ar * c.rv_re - ai * c.rv_im) - (wr * s[3] - wi * s[4]);
-            const double ni = c.rho_im - (ar * c.rv_im + ai * c.rv_re) - (wr * s[4] + wi * s[3]);
+            const double nr = s[6] - (wr * s[3] - wi * s[4]);
+            const double ni = s[7] - (wr * s[4] + wi * s[3]);
             // beta = (rho' / rho) (alpha / omega)
             double qr, qi, er, ei;
             cdiv(nr, ni, c.rho_re, c.rho_im, qr, qi);

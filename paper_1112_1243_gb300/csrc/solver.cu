@@ -101,7 +101,7 @@ __global__ void cg_arm_kernel(int nrhs, CGState* st, const CGState* outer, const
     c.zz = c.qq = c.alpha = c.beta = 0.0;
     const double r0 = rr0 ? rr0[r] : 1.0;  // null: a right-hand side of unit norm
     c.rr = r0;
-    c.rho_re = c.rho_im = c.al_re = c.al_im = c.om_re = c.om_im = c.be_re = c.be_im = c.rv_re = c.rv_im = 0.0;
+    c.rho_re = c.rho_im = c.al_re = c.al_im = c.om_re = c.om_im = c.be_re = c.be_im = 0.0;
     c.last = 0;
     // relative target tol^2 |r0|^2, or a fraction of the outer absolute target.
     // A mixed inner solve is asked for no more than the outer loop still

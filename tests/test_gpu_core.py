@@ -212,3 +212,24 @@ def test_plaquette(api):
     U = synthetic.random_gauge(dims, 0.6, 8)
     got = float(host(api.dd_plaquette(h, dev(U)))[0])
     assert abs(got - heatbath.plaquette_mean(U, lat)) < 1e-14
+
+
+@pytest.mark.parametrize("dims,block,kappa,eps", [((8, 8, 8, 8), (4, 4, 4, 4), 0.13, 0.3),
+                                                  ((16, 16, 16, 16), (8, 8, 8, 8), 0.1355, 0.2)])
+@pytest.mark.parametrize("prec", ["f32", "f16"])
+@pytest.mark.parametrize("tol_inner", [1e-7, 1e-9])
+def test_bicgstab_of_long_inner_solves(api, dims, block, kappa, eps, prec, tol_inner):
+    """An inner target at the accuracy of FP32 and below: rho stays the inner
+    product of the vectors as they are, so that the iteration goes on to the
+    target (150 iterations at most are needed) or stops and restarts."""
+    precision = {"f32": api.DD_PREC_F32, "f16": api.DD_PREC_F16}[prec]
+    lat = geometry.Lattice(dims, block)
+    U = synthetic.random_gauge(dims, eps, 4)
+    b = synthetic.random_spinor(dims, 12)
+    h = api.dd_init(dims, block, kappa, max_rhs=1, inner_prec=precision, krylov=api.DD_KRYLOV_BICGSTAB,
+                    tol_inner=tol_inner, maxit=1000)
+    x = dev(np.zeros_like(b))
+    api.dd_solve(h, x, dev(b), dev(U), 1, precision)
+    res = np.linalg.norm(b - dirac.apply_D(U, host(x).reshape(b.shape), lat, kappa)) / np.linalg.norm(b)
+    assert res <= 1e-10 * 1.01
+    assert api.dd_status(h)[0] == 0
