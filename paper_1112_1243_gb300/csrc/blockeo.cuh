@@ -153,10 +153,10 @@ DD_DEV void df_acc(dfl& a, float t) {
     a.hi = s;
 }
 struct EoSums {
-    dfl v[6];  // Re, Im <rhat, out>; Re, Im <out, in>; |out|^2; |in|^2
+    dfl v[8];  // Re, Im <rhat, out>; Re, Im <out, in>; |out|^2; |in|^2; Re, Im <rhat, in>
 };
 
-// out = Dtilde in (th: odd temporary); with ALL all six sums, else the first
+// out = Dtilde in (th: odd temporary); with all all eight sums, else the first
 // two.  Every thread of the team calls this; in is complete, out is written
 // by the lanes that own its entries (no barrier at the end).
 DD_DEV void eo_dtilde(const EoCtx& c, const EoTeam& T, const float2* in, float2* th, float2* out, const float2* lk,
@@ -174,7 +174,7 @@ DD_DEV void eo_dtilde(const EoCtx& c, const EoTeam& T, const float2* in, float2*
     }
     T.sync();
 #pragma unroll
-    for (int k = 0; k < 6; ++k) S.v[k] = dfl{0.f, 0.f};
+    for (int k = 0; k < 8; ++k) S.v[k] = dfl{0.f, 0.f};
     for (int t0 = first; t0 < c.count; t0 += step) {
         EoSite s;
         const bool ok = eo_site(c, 0, t0 + (lane & 15), s);
@@ -194,6 +194,8 @@ DD_DEV void eo_dtilde(const EoCtx& c, const EoTeam& T, const float2* in, float2*
                 df_acc(S.v[3], o.x * x.y - o.y * x.x);
                 df_acc(S.v[4], o.x * o.x + o.y * o.y);
                 df_acc(S.v[5], x.x * x.x + x.y * x.y);
+                df_acc(S.v[6], h.x * x.x + h.y * x.y);
+                df_acc(S.v[7], h.x * x.y - h.y * x.x);
             }
         }
     }
@@ -201,9 +203,9 @@ DD_DEV void eo_dtilde(const EoCtx& c, const EoTeam& T, const float2* in, float2*
 
 constexpr int EO_CLUSTER = 8;  // thread blocks of a team
 struct EoShared {
-    dfl part[6][8];
-    double tot[6];
-    double all[EO_CLUSTER][6];  // the team's totals, by rank
+    dfl part[8][8];
+    double tot[8];
+    double all[EO_CLUSTER][8];  // the team's totals, by rank
     double sh[34];
     int ex[2][4][X_TILE], hs[2][X_TILE];
     int item;
@@ -260,8 +262,12 @@ DD_DEV double eo_sum(EoShared& M, const EoTeam& T, double v) {
 // ------------------------------------------------ BiCGStab on Dtilde (FP32)
 // x = 0, r holds the right-hand side.  Per iteration two operator
 // applications with their sums, one pass for s and one for x, r and p: rho
-// of the next iteration follows from <rhat, t> and |r|^2 from |s|^2, <t, s>
-// and |t|^2, so the vector updates need no sums of their own.  Stops when
+// of the next iteration follows from <rhat, s> and <rhat, t>, |r|^2 from
+// |s|^2, <t, s> and |t|^2, so the vector updates need no sums of their own.
+// (<rhat, s> carried on as rho - alpha <rhat, v> kept the rounding of all
+// iterations: near the critical mass, 8^4 blocks at kappa 0.16, some solves
+// ran to their cap of 2000 iterations where 40 are enough.  The two sums more
+// cost 4%: batch of 4^4, 6^4 and 8^4 blocks 15.06 -> 15.72 ms.)  Stops when
 // |r|^2 <= tol2rel |r0|^2, after maxit iterations or at a breakdown (the
 // refinement around it restarts from the true residual).
 struct EoVecs {
@@ -287,12 +293,12 @@ DD_DEV int eo_bicgstab(const EoCtx& c, const EoTeam& T, EoShared& M, const EoVec
         df_acc(rr0, r.x * r.x + r.y * r.y);
     });
     S.v[0] = rr0;
-    double d[6];
+    double d[8];
     eo_total(M, T, S, 1, d);
     if (!(d[0] > 0.0)) return 0;
     T.sync();  // p complete
     const double target = tol2rel * d[0];
-    cpx<double> rho = mk<double>(d[0], 0.0), alpha = mk<double>(0.0, 0.0), rv = alpha;
+    cpx<double> rho = mk<double>(d[0], 0.0), alpha = mk<double>(0.0, 0.0);
     cpx<float> aR = mk<float>(0.f, 0.f);
     int it = 0;
     // two passes an iteration, v = Dtilde p and t = Dtilde s, with one copy
@@ -300,9 +306,9 @@ DD_DEV int eo_bicgstab(const EoCtx& c, const EoTeam& T, EoShared& M, const EoVec
 #pragma unroll 1
     for (bool second = false; second || it < maxit; second = !second) {
         eo_dtilde(c, T, second ? V.s : V.p, V.th, second ? V.t : V.v, lk, V.rhat, second, S);
-        eo_total(M, T, S, second ? 6 : 2, d);
+        eo_total(M, T, S, second ? 8 : 2, d);
         if (!second) {
-            rv = mk<double>(d[0], d[1]);
+            const cpx<double> rv = mk<double>(d[0], d[1]);
             if (!(norm2(rv) > 0.0)) break;
             alpha = (1.0 / norm2(rv)) * cmul(rho, conj(rv));
             aR = mk<float>((float)alpha.x, (float)alpha.y);
@@ -320,9 +326,9 @@ DD_DEV int eo_bicgstab(const EoCtx& c, const EoTeam& T, EoShared& M, const EoVec
         const bool stop_s = !(tt > 0.0) || ss <= target;  // s is the residual: x += alpha p
         const cpx<double> omega = stop_s ? mk<double>(0.0, 0.0) : (1.0 / tt) * ts;
         const cpx<float> wR = mk<float>((float)omega.x, (float)omega.y);
-        const cpx<double> ad = mk<double>((double)aR.x, (double)aR.y), wd = mk<double>((double)wR.x, (double)wR.y);
+        const cpx<double> wd = mk<double>((double)wR.x, (double)wR.y);
         const double rr = ss - 2.0 * (wd.x * ts.x + wd.y * ts.y) + norm2(wd) * tt;
-        const cpx<double> rho_new = (rho - cmul(ad, rv)) - cmul(wd, rt);
+        const cpx<double> rho_new = mk<double>(d[6], d[7]) - cmul(wd, rt);
         cpx<double> beta = mk<double>(0.0, 0.0);
         bool last = stop_s || !(rr > target) || !(norm2(omega) > 0.0) || !(norm2(rho_new) > 0.0);
         if (!last) {

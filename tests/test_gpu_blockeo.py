@@ -100,3 +100,24 @@ def test_source_of_small_rotations(api):
     got = host(api.dd_block_ratios_range(h, dev(U), dev(Up), 0, lat.nblocks, 1, 9, 3))
     assert np.all(np.abs(got - ref) <= tol)
     assert api.dd_status(h)[0] == 0
+
+
+def test_no_item_runs_to_its_iteration_cap(api):
+    """Blocks of 8^4 near the critical mass: an inner solve whose rho has lost
+    its accuracy goes on to its cap of 2000 iterations, as many as all 16 items
+    of a launch need together.  Launches with other noise vectors therefore
+    differ by far less than half of their iterations."""
+    dims, block, kappa = (16, 16, 16, 16), (8, 8, 8, 8), 0.16
+    U = dev(synthetic.random_gauge(dims, 0.2, 4))
+    Up = U.clone()
+    h = api.dd_init(dims, block, kappa, max_rhs=1)
+    api.dd_gauge_update(h, Up, 3, 5.3, 1, 0, 21, 4)
+    its = []
+    for ctr in range(12):
+        api.dd_kernel_timer(h, 1, 0, 1)
+        got = host(api.dd_block_ratios_range(h, U, Up, 0, 16, 1, 9, ctr))
+        st = api.dd_solver_stats(h, 2)
+        assert np.all(np.isfinite(got)) and st["items"] == 16
+        its.append(st["inner_iterations"])
+    assert max(its) < 1.5 * min(its), its
+    assert api.dd_status(h)[0] == 0
