@@ -15,8 +15,9 @@
 // residual's stencil, the source from two FP64 links a hop, the noise.  Here
 // the stencils are integer, sums are kept as pairs of FP32 numbers (48 bits)
 // until the block has one, and only the noise, the vector updates of the
-// refinement and the final sum are FP64.  4^4: 1024 items 8.0 -> 4.7
-// ms (noise 13%, source 16%, FP32 iterations 53%, refinement 14%).
+// refinement, the differences of links and the final sum are FP64.  4^4: 1024
+// items 8.0 -> 4.7 ms (noise 9%, source 18%, FP32 iterations 53%, refinement
+// 17%; at 25% of its issue slots, 15 warps an SM waiting for L2 and barriers).
 //
 // Vectors live in the thread block's scratch slot, component-major (component
 // k of site i at [k * half + i]); FP32 work runs two lanes a site, lane pair
@@ -147,6 +148,8 @@ DD_DEV void hops32(const EoCtx& c, bool ok, int par, const EoSite& s, int sp, co
 DD_DEV int lane_comp(int sp, int k) { return k < 3 ? 3 * sp + k : 3 + 3 * sp + k; }
 
 // sums over the lanes' sites kept as (hi, lo) pairs of FP32 numbers
+// (a CPU model of the sums at 4^4, 6^4 and 8^4: the bits of FP64 sums of the
+// same FP32 products, whose own rounding leaves 1e-9 of the summed terms)
 DD_DEV void df_acc(dfl& a, float t) {
     const float s = a.hi + t, bb = s - a.hi;
     a.lo += (a.hi - (s - bb)) + (t - bb);

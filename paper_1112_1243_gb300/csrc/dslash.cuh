@@ -260,8 +260,9 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 0)
 // a chain of 4000 instructions: with all hops in one lane (128 registers, 16
 // warps an SM) 2^20 sites took 537 us, 128 sites 21 us; here 508 and 10 us
 // (8 x 16384 sites: 28 -> 15 us).  Two lanes a site with one spin each took
-// 2.5 times the instructions and 830 us.  At 2^20 sites what is left is
-// latency: 20 warps an SM (96 registers), DRAM at 45%, issue slots at 32%.
+// 2.5 times the instructions and 830 us.  What is left is latency: 20 warps
+// an SM (96 registers); at 2^19 sites DRAM at 50% and issue slots at 40% with
+// out in limbs, 41% and 29% in the residual form.
 
 // sum kept as a pair of FP64 numbers
 struct Pair64 {
